@@ -123,7 +123,7 @@ KParams params(labs_ctx* c)
     p.target_num = c->cfg.target_num;
     p.target_den = c->cfg.target_den;
     p.chunk_steps = c->chunk;
-    p.rmax = c->long_mode ? long_R(c->n_max, c->tile) : lanes_for(c->n_max, c->tile);
+    p.rmax = c->long_mode ? long_R(c->n_max, c->tile) : 0;
     p.tile = c->tile;
     p.long_mode = c->long_mode ? 1 : 0;
     p.cur_bits = c->long_mode ? at<uint32_t>(c, c->off_cur_bits) : nullptr;
@@ -133,7 +133,10 @@ KParams params(labs_ctx* c)
     p.pq_key = p.best_first ? at<uint64_t>(c, c->off_pq_key) : nullptr;
     p.pq_bits = p.best_first ? at<uint32_t>(c, c->off_pq_bits) : nullptr;
     p.tabu2 = (c->cfg.flags & LABS_FLAG_SECOND_HASH) ? at<uint64_t>(c, c->off_tabu2) : nullptr;
-    p.mode = (c->cfg.flags & LABS_FLAG_PSL) ? 3 : p.best_first ? 2 : (c->l_params ? 1 : 0);
+    // the restart-only learned mode keeps the plain walk's kernels
+    p.mode = (c->cfg.flags & LABS_FLAG_PSL) ? 3
+             : p.best_first                 ? 2
+             : c->l_params && (c->cfg.flags & LABS_FLAG_LEARNED) ? 1 : 0;
     return p;
 }
 
@@ -163,7 +166,7 @@ int walker_bits(labs_ctx* c, int64_t w, const WalkerState& ws, bool best, uint32
 int launch_chunk(labs_ctx* c, const KParams& p, int j, cudaStream_t stream)
 {
     if (c->long_mode) return launch_long_walk_chunk(p, j, c->grid, c->smem_bytes, stream);
-    return launch_walk_chunk(p, j, c->grid, c->warps_per_cta, c->smem_bytes, stream);
+    return launch_walk_chunk(p, j, c->grid, c->warps_per_cta, stream);
 }
 
 int need_ws(labs_ctx* c)
@@ -298,15 +301,13 @@ int setup(labs_ctx* c, const int32_t* Ls, const int64_t* counts, int32_t nL, uin
         off = align_up(off + sizeof(uint64_t) * ((size_t)c->W << k.tabu_log2), 256);
     }
     c->total = off;
-    // launch shape of the walk kernel: four walkers per warp (8 lanes each) while 8
-    // lanes cover n with at most kQuadMaxR outputs per lane (n <= 80; measured faster
-    // than two per warp there, equal from n = 88 to 104), two walkers per warp (16 lanes
-    // each, the Toeplitz product on the tensor cores) up to n = 128, else one walker per
-    // warp (tensor-core product; measured 7-12% faster than two walkers per warp with the
-    // FP32 product from n = 129 to 160, which LABS_FLAG_TWO_PER_WARP keeps; the learned
-    // mode and the best-first search run one walker per warp).  The PSL objective runs
-    // two walkers per warp up to n = 128 (LABS_FLAG_WARP_PER_WALKER: one per warp), one
-    // above.
+    // launch shape of the walk kernel (16384 walkers, Gflips/s, both sides measured): four
+    // walkers per warp (8 lanes each) while 8 lanes cover n with at most kQuadMaxR outputs
+    // per lane (n <= 80: L = 101 194 against 152 with two per warp, L = 151 229 against
+    // 226); two per warp (16 lanes each) up to n = 160 (L = 303 253 against 212 with one
+    // per warp; above, two walkers' shared memory leaves an SM too few warps); one above.
+    // The learned mode and the best-first search run one walker per warp, the PSL objective
+    // two up to n = 128 (LABS_FLAG_WARP_PER_WALKER: one) and one above.
     if (c->long_mode) {
         // one walker per CTA of 256 or 512 threads
         c->tile = long_threads(c->n_max, (k.flags & LABS_FLAG_PSL) != 0);
@@ -326,21 +327,21 @@ int setup(labs_ctx* c, const int32_t* Ls, const int64_t* counts, int32_t nL, uin
         if (psl)
             c->tile = c->n_max <= 128 && !(k.flags & LABS_FLAG_WARP_PER_WALKER) ? 16 : 32;
         else if ((k.flags & (LABS_FLAG_WARP_PER_WALKER | LABS_FLAG_LEARNED | LABS_FLAG_BEST_FIRST)) ||
-                 lanes_for(c->n_max, 16) > 10 || (c->n_max > 128 && !(k.flags & LABS_FLAG_TWO_PER_WARP)))
+                 c->n_max > 160)
             c->tile = 32;
-        else if (!(k.flags & LABS_FLAG_TWO_PER_WARP) && lanes_for(c->n_max, 8) <= kQuadMaxR)
+        else if (!(k.flags & LABS_FLAG_TWO_PER_WARP) && block_R(c->n_max, 8) <= kQuadMaxR)
             c->tile = 8;
         else
             c->tile = 16;
-        const size_t per_warp = (size_t)warp_smem(c->n_max, c->tile, psl).words * sizeof(int) * (kWarp / c->tile);
         int warps = k.warps_per_cta ? k.warps_per_cta : 8;
         for (;;) {
-            c->smem_bytes = per_warp * (size_t)warps;
-            int occ = 0;
-            const int mode = (k.flags & LABS_FLAG_PSL) ? 3 : (k.flags & LABS_FLAG_BEST_FIRST) ? 2 : 0;
-            if (walk_kernel_config(c->tile, lanes_for(c->n_max, c->tile), mode, warps, c->smem_bytes, &occ,
-                                   &c->regs) == LABS_OK &&
-                occ > 0) {
+            int occ = 0, occ_l = 1, regs_l = 0;
+            const int mode = psl ? 3 : (k.flags & LABS_FLAG_BEST_FIRST) ? 2 : 0;
+            int rc = walk_kernel_config(c->n_max, c->tile, mode, warps, &occ, &c->regs);
+            // the learned mode is switched on and off at run time
+            if (rc == LABS_OK && (k.flags & LABS_FLAG_LEARNED))
+                rc = walk_kernel_config(c->n_max, c->tile, 1, warps, &occ_l, &regs_l);
+            if (rc == LABS_OK && occ > 0 && occ_l > 0) {
                 c->ctas_per_sm = occ;
                 break;
             }
@@ -862,9 +863,13 @@ int labs_stats(labs_ctx* c, int32_t L, labs_counters* out)
     out->cache_hits = (int64_t)h.st_cache_hits;
     out->walkers_at_target = (int64_t)h.st_at_target;
     out->walkers_per_warp = kWarp / c->tile;  // 0 for long sequences: one walker per CTA
-    out->lane_block = c->long_mode ? long_R(c->n_max, c->tile) : lanes_for(c->n_max, c->tile);
-    out->tensor_cores = (c->long_mode ? long_smem(c->n_max, c->tile).xp
-                                      : warp_smem(c->n_max, c->tile, (c->cfg.flags & LABS_FLAG_PSL) != 0).xp) != 0;
+    const KParams kp = params(c);
+    out->lane_block = c->long_mode   ? long_R(c->n_max, c->tile)
+                      : kp.mode == 0 ? step_R(c->n_max, c->tile)
+                                     : block_R(c->n_max, c->tile);
+    out->tensor_cores = c->long_mode   ? long_smem(c->n_max, c->tile).xp != 0
+                        : kp.mode == 0 ? 1
+                                       : warp_smem(c->n_max, c->tile, kp.mode == 3).xp != 0;
     out->target_step = h.st_target_step == LLONG_MAX ? -1 : (int64_t)h.st_target_step;
     out->best_psl = -1;
     if (h.best_key == ~0ull) {

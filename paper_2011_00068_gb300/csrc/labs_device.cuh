@@ -1283,8 +1283,6 @@ template <class LG, int R, class E>
 __device__ __forceinline__ int lane_dlb_rows(const E* A, const View& V, int n, const Outs<LG, R>& o,
                                              const float (&X)[R], const float (&P)[R], uint32_t (&db)[R])
 {
-    // four walkers per warp: the rows are not padded for the missing outputs' reads
-    constexpr bool kGuard = LG::kSize == 8;
     const int p = o.p, c = n - 1;
     const int rv = (p ? (n >> 1) : ((n + 1) >> 1)) - o.v0;
     const int rc = (c & 1) == p ? ((c - p) >> 1) - o.v0 : -1;  // the centre's r, if this lane has it
@@ -1295,9 +1293,8 @@ __device__ __forceinline__ int lane_dlb_rows(const E* A, const View& V, int n, c
     const float2* Gc = V.G + (c - p - 2 * o.v0);   // C_{q-i}      = Gc[-2r].x
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const bool ok = !kGuard || r < rv;
         const float av = row_value(Av[r]), sq = row_value(Aq[-r]);
-        const float ck0 = ok ? Gc[-2 * r].x : 0.f, st = ok ? row_value(At[3 * r]) : 0.f;
+        const float ck0 = Gc[-2 * r].x, st = row_value(At[3 * r]);
         const bool ctr = r == rc;
         // every partial sum is an integer of magnitude below 2^24: exact
         const float add = ctr ? cbase : fmaf(32.f, fmaf(-sq, st, P[r]), base);
@@ -1408,7 +1405,6 @@ template <class LG, int R>
 __device__ __forceinline__ void apply_flip(const View& V, int n, const Outs<LG, R>& o, int lane, bool moves,
                                            int best_i, float (&P)[R])
 {
-    constexpr bool kQuad = LG::kSize == 8;
     const int c = n - 1;
     const int m0 = 1 + lane * R;  // this lane's lags 2m of the update, m = m0 .. m0+R-1
     const int pb = best_i & 1, vb = best_i >> 1;
@@ -1430,9 +1426,8 @@ __device__ __forceinline__ void apply_flip(const View& V, int n, const Outs<LG, 
     {
         const float* up = Ab + vb + m0;
         const float* dn = Ab + vb - m0;
-        const int ku = kQuad ? (pb ? n - 1 : n) - vb - m0 : R;  // s_{i+2m} inside the class for k < ku
 #pragma unroll
-        for (int k = 0; k < R; ++k) dd[k] = coef * ((k < ku ? up[k] : 0.f) + dn[-k]);
+        for (int k = 0; k < R; ++k) dd[k] = coef * (up[k] + dn[-k]);
     }
     // P_v of the moved class: each pair (v+m, v-m) with exactly one flipped end
     // changes by -2 x its old product; the partner of w is 2v - w
@@ -1458,12 +1453,10 @@ __device__ __forceinline__ void apply_flip(const View& V, int n, const Outs<LG, 
 #pragma unroll
         for (int k = 0; k + 1 < R; ++k) V.G[m0 + k] = make_float2(e[k], e[k + 1]);
         V.G[m0 + R - 1].x = e[R - 1];
-        if (!kQuad || m0 + R <= V.gpad) {
-            V.G[-m0].x = e[0];
+        V.G[-m0].x = e[0];
 #pragma unroll
-            for (int k = 0; k + 1 < R; ++k) V.G[-m0 - k - 1] = make_float2(e[k + 1], e[k]);
-            V.G[-m0 - R].y = e[R - 1];
-        }
+        for (int k = 0; k + 1 < R; ++k) V.G[-m0 - k - 1] = make_float2(e[k + 1], e[k]);
+        V.G[-m0 - R].y = e[R - 1];
     }
     __syncwarp();
     if (moves && lane == 0) {
@@ -1481,200 +1474,6 @@ __device__ __forceinline__ int target_isl(const KParams& p, int L)
 
 // Outcome of probing HT for a candidate.
 enum : int { kProbeFree = 0, kProbeVisited = 1, kProbeUnknown = 2, kProbeNone = 3 };
-
-// TC: the Toeplitz product on the tensor cores (two walkers per warp): 0 never, 1 always,
-// 2 when the layout holds the FP16 rows (n_max <= 128).
-template <class LG, class RT, int R, int TC = 0>
-__device__ void walk_lockstep(const WalkEnv& env, Walker& w, int64_t until, bool real, int* base, const WarpSmem& SL,
-                              const View& V, int trace_slot, int64_t trace_start, labs_log_record* rec, const LG& t,
-                              const RT& tt)
-{
-    constexpr int S = LG::kSize / 2;            // HT slots probed per candidate in a round
-    constexpr unsigned SM = (1u << S) - 1u;
-    const KParams& p = *env.p;
-    const int lane = t.lane, n = env.n;
-    const Outs<LG, R> o(t);
-    const int cap = p.probe_cap;
-    const uint32_t tmask = (uint32_t)env.tmask;  // HT slots <= 2^20
-    // ISL at or below which the target merit factor is met (-1: no target)
-    const int tisl = target_isl(p, env.L);
-    float P[R];
-    p_direct(V, n, o, P);
-    const int64_t first_step = w.steps;
-    int log_first = 0, log_min = w.isl;
-    bool log_live = true;
-    int prev = -1;  // the last flip since the walker's (re)start in this call, or -1
-    StopCheck stop;
-    stop.start(p, (threadIdx.x & 31) == 0);
-    if (real && rec != nullptr) {
-        if (lane < kBitWords) rec->bits[lane] = w.word;
-        if (lane == 0) {
-            rec->isl = w.isl;
-            rec->L = env.L;
-            rec->walker = env.g;
-            rec->step = w.steps;
-        }
-    }
-    for (;;) {
-        const bool act = real && w.steps < until;
-        if (!__any_sync(kFull, act)) break;
-        if (__any_sync(kFull, act && (w.steps & (kCheckEvery - 1)) == 0)) {
-            const int why = __shfl_sync(kFull, stop.poll(p, (threadIdx.x & 31) == 0), 0);
-            if (why) {
-                if (act && lane == 0) raise_error(p.status, why, (int)env.g);
-                break;
-            }
-        }
-        unsigned key[R];
-        {
-            float X[R];
-            if constexpr (TC == 1) {
-                toeplitz_tc(V, SL, n, o, t.h, X);
-            } else if constexpr (TC == 2) {
-                if (SL.xp)
-                    toeplitz_tc(V, SL, n, o, t.h, X);
-                else
-                    toeplitz_one(V, SL, n, o, t, X);
-            } else {
-                toeplitz_one(V, SL, n, o, t, X);
-            }
-            lane_keys(V, n, o, X, P, key);
-            drop_candidate(key, prev, o, 0xFFFFFFFFu);
-        }
-
-        // Best admissible flip, as in walk_steps: candidates in ascending key order, two
-        // per round, the first S HT slots of each probed by one half of the walker's
-        // lanes; keys <= floor are known to lead to visited states.
-        unsigned floor = 0u, kc = 0xFFFFFFFFu;
-        int slot = -1;
-        uint64_t fnew = 0;
-        bool done = !act;
-        do {
-            unsigned b1, b2;
-            top2_above(key, floor, b1, b2);
-            const unsigned k0 = t.rminu(done ? 0xFFFFFFFFu : b1);
-            const unsigned k1 = t.rminu(done ? 0xFFFFFFFFu : (b1 == k0 ? b2 : b1));
-            const bool has0 = k0 != 0xFFFFFFFFu, has1 = k1 != 0xFFFFFFFFu;
-            const uint64_t f0 = w.fp ^ (has0 ? __ldg(env.zk + (k0 & 0xFFu)) : 0ull);
-            const uint64_t f1 = w.fp ^ (has1 ? __ldg(env.zk + (k1 & 0xFFu)) : 0ull);
-            const int hs = lane & (S - 1);
-            const bool second = lane >= S;
-            const uint64_t f = second ? f1 : f0;
-            const bool live = !done && (second ? has1 : has0) && hs < cap;
-            uint64_t e = 0;
-            if (live) e = env.T[((uint32_t)f + (uint32_t)hs) & tmask];
-            const bool match = live && e == ((f & ~kGenMask) | w.gen);
-            const bool hit = live && ((((uint32_t)e & (uint32_t)kGenMask) != w.gen) || match);
-            const unsigned hb = t.ballot(hit), mb = t.ballot(match);
-            const unsigned h0 = hb & SM, h1 = (hb >> S) & SM;
-            int st0 = !has0 ? kProbeNone
-                            : h0 ? ((mb & h0 & (0u - h0)) ? kProbeVisited : kProbeFree)
-                                 : (cap > S ? kProbeUnknown : kProbeFree);
-            int st1 = !has1 ? kProbeNone
-                            : h1 ? (((mb >> S) & h1 & (0u - h1)) ? kProbeVisited : kProbeFree)
-                                 : (cap > S ? kProbeUnknown : kProbeFree);
-            // the slot of a candidate's first hit (its insertion slot when it is free) is
-            // taken below for the candidate chosen; a full probe supplies its own
-            int s0 = -2, s1 = -2;
-            // chains longer than S slots (rare): full probes, of the second candidate only
-            // when the first leads to a visited state
-            const bool need0 = !done && st0 == kProbeUnknown;
-            if (__any_sync(kFull, need0)) {
-                const Probe pf = lockstep_probe_full(env, f0, w.gen, cap, need0, t);
-                if (need0) {
-                    st0 = pf.visited ? kProbeVisited : kProbeFree;
-                    s0 = (int)pf.slot;
-                }
-            }
-            const bool need1 = !done && st0 == kProbeVisited && st1 == kProbeUnknown;
-            if (__any_sync(kFull, need1)) {
-                const Probe pf = lockstep_probe_full(env, f1, w.gen, cap, need1, t);
-                if (need1) {
-                    st1 = pf.visited ? kProbeVisited : kProbeFree;
-                    s1 = (int)pf.slot;
-                }
-            }
-            if (!done) {
-                if (st0 == kProbeFree) {
-                    kc = k0, fnew = f0, done = true;
-                    slot = s0 != -2 ? s0 : (h0 ? (int)(((uint32_t)f0 + (uint32_t)(__ffs(h0) - 1)) & tmask) : -1);
-                } else if (st0 == kProbeNone || st1 == kProbeNone) {
-                    done = true;  // every neighbour is in HT
-                } else if (st1 == kProbeFree) {
-                    kc = k1, fnew = f1, done = true;
-                    slot = s1 != -2 ? s1 : (h1 ? (int)(((uint32_t)f1 + (uint32_t)(__ffs(h1) - 1)) & tmask) : -1);
-                } else {
-                    floor = k1;
-                }
-            }
-        } while (__any_sync(kFull, !done));
-
-        // Apply the move (walkers that have one), from the values before the flip.
-        const bool moves = act && kc != 0xFFFFFFFFu;
-        const int best_i = moves ? (int)(kc & 0xFFu) : 0, best_d = (int)(kc >> 8) - kKeyBias;
-        apply_flip<LG, R>(V, n, o, lane, moves, best_i, P);
-        const bool stored = slot >= 0;
-        if (moves && lane == 0 && stored) env.T[slot] = (fnew & ~kGenMask) | w.gen;
-        if (moves && lane == (best_i >> 5)) w.word ^= 1u << (best_i & 31);
-        __syncwarp();
-        int code = 0;
-        bool again = false;
-        if (act) {
-            w.steps += 1;
-            if (!moves) {
-                w.blocked += 1;
-                again = true;
-                code = LABS_TRACE_BLOCKED;
-            } else {
-                w.fp = fnew;
-                w.isl += best_d;
-                if (!stored) w.overflows += 1;
-                if (w.isl < w.best_isl) {
-                    w.best_isl = w.isl;
-                    w.best_step = w.steps;
-                    if (lane < kBitWords) env.st->best[lane] = w.word;
-                }
-                if (w.target_step < 0 && w.isl <= tisl) w.target_step = w.steps;
-                if (w.isl < w.since) {
-                    w.since = w.isl;
-                    w.stag = 0;
-                } else {
-                    w.stag += 1;
-                }
-                code = best_i;
-                if (w.stag >= env.patience || !stored) {
-                    again = true;
-                    code |= LABS_TRACE_RESTART;
-                }
-            }
-        }
-        if (moves) prev = best_i;
-        if (again) {  // two walkers per warp: divergent, only this half restarts
-            restart_walker(env, w, base, SL, V, tt);
-            p_direct(V, n, o, P);
-            prev = -1;
-        }
-        __syncwarp();
-        if (act) {
-            if (trace_slot >= 0 && lane == 0) {
-                const int64_t s = w.steps - 1 - trace_start;
-                if (s >= 0 && s < p.status->trace_capacity) {
-                    p.status->trace_code[trace_slot * p.status->trace_capacity + s] = code;
-                    p.status->trace_isl[trace_slot * p.status->trace_capacity + s] = w.isl;
-                }
-            }
-            if (rec != nullptr && log_live) {
-                if (w.steps == first_step + 1) log_first = code;
-                if (code == LABS_TRACE_BLOCKED || (code & LABS_TRACE_RESTART)) log_live = false;
-                else log_min = min(log_min, w.isl);
-            }
-        }
-    }
-    if (real && rec != nullptr && lane == 0) {
-        rec->first = log_first;
-        rec->min_isl = log_min;
-    }
-}
 
 // ------------------------------------------------------------- best-first search
 //
@@ -2421,18 +2220,6 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
         env.rdump_count = nullptr;
         env.dump_cap = 0;
         DevStatus* S = p.status;
-        if (MODE == 0 && S->learned) {
-            // restart-only learned mode: the proposed restart state, and its record for
-            // a traced walker
-            env.slot = S->l_slot + wi * kBitWords;
-            env.slot_valid = S->l_slot_valid + wi;
-            if (trace_slot >= 0 && S->d_restart != nullptr) {
-                env.rdump = S->d_restart + (int64_t)trace_slot * S->d_cap * kBitWords;
-                env.rdump_idx = S->d_restart_idx + (int64_t)trace_slot * S->d_cap;
-                env.rdump_count = S->d_restart_count + trace_slot;
-                env.dump_cap = S->d_cap;
-            }
-        }
         if (MODE == 1 && S->learned) {
             env.slot = S->l_slot + wi * kBitWords;
             env.slot_valid = S->l_slot_valid + wi;
@@ -2458,8 +2245,7 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
                 if (idx < S->log_capacity) ex.rec = S->log + idx;
             }
         }
-        // the learned mode's step (walk_steps), the best-first search, or the lockstep
-        // step of the plain walk
+        // the learned mode's step (walk_steps), the best-first search or the PSL walk
         constexpr int R2 = RMAX > 2 ? RMAX - 2 : 1;
         const bool full = RMAX <= 2 || block_R(G.n, TILE) >= RMAX;
         if constexpr (MODE == 3) {
@@ -2487,18 +2273,11 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
                 walk_bestfirst<RMAX>(env, w, until, base, SL, V, trace_slot, trace_start, t, qk, qb);
             else
                 walk_bestfirst<R2>(env, w, until, base, SL, V, trace_slot, trace_start, t, qk, qb);
-        } else if constexpr (MODE == 1) {
+        } else {
             if (full)
                 walk_steps<Tile<TILE>, RMAX>(env, w, until, base, SL, V, trace_slot, trace_start, ex, t);
             else
                 walk_steps<Tile<TILE>, R2>(env, w, until, base, SL, V, trace_slot, trace_start, ex, t);
-        } else {
-            if (full)
-                walk_lockstep<Tile<TILE>, Tile<TILE>, RMAX>(env, w, until, true, base, SL, V, trace_slot, trace_start,
-                                                            ex.rec, t, t);
-            else
-                walk_lockstep<Tile<TILE>, Tile<TILE>, R2>(env, w, until, true, base, SL, V, trace_slot, trace_start,
-                                                          ex.rec, t, t);
         }
         save_walker(st, w, t.lane);
         t.sync();
@@ -2506,17 +2285,16 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
 }
 
 
-// Walk launch with WPW = 32 / LG::kSize walkers per warp (two for n <= 160, four for
-// short sequences): the warp takes WPW consecutive walkers; when their lengths differ
-// (a group boundary) or fewer are left, it runs them one after the other with the other
-// lane groups idle.  RT is the tile type a lane group restarts with (divergently).
-// MODE 0: the plain walk; 3: the walk under the PSL objective (two walkers per warp).
-template <class LG, class RT, int RMAX, int MODE = 0>
-__device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
+// PSL walk with WPW = 32 / LG::kSize (two) walkers per warp: the warp takes WPW consecutive
+// walkers; when their lengths differ (a group boundary) or fewer are left, it runs them
+// one after the other with the other lane group idle.  RT is the tile type a lane group
+// restarts with (divergently).
+template <class LG, class RT, int RMAX>
+__device__ __forceinline__ void walk_psl_group(const KParams& p, int chunk_index)
 {
     constexpr int WPW = 32 / LG::kSize;
     extern __shared__ __align__(16) int smem[];
-    const WarpSmem SL = warp_smem(p.n_max, LG::kSize, MODE == 3);
+    const WarpSmem SL = warp_smem(p.n_max, LG::kSize, true);
     const LG t(threadIdx.x & 31);
     const RT tt(threadIdx.x & 31);
     int* base = smem + (threadIdx.x / LG::kSize) * SL.words;
@@ -2562,18 +2340,6 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
             int64_t until = min(target, steps_done + (int64_t)p.chunk_steps);
             bool real = real0 && steps_done < until;
             const int trace_slot = real ? env.st->trace_slot : -1;
-            if (MODE == 0 && real && S->learned) {
-                // restart-only learned mode: the proposed restart state (and its record
-                // for a traced walker)
-                env.slot = S->l_slot + mine_w * kBitWords;
-                env.slot_valid = S->l_slot_valid + mine_w;
-                if (trace_slot >= 0 && S->d_restart != nullptr) {
-                    env.rdump = S->d_restart + (int64_t)trace_slot * S->d_cap * kBitWords;
-                    env.rdump_idx = S->d_restart_idx + (int64_t)trace_slot * S->d_cap;
-                    env.rdump_count = S->d_restart_count + trace_slot;
-                    env.dump_cap = S->d_cap;
-                }
-            }
             const int64_t trace_start = trace_slot >= 0 ? p.trace_start[trace_slot] : 0;
             const int isl = load_rows(base, SL, V, w.word, G.L, G.n, t);
             if (real && isl != w.isl) {
@@ -2581,22 +2347,12 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
                 real = false;
             }
             PslTrack ps;
-            if constexpr (MODE == 3) {
-                ps.psl = table_psl(V, G.n, t);
-                ps.best_psl = env.st->best_psl;
-                ps.since_psl = env.st->since_psl;
-                if (real && ps.psl != env.st->psl) {
-                    if (t.lane == 0) raise_error(p.status, LABS_ESTATE, (int)mine_w);
-                    real = false;
-                }
-            }
-            labs_log_record* rec = nullptr;
-            if (MODE == 0 && real && S->log != nullptr && p.chunk_steps > 0) {
-                const int64_t since = steps_done - S->log_start;
-                if (since >= 0 && since % p.chunk_steps == 0) {
-                    const int64_t idx = (since / p.chunk_steps) * p.W + mine_w;
-                    if (idx < S->log_capacity) rec = S->log + idx;
-                }
+            ps.psl = table_psl(V, G.n, t);
+            ps.best_psl = env.st->best_psl;
+            ps.since_psl = env.st->since_psl;
+            if (real && ps.psl != env.st->psl) {
+                if (t.lane == 0) raise_error(p.status, LABS_ESTATE, (int)mine_w);
+                real = false;
             }
             // lane block: block_R(n) when it is one of RMAX .. RMAX-3, else the smallest
             // bank-conflict-free one of those.  Two walkers per warp take the Toeplitz
@@ -2605,41 +2361,23 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
             constexpr int TC = LG::kSize != 16 ? 0 : RMAX <= 8 ? 1 : RMAX == 9 ? 2 : 0;
             int R = block_R(G.n, LG::kSize);
             if (R < RMAX - 3) R = conflict_free_R(RMAX - 3, LG::kSize);
-            if constexpr (MODE == 3) {
-                if (R >= RMAX)
-                    walk_psl_lockstep<LG, RT, RMAX, TC>(env, w, ps, until, real, base, SL, V, trace_slot, trace_start,
-                                                        t, tt);
-                else if (R == RMAX - 1)
-                    walk_psl_lockstep<LG, RT, (RMAX > 1 ? RMAX - 1 : 1), TC>(env, w, ps, until, real, base, SL, V,
-                                                                         trace_slot, trace_start, t, tt);
-                else if (R == RMAX - 2)
-                    walk_psl_lockstep<LG, RT, (RMAX > 2 ? RMAX - 2 : 1), TC>(env, w, ps, until, real, base, SL, V,
-                                                                         trace_slot, trace_start, t, tt);
-                else
-                    walk_psl_lockstep<LG, RT, (RMAX > 3 ? RMAX - 3 : 1), TC>(env, w, ps, until, real, base, SL, V,
-                                                                         trace_slot, trace_start, t, tt);
-            } else {
-                if (R >= RMAX)
-                    walk_lockstep<LG, RT, RMAX, TC>(env, w, until, real, base, SL, V, trace_slot, trace_start, rec, t,
-                                                    tt);
-                else if (R == RMAX - 1)
-                    walk_lockstep<LG, RT, (RMAX > 1 ? RMAX - 1 : 1), TC>(env, w, until, real, base, SL, V, trace_slot,
-                                                                     trace_start, rec, t, tt);
-                else if (R == RMAX - 2)
-                    walk_lockstep<LG, RT, (RMAX > 2 ? RMAX - 2 : 1), TC>(env, w, until, real, base, SL, V, trace_slot,
-                                                                     trace_start, rec, t, tt);
-                else
-                    walk_lockstep<LG, RT, (RMAX > 3 ? RMAX - 3 : 1), TC>(env, w, until, real, base, SL, V, trace_slot,
-                                                                     trace_start, rec, t, tt);
-            }
+            if (R >= RMAX)
+                walk_psl_lockstep<LG, RT, RMAX, TC>(env, w, ps, until, real, base, SL, V, trace_slot, trace_start, t, tt);
+            else if (R == RMAX - 1)
+                walk_psl_lockstep<LG, RT, (RMAX > 1 ? RMAX - 1 : 1), TC>(env, w, ps, until, real, base, SL, V, trace_slot,
+                                                                     trace_start, t, tt);
+            else if (R == RMAX - 2)
+                walk_psl_lockstep<LG, RT, (RMAX > 2 ? RMAX - 2 : 1), TC>(env, w, ps, until, real, base, SL, V, trace_slot,
+                                                                     trace_start, t, tt);
+            else
+                walk_psl_lockstep<LG, RT, (RMAX > 3 ? RMAX - 3 : 1), TC>(env, w, ps, until, real, base, SL, V, trace_slot,
+                                                                     trace_start, t, tt);
             if (real) {
                 save_walker(env.st, w, t.lane);
-                if constexpr (MODE == 3) {
-                    if (t.lane == 0) {
-                        env.st->psl = ps.psl;
-                        env.st->best_psl = ps.best_psl;
-                        env.st->since_psl = ps.since_psl;
-                    }
+                if (t.lane == 0) {
+                    env.st->psl = ps.psl;
+                    env.st->best_psl = ps.best_psl;
+                    env.st->since_psl = ps.since_psl;
                 }
             }
             __syncwarp();
@@ -2648,21 +2386,9 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
 }
 
 template <int RMAX>
-__global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_pair_kernel(KParams p, int chunk_index)
-{
-    walk_group<Pair, Tile<16>, RMAX>(p, chunk_index);
-}
-
-template <int RMAX>
 __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_psl_pair_kernel(KParams p, int chunk_index)
 {
-    walk_group<Pair, Tile<16>, RMAX, 3>(p, chunk_index);
-}
-
-template <int RMAX>
-__global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_quad_kernel(KParams p, int chunk_index)
-{
-    walk_group<Quad, Tile<8>, RMAX>(p, chunk_index);
+    walk_psl_group<Pair, Tile<16>, RMAX>(p, chunk_index);
 }
 
 }  // namespace

@@ -130,7 +130,7 @@ struct KParams {
     int32_t patience;         // 0 = 2n
     int32_t target_num, target_den;
     int32_t chunk_steps;
-    int32_t rmax;             // lane block of the walk kernel instantiation (block_R(n_max, tile))
+    int32_t rmax;             // long mode: lane block of the kernel instantiation
     int32_t tile;             // lanes per walker: 32, 16 (two walkers per warp) or 8 (four)
     int32_t best_first;       // 1: best-first search (one walker per warp, queue below)
     int32_t mode;             // walk kernel variant: 0 plain walk, 1 learned mode, 2 best-first,
@@ -186,7 +186,7 @@ struct WarpSmem {
 // (tile/2 lanes per parity class): at least ceil(ceil(n/2) / (tile/2)), raised until
 // the lanes of a class, whose table windows lie 8R bytes apart, read 16 distinct pairs
 // of banks, i.e. until 16 / gcd(R, 16) >= tile/2.
-__host__ __device__ inline int conflict_free_R(int R, int tile)  // smallest such R' >= R
+__host__ __device__ constexpr int conflict_free_R(int R, int tile)  // smallest such R' >= R
 {
     for (;;) {
         const int low = R & -R;  // gcd(R, 16) for R < 32
@@ -194,7 +194,7 @@ __host__ __device__ inline int conflict_free_R(int R, int tile)  // smallest suc
         ++R;
     }
 }
-__host__ __device__ inline int block_R(int n, int tile)
+__host__ __device__ constexpr int block_R(int n, int tile)
 {
     const int h = tile / 2;
     return conflict_free_R((((n + 1) >> 1) + h - 1) / h, tile);
@@ -300,6 +300,98 @@ __host__ __device__ inline WarpSmem warp_smem(int n_max, int tile, bool psl = fa
         if (w.words * 4 * 16 <= kSmemBudget) return w;
     }
     return warp_layout(n_max, tile, false);
+}
+
+// ---- the plain walk's step (labs_step.cuh): compile-time shapes and shared memory.
+
+// Lane block of the plain walk: block_R, except that two walkers per warp above n = 128
+// take the block whose kernel runs two column groups and two lag blocks.
+__host__ __device__ constexpr int step_R(int n, int tile)
+{
+    return tile == 16 && n > 128 && n <= 160 ? 10 : block_R(n, tile);
+}
+
+// Largest n (up to kMaxN) that takes lane block R: a kernel's layout and its product are
+// sized for it, so that every offset and trip count of the step is a compile-time constant
+// (offsets in registers cost the two-walker step at L = 201 about 160 of 868 instructions).
+__host__ __device__ constexpr int step_n(int tile, int R)
+{
+    int n = 1;
+    for (int k = 2; k <= kMaxN; ++k)
+        if (step_R(k, tile) == R) n = k;
+    return n;
+}
+
+// Column groups of 4 output blocks (64 outputs per class) of the tensor-core product, and
+// blocks of 4 lags per lane, of the kernels with `tile` lanes per walker and lane block R.
+__host__ __device__ constexpr int step_groups(int tile, int R)
+{
+    return (tile == 32 && R >= 5) || (tile == 16 && R >= 10) ? 2 : 1;
+}
+__host__ __device__ constexpr int step_lag_blocks(int tile, int R)
+{
+    return (step_n(tile, R) + 4 * tile - 1) / (4 * tile);
+}
+
+// Shared memory of one walker of the plain walk, in 32-bit words from the walker's base
+// (a multiple of 4).  FP16 throughout but for the coefficients and the product's results:
+//   rows: class p's block at p hc holds two copies of the row, entry u of copy 0 at half
+//     index 2 h0 + u (zero below and above the class), and the same entries one half
+//     lower in copy 1, ks words further, so that the pair (u, u+1) of either parity is one
+//     aligned word;
+//   r8:   FP32 coefficients -8 s_i (-4 s_c) of the outputs, class p at r8 + p xp;
+//   g:    pairs G[y] = (E[y], E[y+1]), one word each, y in [-gneg, gpos);
+//   z:    the sums Z_m, half index 2 z + m, infinite for m in [-zneg, 0);
+//   x:    the product's results, class p at x + p xp; the bit vectors of a rebuild (class
+//     p at b + p bvec) share its words.
+struct StepSmem {
+    int h0, hc, ks;
+    int r8;
+    int g, gneg, gpos;
+    int z, zneg;
+    int x, xp;
+    int b, bvec;
+    int words;
+};
+
+__host__ __device__ constexpr StepSmem step_smem(int tile, int R)
+{
+    StepSmem w{};
+    const int n_max = step_n(tile, R), M = step_groups(tile, R), outs = (tile / 2) * R;
+    const int S = (n_max + 15) >> 4, T = (((n_max + 1) >> 1) + 15) >> 4, hw = (n_max + 1) >> 1;
+    // copy 0 below entry 0: s_{3i-L+1} down to -(n-1), the product's row blocks down to
+    // -(T-1).  Above: row blocks S+2 (S+3 with one operand per diagonal pair, S+6 with two
+    // column groups), the update's pairs (words below hw + 2), s_{3i-L+1} of the last lane
+    int lo = n_max - 1 > 16 * (T - 1) ? n_max - 1 : 16 * (T - 1);
+    lo = (lo + 7) & ~7;
+    int hi = 16 * (M == 2 ? S + 7 : tile == 32 ? S + 4 : S + 3);
+    if (2 * (hw + 2) > hi) hi = 2 * (hw + 2);
+    if (hw + 3 * R + 1 > hi) hi = hw + 3 * R + 1;
+    hi = (hi + 7) & ~7;
+    w.h0 = lo / 2;
+    w.ks = hi / 2 + 4;  // entry 0 of copy 1 lies one half below its first word
+    // 4 (mod 8) words per class: the two classes' operand rows use different banks
+    w.hc = ((w.h0 + w.ks + hw + 2 + 3) & ~7) + 4;
+    // class pitch of the coefficients and the results, and below the walkers' pitch, so that
+    // a warp's reads at odd R apart take 32 different banks: two walkers per warp 8 and 16
+    // (mod 32), with the operand columns in block order 0, 2, 1, 3 (step_toeplitz) a store of
+    // the results covers all banks too; four walkers 16 and 4; one walker 16
+    const int tb = (outs + 15) / 16 < 4 * M ? (outs + 15) / 16 : 4 * M;
+    const int need = 16 * tb > outs ? 16 * tb : outs;
+    w.xp = tile == 16 ? ((need + 23) & ~31) + 8 : ((need + 15) & ~31) + 16;
+    w.r8 = 2 * w.hc;
+    w.gneg = 16 * T;
+    w.gpos = 16 * S > 4 * tile ? 16 * S : 4 * tile;
+    w.g = ((w.r8 + w.xp + outs + 3) & ~3) + w.gneg;
+    w.zneg = (2 * R + 7) & ~7;
+    w.z = w.g + w.gpos + w.zneg / 2;
+    w.x = w.z + 2 * tile * step_lag_blocks(tile, R);
+    w.b = w.x;
+    w.bvec = (n_max - 1) / 32 + 2;
+    w.words = (w.x + w.xp + need + 3) & ~3;
+    if (tile == 16) w.words += (48 - (w.words & 31)) & 31;
+    if (tile == 8) w.words += (36 - (w.words & 31)) & 31;
+    return w;
 }
 
 // Layout of one row of the stateless row kernels (labs_neighbor_delta), `tile` lanes per
@@ -505,11 +597,8 @@ int launch_zobrist(const KParams& p, uint64_t* zkeys, const DevGroup* host_group
                    void* stream);
 int launch_reset(const KParams& p, int grid, int block, void* stream);
 int launch_prep_walk(const KParams& p, int64_t steps, int nchunks, void* stream);
-int launch_walk_chunk(const KParams& p, int chunk_index, int grid, int warps_per_cta,
-                      size_t smem_bytes, void* stream);
-int walk_kernel_config(int tile, int rmax, int mode, int warps_per_cta, size_t smem_bytes, int* ctas_per_sm,
-                       int* regs);
-int lanes_for(int n, int tile);  // block_R(n, tile)
+int launch_walk_chunk(const KParams& p, int chunk_index, int grid, int warps_per_cta, void* stream);
+int walk_kernel_config(int n_max, int tile, int mode, int warps_per_cta, int* ctas_per_sm, int* regs);
 int launch_isl(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, DevStatus* status,
                void* stream);
 int launch_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, DevStatus* status,

@@ -804,40 +804,44 @@ static WalkFn walk_fn(int tile, int rmax, int mode)
     }
 }
 
-int lanes_for(int n, int tile)
+// Lane block and shared memory per warp of a walk kernel (mode 0: the plain walk).
+static int walk_R(int n_max, int tile, int mode)
 {
-    return block_R(n, tile);
+    return mode == 0 ? step_R(n_max, tile) : block_R(n_max, tile);
 }
 
-int walk_kernel_config(int tile, int rmax, int mode, int warps_per_cta, size_t smem_bytes, int* ctas_per_sm,
-                       int* regs)
+static size_t walk_warp_bytes(int n_max, int tile, int mode)
 {
-    const WalkFn fn = walk_fn(tile, rmax, mode);
-    // every variant a context of this shape may launch (the learned mode is switched on
-    // and off at run time) gets the shared-memory size
-    for (int m = 0; m < (tile == 32 ? 3 : 1); ++m) {
-        const cudaError_t e = cudaFuncSetAttribute(walk_fn(tile, rmax, m), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem_bytes);
-        if (e != cudaSuccess) return LABS_ECUDA;
-    }
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    const int words = mode == 0 ? step_smem(tile, step_R(n_max, tile)).words : warp_smem(n_max, tile, mode == 3).words;
+    return (size_t)words * sizeof(int) * (kWarp / tile);
+}
+
+int walk_kernel_config(int n_max, int tile, int mode, int warps_per_cta, int* ctas_per_sm, int* regs)
+{
+    const WalkFn fn = walk_fn(tile, walk_R(n_max, tile, mode), mode);
+    const size_t smem_bytes = walk_warp_bytes(n_max, tile, mode) * (size_t)warps_per_cta;
+    // the limit is the device's, not this context's need: contexts share the kernels
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return LABS_ECUDA;
+    *ctas_per_sm = 0;
+    if (smem_bytes > (size_t)most) return LABS_EINVAL;
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, fn);
     if (e != cudaSuccess) return LABS_ECUDA;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    if (e != cudaSuccess) return LABS_ECUDA;
     if (regs) *regs = fa.numRegs;
-    if (warps_per_cta * kWarp > fa.maxThreadsPerBlock) {
-        *ctas_per_sm = 0;
-        return LABS_EINVAL;
-    }
+    if (warps_per_cta * kWarp > fa.maxThreadsPerBlock) return LABS_EINVAL;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, warps_per_cta * kWarp, smem_bytes);
     return status_of(e);
 }
 
-int launch_walk_chunk(const KParams& p, int chunk_index, int grid, int warps_per_cta, size_t smem_bytes,
-                      void* stream)
+int launch_walk_chunk(const KParams& p, int chunk_index, int grid, int warps_per_cta, void* stream)
 {
-    const WalkFn fn = walk_fn(p.tile, p.rmax, p.mode);
+    const WalkFn fn = walk_fn(p.tile, walk_R(p.n_max, p.tile, p.mode), p.mode);
+    const size_t smem_bytes = walk_warp_bytes(p.n_max, p.tile, p.mode) * (size_t)warps_per_cta;
     fn<<<grid, warps_per_cta * kWarp, smem_bytes, (cudaStream_t)stream>>>(p, chunk_index);
     return status_of(cudaGetLastError());
 }

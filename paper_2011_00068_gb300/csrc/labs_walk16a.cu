@@ -1,7 +1,18 @@
-// labs_walk16a.cu -- instantiations of the walk kernel with two walkers per warp, lane blocks 1-5.
-#include "labs_device.cuh"
+// labs_walk16a.cu -- walk kernels with two walkers per warp, lane blocks 1-5:
+// walk_lockstep in labs_step.cuh, compiled in their own unit.
+#include "labs_step.cuh"
 
 namespace labsgpu {
+
+namespace {
+
+template <int RMAX>
+__global__ void __launch_bounds__(256, step_ctas(16, RMAX)) walk_pair_kernel(KParams p, int chunk_index)
+{
+    walk_group<Pair, Tile<16>, RMAX>(p, chunk_index);
+}
+
+}  // namespace
 
 WalkFn walk_fn16a(int rmax)
 {
@@ -9,8 +20,6 @@ WalkFn walk_fn16a(int rmax)
         case 1: return walk_pair_kernel<1>;
         case 2: return walk_pair_kernel<2>;
         case 3: return walk_pair_kernel<3>;
-        case 4: return walk_pair_kernel<4>;
-        case 5: return walk_pair_kernel<5>;
         default: return walk_pair_kernel<5>;
     }
 }

@@ -1,16 +1,27 @@
-// labs_walk32.cu -- instantiations of the walk kernel with one walker per warp: the plain walk.
-#include "labs_device.cuh"
+// labs_walk32.cu -- walk kernels with one walker per warp (lane blocks are odd):
+// walk_lockstep in labs_step.cuh, compiled in their own unit.
+#include "labs_step.cuh"
 
 namespace labsgpu {
 
+namespace {
+
+template <int RMAX>
+__global__ void __launch_bounds__(256, step_ctas(32, RMAX)) walk_chunk_kernel(KParams p, int chunk_index)
+{
+    walk_group<Tile<32>, Tile<32>, RMAX>(p, chunk_index);
+}
+
+}  // namespace
+
 WalkFn walk_fn32(int rmax)
 {
-    switch (rmax) {  // block_R(n, 32) is odd
-        case 1: return walk_chunk_kernel<32, 1, 0>;
-        case 3: return walk_chunk_kernel<32, 3, 0>;
-        case 5: return walk_chunk_kernel<32, 5, 0>;
-        case 7: return walk_chunk_kernel<32, 7, 0>;
-        default: return walk_chunk_kernel<32, 9, 0>;
+    switch (rmax) {
+        case 1: return walk_chunk_kernel<1>;
+        case 3: return walk_chunk_kernel<3>;
+        case 5: return walk_chunk_kernel<5>;
+        case 7: return walk_chunk_kernel<7>;
+        default: return walk_chunk_kernel<9>;
     }
 }
 
