@@ -2,11 +2,21 @@
 // (L <= 63), the exact counterpart of the stochastic search for small L.
 //
 // The centre is fixed to s_c = +1 (negating a whole sequence keeps Eq. 4 and the ISL).
-// Assignment a sets free variable i (i < c) to -1 when bit i of a is set.  Thread t
-// owns the assignments whose high bits equal t and walks its low bits in Gray-code
-// order, so consecutive assignments differ by one free variable; the even-lag C_k are
-// updated by the change of one flip (positions j and q = L-1-j), and the ISL (Eq. 2)
-// is the sum of their squares (odd lags vanish by Eq. 4).
+// Assignment a sets free variable i (i < c) to -1 when bit i of a is set.
+//
+// Every assignment's even-lag C_k come from bit vectors of its two parity classes.  Class p
+// (n_p = n - p entries) is a palindrome or an antipalindrome (Eq. 4), a_{n_p-1-u} = sg_p a_u,
+// so the pairs (u, u+m) of lag m repeat from both ends: with h = floor((n_p - m) / 2) pairs
+// counted and d of them unequal, C^(p)_m = 2 h - 4 d, plus sg_p when n_p - m is odd (the
+// middle pair).  h <= 16 for L <= 63: both classes' pairs share one 32-bit word and one
+// popcount, and C_{2m} is a constant of the lag minus 4 popcounts.  The ISL (Eq. 2) is the
+// sum of the squares (odd lags vanish).
+//
+// What bounds it: about 8 integer instructions per assignment and lag.  A thread takes its
+// 2^low consecutive assignments kEnumLanes at a time, so that a lag's masks and constant
+// are computed once for all of them.  The partial results are reduced by trees of one CTA
+// each (one thread reading 1024 of them took 270 us).  L = 41: the two kernels take about
+// 10 us of the call (333 before).
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -28,122 +38,131 @@ __host__ __device__ inline int enum_low_bits(int free_bits)
     return free_bits > kEnumMaxHighBits ? free_bits - kEnumMaxHighBits : 0;
 }
 
-// +1 / -1 / 0 (outside 0..L-1) from the sequence mask (bit j set <=> s_j = -1).
-__device__ __forceinline__ int sval(uint64_t mask, int L, int j)
+// Every second bit of a, from bit 0, packed.
+__device__ __forceinline__ uint32_t even_bits(uint32_t a)
 {
-    if (j < 0 || j >= L) return 0;
-    return ((mask >> j) & 1ull) ? -1 : 1;
+    a &= 0x55555555u;
+    a = (a | (a >> 1)) & 0x33333333u;
+    a = (a | (a >> 2)) & 0x0F0F0F0Fu;
+    a = (a | (a >> 4)) & 0x00FF00FFu;
+    return (a | (a >> 8)) & 0x0000FFFFu;
 }
 
-__device__ __forceinline__ uint64_t seq_mask(uint64_t a, int L, int n)
+__device__ __forceinline__ uint32_t low_mask(int bits)  // 0 <= bits <= 32
+{
+    return bits >= 32 ? ~0u : (1u << bits) - 1u;
+}
+
+// Bit vector of class p of assignment a: free variables 2v + p, then their mirrors.
+__device__ __forceinline__ uint32_t class_bits(uint32_t a, int n, int p)
+{
+    const int c = n - 1, np = n - p, nv = p ? n >> 1 : (n + 1) >> 1;  // nv entries are free (or the centre)
+    const uint32_t lo = even_bits(a >> p) & low_mask(nv);
+    uint32_t rev = __brev(lo) >> (32 - np);                           // entry np-1-u for entry u
+    if ((c + p) & 1) rev = ~rev;                                      // antipalindrome
+    return lo | (rev & low_mask(np) & ~low_mask(nv));
+}
+
+struct EnumBest {
+    int isl;
+    uint32_t first;
+    unsigned long long count;
+};
+
+__device__ __forceinline__ void enum_take(EnumBest& b, int isl, uint32_t first, unsigned long long count)
+{
+    if (count == 0 || isl > b.isl) return;
+    if (isl < b.isl) {
+        b.isl = isl;
+        b.count = 0;
+        b.first = first;
+    }
+    b.count += count;
+    b.first = min(b.first, first);
+}
+
+// Adds the whole CTA's results into thread 0's.
+template <int THREADS>
+__device__ __forceinline__ EnumBest enum_block_best(EnumBest b)
+{
+    __shared__ EnumBest sh[THREADS];
+    sh[threadIdx.x] = b;
+    for (int h = THREADS / 2; h > 0; h >>= 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < h) {
+            const EnumBest o = sh[threadIdx.x + h];
+            enum_take(b, o.isl, o.first, o.count);
+            sh[threadIdx.x] = b;
+        }
+    }
+    return b;
+}
+
+// ISLs of the K assignments a0 .. a0+K-1.  (ISL <= sum of squares below 63: 2^17.)
+template <int K>
+__device__ __forceinline__ void enum_eval(uint32_t a0, int n, EnumBest& best)
 {
     const int c = n - 1;
-    uint64_t m = 0;
-    for (int j = 0; j < L; ++j) {
-        int f = j <= c ? j : 2 * c - j;
-        int bit = f < c ? (int)((a >> f) & 1ull) : 0;  // centre is +1
-        if (j > c && ((j - c) & 1)) bit ^= 1;
-        m |= (uint64_t)bit << j;
+    uint32_t x0[K], x1[K];
+    int isl[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        x0[k] = class_bits(a0 + k, n, 0);
+        x1[k] = class_bits(a0 + k, n, 1);
+        isl[k] = 0;
     }
-    return m;
+    const int g0 = (c & 1) ? -1 : 1;  // sg of class 0; class 1 has the other sign
+    for (int m = 1; m < n; ++m) {
+        const int q0 = n - m, q1 = n - 1 - m, h0 = q0 >> 1, h1 = q1 >> 1;
+        const uint32_t m0 = low_mask(h0), m1 = low_mask(h1);
+        const int base = 2 * (h0 + h1) + ((q0 & 1) ? g0 : 0) + ((q1 & 1) ? -g0 : 0);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t d0 = (x0[k] ^ (x0[k] >> m)) & m0, d1 = (x1[k] ^ (x1[k] >> m)) & m1;
+            const int cm = base - 4 * __popc(d0 | (d1 << 16));
+            isl[k] += cm * cm;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) enum_take(best, isl[k], a0 + k, 1ull);
 }
+
+constexpr int kEnumLanes = 8;
 
 __global__ void __launch_bounds__(kEnumThreads) enum_kernel(int L, EnumPart* parts)
 {
-    __shared__ int Cs[32][kEnumThreads];  // even-lag C, Cs[m][thread] = C_{2m}
-    __shared__ long long rmin[kEnumThreads];
-    __shared__ unsigned long long rcnt[kEnumThreads], rfirst[kEnumThreads];
-    const int n = (L + 1) / 2, c = n - 1;
-    const int T = n - 1;
-    const int b = enum_low_bits(T);
-    const uint64_t high = (uint64_t)blockIdx.x * kEnumThreads + threadIdx.x;
-    const uint64_t nhigh = 1ull << (T - b);
-    long long best = LLONG_MAX;
-    unsigned long long cnt = 0, first = 0;
-    int* C = &Cs[0][threadIdx.x];
-    if (high < nhigh) {
-        uint64_t a = high << b;
-        uint64_t mask = seq_mask(a, L, n);
-        long long isl = 0;
-        for (int m = 1; m < n; ++m) {
-            int d = 0;
-            for (int j = 0; j + 2 * m < L; ++j) d += sval(mask, L, j) * sval(mask, L, j + 2 * m);
-            C[m * kEnumThreads] = d;
-            isl += (long long)d * d;
-        }
-        best = isl;
-        cnt = 1;
-        first = a;
-        const uint64_t steps = 1ull << b;
-        for (uint64_t t = 1; t < steps; ++t) {
-            const int j = __ffsll((long long)t) - 1;  // Gray code: bit j changes
-            const int q = L - 1 - j;
-            const int sj = sval(mask, L, j);
-            isl = 0;
-            for (int m = 1; m < n; ++m) {
-                const int k = 2 * m;
-                const int up = (j + k == q) ? 0 : sval(mask, L, j + k);
-                const int dC = -4 * sj * (up + sval(mask, L, j - k));
-                const int cm = C[m * kEnumThreads] + dC;
-                C[m * kEnumThreads] = cm;
-                isl += (long long)cm * cm;
-            }
-            mask ^= (1ull << j) | (1ull << q);
-            a ^= 1ull << j;
-            if (isl < best) {
-                best = isl;
-                cnt = 1;
-                first = a;
-            } else if (isl == best) {
-                cnt += 1;
-                if (a < first) first = a;
-            }
+    const int n = (L + 1) / 2, T = n - 1, low = enum_low_bits(T);
+    const uint32_t high = blockIdx.x * kEnumThreads + threadIdx.x;
+    EnumBest best{INT_MAX, ~0u, 0ull};
+    if (high < (1u << (T - low))) {
+        const uint32_t a0 = high << low;
+        if (low >= 3) {
+            for (uint32_t t = 0; t < (1u << low); t += kEnumLanes) enum_eval<kEnumLanes>(a0 + t, n, best);
+        } else {
+            for (uint32_t t = 0; t < (1u << low); ++t) enum_eval<1>(a0 + t, n, best);
         }
     }
-    (void)c;
-    rmin[threadIdx.x] = best;
-    rcnt[threadIdx.x] = cnt;
-    rfirst[threadIdx.x] = first;
-    __syncthreads();
+    best = enum_block_best<kEnumThreads>(best);
     if (threadIdx.x == 0) {
-        long long m = LLONG_MAX;
-        unsigned long long k = 0, f = 0;
-        for (int t = 0; t < kEnumThreads; ++t) {
-            if (rcnt[t] == 0) continue;
-            if (rmin[t] < m) {
-                m = rmin[t];
-                k = rcnt[t];
-                f = rfirst[t];
-            } else if (rmin[t] == m) {
-                k += rcnt[t];
-                if (rfirst[t] < f) f = rfirst[t];
-            }
-        }
-        parts[blockIdx.x].min_isl = m;
-        parts[blockIdx.x].count = k;
-        parts[blockIdx.x].first = f;
+        parts[blockIdx.x].min_isl = best.isl;
+        parts[blockIdx.x].count = best.count;
+        parts[blockIdx.x].first = best.first;
     }
 }
 
-__global__ void enum_reduce_kernel(const EnumPart* parts, int nparts, EnumPart* out)
+constexpr int kEnumReduceThreads = 256;
+
+__global__ void __launch_bounds__(kEnumReduceThreads) enum_reduce_kernel(const EnumPart* parts, int nparts, EnumPart* out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    long long m = LLONG_MAX;
-    unsigned long long k = 0, f = 0;
-    for (int t = 0; t < nparts; ++t) {
-        if (parts[t].count == 0) continue;
-        if (parts[t].min_isl < m) {
-            m = parts[t].min_isl;
-            k = parts[t].count;
-            f = parts[t].first;
-        } else if (parts[t].min_isl == m) {
-            k += parts[t].count;
-            if (parts[t].first < f) f = parts[t].first;
-        }
+    EnumBest best{INT_MAX, ~0u, 0ull};
+    for (int t = threadIdx.x; t < nparts; t += kEnumReduceThreads)
+        enum_take(best, (int)parts[t].min_isl, (uint32_t)parts[t].first, parts[t].count);
+    best = enum_block_best<kEnumReduceThreads>(best);
+    if (threadIdx.x == 0) {
+        out->min_isl = best.isl;
+        out->count = best.count;
+        out->first = best.first;
     }
-    out->min_isl = m;
-    out->count = k;
-    out->first = f;
 }
 
 }  // namespace
@@ -167,7 +186,7 @@ int enum_run(int L, EnumPart* scratch, void* stream, EnumPart* host_out)
     const int blocks = enum_blocks(L);
     cudaStream_t s = (cudaStream_t)stream;
     enum_kernel<<<blocks, kEnumThreads, 0, s>>>(L, scratch);
-    enum_reduce_kernel<<<1, 32, 0, s>>>(scratch, blocks, scratch + blocks);
+    enum_reduce_kernel<<<1, kEnumReduceThreads, 0, s>>>(scratch, blocks, scratch + blocks);
     if (cudaGetLastError() != cudaSuccess) return LABS_ECUDA;
     if (cudaMemcpyAsync(host_out, scratch + blocks, sizeof(EnumPart), cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return LABS_ECUDA;
