@@ -10,11 +10,18 @@
 //   restart = w6 . mean_p(a3_p) + b6                                   (restart score)
 // Loss per sample: wf * CE(softmax(score), t) + 0.5 (restart - y)^2, batch mean.
 //
-// Layouts.  Activations are bf16 [B][P][C] with P = ceil16(n) + 6 rows per sample:
-// row r holds position r-3, rows outside 3..n+2 stay zero (the convolution's padding
-// and the tile tail).  Convolution weights are packed bf16 [64 out][taps x Cin]
-// (tap-major, channel fastest), the layout the products' K-major weight operand takes;
-// the backward-data pass uses the tap-reversed transpose.
+// Tiles.  A tile holds as many whole samples as fit 128 output rows (256 for n > 128) with
+// three zero rows between them (the convolutions' padding), so nothing crosses a tile: one
+// CTA carries it through all layers without leaving shared memory.  A tile's activations
+// are kept as 16-byte rows of 8 channels, one column of rows per 8 channels ([column][row],
+// rows 0-2 zero, row o+3 output row o), in shared and in global memory alike:
+//   - as the K-major operand of a product over channels, tap k of a convolution is the same
+//     operand with its start address 16 k bytes further;
+//   - as the MN-major operand of a weight gradient (the reduction runs over rows), the same
+//     columns serve without a transpose;
+//   - a tile moves between global and shared memory as one contiguous copy.
+// Weights are packed per layer as [K/8][64 outputs][8] bf16, the K-major layout of the second
+// operand; the backward-data products use the tap-reversed transpose.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -41,201 +48,62 @@ constexpr int pWf1 = 0, pWf2 = pWf1 + kC * kTaps * kCin, pWf3 = pWf2 + kC * kTap
               pWb2 = pWf4 + kC * kC, pWb3 = pWb2 + kC * kTaps * kC, pWb4 = pWb3 + kC * kTaps * kC, pW5 = pWb4 + kC * kC,
               pW6 = pW5 + kC, kPacked = pW6 + kC;
 
-__host__ __device__ inline int rows_per_sample(int n)
-{
-    return ((n + 15) & ~15) + 6;
-}
-
 namespace {
 
-enum { EPI_BIAS_RELU = 0, EPI_MASK = 1, EPI_MASK_POOL = 2 };
+constexpr int kTcThreads = 128;  // threads of a tile group: one TMEM lane (output row) each
 
-// out[b][3+p][o] = epi(sum_{k<TAPS, c<CIN} in[b][p+k+RO][c] * Wt[o][k*CIN+c]) for p < n, on
-// the 5th-generation tensor cores.  The B*P activation rows form
-// one long sequence (the zero rows around each sample keep the samples apart), so output
-// row G (sample b = G / P, position G % P - 3) takes input rows G - 3 + RO + k, k < TAPS:
-// a tile of 128 output rows reads 128 + TAPS - 1 consecutive input rows.  TMA stages them
-// once, in the K-major layout without swizzling (16-byte rows back to back, one column
-// of rows per 8 input channels, kRowsPad rows apart), and tap k is the same operand with
-// its start address 16 k bytes further.  The weights (64 outputs x TAPS CIN) are staged
-// once per CTA in the same layout (64 rows per column of 8 K values).  One thread issues
-// TAPS * CIN/16 MMAs of M = 128, N = 64, K = 16 into 64 TMEM columns; every warp reads
-// its 32 rows back (tcgen05.ld) for the epilogue, which writes only rows of real
-// positions (the zero rows stay zero).
-constexpr int kTcThreads = 128;
-constexpr int kTcTile = 128;  // output rows per tile (the MMA's M)
-
-template <int CIN, int TAPS>
-struct TcShape {
-    static constexpr int KK = TAPS * CIN;
-    static constexpr int RO = 3 - (TAPS - 1) / 2;
-    static constexpr int ROWS = kTcTile + TAPS - 1;              // input rows per tile
-    static constexpr int ROWS_PAD = (ROWS + 7) & ~7;              // 128-byte aligned columns
-    static constexpr int A_COL = ROWS_PAD * 16;                   // bytes per 8-channel column
-    static constexpr int A_BYTES = (CIN / 8) * A_COL;
-    static constexpr int W_BYTES = (KK / 8) * 1024;               // 64 rows x 16 bytes per column
-    static constexpr int BAR_OFF = W_BYTES + A_BYTES;             // three barriers, the TMEM slot
-    static constexpr int BIAS_OFF = BAR_OFF + 32;
-    static constexpr int SMEM = BIAS_OFF + 2 * kC * 4 + 128;       // + alignment slack
+// A tile of MT x 128 output rows.
+template <int MT>
+struct Tile {
+    static constexpr int M = 128 * MT;
+    static constexpr int RP = M + 9;            // rows per column: 3 zero rows on each side, 1 (mod 8) rows
+                                                // so that the columns of a row use different banks
+    static constexpr int COL = RP * 16;         // bytes per column
+    static constexpr int ACT = 8 * COL;         // bytes of 64 channels
 };
 
-template <int CIN, int TAPS, int EPI>
-__global__ void __launch_bounds__(kTcThreads) rows_tc_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                             const __grid_constant__ CUtensorMap tmW,
-                                                             const float* __restrict__ bias,
-                                                             const bf16* __restrict__ mask,
-                                                             const float* __restrict__ pool_dr,
-                                                             const bf16* __restrict__ pool_w, bf16* __restrict__ out,
-                                                             int n, int64_t rows_total, int* __restrict__ err)
+__host__ __device__ inline int tile_rows(int n) { return n <= 128 ? 128 : 256; }
+__host__ __device__ inline int tile_samples(int n) { return (tile_rows(n) + 3) / (n + 3); }
+__host__ __device__ inline int64_t tile_count(int64_t B, int n)
 {
-    using S = TcShape<CIN, TAPS>;
-    extern __shared__ unsigned char tc_smem_raw[];
-    // 128-byte aligned base for the TMA destinations
-    unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 127) & ~uintptr_t(127));
-    const uint32_t sW = smem_addr(sm), sA = sW + S::W_BYTES;
-    const uint32_t bar_w = sW + S::BAR_OFF, bar_a = bar_w + 8, bar_m = bar_w + 16, slot = bar_w + 24;
-    float* sbias = reinterpret_cast<float*>(sm + S::BIAS_OFF);
-    float* spool = sbias + kC;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int P = rows_per_sample(n);
-    const int64_t tiles = (rows_total + kTcTile - 1) / kTcTile;
-    if (threadIdx.x < kC) {
-        sbias[threadIdx.x] = (EPI == EPI_BIAS_RELU) ? bias[threadIdx.x] : 0.f;
-        spool[threadIdx.x] = (EPI == EPI_MASK_POOL) ? __bfloat162float(pool_w[threadIdx.x]) / (float)n : 0.f;
-    }
-    if (warp == 0) tmem_alloc(slot, 64);
-    if (threadIdx.x == 0) {
-        mbar_init(bar_w, 1);
-        mbar_init(bar_a, 1);
-        mbar_init(bar_m, 1);
-        mbar_init_fence();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + S::BAR_OFF + 24);
-    bool ok = true;
-    if (threadIdx.x == 0) {
-        mbar_arrive_expect_tx(bar_w, S::W_BYTES);
-        for (int j = 0; j < S::KK / 8; ++j) tma_load_2d(sW + 1024 * j, &tmW, 8 * j, 0, bar_w);
-        ok = mbar_wait(bar_w, 0);
-    }
-    constexpr uint32_t idesc = idesc_bf16_f32(kTcTile, kC);
-    int it = 0;
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
-        const int64_t G0 = tile * kTcTile;
-        if (threadIdx.x == 0 && ok) {
-            mbar_arrive_expect_tx(bar_a, S::A_BYTES / S::ROWS_PAD * S::ROWS);
-            for (int j = 0; j < CIN / 8; ++j)
-                tma_load_2d(sA + S::A_COL * j, &tmA, 8 * j, (int)(G0 - 3 + S::RO), bar_a);
-            ok = mbar_wait(bar_a, it & 1);
-            if (ok) {
-                tc_fence_after();
-#pragma unroll
-                for (int k = 0; k < TAPS; ++k)
-#pragma unroll
-                    for (int s2 = 0; s2 < CIN / 16; ++s2) {
-                        const uint64_t ad = smem_desc(sA + 16 * k + 2 * s2 * S::A_COL, S::A_COL, 128);
-                        const uint64_t bd = smem_desc(sW + (k * (CIN / 8) + 2 * s2) * 1024, 1024, 128);
-                        tc_mma_bf16(tmem, ad, bd, idesc, (k | s2) != 0);
-                    }
-                tc_commit(bar_m);
-            }
-        }
-        // every thread waits for the accumulator (a failed copy or wait skips the tile)
-        ok = __syncthreads_and(ok) && mbar_wait(bar_m, it & 1);
-        ok = __syncthreads_and(ok);
-        if (!ok) {
-            if (threadIdx.x == 0) atomicExch(err, 1);
-            break;
-        }
-        tc_fence_after();
-        float acc[64];
-        const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float v[16];
-            tmem_ld16(trow + 16 * q, v);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) acc[16 * q + i] = v[i];
-        }
-        tc_wait_ld();
-        const int64_t G = G0 + 32 * warp + lane;
-        const int b = (int)(G / P), p = (int)(G % P) - 3;
-        if (G < rows_total && p >= 0 && p < n) {
-            bf16* dst = out + G * kC;
-            const float pdr = (EPI == EPI_MASK_POOL) ? pool_dr[b] : 0.f;
-#pragma unroll
-            for (int c8 = 0; c8 < kC / 8; ++c8) {
-                uint4 mk = make_uint4(0u, 0u, 0u, 0u);
-                if (EPI != EPI_BIAS_RELU) mk = *reinterpret_cast<const uint4*>(mask + G * kC + 8 * c8);
-                const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
-                uint32_t pk[4];
-#pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    const int o = 8 * c8 + 2 * h;
-                    float v0 = acc[o], v1 = acc[o + 1];
-                    if (EPI == EPI_BIAS_RELU) {
-                        v0 = fmaxf(v0 + sbias[o], 0.f);
-                        v1 = fmaxf(v1 + sbias[o + 1], 0.f);
-                    } else {
-                        if (EPI == EPI_MASK_POOL) {
-                            v0 += spool[o] * pdr;
-                            v1 += spool[o + 1] * pdr;
-                        }
-                        const __nv_bfloat162 m2 = *reinterpret_cast<const __nv_bfloat162*>(&mw[h]);
-                        if (!(__bfloat162float(m2.x) > 0.f)) v0 = 0.f;
-                        if (!(__bfloat162float(m2.y) > 0.f)) v1 = 0.f;
-                    }
-                    const __nv_bfloat162 r2 = __floats2bfloat162_rn(v0, v1);
-                    pk[h] = *reinterpret_cast<const uint32_t*>(&r2);
-                }
-                *reinterpret_cast<uint4*>(dst + 8 * c8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            }
-        }
-        // the next tile's copy overwrites the operand and its MMAs the accumulator
-        tc_fence_before();
-        __syncthreads();
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        tmem_dealloc(tmem, 64);
-    }
+    const int k = tile_samples(n);
+    return (B + k - 1) / k;
 }
 
-// Weight gradients on the tensor cores: dW[o][c][k] = sum over the B*P rows r of
-// G[r][o] * IN[r - 3 + RO + k][c] (rows of G outside the positions are zero).  The
-// reduction dimension is the rows, so both operands are MN-major: a staged column of 16-
-// byte rows (8 channels or 8 outputs per row) is the MN-major core-matrix layout without
-// swizzling (8 K rows of 16 bytes each, the next 8 rows 128 bytes further), and columns
-// lie kWgCol bytes apart along M (or N).  M = 128 covers 16 columns of (tap, 8-channel
-// block) pairs: column c holds channels 8 (c % (CIN/8)) .. +7 of tap c / (CIN/8), loaded
-// with that tap's row offset, so every column's shift is in its TMA coordinate; columns
-// past the last tap load tap 0 and their rows of the result are dropped.  N = 64
-// outputs (the 8 columns of G).  A CTA walks blocks of kWgRows rows, accumulating
-// ceil(TAPS CIN / 128) tiles of 128 x 64 in TMEM, and writes its partial sums; a second
-// kernel adds the partials of all CTAs into the gradient.
-constexpr int kWgRows = 64;                 // rows (K) per staged block
-constexpr int kWgCol = kWgRows * 16;        // bytes per staged column
-constexpr int kWgCtasPerSm = 2;
-
-template <int CIN, int TAPS>
-struct WgShape {
-    static constexpr int KK = TAPS * CIN;
-    static constexpr int RO = 3 - (TAPS - 1) / 2;
-    static constexpr int NT = (KK + 127) / 128;           // M tiles
-    static constexpr int NCOL = 16 * NT;                  // staged columns of IN
-    static constexpr int IN_BYTES = NCOL * kWgCol;
-    static constexpr int G_BYTES = 8 * kWgCol;
-    static constexpr int BAR_OFF = IN_BYTES + G_BYTES;
-    static constexpr int TMEM_COLS = NT * 64 <= 64 ? 64 : (NT * 64 <= 128 ? 128 : 256);
-    // a CTA holding 256 of the SM's 512 TMEM columns asks for enough shared memory that
-    // no third CTA fits beside two (its allocation would wait for theirs to end)
-    static constexpr int SMEM_NEED = BAR_OFF + 32 + 128;
-    static constexpr int SMEM = TMEM_COLS > 128 && SMEM_NEED < 80 * 1024 ? 80 * 1024 : SMEM_NEED;
+// Where an output row of a tile stands: its sample (of the tile) and position, in if it is
+// one.
+struct RowPos {
+    int k, p;
+    bool in;
+    __device__ RowPos(int o, int n, int K) : k(o / (n + 3)), p(o % (n + 3)), in(false) { in = p < n && k < K; }
 };
+
+__device__ __forceinline__ void group_sync(int id)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kTcThreads) : "memory");
+}
+
+__device__ __forceinline__ uint32_t pack2(float a, float b)
+{
+    const __nv_bfloat162 r = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+__device__ __forceinline__ float lo_f(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float hi_f(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+
+__device__ __forceinline__ void sts128(uint32_t a, uint4 v)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(a)
+                 : "memory");
+    return v;
+}
 
 // Instruction descriptor of kind::f16 with both operands MN-major (bits 15 and 16).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N)
@@ -243,293 +111,780 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N)
     return idesc_bf16_f32(M, N) | (1u << 15) | (1u << 16);
 }
 
-template <int CIN, int TAPS>
-__global__ void __launch_bounds__(kTcThreads) wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmIN,
-                                                              const __grid_constant__ CUtensorMap tmG,
-                                                              float* __restrict__ part, int64_t rows,
-                                                              int* __restrict__ err)
+// D (128 rows, 64 columns at TMEM address d) = TAPS-tap product of the rows from byte
+// address a (column pitch COL) with the packed weights at w.  One thread.
+template <int CIN, int TAPS, int COL>
+__device__ __forceinline__ void issue_product(uint32_t d, uint32_t a, uint32_t w)
 {
-    using S = WgShape<CIN, TAPS>;
+    constexpr uint32_t id = idesc_bf16_f32(128, kC);
+#pragma unroll
+    for (int k = 0; k < TAPS; ++k)
+#pragma unroll
+        for (int s2 = 0; s2 < CIN / 16; ++s2)
+            tc_mma_bf16(d, smem_desc(a + 16 * k + 2 * s2 * COL, COL, 128),
+                        smem_desc(w + (k * (CIN / 8) + 2 * s2) * 1024, 1024, 128), id, (k | s2) != 0);
+}
+
+// D (128 x 64 at TMEM address d) += over the rows r < M: A columns (16 of them, pitch COL,
+// from address a) x G columns (8, from address g): a weight gradient, both operands
+// MN-major (the next 8 rows 128 bytes on, the next 8 channels one column on).
+template <int M, int COL>
+__device__ __forceinline__ void issue_wgrad(uint32_t d, uint32_t a, uint32_t g, bool fresh)
+{
+    constexpr uint32_t id = idesc_bf16_f32_mn(128, kC);
+#pragma unroll
+    for (int ks = 0; ks < M / 16; ++ks)
+        tc_mma_bf16(d, smem_desc(a + 256 * ks, 128, COL), smem_desc(g + 256 * ks, 128, COL), id, !fresh || ks > 0);
+}
+
+// This thread's 64 accumulators (TMEM lane 32 (warp mod 4) + lane).
+__device__ __forceinline__ void load_acc(uint32_t d, int wq, float (&acc)[64])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float v[16];
+        tmem_ld16(d + ((uint32_t)(32 * wq) << 16) + 16 * q, v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[16 * q + i] = v[i];
+    }
+    tc_wait_ld();
+}
+
+// Sums v over the warp's 32 lanes: lane l returns the sums of entries 2l and 2l+1 (each
+// round exchanges half of what a lane still holds).
+__device__ __forceinline__ float2 warp_colsum(float (&v)[64], int lane)
+{
+#pragma unroll
+    for (int h = 32, off = 16; h >= 2; h >>= 1, off >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, off);
+        }
+    }
+    return make_float2(v[0], v[1]);
+}
+
+// Adds a lane's channel sums (2 lane, 2 lane + 1) to the CTA's.
+__device__ __forceinline__ void add_channels(float* sums, int lane, float2 v)
+{
+    atomicAdd(sums + 2 * lane, v.x);
+    atomicAdd(sums + 2 * lane + 1, v.y);
+}
+
+// ------------------------------------------------------------------ forward
+//
+// One kernel from the inputs to the scores: conv1..3, the MLP and the heads of a tile stay
+// in shared memory (a convolution's result overwrites its input once its product has
+// completed), the weights of all layers are loaded once per CTA.  NG tile groups of 128
+// threads share a CTA and its weights, each with its own tile, accumulators and barriers,
+// so one group's epilogue runs beside another's products.  TRAIN goes on to the loss and the
+// gradients that need the scores of whole samples: the softmax, dh, the MLP's and the heads'
+// gradients and da3; a1, a2 and da3 go to global memory for the convolutions' backward
+// kernels, a3 and h never leave the CTA.
+//
+// What bounds it: the products' shared-memory reads (6 KB per 128 x 64 x 16 product, 67
+// products a tile) and the epilogues between them.  It replaces one launch per layer over
+// global activations (read and written 70 MB each for 4096 samples of n = 128) cleared by a
+// memset before every pass.
+template <int MT, bool TRAIN>
+struct FwdShape {
+    using T = Tile<MT>;
+    static constexpr int NG = TRAIN ? (MT == 1 ? 2 : 1) : (MT == 1 ? 3 : 2);
+    static constexpr int THREADS = NG * kTcThreads;
+    static constexpr int W1 = 0, W2 = W1 + kTaps * kCin * 128, W3 = W2 + kTaps * kC * 128, W4 = W3 + kTaps * kC * 128,
+                         WB4 = W4 + kC * 128, W_END = TRAIN ? WB4 + kC * 128 : WB4;
+    static constexpr int X0 = 0, ACT = 2 * T::COL, DH = ACT + T::ACT;  // within a group
+    static constexpr int GROUP = TRAIN ? DH + T::ACT : DH;
+    static constexpr int GROUPS = W_END;
+    static constexpr int MISC = GROUPS + NG * GROUP;
+    // misc: biases b1..b4, w5, w6 (float), barriers, the TMEM slot; then per group scores, ds
+    // (M floats each) and dr per sample (M/4 floats), the CTA's sums of b3, b4, w5, w6 gradients
+    static constexpr int BIAS = MISC, BAR = BIAS + 6 * kC * 4, SC = BAR + 64;
+    static constexpr int SCB = (2 * T::M + T::M / 4 + 32) * 4;
+    static constexpr int SUMS = SC + (TRAIN ? NG * SCB : 0);
+    static constexpr int SMEM = SUMS + (TRAIN ? 4 * kC * 4 : 0) + 128;  // + alignment slack
+    static constexpr int TMEM_USED = NG * MT * 64 + (TRAIN ? NG * 64 : 0);
+    static constexpr int TMEM = TMEM_USED <= 128 ? 128 : 256;
+};
+
+struct FwdArgs {
+    const float* x;
+    const bf16* wpk;
+    const float* prm;
+    float* score;
+    float* restart;
+    int* err;
+    int64_t B;
+    int n;
+    // training
+    const int32_t* target;
+    const float* y;
+    const float* wf;
+    bf16 *X0, *A1, *A2, *dA3;  // tiles in global memory
+    float* part4;              // [CTA x group][64 channels][64 outputs] partial dW4
+    float* grad;
+    float* loss;
+};
+
+// Row o of a tile: 64 bf16 values (as 32 words) to the columns at address col (this row's
+// first 16 bytes) and, when g is given, to the same place of a tile in global memory.
+template <int COL>
+__device__ __forceinline__ void store_row(uint32_t col, unsigned char* g, const uint32_t (&w)[32])
+{
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const uint4 v = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+        if (col != 0u) sts128(col + c * COL, v);
+        if (g != nullptr) *reinterpret_cast<uint4*>(g + c * COL) = v;
+    }
+}
+
+// Zero rows of a tile in global memory (rows outside its output rows), by the first threads
+// of a group.
+template <int MT, int COLS>
+__device__ __forceinline__ void zero_pad_rows(unsigned char* g, int t)
+{
+    if (t < 9) {
+        const int r = t < 3 ? t : Tile<MT>::M + t;
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) *reinterpret_cast<uint4*>(g + c * Tile<MT>::COL + 16 * r) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+template <int MT, bool TRAIN>
+__global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_kernel(FwdArgs a)
+{
+    using S = FwdShape<MT, TRAIN>;
+    using T = Tile<MT>;
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 127) & ~uintptr_t(127));
-    const uint32_t sIN = smem_addr(sm), sG = sIN + S::IN_BYTES;
-    const uint32_t bar_a = sIN + S::BAR_OFF, bar_m = bar_a + 8, slot = bar_a + 16;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) tmem_alloc(slot, S::TMEM_COLS);
+    const uint32_t sb = smem_addr(sm);
+    const int t = threadIdx.x % kTcThreads, grp = threadIdx.x / kTcThreads, wq = t >> 5, lane = t & 31;
+    float* bias = reinterpret_cast<float*>(sm + S::BIAS);
+    const uint32_t bar_w = sb + S::BAR, bar = bar_w + 8 + 8 * grp, slot = sb + S::BAR + 48;
+    volatile int* failed = reinterpret_cast<volatile int*>(sm + S::BAR + 56);
+    const uint32_t gx = sb + S::GROUPS + grp * S::GROUP + S::X0, ga = sb + S::GROUPS + grp * S::GROUP + S::ACT,
+                   gd = sb + S::GROUPS + grp * S::GROUP + S::DH;
+    float* s_score = reinterpret_cast<float*>(sm + S::SC + grp * S::SCB);
+    float* s_ds = s_score + T::M;
+    float* s_dr = s_ds + T::M;
+    float* sums = reinterpret_cast<float*>(sm + S::SUMS);  // b3, b4, w5, w6
+    const int n = a.n, K = tile_samples(n);
+    const int64_t tiles = tile_count(a.B, n);
+
+    for (int i = threadIdx.x; i < kC; i += S::THREADS) {
+        bias[i] = a.prm[oB1 + i];
+        bias[kC + i] = a.prm[oB2 + i];
+        bias[2 * kC + i] = a.prm[oB3 + i];
+        bias[3 * kC + i] = a.prm[oB4 + i];
+        bias[4 * kC + i] = __bfloat162float(a.wpk[pW5 + i]);
+        bias[5 * kC + i] = __bfloat162float(a.wpk[pW6 + i]);
+    }
+    if (TRAIN)
+        for (int i = threadIdx.x; i < 4 * kC; i += S::THREADS) sums[i] = 0.f;
+    for (int i = threadIdx.x; i < S::NG * S::GROUP / 16; i += S::THREADS)
+        sts128(sb + S::GROUPS + 16 * i, make_uint4(0u, 0u, 0u, 0u));
+    if (threadIdx.x < 32) tmem_alloc(slot, S::TMEM);
     if (threadIdx.x == 0) {
-        mbar_init(bar_a, 1);
-        mbar_init(bar_m, 1);
+        *failed = 0;
+        mbar_init(bar_w, 1);
+        for (int g = 0; g < S::NG; ++g) mbar_init(bar_w + 8 + 8 * g, 1);
         mbar_init_fence();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + S::BAR_OFF + 16);
-    constexpr uint32_t idesc = idesc_bf16_f32_mn(128, kC);
-    const int64_t blocks = (rows + kWgRows - 1) / kWgRows;
-    bool ok = true;
-    int it = 0;
-    for (int64_t blk = blockIdx.x; blk < blocks; blk += gridDim.x, ++it) {
-        if (threadIdx.x == 0 && ok) {
-            const int R0 = (int)(blk * kWgRows);
-            mbar_arrive_expect_tx(bar_a, (uint32_t)(S::IN_BYTES + S::G_BYTES));
-            for (int c = 0; c < S::NCOL; ++c) {
-                const int tap = c / (CIN / 8), ch = c % (CIN / 8);
-                tma_load_2d(sIN + c * kWgCol, &tmIN, 8 * ch, R0 - 3 + S::RO + (tap < TAPS ? tap : 0), bar_a);
-            }
-            for (int j = 0; j < 8; ++j) tma_load_2d(sG + j * kWgCol, &tmG, 8 * j, R0, bar_a);
-            ok = mbar_wait(bar_a, it & 1);
-            if (ok) {
-                tc_fence_after();
-#pragma unroll
-                for (int t = 0; t < S::NT; ++t)
-#pragma unroll
-                    for (int ks = 0; ks < kWgRows / 16; ++ks) {
-                        // MN-major without swizzling: the leading byte offset steps along K
-                        // (the next 8 rows, 128 bytes on), the stride byte offset along M or
-                        // N (the next column of 8 values)
-                        const uint64_t ad = smem_desc(sIN + t * 16 * kWgCol + 256 * ks, 128, kWgCol);
-                        const uint64_t bd = smem_desc(sG + 256 * ks, 128, kWgCol);
-                        tc_mma_bf16(tmem + 64 * t, ad, bd, idesc, it > 0 || ks > 0);
-                    }
-                tc_commit(bar_m);
-                // the next block's copies overwrite the operands: wait for these MMAs
-                ok = mbar_wait(bar_m, it & 1);
-            }
-        }
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + S::BAR + 48);
+    const uint32_t acc0 = tmem + grp * MT * 64, acc4 = tmem + S::NG * MT * 64 + grp * 64;
+    if (threadIdx.x == 0) {
+        mbar_arrive_expect_tx(bar_w, S::W_END);
+        bulk_copy_g2s(sb + S::W1, a.wpk + pWf1, S::W2 - S::W1, bar_w);
+        bulk_copy_g2s(sb + S::W2, a.wpk + pWf2, S::W3 - S::W2, bar_w);
+        bulk_copy_g2s(sb + S::W3, a.wpk + pWf3, S::W4 - S::W3, bar_w);
+        bulk_copy_g2s(sb + S::W4, a.wpk + pWf4, kC * 128, bar_w);
+        if (TRAIN) bulk_copy_g2s(sb + S::WB4, a.wpk + pWb4, kC * 128, bar_w);
     }
-    tc_fence_before();
-    ok = __syncthreads_and(ok);
-    if (!ok && threadIdx.x == 0) atomicExch(err, 1);
-    tc_fence_after();
-    // partial sums of this CTA: row m of tile t is (tap, channel) = ((128 t + m) / CIN,
-    // (128 t + m) % CIN); columns are the 64 outputs
-    if (ok && it > 0) {
-        float* dst = part + (int64_t)blockIdx.x * S::NT * 128 * kC;
-        for (int t = 0; t < S::NT; ++t) {
-            const int m = 128 * t + 32 * warp + lane;
-            float4* d4 = reinterpret_cast<float4*>(dst + (int64_t)m * kC);
+    bool ok = mbar_wait(bar_w, 0);
+    uint32_t phase = 0;
+    int done = 0;           // tiles of this group
+    float2 gw6 = {0.f, 0.f};  // sums over this warp's samples: w6 (channels 2 lane, 2 lane + 1)
+    float gb5 = 0.f, gb6 = 0.f, lsum = 0.f;
+    const float inv = TRAIN ? 1.f / (float)a.B : 0.f;
+
+    // the group's inputs of a tile: three features per row
+    float xin[MT][3];
+    auto fetch = [&](int64_t tile) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + 64 * t + 16 * q, v);
-                tc_wait_ld();
-                if (m < S::KK) {
+        for (int mt = 0; mt < MT; ++mt) {
+            const RowPos rp(t + 128 * mt, n, K);
+            const int64_t b = tile * K + rp.k;
+            const bool in = rp.in && tile < tiles && b < a.B;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        d4[4 * q + i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                }
-            }
+            for (int f = 0; f < 3; ++f) xin[mt][f] = in ? a.x[(b * 3 + f) * n + rp.p] : 0.f;
         }
-    } else if (ok) {
-        // no block for this CTA: zero partials
-        float* dst = part + (int64_t)blockIdx.x * S::NT * 128 * kC;
-        for (int i = threadIdx.x; i < S::KK * kC; i += blockDim.x) dst[i] = 0.f;
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
+    };
+    // waits for the group's products; a wait that gives up ends the CTA's work
+    auto wait_products = [&]() {
+        if (!mbar_wait(bar, phase)) *failed = 1;
+        phase ^= 1;
         tc_fence_after();
-        tmem_dealloc(tmem, S::TMEM_COLS);
-    }
-}
+    };
+    // the epilogue's shared-memory rows are visible to the next product, the accumulators read
+    auto rows_ready = [&]() {
+        fence_async_shared();
+        tc_fence_before();
+        group_sync(1 + grp);
+        tc_fence_after();
+    };
 
-// dW[o][c][k] += sum over CTAs of part[cta][k CIN + c][o].
-template <int CIN, int TAPS>
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int ctas, float* __restrict__ dW)
-{
-    using S = WgShape<CIN, TAPS>;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < S::KK * kC; i += gridDim.x * blockDim.x) {
-        const int m = i / kC, o = i % kC;
-        float t = 0.f;
-        for (int c = 0; c < ctas; ++c) t += part[(int64_t)c * S::NT * 128 * kC + i];
-        const int k = m / CIN, ch = m % CIN;
-        dW[((int64_t)o * CIN + ch) * TAPS + k] += t;
-    }
-}
-
-// Bias gradient: db[o] += sum_{b, p<n} G[b][p+3][o], summed over all B*P rows (the rows
-// outside 0 <= p < n hold zeros).  Thread t reads channels 8 (t % 8) .. +7 of rows
-// t / 8, t / 8 + 32, ... as one 16-byte load; the CTA's 32 row lanes are added in shared
-// memory and each CTA adds its 64 sums to db.
-__global__ void __launch_bounds__(256) colsum_kernel(const bf16* __restrict__ G, float* __restrict__ db,
-                                                     int64_t rows)
-{
-    __shared__ float part[32][kC + 1];
-    const int cg = threadIdx.x & 7, rl = threadIdx.x >> 3;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int64_t r = (int64_t)blockIdx.x * 32 + rl; r < rows; r += (int64_t)gridDim.x * 32) {
-        const uint4 v = *reinterpret_cast<const uint4*>(G + r * kC + 8 * cg);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const __nv_bfloat162 b2 = *reinterpret_cast<const __nv_bfloat162*>(&w[h]);
-            acc[2 * h] += __bfloat162float(b2.x);
-            acc[2 * h + 1] += __bfloat162float(b2.y);
+    const int64_t stride = (int64_t)gridDim.x * S::NG;
+    int64_t tile = (int64_t)grp * gridDim.x + blockIdx.x;
+    fetch(tile);
+    for (; tile < tiles && ok; tile += stride, ++done) {
+        unsigned char* const gA1 = TRAIN ? reinterpret_cast<unsigned char*>(a.A1) + tile * T::ACT : nullptr;
+        unsigned char* const gA2 = TRAIN ? reinterpret_cast<unsigned char*>(a.A2) + tile * T::ACT : nullptr;
+        unsigned char* const gA3 = TRAIN ? reinterpret_cast<unsigned char*>(a.dA3) + tile * T::ACT : nullptr;
+        if (TRAIN) {
+            zero_pad_rows<MT, 8>(gA1, t);
+            zero_pad_rows<MT, 8>(gA2, t);
+            zero_pad_rows<MT, 8>(gA3, t);
+            zero_pad_rows<MT, 1>(reinterpret_cast<unsigned char*>(a.X0) + tile * T::COL, t);
         }
-    }
+        bool in[MT];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) part[rl][8 * cg + i] = acc[i];
-    __syncthreads();
-    if (threadIdx.x < kC) {
-        float t = 0.f;
-        for (int k = 0; k < 32; ++k) t += part[k][threadIdx.x];
-        atomicAdd(db + threadIdx.x, t);
-    }
-}
-
-// x (float32 [B][3][n]) -> bf16 input rows [B][P][16].
-__global__ void input_kernel(const float* __restrict__ x, bf16* __restrict__ X0, int B, int n)
-{
-    const int P = rows_per_sample(n);
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)B * n * 3;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int b = (int)(t / (3 * n)), rem = (int)(t % (3 * n)), f = rem / n, p = rem % n;
-        X0[((int64_t)b * P + p + 3) * kCin + f] = __float2bfloat16_rn(x[t]);
-    }
-}
-
-// Heads: score[b][p] = b5 + sum_j h[b][p][j] w5[j]; pooled[b][c] = mean_p a3[b][p][c];
-// restart[b] = b6 + sum_c pooled[b][c] w6[c].  One warp per sample: lane l scores
-// positions l, l+32, ... (its row of h as 16-byte loads) and sums channels 2l, 2l+1 of a3
-// over the positions (one 4-byte load per row).
-__global__ void head_kernel(const bf16* __restrict__ H, const bf16* __restrict__ A3, const bf16* __restrict__ wpk,
-                            const float* __restrict__ params, float* __restrict__ score,
-                            float* __restrict__ pooled, float* __restrict__ restart, int B, int n)
-{
-    __shared__ float w5[kC];
-    for (int j = threadIdx.x; j < kC; j += blockDim.x) w5[j] = __bfloat162float(wpk[pW5 + j]);
-    __syncthreads();
-    const int P = rows_per_sample(n);
-    const int lane = threadIdx.x & 31;
-    const float b5 = params[oB5], b6 = params[oB6];
-    const float w6a = __bfloat162float(wpk[pW6 + 2 * lane]), w6b = __bfloat162float(wpk[pW6 + 2 * lane + 1]);
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < B; b += nw) {
-        const bf16* hb = H + b * P * kC;
-        for (int p = lane; p < n; p += 32) {
-            const uint4* row = reinterpret_cast<const uint4*>(hb + (int64_t)(p + 3) * kC);
+        for (int mt = 0; mt < MT; ++mt) {
+            const int o = t + 128 * mt;
+            const RowPos rp(o, n, K);
+            in[mt] = rp.in && tile * K + rp.k < a.B;
+            const uint4 v = make_uint4(pack2(xin[mt][0], xin[mt][1]), pack2(xin[mt][2], 0.f), 0u, 0u);
+            sts128(gx + 16 * (o + 3), v);
+            if (TRAIN) *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(a.X0) + tile * T::COL + 16 * (o + 3)) = v;
+        }
+        rows_ready();
+        if (t == 0) {
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) issue_product<kCin, kTaps, T::COL>(acc0 + 64 * mt, gx + 2048 * mt, sb + S::W1);
+            tc_commit(bar);
+        }
+        fetch(tile + stride);
+        // conv1..3: bias, ReLU, the rows replace the layer's input
+#pragma unroll 1
+        for (int l = 0; l < 3; ++l) {
+            wait_products();
+            unsigned char* const gl = l == 0 ? gA1 : l == 1 ? gA2 : nullptr;
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                float acc[64];
+                load_acc(acc0 + 64 * mt, wq, acc);
+                const int o = t + 128 * mt;
+                uint32_t w[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const float v0 = fmaxf(acc[2 * i] + bias[l * kC + 2 * i], 0.f),
+                                v1 = fmaxf(acc[2 * i + 1] + bias[l * kC + 2 * i + 1], 0.f);
+                    w[i] = in[mt] ? pack2(v0, v1) : 0u;
+                }
+                store_row<T::COL>(ga + 16 * (o + 3), gl ? gl + 16 * (o + 3) : nullptr, w);
+            }
+            rows_ready();
+            if (t == 0) {
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    if (l < 2)
+                        issue_product<kC, kTaps, T::COL>(acc0 + 64 * mt, ga + 2048 * mt, sb + (l == 0 ? S::W2 : S::W3));
+                    else
+                        issue_product<kC, 1, T::COL>(acc0 + 64 * mt, ga + 48 + 2048 * mt, sb + S::W4);
+                }
+                tc_commit(bar);
+            }
+        }
+        // restart scores from the pooled a3 (beside the MLP's product): a warp per sample,
+        // lane l sums channels 2l and 2l+1 over the positions
+        for (int k = wq; k < K; k += 4) {
+            const int64_t b = tile * K + k;
+            if (b >= a.B) break;
+            const uint32_t col = ga + (lane >> 2) * T::COL + 4 * (lane & 3) + 16 * (k * (n + 3) + 3);
+            float ma = 0.f, mb = 0.f;
+#pragma unroll 8
+            for (int p = 0; p < n; ++p) {
+                uint32_t v;
+                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(col + 16 * p) : "memory");
+                ma += lo_f(v);
+                mb += hi_f(v);
+            }
+            ma /= (float)n;
+            mb /= (float)n;
+            float r = ma * bias[5 * kC + 2 * lane] + mb * bias[5 * kC + 2 * lane + 1];
+#pragma unroll
+            for (int off = 16; off; off >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, off);
+            r += a.prm[oB6];
+            if (TRAIN) {
+                const float e = r - a.y[b], dr = e * inv;
+                gw6.x += ma * dr;
+                gw6.y += mb * dr;
+                if (lane == 0) {
+                    s_dr[k] = dr;
+                    gb6 += dr;
+                    lsum += 0.5f * e * e * inv;
+                }
+            } else if (lane == 0) {
+                a.restart[b] = r;
+            }
+        }
+        wait_products();
+        uint32_t h[TRAIN ? MT : 1][32];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            float acc[64];
+            load_acc(acc0 + 64 * mt, wq, acc);
+            const int o = t + 128 * mt;
+            const RowPos rp(o, n, K);
             float sacc = 0.f;
 #pragma unroll
-            for (int c8 = 0; c8 < kC / 8; ++c8) {
-                const uint4 v = row[c8];
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            for (int i = 0; i < 32; ++i) {
+                const uint32_t w = pack2(fmaxf(acc[2 * i] + bias[3 * kC + 2 * i], 0.f),
+                                         fmaxf(acc[2 * i + 1] + bias[3 * kC + 2 * i + 1], 0.f));
+                if (TRAIN) h[mt][i] = w;
+                sacc += lo_f(w) * bias[4 * kC + 2 * i] + hi_f(w) * bias[4 * kC + 2 * i + 1];
+            }
+            sacc += a.prm[oB5];
+            if (TRAIN)
+                s_score[o] = sacc;
+            else if (in[mt])
+                a.score[(tile * K + rp.k) * n + rp.p] = sacc;
+        }
+        if constexpr (TRAIN) {
+            group_sync(1 + grp);
+            // softmax cross-entropy and its gradient, a warp per sample
+            for (int k = wq; k < K; k += 4) {
+                const int64_t b = tile * K + k;
+                if (b >= a.B) break;
+                const float* s = s_score + k * (n + 3);
+                float m = -INFINITY;
+                for (int p = lane; p < n; p += 32) m = fmaxf(m, s[p]);
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    const __nv_bfloat162 b2 = *reinterpret_cast<const __nv_bfloat162*>(&w[h]);
-                    sacc += __bfloat162float(b2.x) * w5[8 * c8 + 2 * h] + __bfloat162float(b2.y) * w5[8 * c8 + 2 * h + 1];
+                for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
+                float z = 0.f;
+                for (int p = lane; p < n; p += 32) z += expf(s[p] - m);
+#pragma unroll
+                for (int off = 16; off; off >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, off);
+                const int tg = min(max(a.target[b], 0), n - 1);
+                const float w = a.wf[b];
+                for (int p = lane; p < n; p += 32)
+                    s_ds[k * (n + 3) + p] = w * (expf(s[p] - m) / z - (p == tg ? 1.f : 0.f)) * inv;
+                if (lane == 0) lsum += w * (logf(z) + m - s[tg]) * inv;
+            }
+            group_sync(1 + grp);
+            // dh = w5 ds where h > 0; gradients of w5, b5 and b4
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                const int o = t + 128 * mt;
+                const float d = in[mt] ? s_ds[o] : 0.f;
+                gb5 += d;
+                float v[64];
+                uint32_t w[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    v[2 * i] = lo_f(h[mt][i]) * d;
+                    v[2 * i + 1] = hi_f(h[mt][i]) * d;
+                }
+                add_channels(sums + 2 * kC, lane, warp_colsum(v, lane));
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    w[i] = pack2(lo_f(h[mt][i]) > 0.f ? bias[4 * kC + 2 * i] * d : 0.f,
+                                 hi_f(h[mt][i]) > 0.f ? bias[4 * kC + 2 * i + 1] * d : 0.f);
+                    if (!in[mt]) w[i] = 0u;
+                    v[2 * i] = lo_f(w[i]);
+                    v[2 * i + 1] = hi_f(w[i]);
+                }
+                store_row<T::COL>(gd + 16 * (o + 3), nullptr, w);
+                add_channels(sums + kC, lane, warp_colsum(v, lane));
+            }
+            rows_ready();
+            if (t == 0) {
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) issue_product<kC, 1, T::COL>(acc0 + 64 * mt, gd + 48 + 2048 * mt, sb + S::WB4);
+                // dW4: its rows 64-127 (the columns after a3's, i.e. dh's) are dropped
+                issue_wgrad<T::M, T::COL>(acc4, ga + 48, gd + 48, done == 0);
+                tc_commit(bar);
+            }
+            wait_products();
+            // da3 = (W4^T dh + w6 dr / n) where a3 > 0; gradient of b3
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                float acc[64];
+                load_acc(acc0 + 64 * mt, wq, acc);
+                const int o = t + 128 * mt;
+                const RowPos rp(o, n, K);
+                const float pdr = in[mt] ? s_dr[rp.k] / (float)n : 0.f;
+                uint32_t w[32];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 q = lds128(ga + c * T::COL + 16 * (o + 3));
+                    const uint32_t mw[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int i = 8 * c + 2 * j;
+                        const float v0 = acc[i] + bias[5 * kC + i] * pdr, v1 = acc[i + 1] + bias[5 * kC + i + 1] * pdr;
+                        w[4 * c + j] = pack2(lo_f(mw[j]) > 0.f ? v0 : 0.f, hi_f(mw[j]) > 0.f ? v1 : 0.f);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    if (!in[mt]) w[i] = 0u;
+                    acc[2 * i] = lo_f(w[i]);
+                    acc[2 * i + 1] = hi_f(w[i]);
+                }
+                store_row<T::COL>(0u, gA3 + 16 * (o + 3), w);
+                add_channels(sums, lane, warp_colsum(acc, lane));
+            }
+        }
+        tc_fence_before();
+        group_sync(1 + grp);
+        tc_fence_after();
+        ok = *failed == 0;
+    }
+    if (!ok || *failed) atomicExch(a.err, 1);
+    if constexpr (TRAIN) {
+        add_channels(sums + 3 * kC, lane, gw6);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) gb5 += __shfl_xor_sync(0xFFFFFFFFu, gb5, off);
+        if (lane == 0) {
+            atomicAdd(a.grad + oB5, gb5);
+            atomicAdd(a.grad + oB6, gb6);
+            atomicAdd(a.loss, lsum);
+        }
+        // this group's partial dW4 (channel x output)
+        float4* dst = reinterpret_cast<float4*>(a.part4 + ((int64_t)blockIdx.x * S::NG + grp) * kC * kC) + t * (kC / 4);
+        float acc[64];
+        if (done > 0) load_acc(acc4, wq, acc);  // a warp-wide load: done is the same for the group
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (t < kC)
+                dst[i] = done > 0 ? make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3])
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (TRAIN && threadIdx.x < kC) {
+        atomicAdd(a.grad + oB3 + threadIdx.x, sums[threadIdx.x]);
+        atomicAdd(a.grad + oB4 + threadIdx.x, sums[kC + threadIdx.x]);
+        atomicAdd(a.grad + oW5 + threadIdx.x, sums[2 * kC + threadIdx.x]);
+        atomicAdd(a.grad + oW6 + threadIdx.x, sums[3 * kC + threadIdx.x]);
+    }
+    if (threadIdx.x < 32) {
+        tc_fence_after();
+        tmem_dealloc(tmem, S::TMEM);
+    }
+}
+
+// ------------------------------------------------------------------ backward of a convolution
+//
+// Per tile, from the gradient G of a convolution's output (rows outside the positions zero)
+// and its input IN:
+//   dIN = (G convolved with the tap-reversed transpose) where IN > 0,
+//   dW[o][c][k] += sum over rows r of G[r][o] IN[r + k][c],
+//   the bias gradient of the layer below (the column sums of dIN).
+// FIRST: IN is a1, and dIN = da1 stays in shared memory for conv1's weight gradient against
+// the inputs; else dIN goes to global memory.
+//
+// A warp of its own issues every product: the weight gradient's accumulators are shared by
+// the CTA's tile groups, and one thread's products on an accumulator complete in order.  The
+// weight gradient takes taps in pairs (M = 128): the tile of IN is loaded twice, the second
+// copy one row up and right behind the first, so that columns 8-15 of the operand are the
+// next tap's.  conv1's takes one column (8 channels, 3 in use) per tap from 8 copies of the
+// inputs, each one row further up.
+template <int MT, bool FIRST>
+struct BwdShape {
+    using T = Tile<MT>;
+    static constexpr int NG = MT == 1 ? (FIRST ? 2 : 3) : 1;
+    static constexpr int THREADS = NG * kTcThreads + 32;
+    static constexpr int WB = 0, GROUPS = kTaps * kC * 128;
+    // the 8 input copies (column k one row further up than column k-1; the operand's columns
+    // 8-15 fall on G and their rows of the result are dropped), G, IN, IN one row up (its
+    // first row lies 16 bytes before it)
+    static constexpr int XC = 0, G = FIRST ? 8 * T::COL : 0, IN = G + T::ACT, GROUP = IN + 2 * T::ACT;
+    static constexpr int BAR = GROUPS + NG * GROUP, SUMS = BAR + 160;
+    static constexpr int SMEM = SUMS + kC * 4 + 128;
+    static constexpr int ACC_W = 0, ACC_W1 = 256, ACC_D = FIRST ? 320 : 256;  // TMEM columns
+    static constexpr int TMEM = 512;
+    static_assert(ACC_D + NG * MT * 64 <= TMEM, "TMEM columns");
+};
+
+struct BwdArgs {
+    const bf16 *G, *IN, *X0, *wb;
+    bf16* dIN;
+    float* part;   // [CTA][448][64] partial dW (row tap * 64 + channel)
+    float* part1;  // FIRST: [CTA][64][64] partial dW1 (row tap * 8 + channel)
+    float* db;
+    int* err;
+    int64_t tiles;
+    int64_t B;
+    int n;
+};
+
+template <int MT, bool FIRST>
+__global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward_kernel(BwdArgs a)
+{
+    using S = BwdShape<MT, FIRST>;
+    using T = Tile<MT>;
+    extern __shared__ unsigned char tc_smem_raw[];
+    unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 127) & ~uintptr_t(127));
+    const uint32_t sb = smem_addr(sm);
+    const int t = threadIdx.x % kTcThreads, grp = threadIdx.x / kTcThreads, wq = t >> 5, lane = t & 31;
+    const bool issuer = grp == S::NG;
+    // barriers per group: operands loaded, dIN product done, weight gradient done, da1 ready,
+    // conv1's weight gradient done
+    const uint32_t bar_w = sb + S::BAR, bars = bar_w + 8, slot = sb + S::BAR + 144;
+    auto full = [&](int g) { return bars + 40 * g; };
+    auto dbar = [&](int g) { return bars + 40 * g + 8; };
+    auto wbar = [&](int g) { return bars + 40 * g + 16; };
+    auto rbar = [&](int g) { return bars + 40 * g + 24; };
+    auto fbar = [&](int g) { return bars + 40 * g + 32; };
+    volatile int* failed = reinterpret_cast<volatile int*>(sm + S::BAR + 152);
+    float* sums = reinterpret_cast<float*>(sm + S::SUMS);
+    auto buf = [&](int g) { return sb + S::GROUPS + g * S::GROUP; };
+    if (threadIdx.x < kC) sums[threadIdx.x] = 0.f;
+    // the operands' unwritten rows and columns hold finite values
+    for (int i = threadIdx.x; i < S::NG * S::GROUP / 16; i += S::THREADS)
+        sts128(sb + S::GROUPS + 16 * i, make_uint4(0u, 0u, 0u, 0u));
+    if (issuer) tmem_alloc(slot, S::TMEM);
+    if (threadIdx.x == 0) {
+        *failed = 0;
+        mbar_init(bar_w, 1);
+        for (int i = 0; i < 5 * S::NG; ++i) mbar_init(bars + 8 * i, 1);
+        mbar_init_fence();
+    }
+    fence_async_shared();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + S::BAR + 144);
+    const int64_t first = (int64_t)blockIdx.x, stride = (int64_t)gridDim.x * S::NG;
+    auto tile_of = [&](int g, int it) { return first + (int64_t)g * gridDim.x + it * stride; };
+    // one thread: the group's operands of a tile
+    auto load = [&](int g, int64_t tile) {
+        const uint32_t b = buf(g), f = full(g);
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(a.IN) + tile * T::ACT;
+        mbar_arrive_expect_tx(f, 3 * T::ACT + (FIRST ? 8 * T::COL : 0));
+        bulk_copy_g2s(b + S::G, reinterpret_cast<const unsigned char*>(a.G) + tile * T::ACT, T::ACT, f);
+        bulk_copy_g2s(b + S::IN, src, T::ACT, f);
+        bulk_copy_g2s(b + S::IN + T::ACT - 16, src, T::ACT, f);
+        if (FIRST)
+            for (int k = 0; k < 8; ++k)
+                bulk_copy_g2s(b + S::XC + k * (T::COL - 16),
+                              reinterpret_cast<const unsigned char*>(a.X0) + tile * T::COL, T::COL, f);
+    };
+    if (issuer) {
+        if (lane == 0) {
+            bool ok = true, fresh = true, fresh1 = true;
+            mbar_arrive_expect_tx(bar_w, kTaps * kC * 128);
+            bulk_copy_g2s(sb + S::WB, a.wb, kTaps * kC * 128, bar_w);
+            for (int g = 0; g < S::NG; ++g)
+                if (tile_of(g, 0) < a.tiles) load(g, tile_of(g, 0));
+            ok = mbar_wait(bar_w, 0);
+            for (int it = 0; ok && tile_of(0, it) < a.tiles; ++it) {
+                for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
+                    ok = mbar_wait(full(g), it & 1);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t b = buf(g);
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt)
+                        issue_product<kC, kTaps, T::COL>(tmem + S::ACC_D + 64 * (g * MT + mt), b + S::G + 2048 * mt, sb + S::WB);
+                    tc_commit(dbar(g));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)  // taps 2q, 2q+1 (the eighth is dropped)
+                        issue_wgrad<T::M, T::COL>(tmem + S::ACC_W + 64 * q, b + S::IN + 32 * q, b + S::G + 48, fresh);
+                    fresh = false;
+                    tc_commit(wbar(g));
+                }
+                if (FIRST)
+                    for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
+                        ok = mbar_wait(rbar(g), it & 1);
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_wgrad<T::M, T::COL>(tmem + S::ACC_W1, buf(g) + S::XC, buf(g) + S::G + 48, fresh1);
+                        fresh1 = false;
+                        tc_commit(fbar(g));
+                    }
+            }
+            if (!ok) *failed = 1;
+        }
+    } else {
+        const int K = tile_samples(a.n);
+        for (int it = 0; tile_of(grp, it) < a.tiles; ++it) {
+            const int64_t tile = tile_of(grp, it);
+            if (!mbar_wait(dbar(grp), it & 1)) *failed = 1;
+            tc_fence_after();
+            unsigned char* const gout = FIRST ? nullptr : reinterpret_cast<unsigned char*>(a.dIN) + tile * T::ACT;
+            if (!FIRST) zero_pad_rows<MT, 8>(gout, t);
+            if (FIRST) {
+                // da1 takes G's place: the weight gradient has read it
+                if (!mbar_wait(wbar(grp), it & 1)) *failed = 1;
+                tc_fence_after();
+            }
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                float acc[64];
+                load_acc(tmem + S::ACC_D + 64 * (grp * MT + mt), wq, acc);
+                const int o = t + 128 * mt;
+                const RowPos rp(o, a.n, K);
+                const bool in = rp.in && tile * K + rp.k < a.B;
+                uint32_t w[32];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 q = lds128(buf(grp) + S::IN + c * T::COL + 16 * (o + 3));
+                    const uint32_t mw[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int i = 8 * c + 2 * j;
+                        w[4 * c + j] = pack2(lo_f(mw[j]) > 0.f ? acc[i] : 0.f, hi_f(mw[j]) > 0.f ? acc[i + 1] : 0.f);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    if (!in) w[i] = 0u;
+                    acc[2 * i] = lo_f(w[i]);
+                    acc[2 * i + 1] = hi_f(w[i]);
+                }
+                store_row<T::COL>(FIRST ? buf(grp) + S::G + 16 * (o + 3) : 0u, FIRST ? nullptr : gout + 16 * (o + 3), w);
+                add_channels(sums, lane, warp_colsum(acc, lane));
+            }
+            if (FIRST) {
+                fence_async_shared();
+                tc_fence_before();
+                group_sync(1 + grp);
+                if (t == 0) {
+                    mbar_arrive(rbar(grp));
+                    if (!mbar_wait(fbar(grp), it & 1)) *failed = 1;
+                    if (tile_of(grp, it + 1) < a.tiles && *failed == 0) {
+                        fence_async_shared();
+                        load(grp, tile_of(grp, it + 1));
+                    }
+                }
+            } else {
+                tc_fence_before();
+                group_sync(1 + grp);  // every row's mask has been read
+                if (t == 0) {
+                    if (!mbar_wait(wbar(grp), it & 1)) *failed = 1;
+                    if (tile_of(grp, it + 1) < a.tiles && *failed == 0) {
+                        fence_async_shared();
+                        load(grp, tile_of(grp, it + 1));
+                    }
                 }
             }
-            score[b * n + p] = sacc + b5;
+            if (*failed) break;
         }
-        const bf16* ab = A3 + b * P * kC + 2 * lane;
-        float ma = 0.f, mb = 0.f;
-        for (int p = 0; p < n; ++p) {
-            const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(ab + (int64_t)(p + 3) * kC);
-            ma += __bfloat162float(v.x);
-            mb += __bfloat162float(v.y);
-        }
-        ma /= (float)n;
-        mb /= (float)n;
-        pooled[b * kC + 2 * lane] = ma;
-        pooled[b * kC + 2 * lane + 1] = mb;
-        float r = ma * w6a + mb * w6b;
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (*failed) {
+        if (threadIdx.x == 0) atomicExch(a.err, 1);
+    } else if (grp == 0) {
+        // every product has completed: each group's last waits covered its own
+        for (int q = 0; q < 4; ++q) {
+            float acc[64];
+            load_acc(tmem + S::ACC_W + 64 * q, wq, acc);
+            const int m = 128 * q + t;  // tap * 64 + channel
+            if (m < kTaps * kC) {
+                float4* dst = reinterpret_cast<float4*>(a.part + ((int64_t)blockIdx.x * kTaps * kC + m) * kC);
 #pragma unroll
-        for (int off = 16; off; off >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, off);
-        if (lane == 0) restart[b] = r + b6;
+                for (int i = 0; i < 16; ++i) dst[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+            }
+        }
+        if (FIRST) {
+            float acc[64];
+            load_acc(tmem + S::ACC_W1, wq, acc);
+            if (t < 64) {
+                float4* dst = reinterpret_cast<float4*>(a.part1 + ((int64_t)blockIdx.x * 64 + t) * kC);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) dst[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+            }
+        }
+    }
+    if (threadIdx.x < kC) atomicAdd(a.db + threadIdx.x, sums[threadIdx.x]);
+    tc_fence_before();
+    __syncthreads();
+    if (issuer) {
+        tc_fence_after();
+        tmem_dealloc(tmem, S::TMEM);
     }
 }
 
-// Loss and its gradients w.r.t. the scores and the restart output (batch mean).
-__global__ void loss_kernel(const float* __restrict__ score, const float* __restrict__ restart,
-                            const int32_t* __restrict__ target, const float* __restrict__ y,
-                            const float* __restrict__ wf, float* __restrict__ ds, float* __restrict__ dr,
-                            float* __restrict__ loss, int B, int n)
+// Gradients of W1..W4 from the CTAs' partial sums: 16 outputs x 4 of them per block, 16
+// slices of the CTAs each.
+struct ReduceArgs {
+    const float *p1, *p2, *p3, *p4;
+    int c23, c4;  // CTAs of the convolutions' partials, CTA groups of W4's
+    float* grad;
+};
+
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(ReduceArgs a)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const float inv = 1.f / (float)B;
-    for (int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < B; b += nw) {
-        const float* s = score + b * n;
-        float m = -INFINITY;
-        for (int p = lane; p < n; p += 32) m = fmaxf(m, s[p]);
-#pragma unroll
-        for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
-        float z = 0.f;
-        for (int p = lane; p < n; p += 32) z += expf(s[p] - m);
-#pragma unroll
-        for (int off = 16; off; off >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, off);
-        const int t = min(max(target[b], 0), n - 1);
-        const float w = wf[b];
-        for (int p = lane; p < n; p += 32) ds[b * n + p] = w * (expf(s[p] - m) / z - (p == t ? 1.f : 0.f)) * inv;
-        if (lane == 0) {
-            const float e = restart[b] - y[b];
-            dr[b] = e * inv;
-            const float ce = logf(z) + m - s[t];
-            atomicAdd(loss, (w * ce + 0.5f * e * e) * inv);
+    __shared__ float4 sh[16][17];
+    const int col = threadIdx.x & 15, sl = threadIdx.x >> 4;
+    // rows of 64 outputs: W2 448, W3 448, W1 64 (tap * 8 + channel), W4 64
+    int row = blockIdx.x, ctas = a.c23, rows = kTaps * kC;
+    const float* p = a.p2;
+    int which = 2;
+    if (row >= 2 * kTaps * kC + 64) {
+        which = 4, row -= 2 * kTaps * kC + 64, p = a.p4, ctas = a.c4, rows = 64;
+    } else if (row >= 2 * kTaps * kC) {
+        which = 1, row -= 2 * kTaps * kC, p = a.p1, rows = 64;
+    } else if (row >= kTaps * kC) {
+        which = 3, row -= kTaps * kC, p = a.p3;
+    }
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = sl; c < ctas; c += 16) {
+        const float4 v = reinterpret_cast<const float4*>(p + ((int64_t)c * rows + row) * kC)[col];
+        s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+    }
+    sh[sl][col] = s;
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        const int o = threadIdx.x;
+        float t = 0.f;
+        for (int k = 0; k < 16; ++k) t += reinterpret_cast<const float*>(&sh[k][o >> 2])[o & 3];
+        if (which == 4) {
+            a.grad[oW4 + o * kC + row] = t;  // dW4[j][c]
+        } else if (which == 1) {
+            const int k = row >> 3, c = row & 7;
+            if (k < kTaps) {
+                a.grad[oW1 + (o * kCin + c) * kTaps + k] = t;
+                a.grad[oW1 + (o * kCin + c + 8) * kTaps + k] = 0.f;  // channels 8-15 carry no input
+            }
+        } else {
+            const int k = row / kC, c = row % kC;
+            a.grad[(which == 2 ? oW2 : oW3) + (o * kC + c) * kTaps + k] = t;
         }
     }
 }
 
-// Head backward: dh = bf16(w5 ds (h > 0)); dw5, db5, dw6, db6 accumulated.
-__global__ void head_back_kernel(const bf16* __restrict__ H, const float* __restrict__ pooled,
-                                 const bf16* __restrict__ wpk, const float* __restrict__ ds,
-                                 const float* __restrict__ dr, bf16* __restrict__ dH, float* __restrict__ grad,
-                                 int B, int n)
-{
-    const int P = rows_per_sample(n);
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-    float gw5a = 0.f, gw5b = 0.f, gw6a = 0.f, gw6b = 0.f, gb5 = 0.f, gb6 = 0.f;
-    const float w5a = __bfloat162float(wpk[pW5 + lane]), w5b = __bfloat162float(wpk[pW5 + lane + 32]);
-    for (int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < B; b += nw) {
-        const bf16* hb = H + b * P * kC;
-        bf16* db = dH + b * P * kC;
-        for (int p = 0; p < n; ++p) {
-            const float d = ds[b * n + p];
-            const float ha = __bfloat162float(hb[(int64_t)(p + 3) * kC + lane]);
-            const float hbv = __bfloat162float(hb[(int64_t)(p + 3) * kC + lane + 32]);
-            gw5a += ha * d;
-            gw5b += hbv * d;
-            if (lane == 0) gb5 += d;
-            db[(int64_t)(p + 3) * kC + lane] = __float2bfloat16_rn(ha > 0.f ? w5a * d : 0.f);
-            db[(int64_t)(p + 3) * kC + lane + 32] = __float2bfloat16_rn(hbv > 0.f ? w5b * d : 0.f);
-        }
-        const float r = dr[b];
-        gw6a += pooled[b * kC + lane] * r;
-        gw6b += pooled[b * kC + lane + 32] * r;
-        if (lane == 0) gb6 += r;
-    }
-    atomicAdd(grad + oW5 + lane, gw5a);
-    atomicAdd(grad + oW5 + lane + 32, gw5b);
-    atomicAdd(grad + oW6 + lane, gw6a);
-    atomicAdd(grad + oW6 + lane + 32, gw6b);
-    if (lane == 0) {
-        atomicAdd(grad + oB5, gb5);
-        atomicAdd(grad + oB6, gb6);
-    }
-}
-
-// bf16 operand copies of the float32 master weights.
+// Packed bf16 copies of the float32 master weights: element e of a layer's K x 64 operand is
+// K index 8 (e / 512) + e % 8 of output (e / 8) % 64.
 __global__ void pack_kernel(const float* __restrict__ prm, bf16* __restrict__ wpk)
 {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < kPacked; t += gridDim.x * blockDim.x) {
         float v;
-        if (t < pWf2) {  // Wf1[o][k*16+c] = W1[o][c][k]
-            const int o = t / (kTaps * kCin), kk = t % (kTaps * kCin), k = kk / kCin, c = kk % kCin;
+        if (t < pWf2) {  // Wf1: K index k*16+c, W1[o][c][k]
+            const int e = t - pWf1, o = (e >> 3) & 63, kk = 8 * (e >> 9) + (e & 7), k = kk / kCin, c = kk % kCin;
             v = prm[oW1 + (o * kCin + c) * kTaps + k];
-        } else if (t < pWf4) {  // Wf2 / Wf3
-            const int base = t < pWf3 ? oW2 : oW3, u = t - (t < pWf3 ? pWf2 : pWf3);
-            const int o = u / (kTaps * kC), kk = u % (kTaps * kC), k = kk / kC, c = kk % kC;
-            v = prm[base + (o * kC + c) * kTaps + k];
-        } else if (t < pWb2) {  // Wf4[j][c] = W4[j][c]
-            v = prm[oW4 + (t - pWf4)];
-        } else if (t < pWb4) {  // Wb[c][k'*64+o] = W[o][c][6-k']
-            const int base = t < pWb3 ? oW2 : oW3, u = t - (t < pWb3 ? pWb2 : pWb3);
-            const int c = u / (kTaps * kC), kk = u % (kTaps * kC), kr = kk / kC, o = kk % kC;
-            v = prm[base + (o * kC + c) * kTaps + (kTaps - 1 - kr)];
-        } else if (t < pW5) {  // Wb4[c][j] = W4[j][c]
-            const int u = t - pWb4, c = u / kC, j = u % kC;
+        } else if (t < pWf4) {  // Wf2 / Wf3: K index k*64+c
+            const int e = t - (t < pWf3 ? pWf2 : pWf3), o = (e >> 3) & 63, kk = 8 * (e >> 9) + (e & 7), k = kk / kC, c = kk % kC;
+            v = prm[(t < pWf3 ? oW2 : oW3) + (o * kC + c) * kTaps + k];
+        } else if (t < pWb2) {  // Wf4: K index c, W4[j][c]
+            const int e = t - pWf4, o = (e >> 3) & 63, c = 8 * (e >> 9) + (e & 7);
+            v = prm[oW4 + o * kC + c];
+        } else if (t < pWb4) {  // Wb2 / Wb3: outputs c, K index k'*64+o, W[o][c][6-k']
+            const int e = t - (t < pWb3 ? pWb2 : pWb3), c = (e >> 3) & 63, kk = 8 * (e >> 9) + (e & 7), kr = kk / kC, o = kk % kC;
+            v = prm[(t < pWb3 ? oW2 : oW3) + (o * kC + c) * kTaps + (kTaps - 1 - kr)];
+        } else if (t < pW5) {  // Wb4: outputs c, K index j, W4[j][c]
+            const int e = t - pWb4, c = (e >> 3) & 63, j = 8 * (e >> 9) + (e & 7);
             v = prm[oW4 + j * kC + c];
         } else if (t < pW6) {
             v = prm[oW5 + (t - pW5)];
@@ -594,133 +949,20 @@ __global__ void init_kernel(float* __restrict__ prm, uint64_t seed)
     }
 }
 
-// cuTensorMapEncodeTiled from the driver, looked up once through the runtime (the
-// library links no driver library of its own).
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_tiled()
-{
-    static std::once_flag once;
-    static EncodeTiledFn fn = nullptr;
-    std::call_once(once, [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(f);
-    });
-    return fn;
-}
-
-// Row-major BF16 matrix [outer][inner] (rows 2 inner bytes apart, a multiple of 16), read
-// in boxes of box_outer rows x box_inner values; reads outside the matrix give zeros.
-bool map_rows(CUtensorMap* m, const bf16* base, uint64_t inner, uint64_t outer, uint32_t box_inner,
-              uint32_t box_outer)
-{
-    const EncodeTiledFn fn = encode_tiled();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {inner, outer};
-    const cuuint64_t strides[1] = {inner * sizeof(bf16)};
-    const cuuint32_t box[2] = {box_inner, box_outer};
-    const cuuint32_t es[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16*>(base), dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-template <int CIN, int TAPS, int EPI>
-int launch_rows_tc(const bf16* in, const bf16* Wt, const float* bias, const bf16* mask, const float* pdr,
-                   const bf16* pw, bf16* out, int B, int n, int sms, int* err, cudaStream_t s)
-{
-    using S = TcShape<CIN, TAPS>;
-    const int64_t rows = (int64_t)B * rows_per_sample(n);
-    CUtensorMap ma, mw;
-    if (!map_rows(&ma, in, CIN, (uint64_t)rows, 8, S::ROWS) || !map_rows(&mw, Wt, S::KK, kC, 8, kC))
-        return LABS_ECUDA;
-    auto fn = rows_tc_kernel<CIN, TAPS, EPI>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM) != cudaSuccess)
-        return LABS_ECUDA;
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kTcThreads, S::SMEM) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    const int64_t tiles = (rows + kTcTile - 1) / kTcTile;
-    const int grid = (int)std::min<int64_t>(tiles, (int64_t)sms * per_sm);
-    fn<<<grid, kTcThreads, S::SMEM, s>>>(ma, mw, bias, mask, pdr, pw, out, n, rows, err);
-    return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
-}
-
-template <int CIN, int TAPS>
-int launch_wgrad_tc(const bf16* G, const bf16* IN, float* dW, float* part, int B, int n, int sms, int* err,
-                    cudaStream_t s)
-{
-    using S = WgShape<CIN, TAPS>;
-    const int64_t rows = (int64_t)B * rows_per_sample(n);
-    CUtensorMap mi, mg;
-    if (!map_rows(&mi, IN, CIN, (uint64_t)rows, 8, kWgRows) || !map_rows(&mg, G, kC, (uint64_t)rows, 8, kWgRows))
-        return LABS_ECUDA;
-    auto fn = wgrad_tc_kernel<CIN, TAPS>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM) != cudaSuccess)
-        return LABS_ECUDA;
-    const int ctas = sms * kWgCtasPerSm;
-    fn<<<ctas, kTcThreads, S::SMEM, s>>>(mi, mg, part, rows, err);
-    wgrad_reduce_kernel<CIN, TAPS><<<(S::KK * kC + 255) / 256, 256, 0, s>>>(part, ctas, dW);
-    return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
-}
-
 }  // namespace
 
 // Workspace carve-up for a batch of B states of n free variables.
 struct NetWs {
-    bf16 *X0, *A1, *A2, *A3, *H, *dH, *dA3, *dA2, *dA1, *wpk;
-    float *score, *restart, *pooled, *ds, *dr, *loss;
-    int* err;  // set by a tensor-core kernel whose copy or MMA wait gave up
-    float* part;  // per-CTA partial weight gradients
+    bf16 *X0, *A1, *A2, *dA3, *dA2, *wpk;
+    float *score, *restart, *loss;
+    int* err;  // set by a tensor-core kernel whose copy or product wait gave up
+    float *part1, *part2, *part3, *part4;  // per-CTA partial weight gradients
     size_t bytes;
 };
 
 static size_t align256(size_t x)
 {
     return (x + 255) & ~(size_t)255;
-}
-
-static int sm_count();
-
-NetWs carve(void* base, int64_t B, int n)
-{
-    NetWs w;
-    const size_t P = (size_t)rows_per_sample(n);
-    const size_t act = align256((size_t)B * P * kC * sizeof(bf16));
-    char* p = static_cast<char*>(base);
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        char* q = p ? p + off : nullptr;
-        off += align256(bytes);
-        return q;
-    };
-    w.X0 = (bf16*)take((size_t)B * P * kCin * sizeof(bf16));
-    w.A1 = (bf16*)take(act);
-    w.A2 = (bf16*)take(act);
-    w.A3 = (bf16*)take(act);
-    w.H = (bf16*)take(act);
-    w.dH = (bf16*)take(act);
-    w.dA3 = (bf16*)take(act);
-    w.dA2 = (bf16*)take(act);
-    w.dA1 = (bf16*)take(act);
-    w.wpk = (bf16*)take(kPacked * sizeof(bf16));
-    w.score = (float*)take((size_t)B * n * 4);
-    w.ds = (float*)take((size_t)B * n * 4);
-    w.restart = (float*)take((size_t)B * 4);
-    w.dr = (float*)take((size_t)B * 4);
-    w.pooled = (float*)take((size_t)B * kC * 4);
-    w.loss = (float*)take(4);
-    w.err = (int*)take(4);
-    // per-CTA partial weight gradients (the largest product's M tiles x 64 outputs)
-    w.part = (float*)take((size_t)sm_count() * kWgCtasPerSm * WgShape<kC, kTaps>::NT * 128 * kC * 4);
-    w.bytes = off;
-    return w;
 }
 
 static int sm_count()
@@ -731,66 +973,134 @@ static int sm_count()
     return sms > 0 ? sms : 1;
 }
 
-// Forward of a batch whose inputs are already in w.X0 (activations zeroed by the caller).
-int forward(const float* prm, const NetWs& w, int B, int n, cudaStream_t s)
+NetWs carve(void* base, int64_t B, int n)
 {
-    const int sms = sm_count();
-    pack_kernel<<<64, 256, 0, s>>>(prm, w.wpk);
-    int rc = launch_rows_tc<kCin, kTaps, EPI_BIAS_RELU>(w.X0, w.wpk + pWf1, prm + oB1, nullptr, nullptr, nullptr, w.A1,
-                                                        B, n, sms, w.err, s);
-    if (!rc) rc = launch_rows_tc<kC, kTaps, EPI_BIAS_RELU>(w.A1, w.wpk + pWf2, prm + oB2, nullptr, nullptr, nullptr,
-                                                           w.A2, B, n, sms, w.err, s);
-    if (!rc) rc = launch_rows_tc<kC, kTaps, EPI_BIAS_RELU>(w.A2, w.wpk + pWf3, prm + oB3, nullptr, nullptr, nullptr,
-                                                           w.A3, B, n, sms, w.err, s);
-    if (!rc) rc = launch_rows_tc<kC, 1, EPI_BIAS_RELU>(w.A3, w.wpk + pWf4, prm + oB4, nullptr, nullptr, nullptr, w.H,
-                                                       B, n, sms, w.err, s);
-    if (rc) return rc;
-    head_kernel<<<std::min(B, sms * 8), 128, 0, s>>>(w.H, w.A3, w.wpk, prm, w.score, w.pooled, w.restart, B, n);
+    NetWs w;
+    const size_t tiles = (size_t)tile_count(B, n), col = (size_t)(tile_rows(n) + 9) * 16, sms = (size_t)sm_count();
+    char* p = static_cast<char*>(base);
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* q = p ? p + off : nullptr;
+        off += align256(bytes);
+        return q;
+    };
+    w.X0 = (bf16*)take(tiles * col);
+    w.A1 = (bf16*)take(tiles * 8 * col);
+    w.A2 = (bf16*)take(tiles * 8 * col);
+    w.dA3 = (bf16*)take(tiles * 8 * col);
+    w.dA2 = (bf16*)take(tiles * 8 * col);
+    w.wpk = (bf16*)take(kPacked * sizeof(bf16));
+    w.score = (float*)take((size_t)B * n * 4);
+    w.restart = (float*)take((size_t)B * 4);
+    w.loss = (float*)take(4);
+    w.err = (int*)take(4);
+    w.part1 = (float*)take(sms * 64 * kC * 4);
+    w.part2 = (float*)take(sms * kTaps * kC * kC * 4);
+    w.part3 = (float*)take(sms * kTaps * kC * kC * 4);
+    w.part4 = (float*)take(sms * 2 * kC * kC * 4);
+    w.bytes = off;
+    return w;
+}
+
+template <class S>
+static int allow_smem(void (*fn)(FwdArgs))
+{
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM) == cudaSuccess ? LABS_OK : LABS_ECUDA;
+}
+
+template <int MT, bool TRAIN>
+static int launch_forward(const FwdArgs& a, int sms, cudaStream_t s)
+{
+    using S = FwdShape<MT, TRAIN>;
+    static_assert(S::SMEM <= 227 * 1024, "shared memory");
+    if (allow_smem<S>(net_forward_kernel<MT, TRAIN>)) return LABS_ECUDA;
+    const int grid = (int)std::min<int64_t>(tile_count(a.B, a.n), sms);
+    net_forward_kernel<MT, TRAIN><<<grid, S::THREADS, S::SMEM, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
 }
 
-int zero_acts(const NetWs& w, int B, int n, cudaStream_t s)
+template <int MT, bool FIRST>
+static int launch_conv_backward(const BwdArgs& a, int sms, cudaStream_t s)
 {
-    // X0 .. dA1 are contiguous at the start of the workspace
-    const size_t bytes = (size_t)((char*)w.wpk - (char*)w.X0);
-    return cudaMemsetAsync(w.X0, 0, bytes, s) == cudaSuccess ? LABS_OK : LABS_ECUDA;
+    using S = BwdShape<MT, FIRST>;
+    static_assert(S::SMEM <= 227 * 1024, "shared memory");
+    if (cudaFuncSetAttribute(conv_backward_kernel<MT, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM) !=
+        cudaSuccess)
+        return LABS_ECUDA;
+    const int grid = (int)std::min<int64_t>(a.tiles, sms);
+    conv_backward_kernel<MT, FIRST><<<grid, S::THREADS, S::SMEM, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
 }
 
-int backward(const float* prm, const NetWs& w, const int32_t* target, const float* y, const float* wf, float* grad,
-             int B, int n, cudaStream_t s)
+static FwdArgs forward_args(const float* prm, const float* x, const NetWs& w, int64_t B, int n, float* score, float* restart)
 {
-    const int sms = sm_count();
-    if (cudaMemsetAsync(grad, 0, kParams * sizeof(float), s) != cudaSuccess) return LABS_ECUDA;
-    if (cudaMemsetAsync(w.loss, 0, sizeof(float), s) != cudaSuccess) return LABS_ECUDA;
-    loss_kernel<<<std::min(B, sms * 8), 128, 0, s>>>(w.score, w.restart, target, y, wf, w.ds, w.dr, w.loss, B, n);
-    head_back_kernel<<<std::min(B, sms * 4), 128, 0, s>>>(w.H, w.pooled, w.wpk, w.ds, w.dr, w.dH, grad, B, n);
-    int rc = cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
-    // h = relu(W4 a3 + b4): dW4, db4, then da3 = (W4^T dh + w6 dr / n) * (a3 > 0)
-    if (!rc) rc = launch_wgrad_tc<kC, 1>(w.dH, w.A3, grad + oW4, w.part, B, n, sms, w.err, s);
-    colsum_kernel<<<sms * 4, 256, 0, s>>>(w.dH, grad + oB4, (int64_t)B * rows_per_sample(n));
-    if (!rc) rc = launch_rows_tc<kC, 1, EPI_MASK_POOL>(w.dH, w.wpk + pWb4, nullptr, w.A3, w.dr, w.wpk + pW6, w.dA3,
-                                                       B, n, sms, w.err, s);
-    // conv3
-    if (!rc) rc = launch_wgrad_tc<kC, kTaps>(w.dA3, w.A2, grad + oW3, w.part, B, n, sms, w.err, s);
-    colsum_kernel<<<sms * 4, 256, 0, s>>>(w.dA3, grad + oB3, (int64_t)B * rows_per_sample(n));
-    if (!rc) rc = launch_rows_tc<kC, kTaps, EPI_MASK>(w.dA3, w.wpk + pWb3, nullptr, w.A2, nullptr, nullptr, w.dA2, B,
-                                                      n, sms, w.err, s);
-    // conv2
-    if (!rc) rc = launch_wgrad_tc<kC, kTaps>(w.dA2, w.A1, grad + oW2, w.part, B, n, sms, w.err, s);
-    colsum_kernel<<<sms * 4, 256, 0, s>>>(w.dA2, grad + oB2, (int64_t)B * rows_per_sample(n));
-    if (!rc) rc = launch_rows_tc<kC, kTaps, EPI_MASK>(w.dA2, w.wpk + pWb2, nullptr, w.A1, nullptr, nullptr, w.dA1, B,
-                                                      n, sms, w.err, s);
-    // conv1
-    if (!rc) rc = launch_wgrad_tc<kCin, kTaps>(w.dA1, w.X0, grad + oW1, w.part, B, n, sms, w.err, s);
-    colsum_kernel<<<sms * 4, 256, 0, s>>>(w.dA1, grad + oB1, (int64_t)B * rows_per_sample(n));
+    FwdArgs a{};
+    a.x = x;
+    a.wpk = w.wpk;
+    a.prm = prm;
+    a.score = score;
+    a.restart = restart;
+    a.err = w.err;
+    a.B = B;
+    a.n = n;
+    return a;
+}
+
+int pack(const float* prm, const NetWs& w, cudaStream_t s)
+{
+    pack_kernel<<<4 * sm_count(), 256, 0, s>>>(prm, w.wpk);
+    return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
+}
+
+int forward(const float* prm, const float* x, const NetWs& w, int64_t B, int n, float* score, float* restart, cudaStream_t s)
+{
+    int rc = pack(prm, w, s);
+    if (rc) return rc;
+    const FwdArgs a = forward_args(prm, x, w, B, n, score, restart);
+    return n <= 128 ? launch_forward<1, false>(a, sm_count(), s) : launch_forward<2, false>(a, sm_count(), s);
+}
+
+template <int MT>
+static int gradients_tiles(FwdArgs a, const NetWs& w, float* grad, int sms, cudaStream_t s)
+{
+    int rc = launch_forward<MT, true>(a, sms, s);
+    const int64_t tiles = tile_count(a.B, a.n);
+    BwdArgs b{};
+    b.err = w.err;
+    b.tiles = tiles;
+    b.B = a.B;
+    b.n = a.n;
+    b.G = w.dA3, b.IN = w.A2, b.wb = w.wpk + pWb3, b.dIN = w.dA2, b.part = w.part3, b.db = grad + oB2;
+    if (!rc) rc = launch_conv_backward<MT, false>(b, sms, s);
+    b.G = w.dA2, b.IN = w.A1, b.X0 = w.X0, b.wb = w.wpk + pWb2, b.dIN = nullptr, b.part = w.part2, b.part1 = w.part1;
+    b.db = grad + oB1;
+    if (!rc) rc = launch_conv_backward<MT, true>(b, sms, s);
+    const int ctas = (int)std::min<int64_t>(tiles, sms);
+    const ReduceArgs r{w.part1, w.part2, w.part3, w.part4, ctas, ctas * FwdShape<MT, true>::NG, grad};
+    wgrad_reduce_kernel<<<2 * kTaps * kC + 128, 256, 0, s>>>(r);
     if (!rc && cudaGetLastError() != cudaSuccess) rc = LABS_ECUDA;
     return rc;
 }
 
-int load_inputs(const float* x, const NetWs& w, int B, int n, cudaStream_t s)
+int gradients(const float* prm, const float* x, const NetWs& w, const int32_t* target, const float* y, const float* wf,
+              float* grad, int64_t B, int n, cudaStream_t s)
 {
-    input_kernel<<<std::min<int64_t>(((int64_t)B * n * 3 + 255) / 256, sm_count() * 16), 256, 0, s>>>(x, w.X0, B, n);
-    return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
+    if (cudaMemsetAsync(grad, 0, kParams * sizeof(float), s) != cudaSuccess) return LABS_ECUDA;
+    if (cudaMemsetAsync(w.loss, 0, sizeof(float), s) != cudaSuccess) return LABS_ECUDA;
+    const int rc = pack(prm, w, s);
+    if (rc) return rc;
+    FwdArgs a = forward_args(prm, x, w, B, n, w.score, w.restart);
+    a.target = target;
+    a.y = y;
+    a.wf = wf;
+    a.X0 = w.X0;
+    a.A1 = w.A1;
+    a.A2 = w.A2;
+    a.dA3 = w.dA3;
+    a.part4 = w.part4;
+    a.grad = grad;
+    a.loss = w.loss;
+    return n <= 128 ? gradients_tiles<1>(a, w, grad, sm_count(), s) : gradients_tiles<2>(a, w, grad, sm_count(), s);
 }
 
 int init_params(float* prm, uint64_t seed, cudaStream_t s)
@@ -820,10 +1130,7 @@ int net_forward_ws(const float* params, const float* x, int64_t B, int n, void* 
                    const float** restart, void* stream)
 {
     const net::NetWs w = net::carve(ws, B, n);
-    cudaStream_t s = (cudaStream_t)stream;
-    int rc = net::zero_acts(w, (int)B, n, s);
-    if (!rc) rc = net::load_inputs(x, w, (int)B, n, s);
-    if (!rc) rc = net::forward(params, w, (int)B, n, s);
+    const int rc = net::forward(params, x, w, B, n, w.score, w.restart, (cudaStream_t)stream);
     if (scores) *scores = w.score;
     if (restart) *restart = w.restart;
     return rc;
@@ -858,15 +1165,8 @@ int labs_net_forward(const float* dev_params, const float* dev_x, int64_t batch,
     if (batch == 0) return LABS_OK;
     const net::NetWs w = net::carve(dev_ws, batch, n);
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
-    cudaStream_t s = (cudaStream_t)cuda_stream;
-    int rc = net::zero_acts(w, (int)batch, n, s);
-    if (!rc) rc = net::load_inputs(dev_x, w, (int)batch, n, s);
-    if (!rc) rc = net::forward(dev_params, w, (int)batch, n, s);
-    if (!rc && dev_scores)
-        rc = cudaMemcpyAsync(dev_scores, w.score, (size_t)batch * n * 4, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
-    if (!rc && dev_restart)
-        rc = cudaMemcpyAsync(dev_restart, w.restart, (size_t)batch * 4, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
-    return rc;
+    return net::forward(dev_params, dev_x, w, batch, n, dev_scores ? dev_scores : w.score,
+                        dev_restart ? dev_restart : w.restart, (cudaStream_t)cuda_stream);
 }
 
 int labs_net_gradients(const float* dev_params, const float* dev_x, const int32_t* dev_target, const float* dev_y,
@@ -880,10 +1180,7 @@ int labs_net_gradients(const float* dev_params, const float* dev_x, const int32_
     const net::NetWs w = net::carve(dev_ws, batch, n);
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    int rc = net::zero_acts(w, (int)batch, n, s);
-    if (!rc) rc = net::load_inputs(dev_x, w, (int)batch, n, s);
-    if (!rc) rc = net::forward(dev_params, w, (int)batch, n, s);
-    if (!rc) rc = net::backward(dev_params, w, dev_target, dev_y, dev_wf, dev_grads, (int)batch, n, s);
+    int rc = net::gradients(dev_params, dev_x, w, dev_target, dev_y, dev_wf, dev_grads, batch, n, s);
     if (!rc && dev_loss) rc = cudaMemcpyAsync(dev_loss, w.loss, 4, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
     return rc;
 }
