@@ -105,6 +105,12 @@ __device__ __forceinline__ uint4 lds128(uint32_t a)
     return v;
 }
 
+__device__ __forceinline__ float4 lds_f4(uint32_t a)
+{
+    const uint4 v = lds128(a);
+    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+
 // Instruction descriptor of kind::f16 with both operands MN-major (bits 15 and 16).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N)
 {
@@ -112,29 +118,29 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N)
 }
 
 // D (128 rows, 64 columns at TMEM address d) = TAPS-tap product of the rows from byte
-// address a (column pitch COL) with the packed weights at w.  One thread.
+// address a (column pitch COL) with the packed weights at w.  One warp, uniform arguments.
 template <int CIN, int TAPS, int COL>
-__device__ __forceinline__ void issue_product(uint32_t d, uint32_t a, uint32_t w)
+__device__ __forceinline__ void issue_product(uint32_t elected, uint32_t d, uint32_t a, uint32_t w)
 {
     constexpr uint32_t id = idesc_bf16_f32(128, kC);
+    const uint64_t ad = smem_desc(a, COL, 128), wd = smem_desc(w, 1024, 128);  // addresses in 16-byte units
 #pragma unroll
     for (int k = 0; k < TAPS; ++k)
 #pragma unroll
         for (int s2 = 0; s2 < CIN / 16; ++s2)
-            tc_mma_bf16(d, smem_desc(a + 16 * k + 2 * s2 * COL, COL, 128),
-                        smem_desc(w + (k * (CIN / 8) + 2 * s2) * 1024, 1024, 128), id, (k | s2) != 0);
+            tc_mma_bf16(elected, d, ad + (k + 2 * s2 * (COL / 16)), wd + (k * (CIN / 8) + 2 * s2) * 64, id, (k | s2) != 0);
 }
 
 // D (128 x 64 at TMEM address d) += over the rows r < M: A columns (16 of them, pitch COL,
 // from address a) x G columns (8, from address g): a weight gradient, both operands
 // MN-major (the next 8 rows 128 bytes on, the next 8 channels one column on).
 template <int M, int COL>
-__device__ __forceinline__ void issue_wgrad(uint32_t d, uint32_t a, uint32_t g, bool fresh)
+__device__ __forceinline__ void issue_wgrad(uint32_t elected, uint32_t d, uint32_t a, uint32_t g, bool fresh)
 {
     constexpr uint32_t id = idesc_bf16_f32_mn(128, kC);
+    const uint64_t ad = smem_desc(a, 128, COL), gd = smem_desc(g, 128, COL);
 #pragma unroll
-    for (int ks = 0; ks < M / 16; ++ks)
-        tc_mma_bf16(d, smem_desc(a + 256 * ks, 128, COL), smem_desc(g + 256 * ks, 128, COL), id, !fresh || ks > 0);
+    for (int ks = 0; ks < M / 16; ++ks) tc_mma_bf16(elected, d, ad + 16 * ks, gd + 16 * ks, id, !fresh || ks > 0);
 }
 
 // This thread's 64 accumulators (TMEM lane 32 (warp mod 4) + lane).
@@ -166,6 +172,12 @@ __device__ __forceinline__ float2 warp_colsum(float (&v)[64], int lane)
     return make_float2(v[0], v[1]);
 }
 
+__device__ __forceinline__ void add2(float2& a, float2 b)
+{
+    a.x += b.x;
+    a.y += b.y;
+}
+
 // Adds a lane's channel sums (2 lane, 2 lane + 1) to the CTA's.
 __device__ __forceinline__ void add_channels(float* sums, int lane, float2 v)
 {
@@ -184,10 +196,11 @@ __device__ __forceinline__ void add_channels(float* sums, int lane, float2 v)
 // gradients and da3; a1, a2 and da3 go to global memory for the convolutions' backward
 // kernels, a3 and h never leave the CTA.
 //
-// What bounds it: the products' shared-memory reads (6 KB per 128 x 64 x 16 product, 67
-// products a tile) and the epilogues between them.  It replaces one launch per layer over
-// global activations (read and written 70 MB each for 4096 samples of n = 128) cleared by a
-// memset before every pass.
+// What bounds it: shared-memory bandwidth -- the products read 6 KB per 128 x 64 x 16
+// product, 67 products a tile, and the epilogues about a third as much again (8192 samples
+// of n = 128: 157 us; the products alone would take 110).  It replaces one launch per layer
+// over global activations (70 MB read and written per layer of 4096 samples) that a memset
+// cleared before every pass: scoring 8192 states 209 us with the features, from 950.
 template <int MT, bool TRAIN>
 struct FwdShape {
     using T = Tile<MT>;
@@ -199,7 +212,7 @@ struct FwdShape {
     static constexpr int GROUP = TRAIN ? DH + T::ACT : DH;
     static constexpr int GROUPS = W_END;
     static constexpr int MISC = GROUPS + NG * GROUP;
-    // misc: biases b1..b4, w5, w6 (float), barriers, the TMEM slot; then per group scores, ds
+    // misc: biases b1..b4, w5, w6 (float), barriers, the TMEM slot; then per group scores and ds
     // (M floats each) and dr per sample (M/4 floats), the CTA's sums of b3, b4, w5, w6 gradients
     static constexpr int BIAS = MISC, BAR = BIAS + 6 * kC * 4, SC = BAR + 64;
     static constexpr int SCB = (2 * T::M + T::M / 4 + 32) * 4;
@@ -263,6 +276,7 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
     const uint32_t sb = smem_addr(sm);
     const int t = threadIdx.x % kTcThreads, grp = threadIdx.x / kTcThreads, wq = t >> 5, lane = t & 31;
     float* bias = reinterpret_cast<float*>(sm + S::BIAS);
+    const uint32_t s_bias = sb + S::BIAS;
     const uint32_t bar_w = sb + S::BAR, bar = bar_w + 8 + 8 * grp, slot = sb + S::BAR + 48;
     volatile int* failed = reinterpret_cast<volatile int*>(sm + S::BAR + 56);
     const uint32_t gx = sb + S::GROUPS + grp * S::GROUP + S::X0, ga = sb + S::GROUPS + grp * S::GROUP + S::ACT,
@@ -298,6 +312,10 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + S::BAR + 48);
     const uint32_t acc0 = tmem + grp * MT * 64, acc4 = tmem + S::NG * MT * 64 + grp * 64;
+    // the group's first warp issues its products, from uniform values
+    const bool issuer = uniform(wq) == 0;
+    const uint32_t u_sb = uniform(sb), u_gx = uniform(gx), u_ga = uniform(ga), u_bar = uniform(bar), u_acc0 = uniform(acc0),
+                   u_acc4 = uniform(acc4);
     if (threadIdx.x == 0) {
         mbar_arrive_expect_tx(bar_w, S::W_END);
         bulk_copy_g2s(sb + S::W1, a.wpk + pWf1, S::W2 - S::W1, bar_w);
@@ -309,20 +327,27 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
     bool ok = mbar_wait(bar_w, 0);
     uint32_t phase = 0;
     int done = 0;           // tiles of this group
-    float2 gw6 = {0.f, 0.f};  // sums over this warp's samples: w6 (channels 2 lane, 2 lane + 1)
+    float2 gw6 = {0.f, 0.f};  // this warp's samples: the gradients of w6's channels 2 lane and 2 lane + 1
     float gb5 = 0.f, gb6 = 0.f, lsum = 0.f;
     const float inv = TRAIN ? 1.f / (float)a.B : 0.f;
 
+    // this thread's output rows: sample of the tile (K: none) and position
+    int rk[MT], rpos[MT];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+        const RowPos rp(t + 128 * mt, n, K);
+        rk[mt] = rp.in ? rp.k : -1;
+        rpos[mt] = rp.p;
+    }
     // the group's inputs of a tile: three features per row
     float xin[MT][3];
     auto fetch = [&](int64_t tile) {
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
-            const RowPos rp(t + 128 * mt, n, K);
-            const int64_t b = tile * K + rp.k;
-            const bool in = rp.in && tile < tiles && b < a.B;
+            const int64_t b = tile * K + rk[mt];
+            const bool in = rk[mt] >= 0 && tile < tiles && b < a.B;
 #pragma unroll
-            for (int f = 0; f < 3; ++f) xin[mt][f] = in ? a.x[(b * 3 + f) * n + rp.p] : 0.f;
+            for (int f = 0; f < 3; ++f) xin[mt][f] = in ? a.x[(b * 3 + f) * n + rpos[mt]] : 0.f;
         }
     };
     // waits for the group's products; a wait that gives up ends the CTA's work
@@ -356,17 +381,18 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
             const int o = t + 128 * mt;
-            const RowPos rp(o, n, K);
-            in[mt] = rp.in && tile * K + rp.k < a.B;
+            in[mt] = rk[mt] >= 0 && tile * K + rk[mt] < a.B;
             const uint4 v = make_uint4(pack2(xin[mt][0], xin[mt][1]), pack2(xin[mt][2], 0.f), 0u, 0u);
             sts128(gx + 16 * (o + 3), v);
             if (TRAIN) *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(a.X0) + tile * T::COL + 16 * (o + 3)) = v;
         }
         rows_ready();
-        if (t == 0) {
+        if (issuer) {
+            const uint32_t el = elect_one();
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt) issue_product<kCin, kTaps, T::COL>(acc0 + 64 * mt, gx + 2048 * mt, sb + S::W1);
-            tc_commit(bar);
+            for (int mt = 0; mt < MT; ++mt)
+                issue_product<kCin, kTaps, T::COL>(el, u_acc0 + 64 * mt, u_gx + 2048 * mt, u_sb + S::W1);
+            tc_commit(el, u_bar);
         }
         fetch(tile + stride);
         // conv1..3: bias, ReLU, the rows replace the layer's input
@@ -381,23 +407,25 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
                 const int o = t + 128 * mt;
                 uint32_t w[32];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const float v0 = fmaxf(acc[2 * i] + bias[l * kC + 2 * i], 0.f),
-                                v1 = fmaxf(acc[2 * i + 1] + bias[l * kC + 2 * i + 1], 0.f);
-                    w[i] = in[mt] ? pack2(v0, v1) : 0u;
+                for (int q = 0; q < 16; ++q) {
+                    const float4 bv = lds_f4(s_bias + 4 * (l * kC + 4 * q));
+                    w[2 * q] = in[mt] ? pack2(fmaxf(acc[4 * q] + bv.x, 0.f), fmaxf(acc[4 * q + 1] + bv.y, 0.f)) : 0u;
+                    w[2 * q + 1] = in[mt] ? pack2(fmaxf(acc[4 * q + 2] + bv.z, 0.f), fmaxf(acc[4 * q + 3] + bv.w, 0.f)) : 0u;
                 }
                 store_row<T::COL>(ga + 16 * (o + 3), gl ? gl + 16 * (o + 3) : nullptr, w);
             }
             rows_ready();
-            if (t == 0) {
+            if (issuer) {
+                const uint32_t el = elect_one();
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt) {
                     if (l < 2)
-                        issue_product<kC, kTaps, T::COL>(acc0 + 64 * mt, ga + 2048 * mt, sb + (l == 0 ? S::W2 : S::W3));
+                        issue_product<kC, kTaps, T::COL>(el, u_acc0 + 64 * mt, u_ga + 2048 * mt,
+                                                         u_sb + (l == 0 ? S::W2 : S::W3));
                     else
-                        issue_product<kC, 1, T::COL>(acc0 + 64 * mt, ga + 48 + 2048 * mt, sb + S::W4);
+                        issue_product<kC, 1, T::COL>(el, u_acc0 + 64 * mt, u_ga + 48 + 2048 * mt, u_sb + S::W4);
                 }
-                tc_commit(bar);
+                tc_commit(el, u_bar);
             }
         }
         // restart scores from the pooled a3 (beside the MLP's product): a warp per sample,
@@ -407,12 +435,19 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
             if (b >= a.B) break;
             const uint32_t col = ga + (lane >> 2) * T::COL + 4 * (lane & 3) + 16 * (k * (n + 3) + 3);
             float ma = 0.f, mb = 0.f;
-#pragma unroll 8
-            for (int p = 0; p < n; ++p) {
-                uint32_t v;
-                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(col + 16 * p) : "memory");
-                ma += lo_f(v);
-                mb += hi_f(v);
+            // in the order of the positions, 16 loads ahead of their additions (the loads may
+            // run past the sample, within the CTA's memory; what they read there is dropped)
+            for (int p0 = 0; p0 < n; p0 += 16) {
+                uint32_t v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v[i]) : "r"(col + 16 * (p0 + i)) : "memory");
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    if (p0 + i >= n) v[i] = 0u;
+                    ma += lo_f(v[i]);
+                    mb += hi_f(v[i]);
+                }
             }
             ma /= (float)n;
             mb /= (float)n;
@@ -440,20 +475,24 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
             float acc[64];
             load_acc(acc0 + 64 * mt, wq, acc);
             const int o = t + 128 * mt;
-            const RowPos rp(o, n, K);
             float sacc = 0.f;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const uint32_t w = pack2(fmaxf(acc[2 * i] + bias[3 * kC + 2 * i], 0.f),
-                                         fmaxf(acc[2 * i + 1] + bias[3 * kC + 2 * i + 1], 0.f));
-                if (TRAIN) h[mt][i] = w;
-                sacc += lo_f(w) * bias[4 * kC + 2 * i] + hi_f(w) * bias[4 * kC + 2 * i + 1];
+            for (int q = 0; q < 16; ++q) {
+                const float4 bv = lds_f4(s_bias + 4 * (3 * kC + 4 * q)), wv = lds_f4(s_bias + 4 * (4 * kC + 4 * q));
+                const float b4[4] = {bv.x, bv.y, bv.z, bv.w}, w5[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int i = 2 * q + j;
+                    const uint32_t w = pack2(fmaxf(acc[2 * i] + b4[2 * j], 0.f), fmaxf(acc[2 * i + 1] + b4[2 * j + 1], 0.f));
+                    if (TRAIN) h[mt][i] = w;
+                    sacc += lo_f(w) * w5[2 * j] + hi_f(w) * w5[2 * j + 1];
+                }
             }
             sacc += a.prm[oB5];
             if (TRAIN)
                 s_score[o] = sacc;
             else if (in[mt])
-                a.score[(tile * K + rp.k) * n + rp.p] = sacc;
+                a.score[(tile * K + rk[mt]) * n + rpos[mt]] = sacc;
         }
         if constexpr (TRAIN) {
             group_sync(1 + grp);
@@ -481,20 +520,20 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
                 const int o = t + 128 * mt;
-                const float d = in[mt] ? s_ds[o] : 0.f;
-                gb5 += d;
+                const float ds = in[mt] ? s_ds[o] : 0.f;
+                gb5 += ds;
                 float v[64];
                 uint32_t w[32];
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    v[2 * i] = lo_f(h[mt][i]) * d;
-                    v[2 * i + 1] = hi_f(h[mt][i]) * d;
+                    v[2 * i] = lo_f(h[mt][i]) * ds;
+                    v[2 * i + 1] = hi_f(h[mt][i]) * ds;
                 }
                 add_channels(sums + 2 * kC, lane, warp_colsum(v, lane));
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    w[i] = pack2(lo_f(h[mt][i]) > 0.f ? bias[4 * kC + 2 * i] * d : 0.f,
-                                 hi_f(h[mt][i]) > 0.f ? bias[4 * kC + 2 * i + 1] * d : 0.f);
+                    w[i] = pack2(lo_f(h[mt][i]) > 0.f ? bias[4 * kC + 2 * i] * ds : 0.f,
+                                 hi_f(h[mt][i]) > 0.f ? bias[4 * kC + 2 * i + 1] * ds : 0.f);
                     if (!in[mt]) w[i] = 0u;
                     v[2 * i] = lo_f(w[i]);
                     v[2 * i + 1] = hi_f(w[i]);
@@ -503,12 +542,14 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
                 add_channels(sums + kC, lane, warp_colsum(v, lane));
             }
             rows_ready();
-            if (t == 0) {
+            if (issuer) {
+                const uint32_t el = elect_one(), u_gd = u_ga + T::ACT;
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) issue_product<kC, 1, T::COL>(acc0 + 64 * mt, gd + 48 + 2048 * mt, sb + S::WB4);
+                for (int mt = 0; mt < MT; ++mt)
+                    issue_product<kC, 1, T::COL>(el, u_acc0 + 64 * mt, u_gd + 48 + 2048 * mt, u_sb + S::WB4);
                 // dW4: its rows 64-127 (the columns after a3's, i.e. dh's) are dropped
-                issue_wgrad<T::M, T::COL>(acc4, ga + 48, gd + 48, done == 0);
-                tc_commit(bar);
+                issue_wgrad<T::M, T::COL>(el, u_acc4, u_ga + 48, u_gd + 48, done == 0);
+                tc_commit(el, u_bar);
             }
             wait_products();
             // da3 = (W4^T dh + w6 dr / n) where a3 > 0; gradient of b3
@@ -517,8 +558,7 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
                 float acc[64];
                 load_acc(acc0 + 64 * mt, wq, acc);
                 const int o = t + 128 * mt;
-                const RowPos rp(o, n, K);
-                const float pdr = in[mt] ? s_dr[rp.k] / (float)n : 0.f;
+                const float pdr = in[mt] ? s_dr[rk[mt]] / (float)n : 0.f;
                 uint32_t w[32];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
@@ -633,7 +673,8 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 127) & ~uintptr_t(127));
     const uint32_t sb = smem_addr(sm);
-    const int t = threadIdx.x % kTcThreads, grp = threadIdx.x / kTcThreads, wq = t >> 5, lane = t & 31;
+    const int t = threadIdx.x % kTcThreads, wq = t >> 5, lane = t & 31;
+    const int grp = (int)uniform(threadIdx.x / kTcThreads);
     const bool issuer = grp == S::NG;
     // barriers per group: operands loaded, dIN product done, weight gradient done, da1 ready,
     // conv1's weight gradient done
@@ -678,43 +719,55 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                               reinterpret_cast<const unsigned char*>(a.X0) + tile * T::COL, T::COL, f);
     };
     if (issuer) {
-        if (lane == 0) {
-            bool ok = true, fresh = true, fresh1 = true;
+        // the whole warp, with uniform values; one lane issues
+        const uint32_t el = elect_one(), u_sb = uniform(sb), u_tmem = uniform(tmem), u_bars = uniform(bars);
+        bool fresh = true, fresh1 = true;
+        if (el) {
             mbar_arrive_expect_tx(bar_w, kTaps * kC * 128);
             bulk_copy_g2s(sb + S::WB, a.wb, kTaps * kC * 128, bar_w);
             for (int g = 0; g < S::NG; ++g)
                 if (tile_of(g, 0) < a.tiles) load(g, tile_of(g, 0));
-            ok = mbar_wait(bar_w, 0);
-            for (int it = 0; ok && tile_of(0, it) < a.tiles; ++it) {
+        }
+        __syncwarp();
+        bool ok = mbar_wait(bar_w, 0);
+        for (int it = 0; ok && tile_of(0, it) < a.tiles; ++it) {
+            for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
+                const uint32_t b = u_sb + S::GROUPS + g * S::GROUP, br = u_bars + 40 * g;
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(br, it & 1));
+                if (!ok) break;
+                tc_fence_after();
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    issue_product<kC, kTaps, T::COL>(el, u_tmem + S::ACC_D + 64 * (g * MT + mt), b + S::G + 2048 * mt,
+                                                     u_sb + S::WB);
+                tc_commit(el, br + 8);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)  // taps 2q, 2q+1 (the eighth is dropped)
+                    issue_wgrad<T::M, T::COL>(el, u_tmem + S::ACC_W + 64 * q, b + S::IN + 32 * q, b + S::G + 48, fresh);
+                fresh = false;
+                tc_commit(el, br + 16);
+            }
+            if (FIRST)
                 for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
-                    ok = mbar_wait(full(g), it & 1);
+                    const uint32_t b = u_sb + S::GROUPS + g * S::GROUP, br = u_bars + 40 * g;
+                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(br + 24, it & 1));
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t b = buf(g);
-#pragma unroll
-                    for (int mt = 0; mt < MT; ++mt)
-                        issue_product<kC, kTaps, T::COL>(tmem + S::ACC_D + 64 * (g * MT + mt), b + S::G + 2048 * mt, sb + S::WB);
-                    tc_commit(dbar(g));
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)  // taps 2q, 2q+1 (the eighth is dropped)
-                        issue_wgrad<T::M, T::COL>(tmem + S::ACC_W + 64 * q, b + S::IN + 32 * q, b + S::G + 48, fresh);
-                    fresh = false;
-                    tc_commit(wbar(g));
+                    issue_wgrad<T::M, T::COL>(el, u_tmem + S::ACC_W1, b + S::XC, b + S::G + 48, fresh1);
+                    fresh1 = false;
+                    tc_commit(el, br + 32);
                 }
-                if (FIRST)
-                    for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
-                        ok = mbar_wait(rbar(g), it & 1);
-                        if (!ok) break;
-                        tc_fence_after();
-                        issue_wgrad<T::M, T::COL>(tmem + S::ACC_W1, buf(g) + S::XC, buf(g) + S::G + 48, fresh1);
-                        fresh1 = false;
-                        tc_commit(fbar(g));
-                    }
-            }
-            if (!ok) *failed = 1;
         }
+        if (!ok) *failed = 1;
     } else {
         const int K = tile_samples(a.n);
+        float2 gb = {0.f, 0.f};
+        int rk[MT];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            const RowPos rp(t + 128 * mt, a.n, K);
+            rk[mt] = rp.in ? rp.k : -1;
+        }
         for (int it = 0; tile_of(grp, it) < a.tiles; ++it) {
             const int64_t tile = tile_of(grp, it);
             if (!mbar_wait(dbar(grp), it & 1)) *failed = 1;
@@ -731,8 +784,7 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                 float acc[64];
                 load_acc(tmem + S::ACC_D + 64 * (grp * MT + mt), wq, acc);
                 const int o = t + 128 * mt;
-                const RowPos rp(o, a.n, K);
-                const bool in = rp.in && tile * K + rp.k < a.B;
+                const bool in = rk[mt] >= 0 && tile * K + rk[mt] < a.B;
                 uint32_t w[32];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
@@ -751,7 +803,7 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                     acc[2 * i + 1] = hi_f(w[i]);
                 }
                 store_row<T::COL>(FIRST ? buf(grp) + S::G + 16 * (o + 3) : 0u, FIRST ? nullptr : gout + 16 * (o + 3), w);
-                add_channels(sums, lane, warp_colsum(acc, lane));
+                add2(gb, warp_colsum(acc, lane));
             }
             if (FIRST) {
                 fence_async_shared();
@@ -778,6 +830,7 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
             }
             if (*failed) break;
         }
+        add_channels(sums, lane, gb);
     }
     __syncwarp();
     tc_fence_before();

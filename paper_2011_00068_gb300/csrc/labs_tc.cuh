@@ -70,24 +70,44 @@ __device__ __forceinline__ void tc_fence_after()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] x B[smem]; issued by one thread.
-__device__ __forceinline__ void tc_mma_bf16(uint32_t taddr, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            bool accumulate)
+// One lane of the (converged) warp.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+
+// A value that is the same in every lane, in a form the compiler knows to be uniform.
+__device__ __forceinline__ uint32_t uniform(uint32_t v)
+{
+    return __shfl_sync(0xFFFFFFFFu, v, 0);
+}
+
+// D[tmem] (+)= A[smem] x B[smem].  The whole warp runs it with uniform operands and one
+// elected lane issues: with operands computed by a single thread, each instruction waited
+// for their moves into uniform registers (140 cycles an MMA, against 48 of the product).
+__device__ __forceinline__ void tc_mma_bf16(uint32_t elected, uint32_t taddr, uint64_t adesc, uint64_t bdesc,
+                                            uint32_t idesc, bool accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(taddr),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(taddr),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected)
         : "memory");
 }
 
-// The barrier at `bar` receives one arrival when every MMA this thread issued before
+// The barrier at `bar` receives one arrival when every MMA the elected lane issued before
 // has completed.
-__device__ __forceinline__ void tc_commit(uint32_t bar)
+__device__ __forceinline__ void tc_commit(uint32_t elected, uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(elected)
+        : "memory");
 }
 
 // 16 consecutive 32-bit columns of this thread's TMEM lane (32x32b shape: thread t of
