@@ -1341,61 +1341,6 @@ __device__ __forceinline__ void lane_keys(const View& V, int n, const Outs<LG, R
     for (int r = 0; r < R; ++r) key[r] = r < rv ? (db[r] << 8) + i0 + 2u * r : 0xFFFFFFFFu;
 }
 
-// The lane's two lowest keys above `floor` (0xFFFFFFFF where there are fewer).
-template <int R>
-__device__ __forceinline__ void top2_above(const unsigned (&key)[R], unsigned floor, unsigned& b1, unsigned& b2)
-{
-    b1 = 0xFFFFFFFFu;
-    b2 = 0xFFFFFFFFu;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const unsigned k = key[r] > floor ? key[r] : 0xFFFFFFFFu;
-        b2 = min(b2, max(b1, k));
-        b1 = min(b1, k);
-    }
-}
-
-// Removes free variable j from the lane's candidates (key `none`) when it is one of the
-// lane's outputs; j < 0: none.  The lockstep steps drop the move back to the previous
-// state this way: that state is in HT (every state of the walk since the last start
-// was inserted, and a failed insertion restarts the walker), so the probe would find
-// it visited, and leaving it out changes no choice while it saves most second rounds.
-template <class LG, int R, class K>
-__device__ __forceinline__ void drop_candidate(K (&key)[R], int j, const Outs<LG, R>& o, K none)
-{
-    const int d = (j >> 1) - o.v0;
-    const bool mine = j >= 0 && (j & 1) == o.p;
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (mine && d == r) key[r] = none;
-}
-
-// Full probe of f for the walkers (halves) with need set: every lane runs the same rounds.
-template <class LG>
-__device__ __forceinline__ Probe lockstep_probe_full(const WalkEnv& env, uint64_t f, uint32_t gen, int cap, bool need,
-                                                     const LG& t)
-{
-    const uint64_t tag = (f & ~kGenMask) | gen;
-    Probe pr{false, -1};
-    bool found = false;
-    for (int s0 = 0; s0 < cap; s0 += LG::kSize) {
-        const int s = s0 + t.lane;
-        uint64_t e = 0;
-        const bool live = need && !found && s < cap;
-        if (live) e = env.T[(f + (uint64_t)s) & env.tmask];
-        const bool match = e == tag;
-        const unsigned bal = t.ballot(live && (((e & kGenMask) != gen) || match));
-        const int fl = bal ? __ffs(bal) - 1 : 0;
-        const bool vis = t.shfl(match ? 1 : 0, fl) != 0;
-        if (bal && !found) {
-            found = true;
-            pr.visited = vis;
-            pr.slot = (int64_t)((f + (uint64_t)(s0 + fl)) & env.tmask);
-        }
-    }
-    return pr;
-}
-
 // Flips free variable best_i (and its mirror) in the walker's rows, even-lag table and
 // P, all from the values before the flip, when `moves` (the lanes of a walker without a
 // move rewrite unchanged values).  The rows are padded so that no read or write needs a
@@ -1471,9 +1416,6 @@ __device__ __forceinline__ int target_isl(const KParams& p, int L)
     if (p.target_num <= 0 || p.target_den <= 0) return -1;
     return (int)min((int64_t)INT_MAX, (int64_t)p.target_den * L * L / (2 * (int64_t)p.target_num));
 }
-
-// Outcome of probing HT for a candidate.
-enum : int { kProbeFree = 0, kProbeVisited = 1, kProbeUnknown = 2, kProbeNone = 3 };
 
 // ------------------------------------------------------------- best-first search
 //
@@ -1866,122 +1808,6 @@ __device__ __forceinline__ void psl_eval(const View& V, int n, const Outs<TL, R>
     }
 }
 
-// The walk under the PSL objective, one walker per warp: evaluate all n flips (dISL by
-// the Toeplitz step of the plain walk, PSL by psl_eval), move to the lowest
-// (PSL, ISL, i) whose result is not in HT, and keep the best sequence, the stagnation
-// count and the restarts on (PSL, ISL) pairs; HT and the restart rules are the walk's.
-template <int R>
-__device__ void walk_psl(const WalkEnv& env, Walker& w, PslTrack& ps, int64_t until, int* base, const WarpSmem& SL,
-                         const View& V, int trace_slot, int64_t trace_start, const Tile<32>& t)
-{
-    using TL = Tile<32>;
-    const KParams& p = *env.p;
-    const int lane = t.lane, n = env.n;
-    const Outs<TL, R> o(t);
-    const int cap = p.probe_cap;
-    float P[R];
-    p_direct(V, n, o, P);
-    StopCheck stop;
-    stop.start(p, lane == 0);
-    while (w.steps < until) {
-        if ((w.steps & (kCheckEvery - 1)) == 0) {
-            const int why = t.shfl(stop.poll(p, lane == 0), 0);
-            if (why) {
-                if (lane == 0) raise_error(p.status, why, (int)env.g);
-                break;
-            }
-        }
-        int dl[R], pl[R];
-        {
-            float X[R];
-            toeplitz_one(V, SL, n, o, t, X);
-            assemble(V, n, o, X, P, dl);
-        }
-        psl_eval(V, n, o, pl);
-        uint64_t key[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            key[r] = dl[r] == INT_MAX ? ~0ull : psl_key(pl[r], w.isl + dl[r], 2 * (o.v0 + r) + o.p);
-        uint32_t excl = 0;
-        int best_i = -1;
-        uint64_t best_key = 0, fnew = 0;
-        int64_t slot = -1;
-        for (;;) {
-            uint64_t lm = ~0ull;
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if (!((excl >> r) & 1u) && key[r] < lm) lm = key[r];
-            const uint64_t km = warp_min64(lm);
-            if (km == ~0ull) break;
-            const int bi = psl_key_i(km);
-            const uint64_t f = w.fp ^ __ldg(env.zk + bi);
-            const Probe pr = probe_full(env, f, w.gen, cap, t);
-            if (!pr.visited) {
-                best_i = bi;
-                best_key = km;
-                slot = pr.slot;
-                fnew = f;
-                break;
-            }
-            exclude<TL, R>(excl, bi, t);
-        }
-
-        w.steps += 1;
-        int code;
-        if (best_i < 0) {
-            w.blocked += 1;
-            restart_walker(env, w, base, SL, V, t, &ps);
-            p_direct(V, n, o, P);
-            code = LABS_TRACE_BLOCKED;
-        } else {
-            flip_rows_table(V, n, o, P, best_i, t);
-            const bool stored = slot >= 0;
-            if (lane == 0 && stored) env.T[slot] = (fnew & ~kGenMask) | w.gen;
-            if (lane == (best_i >> 5)) w.word ^= 1u << (best_i & 31);
-            t.sync();
-            w.fp = fnew;
-            w.isl = psl_key_isl(best_key);
-            ps.psl = psl_key_psl(best_key);
-            if (!stored) w.overflows += 1;
-            note_best(env, w, t, &ps);
-            if (psl_better(ps.psl, w.isl, ps.since_psl, w.since)) {
-                w.since = w.isl;
-                ps.since_psl = ps.psl;
-                w.stag = 0;
-            } else {
-                w.stag += 1;
-            }
-            code = best_i;
-            if (w.stag >= env.patience || !stored) {
-                restart_walker(env, w, base, SL, V, t, &ps);
-                p_direct(V, n, o, P);
-                code |= LABS_TRACE_RESTART;
-            }
-        }
-        if (trace_slot >= 0 && lane == 0) {
-            const int64_t s = w.steps - 1 - trace_start;
-            if (s >= 0 && s < p.status->trace_capacity) {
-                p.status->trace_code[trace_slot * p.status->trace_capacity + s] = code;
-                p.status->trace_isl[trace_slot * p.status->trace_capacity + s] = w.isl;
-            }
-        }
-    }
-}
-
-// The lane's two lowest 64-bit keys above `floor` (~0 where there are fewer).
-template <int R>
-__device__ __forceinline__ void top2_above64(const uint64_t (&key)[R], uint64_t floor, uint64_t& b1, uint64_t& b2)
-{
-    b1 = ~0ull;
-    b2 = ~0ull;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint64_t k = key[r] > floor ? key[r] : ~0ull;
-        b2 = min(b2, max(b1, k));
-        b1 = min(b1, k);
-    }
-}
-
 // Lowest 64-bit value of the lane group: the lowest high word, then the lowest low word
 // among the lanes that hold it.
 template <class LG>
@@ -1990,181 +1816,6 @@ __device__ __forceinline__ uint64_t group_min64(uint64_t v, const LG& t)
     const uint32_t hi = t.rminu((uint32_t)(v >> 32));
     const uint32_t lo = t.rminu((uint32_t)(v >> 32) == hi ? (uint32_t)v : 0xFFFFFFFFu);
     return ((uint64_t)hi << 32) | lo;
-}
-
-// The walk under the PSL objective with two walkers per warp in lockstep (Pair): the
-// dISL of every flip from the lockstep Toeplitz step (on the tensor cores when TC says
-// so, as in walk_lockstep), the PSL of every neighbour from psl_eval, and the candidate
-// rounds of walk_lockstep on the (PSL', ISL', i) keys: two candidates per round, the
-// first S HT slots of each probed by half of the walker's lanes, full probes for longer
-// chains.  The trajectory of each walker is exactly that of walk_psl: the lowest key
-// whose state is not in HT is taken, and the best, stagnation and restart rules are the
-// same.  Restarts run divergently per half (RT = Tile<16>).
-template <class LG, class RT, int R, int TC>
-__device__ void walk_psl_lockstep(const WalkEnv& env, Walker& w, PslTrack& ps, int64_t until, bool real, int* base,
-                                  const WarpSmem& SL, const View& V, int trace_slot, int64_t trace_start,
-                                  const LG& t, const RT& tt)
-{
-    constexpr int S = LG::kSize / 2;  // HT slots probed per candidate in a round
-    constexpr unsigned SM = (1u << S) - 1u;
-    const KParams& p = *env.p;
-    const int lane = t.lane, n = env.n;
-    const Outs<LG, R> o(t);
-    const int cap = p.probe_cap;
-    const uint32_t tmask = (uint32_t)env.tmask;  // HT slots <= 2^20
-    float P[R];
-    p_direct(V, n, o, P);
-    int prev = -1;  // the last flip since the walker's (re)start in this call, or -1
-    StopCheck stop;
-    stop.start(p, (threadIdx.x & 31) == 0);
-    for (;;) {
-        const bool act = real && w.steps < until;
-        if (!__any_sync(kFull, act)) break;
-        if (__any_sync(kFull, act && (w.steps & (kCheckEvery - 1)) == 0)) {
-            const int why = __shfl_sync(kFull, stop.poll(p, (threadIdx.x & 31) == 0), 0);
-            if (why) {
-                if (act && lane == 0) raise_error(p.status, why, (int)env.g);
-                break;
-            }
-        }
-        uint64_t key[R];
-        {
-            int dl[R], pl[R];
-            int rv;
-            {
-                float X[R];
-                if constexpr (TC == 1) {
-                    toeplitz_tc(V, SL, n, o, t.h, X);
-                } else if constexpr (TC == 2) {
-                    if (SL.xp)
-                        toeplitz_tc(V, SL, n, o, t.h, X);
-                    else
-                        toeplitz(V, n, o, X);
-                } else {
-                    toeplitz(V, n, o, X);
-                }
-                rv = lane_dl(V, n, o, X, P, dl);
-            }
-            psl_eval<LG, R>(V, n, o, pl);
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                key[r] = r < rv ? psl_key(pl[r], w.isl + dl[r], 2 * (o.v0 + r) + o.p) : ~0ull;
-            drop_candidate(key, prev, o, ~(uint64_t)0);
-        }
-
-        // Best admissible flip: candidates in ascending key order, two per round; keys
-        // <= floor are known to lead to visited states.
-        uint64_t floor = 0ull, kc = ~0ull;
-        int slot = -1;
-        uint64_t fnew = 0;
-        bool done = !act;
-        do {
-            uint64_t b1, b2;
-            top2_above64(key, floor, b1, b2);
-            const uint64_t k0 = group_min64(done ? ~0ull : b1, t);
-            const uint64_t k1 = group_min64(done ? ~0ull : (b1 == k0 ? b2 : b1), t);
-            const bool has0 = k0 != ~0ull, has1 = k1 != ~0ull;
-            const uint64_t f0 = w.fp ^ (has0 ? __ldg(env.zk + psl_key_i(k0)) : 0ull);
-            const uint64_t f1 = w.fp ^ (has1 ? __ldg(env.zk + psl_key_i(k1)) : 0ull);
-            const int hs = lane & (S - 1);
-            const bool second = lane >= S;
-            const uint64_t f = second ? f1 : f0;
-            const bool live = !done && (second ? has1 : has0) && hs < cap;
-            uint64_t e = 0;
-            if (live) e = env.T[((uint32_t)f + (uint32_t)hs) & tmask];
-            const bool match = live && e == ((f & ~kGenMask) | w.gen);
-            const bool hit = live && ((((uint32_t)e & (uint32_t)kGenMask) != w.gen) || match);
-            const unsigned hb = t.ballot(hit), mb = t.ballot(match);
-            const unsigned h0 = hb & SM, h1 = (hb >> S) & SM;
-            int st0 = !has0 ? kProbeNone
-                            : h0 ? ((mb & h0 & (0u - h0)) ? kProbeVisited : kProbeFree)
-                                 : (cap > S ? kProbeUnknown : kProbeFree);
-            int st1 = !has1 ? kProbeNone
-                            : h1 ? (((mb >> S) & h1 & (0u - h1)) ? kProbeVisited : kProbeFree)
-                                 : (cap > S ? kProbeUnknown : kProbeFree);
-            int s0 = -2, s1 = -2;
-            const bool need0 = !done && st0 == kProbeUnknown;
-            if (__any_sync(kFull, need0)) {
-                const Probe pf = lockstep_probe_full(env, f0, w.gen, cap, need0, t);
-                if (need0) {
-                    st0 = pf.visited ? kProbeVisited : kProbeFree;
-                    s0 = (int)pf.slot;
-                }
-            }
-            const bool need1 = !done && st0 == kProbeVisited && st1 == kProbeUnknown;
-            if (__any_sync(kFull, need1)) {
-                const Probe pf = lockstep_probe_full(env, f1, w.gen, cap, need1, t);
-                if (need1) {
-                    st1 = pf.visited ? kProbeVisited : kProbeFree;
-                    s1 = (int)pf.slot;
-                }
-            }
-            if (!done) {
-                if (st0 == kProbeFree) {
-                    kc = k0, fnew = f0, done = true;
-                    slot = s0 != -2 ? s0 : (h0 ? (int)(((uint32_t)f0 + (uint32_t)(__ffs(h0) - 1)) & tmask) : -1);
-                } else if (st0 == kProbeNone || st1 == kProbeNone) {
-                    done = true;  // every neighbour is in HT
-                } else if (st1 == kProbeFree) {
-                    kc = k1, fnew = f1, done = true;
-                    slot = s1 != -2 ? s1 : (h1 ? (int)(((uint32_t)f1 + (uint32_t)(__ffs(h1) - 1)) & tmask) : -1);
-                } else {
-                    floor = k1;
-                }
-            }
-        } while (__any_sync(kFull, !done));
-
-        // Apply the move (walkers that have one), from the values before the flip.
-        const bool moves = act && kc != ~0ull;
-        const int best_i = moves ? psl_key_i(kc) : 0;
-        apply_flip<LG, R>(V, n, o, lane, moves, best_i, P);
-        const bool stored = slot >= 0;
-        if (moves && lane == 0 && stored) env.T[slot] = (fnew & ~kGenMask) | w.gen;
-        if (moves && lane == (best_i >> 5)) w.word ^= 1u << (best_i & 31);
-        __syncwarp();
-        int code = 0;
-        bool again = false;
-        if (act) {
-            w.steps += 1;
-            if (!moves) {
-                w.blocked += 1;
-                again = true;
-                code = LABS_TRACE_BLOCKED;
-            } else {
-                w.fp = fnew;
-                w.isl = psl_key_isl(kc);
-                ps.psl = psl_key_psl(kc);
-                if (!stored) w.overflows += 1;
-                note_best(env, w, t, &ps);
-                if (psl_better(ps.psl, w.isl, ps.since_psl, w.since)) {
-                    w.since = w.isl;
-                    ps.since_psl = ps.psl;
-                    w.stag = 0;
-                } else {
-                    w.stag += 1;
-                }
-                code = best_i;
-                if (w.stag >= env.patience || !stored) {
-                    again = true;
-                    code |= LABS_TRACE_RESTART;
-                }
-            }
-        }
-        if (moves) prev = best_i;
-        if (again) {  // divergent: only this half restarts
-            restart_walker(env, w, base, SL, V, tt, &ps);
-            p_direct(V, n, o, P);
-            prev = -1;
-        }
-        __syncwarp();
-        if (act && trace_slot >= 0 && lane == 0) {
-            const int64_t s = w.steps - 1 - trace_start;
-            if (s >= 0 && s < p.status->trace_capacity) {
-                p.status->trace_code[trace_slot * p.status->trace_capacity + s] = code;
-                p.status->trace_isl[trace_slot * p.status->trace_capacity + s] = w.isl;
-            }
-        }
-    }
 }
 
 template <int TILE, int RMAX, int MODE>
@@ -2245,28 +1896,10 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
                 if (idx < S->log_capacity) ex.rec = S->log + idx;
             }
         }
-        // the learned mode's step (walk_steps), the best-first search or the PSL walk
+        // the learned mode's step (walk_steps) or the best-first search
         constexpr int R2 = RMAX > 2 ? RMAX - 2 : 1;
         const bool full = RMAX <= 2 || block_R(G.n, TILE) >= RMAX;
-        if constexpr (MODE == 3) {
-            PslTrack ps;
-            ps.psl = table_psl(V, G.n, t);
-            ps.best_psl = st->best_psl;
-            ps.since_psl = st->since_psl;
-            if (ps.psl != st->psl) {
-                if (t.lane == 0) raise_error(p.status, LABS_ESTATE, (int)wi);
-                continue;
-            }
-            if (full)
-                walk_psl<RMAX>(env, w, ps, until, base, SL, V, trace_slot, trace_start, t);
-            else
-                walk_psl<R2>(env, w, ps, until, base, SL, V, trace_slot, trace_start, t);
-            if (t.lane == 0) {
-                st->psl = ps.psl;
-                st->best_psl = ps.best_psl;
-                st->since_psl = ps.since_psl;
-            }
-        } else if constexpr (MODE == 2) {
+        if constexpr (MODE == 2) {
             uint64_t* qk = p.pq_key + wi * LABS_QUEUE_SIZE;
             uint32_t* qb = p.pq_bits + wi * LABS_QUEUE_SIZE * kBitWords;
             if (full)
@@ -2284,112 +1917,6 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
     }
 }
 
-
-// PSL walk with WPW = 32 / LG::kSize (two) walkers per warp: the warp takes WPW consecutive
-// walkers; when their lengths differ (a group boundary) or fewer are left, it runs them
-// one after the other with the other lane group idle.  RT is the tile type a lane group
-// restarts with (divergently).
-template <class LG, class RT, int RMAX>
-__device__ __forceinline__ void walk_psl_group(const KParams& p, int chunk_index)
-{
-    constexpr int WPW = 32 / LG::kSize;
-    extern __shared__ __align__(16) int smem[];
-    const WarpSmem SL = warp_smem(p.n_max, LG::kSize, true);
-    const LG t(threadIdx.x & 31);
-    const RT tt(threadIdx.x & 31);
-    int* base = smem + (threadIdx.x / LG::kSize) * SL.words;
-    const View V = make_view(base, SL);
-    const int64_t target = p.status->target_steps;
-    DevStatus* S = p.status;
-    for (;;) {
-        uint32_t q = 0;
-        if ((threadIdx.x & 31) == 0) q = atomicAdd(&p.queue[chunk_index], (uint32_t)WPW);
-        q = __shfl_sync(kFull, q, 0);
-        if ((int64_t)q >= p.W) break;
-        const int64_t mine_w = (int64_t)q + t.h;
-        const bool exists = mine_w < p.W;
-        const int my_n = exists ? p.groups[p.states[mine_w].group].n : -1;
-        const int n0 = __shfl_sync(kFull, my_n, 0);
-        const bool together = __all_sync(kFull, exists && my_n == n0);
-        const int passes = together ? 1 : (int)min((int64_t)WPW, p.W - (int64_t)q);
-        for (int pass = 0; pass < passes; ++pass) {
-            // together: every group runs its walker; else pass k runs group k alone
-            const bool real0 = exists && (together || pass == t.h);
-            // the idle groups mirror the running group's length so that loops match
-            const int64_t lead_w = together ? mine_w : (int64_t)q + pass;
-            const DevGroup G = p.groups[p.states[lead_w].group];
-            WalkEnv env;
-            env.p = &p;
-            env.tmask = (1ull << p.tabu_log2) - 1ull;
-            env.T = p.tabu + ((uint64_t)mine_w << p.tabu_log2);
-            env.L = G.L;
-            env.n = G.n;
-            env.patience = p.patience > 0 ? p.patience : 2 * G.n;
-            env.g = (uint32_t)mine_w;
-            env.st = p.states + (exists ? mine_w : lead_w);
-            env.slot = nullptr;
-            env.slot_valid = nullptr;
-            env.rdump = nullptr;
-            env.rdump_idx = nullptr;
-            env.rdump_count = nullptr;
-            env.dump_cap = 0;
-            env.zk = p.zkeys + G.zkey_off;
-            Walker w;
-            load_walker(env.st, w, t.lane);
-            int64_t steps_done = w.steps;
-            int64_t until = min(target, steps_done + (int64_t)p.chunk_steps);
-            bool real = real0 && steps_done < until;
-            const int trace_slot = real ? env.st->trace_slot : -1;
-            const int64_t trace_start = trace_slot >= 0 ? p.trace_start[trace_slot] : 0;
-            const int isl = load_rows(base, SL, V, w.word, G.L, G.n, t);
-            if (real && isl != w.isl) {
-                if (t.lane == 0) raise_error(p.status, LABS_ESTATE, (int)mine_w);
-                real = false;
-            }
-            PslTrack ps;
-            ps.psl = table_psl(V, G.n, t);
-            ps.best_psl = env.st->best_psl;
-            ps.since_psl = env.st->since_psl;
-            if (real && ps.psl != env.st->psl) {
-                if (t.lane == 0) raise_error(p.status, LABS_ESTATE, (int)mine_w);
-                real = false;
-            }
-            // lane block: block_R(n) when it is one of RMAX .. RMAX-3, else the smallest
-            // bank-conflict-free one of those.  Two walkers per warp take the Toeplitz
-            // product to the tensor cores while n_max <= 128 (lane blocks up to 9; the
-            // second product for n > 128 would be mostly padding)
-            constexpr int TC = LG::kSize != 16 ? 0 : RMAX <= 8 ? 1 : RMAX == 9 ? 2 : 0;
-            int R = block_R(G.n, LG::kSize);
-            if (R < RMAX - 3) R = conflict_free_R(RMAX - 3, LG::kSize);
-            if (R >= RMAX)
-                walk_psl_lockstep<LG, RT, RMAX, TC>(env, w, ps, until, real, base, SL, V, trace_slot, trace_start, t, tt);
-            else if (R == RMAX - 1)
-                walk_psl_lockstep<LG, RT, (RMAX > 1 ? RMAX - 1 : 1), TC>(env, w, ps, until, real, base, SL, V, trace_slot,
-                                                                     trace_start, t, tt);
-            else if (R == RMAX - 2)
-                walk_psl_lockstep<LG, RT, (RMAX > 2 ? RMAX - 2 : 1), TC>(env, w, ps, until, real, base, SL, V, trace_slot,
-                                                                     trace_start, t, tt);
-            else
-                walk_psl_lockstep<LG, RT, (RMAX > 3 ? RMAX - 3 : 1), TC>(env, w, ps, until, real, base, SL, V, trace_slot,
-                                                                     trace_start, t, tt);
-            if (real) {
-                save_walker(env.st, w, t.lane);
-                if (t.lane == 0) {
-                    env.st->psl = ps.psl;
-                    env.st->best_psl = ps.best_psl;
-                    env.st->since_psl = ps.since_psl;
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
-template <int RMAX>
-__global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_psl_pair_kernel(KParams p, int chunk_index)
-{
-    walk_psl_group<Pair, Tile<16>, RMAX>(p, chunk_index);
-}
 
 }  // namespace
 }  // namespace labsgpu

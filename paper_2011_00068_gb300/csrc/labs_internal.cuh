@@ -343,7 +343,9 @@ __host__ __device__ constexpr int step_lag_blocks(int tile, int R)
 //   g:    pairs G[y] = (E[y], E[y+1]), one word each, y in [-gneg, gpos);
 //   z:    the sums Z_m, half index 2 z + m, infinite for m in [-zneg, 0);
 //   x:    the product's results, class p at x + p xp; the bit vectors of a rebuild (class
-//     p at b + p bvec) share its words.
+//     p at b + p bvec) and, under the PSL objective, the list of critical lags share its
+//     words.
+// psl: both row copies zero-padded for the PSL terms, entries -(n+1) .. outputs + n + 1.
 struct StepSmem {
     int h0, hc, ks;
     int r8;
@@ -354,7 +356,7 @@ struct StepSmem {
     int words;
 };
 
-__host__ __device__ constexpr StepSmem step_smem(int tile, int R)
+__host__ __device__ constexpr StepSmem step_smem(int tile, int R, bool psl = false)
 {
     StepSmem w{};
     const int n_max = step_n(tile, R), M = step_groups(tile, R), outs = (tile / 2) * R;
@@ -363,15 +365,19 @@ __host__ __device__ constexpr StepSmem step_smem(int tile, int R)
     // -(T-1).  Above: row blocks S+2 (S+3 with one operand per diagonal pair, S+6 with two
     // column groups), the update's pairs (words below hw + 2), s_{3i-L+1} of the last lane
     int lo = n_max - 1 > 16 * (T - 1) ? n_max - 1 : 16 * (T - 1);
+    if (psl) lo = n_max + 2;
     lo = (lo + 7) & ~7;
     int hi = 16 * (M == 2 ? S + 7 : tile == 32 ? S + 4 : S + 3);
     if (2 * (hw + 2) > hi) hi = 2 * (hw + 2);
     if (hw + 3 * R + 1 > hi) hi = hw + 3 * R + 1;
+    if (psl && outs + n_max + 4 > hi) hi = outs + n_max + 4;
     hi = (hi + 7) & ~7;
     w.h0 = lo / 2;
-    w.ks = hi / 2 + 4;  // entry 0 of copy 1 lies one half below its first word
+    // entry 0 of copy 1 lies one half below its first word
+    w.ks = psl ? hi / 2 + lo / 2 : hi / 2 + 4;
+    const int hi1 = psl ? hi / 2 : hw + 2;
     // 4 (mod 8) words per class: the two classes' operand rows use different banks
-    w.hc = ((w.h0 + w.ks + hw + 2 + 3) & ~7) + 4;
+    w.hc = ((w.h0 + w.ks + hi1 + 3) & ~7) + 4;
     // class pitch of the coefficients and the results, and below the walkers' pitch, so that
     // a warp's reads at odd R apart take 32 different banks: two walkers per warp 8 and 16
     // (mod 32), with the operand columns in block order 0, 2, 1, 3 (step_toeplitz) a store of
@@ -389,6 +395,7 @@ __host__ __device__ constexpr StepSmem step_smem(int tile, int R)
     w.b = w.x;
     w.bvec = (n_max - 1) / 32 + 2;
     w.words = (w.x + w.xp + need + 3) & ~3;
+    if (psl && w.x + n_max + 4 > w.words) w.words = (w.x + n_max + 7) & ~3;
     if (tile == 16) w.words += (48 - (w.words & 31)) & 31;
     if (tile == 8) w.words += (36 - (w.words & 31)) & 31;
     return w;
@@ -580,7 +587,7 @@ WalkFn walk_fn8b(int rmax);
 WalkFn walk_fn16a(int rmax);
 WalkFn walk_fn16b(int rmax);
 WalkFn walk_fn16p(int rmax);  // two walkers per warp, PSL objective, lane blocks 1-5 (labs_walk16p.cu)
-WalkFn walk_fn16q(int rmax);  // the same, lane blocks 6-9 (labs_walk16q.cu)
+WalkFn walk_fn16q(int rmax);  // the same, lane blocks 6-10 (labs_walk16q.cu)
 WalkFn walk_fn32(int rmax);   // one walker per warp: plain walk
 WalkFn walk_fn32l(int rmax);  // learned mode (labs_walk32l.cu)
 WalkFn walk_fn32b(int rmax);  // best-first search (labs_walk32b.cu)

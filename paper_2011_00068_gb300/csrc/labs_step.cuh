@@ -1,8 +1,8 @@
-// labs_step.cuh -- the plain walk's step (Algorithm 1, self-avoiding form) for lengths up
-// to LABS_MAX_L: four, two or one walkers per warp (LG = Quad, Pair or Tile<32>), the
-// Toeplitz product on the tensor cores in all three.  The step rule is the one stated at
-// labs_walk in labs.h.  Included by the labs_walk8*.cu, labs_walk16a/b.cu and
-// labs_walk32.cu units.
+// labs_step.cuh -- the walk's step (Algorithm 1, self-avoiding form) for lengths up to
+// LABS_MAX_L under the ISL or the PSL objective: four, two or one walkers per warp (LG =
+// Quad, Pair or Tile<32>), the Toeplitz product on the tensor cores in all three.  The step
+// rule is the one stated at labs_walk in labs.h.  Included by the labs_walk8*.cu,
+// labs_walk16*.cu, labs_walk32.cu and labs_walk32p.cu units.
 //
 // The neighbourhood in the form this step evaluates.  With p = i mod 2, v = i / 2, n_p
 // entries in class p, c = n-1, m = c - i and sg = (-1)^m:
@@ -161,18 +161,19 @@ struct StepShape {
 };
 
 // Layout of a kernel's walkers: that of its largest lane block.
-template <int NL, int RMAX>
+template <int NL, int RMAX, bool PSL>
 struct StepLayout {
-    static constexpr StepSmem SL = step_smem(NL, RMAX);
+    static constexpr StepSmem SL = step_smem(NL, RMAX, PSL);
+    static constexpr bool kPsl = PSL;
 };
 
 // ------------------------------------------------------------------ rebuild from bits
 
 // Rows, table and Z of the walker at word offset wb from its free-variable bits (word j in
-// lane j of the tile); returns the ISL.  Every word of the walker's shared memory is
-// rewritten.
+// lane j of the tile); returns the ISL, and under the PSL objective max |C_{2m}|.  Every
+// word of the walker's shared memory is rewritten.
 template <class LAY, class TL>
-__device__ int step_build(int wb, uint32_t word, int L, int n, const TL& t)
+__device__ int step_build(int wb, uint32_t word, int L, int n, const TL& t, int* psl)
 {
     constexpr StepSmem SL = LAY::SL;
     constexpr int NL = TL::kSize;
@@ -216,7 +217,7 @@ __device__ int step_build(int wb, uint32_t word, int L, int n, const TL& t)
     }
     t.sync();
     // autocorrelations of both classes at every lag, four lags per lane and pass
-    int part = 0;
+    int part = 0, top = 0;
     const uint32_t x0 = base + 4 * SL.b, x1 = x0 + 4 * SL.bvec;
     constexpr int kG = 4;
     for (int mb = 1 + t.lane; mb < n; mb += kG * NL) {
@@ -243,6 +244,7 @@ __device__ int step_build(int wb, uint32_t word, int L, int n, const TL& t)
                 const int a0 = (n - m) - 2 * c0[g], a1 = m < c ? (c - m) - 2 * c1[g] : 0;
                 const int d = a0 + a1;
                 part += d * d;
+                if (LAY::kPsl) top = max(top, abs(d));
                 const uint32_t e = half_bits(d), gb = base + 4 * SL.g;
                 sts_u16(gb + 4 * m, e);
                 sts_u16(gb + 4 * m - 2, e);
@@ -256,6 +258,7 @@ __device__ int step_build(int wb, uint32_t word, int L, int n, const TL& t)
     }
     if (t.lane == 0) sts_u16(base + 4 * SL.z, half_bits(6 - c + (c & 1)));
     t.sync();
+    if (LAY::kPsl) *psl = t.rmax(top);
     return t.radd(part);
 }
 
@@ -383,7 +386,25 @@ struct StepWalker {
     int isl, best, since, stag;
     uint32_t gen;
     int tisl;       // the target's ISL while it has not been met, else -1
+    int psl, best_psl, since_psl;  // PSL objective: the PSL halves of the (PSL, ISL) pairs
 };
+
+template <bool PSL>
+struct StepKey {
+    using type = unsigned;
+};
+template <>
+struct StepKey<true> {
+    using type = uint64_t;
+};
+
+// Strictly lower objective: the ISL, or the (PSL, ISL) pair.
+template <bool PSL>
+__device__ __forceinline__ bool step_better(int psl, int isl, int psl0, int isl0)
+{
+    if constexpr (PSL) return psl_better(psl, isl, psl0, isl0);
+    return isl < isl0;
+}
 
 struct StepEnv {
     const KParams* p;
@@ -459,14 +480,16 @@ __device__ __forceinline__ void step_restart(const StepEnv& env, StepWalker& w, 
     } else {
         w.word = lane < kBitWords ? start_word(p.seed, env.g, ridx, lane, env.n) : 0u;
     }
-    w.isl = step_build<LAY>(wb, w.word, 2 * env.n - 1, env.n, t);
+    w.isl = step_build<LAY>(wb, w.word, 2 * env.n - 1, env.n, t, &w.psl);
     w.fp = fingerprint_all(w.word, env.zk, env.n, t);
     if (lane == 0) env.T[(uint32_t)w.fp & tmask] = (w.fp & ~kGenMask) | w.gen;
     t.sync();
     w.since = w.isl;
+    w.since_psl = w.psl;
     w.stag = 0;
-    if (w.isl < w.best) {
+    if (step_better<LAY::kPsl>(w.psl, w.isl, w.best_psl, w.best)) {
         w.best = w.isl;
+        w.best_psl = w.psl;
         if (lane == 0) st->best_step = steps;
         if (lane < kBitWords) st->best[lane] = w.word;
     }
@@ -498,6 +521,35 @@ __device__ __forceinline__ void step_min2(unsigned b1, unsigned b2, const LG& t,
 }
 
 template <class LG>
+__device__ __forceinline__ void step_min2(uint64_t b1, uint64_t b2, const LG& t, uint64_t& k0, uint64_t& k1)
+{
+    k0 = group_min64(b1, t);
+    k1 = group_min64(b1 == k0 ? b2 : b1, t);
+}
+
+// Keys: the plain walk's 32 bits (below 2^31 for a candidate), or under the PSL objective
+// the PSL above them (below 2^63).
+__device__ __forceinline__ bool key_none(unsigned k) { return (int)k < 0; }
+__device__ __forceinline__ bool key_none(uint64_t k) { return (int64_t)k < 0; }
+template <class LG>
+__device__ __forceinline__ unsigned group_min(unsigned v, const LG& t) { return t.rminu(v); }
+template <class LG>
+__device__ __forceinline__ uint64_t group_min(uint64_t v, const LG& t) { return group_min64(v, t); }
+
+// The lane's two lowest keys (all ones where there are fewer).
+template <class KT, int R>
+__device__ __forceinline__ void key_top2(const KT (&key)[R], KT& b1, KT& b2)
+{
+    b1 = key[0];
+    b2 = ~(KT)0;
+#pragma unroll
+    for (int r = 1; r < R; ++r) {
+        b2 = min(b2, max(b1, key[r]));
+        b1 = min(b1, key[r]);
+    }
+}
+
+template <class LG>
 __device__ __forceinline__ int group_of(const LG& t)
 {
     if constexpr (LG::kSize == 32)
@@ -509,22 +561,23 @@ __device__ __forceinline__ int group_of(const LG& t)
 // The rest of the candidate search when the two best candidates' first HT slots did not
 // settle it (a chain longer than the probed slots, or both states visited): the walkers
 // with need set try their keys above floor one by one with full probes and insert the
-// state they choose.  kc: the chosen key, 0xFFFFFFFF when every neighbour is in HT; stored:
+// state they choose.  kc: the chosen key, all ones when every neighbour is in HT; stored:
 // the state found a free slot.
-template <class LG, int R>
-__device__ __forceinline__ void step_search(const StepEnv& env, uint64_t fp, uint32_t gen, const unsigned (&key)[R],
-                                         unsigned floor, bool need, const LG& t, unsigned& kc, bool& stored)
+template <class LG, class KT, int R>
+__device__ __forceinline__ void step_search(const StepEnv& env, uint64_t fp, uint32_t gen, const KT (&key)[R], KT floor,
+                                            bool need, const LG& t, KT& kc, bool& stored)
 {
+    constexpr KT none = ~(KT)0;
     const KParams& p = *env.p;
     const uint32_t tmask = (1u << p.tabu_log2) - 1u;
     const int cap = p.probe_cap;
     do {
-        unsigned b = 0xFFFFFFFFu;
+        KT b = none;
 #pragma unroll
-        for (int r = 0; r < R; ++r) b = min(b, key[r] > floor ? key[r] : 0xFFFFFFFFu);
-        const unsigned k = t.rminu(need ? b : 0xFFFFFFFFu);
-        if ((int)k < 0) need = false;  // no candidate left (or the walker is done)
-        const uint64_t f = fp ^ (need ? __ldg(env.zk + (k & 0xFFu)) : 0ull);
+        for (int r = 0; r < R; ++r) b = min(b, key[r] > floor ? key[r] : none);
+        const KT k = group_min(need ? b : none, t);
+        if (key_none(k)) need = false;  // no candidate left (or the walker is done)
+        const uint64_t f = fp ^ (need ? __ldg(env.zk + ((uint32_t)k & 0xFFu)) : 0ull);
         const uint64_t tag = (f & ~kGenMask) | gen;
         bool found = !need;
         for (int s0 = 0; s0 < cap; s0 += LG::kSize) {
@@ -592,6 +645,72 @@ __device__ __forceinline__ bool step_note(const StepEnv& env, int it, int code, 
     return true;
 }
 
+// ------------------------------------------------------------------ PSL of the neighbours
+//
+// Flipping output v of class p changes C_{2m} by ms (a_{v+m} + a_{v-m}), ms = -4 s_i (centre
+// -2 s_c), the mirror's own term a_{v+m} (m = c - i) left out: by at most 8.  So of all lags
+// only those within 8 of the sequence's PSL can decide a neighbour's unless the neighbour is
+// better than the sequence, and then those within 8 of the best neighbour's bound: about 31
+// and 1.4 of 100 lags at L = 201 (28% of the steps need the second band).  The lags of a
+// band are listed in shared memory (lag and C as one word) and every lane takes its R
+// outputs through them in FP16 pairs, exact on these small integers.  All lags of all
+// outputs in FP32 took 59.5 ms for 16384 walkers x 1000 steps at L = 201.
+
+// Lists the walker's lags with lo <= |C| < hi (both groups of a warp together: returns the
+// longer list's length, the shorter one filled with lag n, whose terms are all zero).
+template <class LAY, class LG, int R>
+__device__ __forceinline__ int psl_list(uint32_t list, const StepLags<StepShape<LG, R>::NB>& lg, int n, int lo, int hi,
+                                        const LG& t)
+{
+    constexpr int NL = LG::kSize;
+    const uint32_t lob = half_bits(max(lo, 0)), hib = half_bits(max(hi, 0));
+    const unsigned below = ((1u << t.lane) - 1u);
+    int count = 0;
+#pragma unroll
+    for (int b = 0; b < StepShape<LG, R>::NB; ++b)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t e = (j & 1) ? lg.e[b][j >> 1] >> 16 : lg.e[b][j >> 1] & 0xFFFFu, ab = e & 0x7FFFu;
+            const int m = 4 * (t.lane + NL * b) + j;
+            const bool in = ab >= lob && ab < hib && m > 0 && m < n;
+            const unsigned bal = t.ballot(in);
+            if (in) sts_u32(list + 4 * (count + __popc(bal & below)), (uint32_t)m | (e << 16));
+            count += __popc(bal);
+        }
+    const int top = __reduce_max_sync(kFull, count);
+    for (int k = count + t.lane; k < top; k += NL) sts_u32(list + 4 * k, (uint32_t)n);
+    __syncwarp();
+    return top;
+}
+
+// Takes the lane's outputs through a list: mx = max(mx, |C'|), outputs 2j and 2j+1 in pair j.
+template <class LAY, class LG, int R>
+__device__ __forceinline__ void psl_terms(uint32_t list, int top, uint32_t rows, int v0, int z0, uint32_t corr,
+                                          const uint32_t (&ms)[(R + 1) / 2], uint32_t (&mx)[(R + 1) / 2])
+{
+    constexpr StepSmem SL = LAY::SL;
+    constexpr int J = (R + 1) / 2;
+    for (int k = 0; k < top; ++k) {
+        const uint32_t w = lds_u32(list + 4 * k);
+        const int m = (int)(w & 0xFFFFu);
+        const uint32_t c2 = __byte_perm(w, w, 0x3232);
+        // entries v0 + m and v0 - m have the same parity: the same copy; entry u of copy 1 is
+        // at half u - 1
+        const uint32_t r = rows + ((v0 + m) & 1 ? 4 * SL.ks - 2 : 0);
+        const uint32_t up = r + 2 * (v0 + m), dn = r + 2 * (v0 - m);
+        // the output whose mirror this lag reaches (its a_{v+m} is sg s_i): z / 2, if even
+        const int z = z0 - m;
+        const uint32_t cx = as_u32(__hadd2(as_half2(c2), as_half2((z & 2) ? corr << 16 : corr)));
+        const int zj = (z & 1) ? -1 : z >> 2;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const __half2 s2 = __hadd2(as_half2(lds_u32(up + 4 * j)), as_half2(lds_u32(dn + 4 * j)));
+            const __half2 e = __hfma2(as_half2(ms[j]), s2, as_half2(zj == j ? cx : c2));
+            mx[j] = as_u32(__hmax2(as_half2(mx[j]), __habs2(e)));
+        }
+    }
+}
+
 // ------------------------------------------------------------------ the walk's steps
 
 // Advances the warp's walkers by up to len steps each (one per lane group; `real`: the
@@ -606,6 +725,8 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
     constexpr StepSmem SL = LAY::SL;
     constexpr int NL = SH::NL, NB = SH::NB;
     constexpr int S = NL / 2;  // HT slots probed per candidate in a round
+    constexpr bool PSL = LAY::kPsl;
+    using KT = typename StepKey<PSL>::type;
     const KParams& p = *env.p;
     const int lane = t.lane, l = lane + t.base, n = env.n, c = n - 1;
     const int wb = wb0 + group_of(t) * SL.words;
@@ -645,39 +766,78 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
         // holds the integer in its low bits, and one byte permute puts i below its low
         // three bytes.  Outputs that do not exist and the move back to the state just left
         // (marked below; that state is always in HT) have an infinite Z, whose bytes give a
-        // key of at least 2^31.
-        unsigned key[R];
+        // key of at least 2^31.  Under the PSL objective the PSL (as FP16 bits, which order
+        // as the integers do) goes above it.
+        KT key[R];
+        {
+            unsigned kl[R];
+            uint32_t ms[(R + 1) / 2];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float x = lds_f32(xr + 4 * r), r8 = lds_f32(xr - 4u * (uint32_t)(SL.x - SL.r8) + 4 * r);
-            const float z = lds_f16(zr - 4 * r), s3 = lds_f16(sr + 6 * r);
-            const float v = fmaf(r8, fmaf(sig4, s3, x), fmaf(8.f, z, bias));
-            key[r] = __byte_perm(__float_as_uint(v), r < 4 ? ib : r < 8 ? ib + 0x08080808u : ib + 0x10101010u, 0x2104 + (r & 3));
-        }
-        unsigned b1 = key[0], b2 = 0xFFFFFFFFu;
+            for (int r = 0; r < R; ++r) {
+                const float x = lds_f32(xr + 4 * r), r8 = lds_f32(xr - 4u * (uint32_t)(SL.x - SL.r8) + 4 * r);
+                const float z = lds_f16(zr - 4 * r), s3 = lds_f16(sr + 6 * r);
+                const float v = fmaf(r8, fmaf(sig4, s3, x), fmaf(8.f, z, bias));
+                kl[r] = __byte_perm(__float_as_uint(v), r < 4 ? ib : r < 8 ? ib + 0x08080808u : ib + 0x10101010u,
+                                    0x2104 + (r & 3));
+                if (PSL) {  // -8 s_i / 2
+                    const uint32_t h = __half_as_ushort(__float2half_rn(0.5f * r8));
+                    ms[r >> 1] = (r & 1) ? ms[r >> 1] | (h << 16) : h;
+                }
+            }
+            if constexpr (PSL) {
+                uint32_t mx[(R + 1) / 2];
 #pragma unroll
-        for (int r = 1; r < R; ++r) {
-            b2 = min(b2, max(b1, key[r]));
-            b1 = min(b1, key[r]);
+                for (int j = 0; j < (R + 1) / 2; ++j) mx[j] = 0u;
+                const uint32_t list = sbyte(wb + SL.x), prow = sbyte(wb + SL.h0 + o.p * SL.hc);
+                const uint32_t corr = ((c - o.p) & 1) ? 0xC400u : 0x4400u;  // 4 sg
+                const int z0 = c - o.p - 2 * o.v0;
+                __syncwarp();  // the list takes the results' place
+                int top_k = psl_list<LAY, LG, R>(list, lg, n, w.psl - 8, 0x7FF, t);
+                psl_terms<LAY, LG, R>(list, top_k, prow, o.v0, z0, corr, ms, mx);
+                uint32_t lb = 0x7FFFu;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t h = (r & 1) ? mx[r >> 1] >> 16 : mx[r >> 1] & 0xFFFFu;
+                    lb = min(lb, (int)kl[r] < 0 ? 0x7FFFu : h);
+                }
+                lb = t.rminu(lb);
+                const int low = (int)__half2float(__ushort_as_half((unsigned short)lb));
+                if (__any_sync(kFull, act && low < w.psl)) {
+                    __syncwarp();
+                    const bool more = low < w.psl;
+                    top_k = psl_list<LAY, LG, R>(list, lg, n, more ? low - 7 : 0, more ? w.psl - 8 : 0, t);
+                    psl_terms<LAY, LG, R>(list, top_k, prow, o.v0, z0, corr, ms, mx);
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t h = (r & 1) ? mx[r >> 1] >> 16 : mx[r >> 1] & 0xFFFFu;
+                    key[r] = ((uint64_t)(h | (uint32_t)((int)kl[r] >> 31)) << 32) | kl[r];
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) key[r] = kl[r];
+            }
         }
+        KT b1, b2;
+        key_top2(key, b1, b2);
 
         // Best admissible flip: the lowest key whose state is not in HT.  The two lowest
         // are probed at once, the first S HT slots of each by one half of the walker's
         // lanes; that settles nearly every step, step_search does the others.
-        unsigned k0, k1;
+        KT k0, k1;
         step_min2(b1, b2, t, k0, k1);
         const int hs = lane & (S - 1);
-        const unsigned km = lane >= S ? k1 : k0;
-        const bool live = act && (int)km >= 0 && hs < p.probe_cap;
+        const KT km = lane >= S ? k1 : k0;
+        const bool live = act && !key_none(km) && hs < p.probe_cap;
         // a key without an output reads past the length's fingerprint keys, within the workspace
-        const uint64_t f = w.fp ^ __ldg(env.zk + (km & 0xFFu));
+        const uint64_t f = w.fp ^ __ldg(env.zk + ((uint32_t)km & 0xFFu));
         const uint32_t at = ((uint32_t)f + (uint32_t)hs) & ((1u << p.tabu_log2) - 1u);
         const uint64_t e = env.T[at], tag = (f & ~kGenMask) | w.gen;
         const bool match = live && e == tag;
         const unsigned hb = __ballot_sync(kFull, match || (live && ((uint32_t)e & (uint32_t)kGenMask) != w.gen));
         const unsigned mb = __ballot_sync(kFull, match);
         unsigned pick;  // the lane that saw the free slot of the chosen state (0: not settled)
-        unsigned kc;
+        KT kc;
         bool stored = true;
         {
             const unsigned g0 = hb & (((1u << S) - 1u) << t.base), g1 = hb & (((1u << S) - 1u) << (t.base + S));
@@ -687,21 +847,21 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
             pick = v0 ? (v1 ? 0u : p1) : p0;
             if (__any_sync(kFull, act && pick == 0u)) {
                 const bool need = act && pick == 0u;
-                unsigned ks = 0xFFFFFFFFu;
+                KT ks = ~(KT)0;
                 bool st = false;
-                step_search<LG, R>(env, w.fp, w.gen, key, v0 ? (v1 ? k1 : k0) : 0u, need, t, ks, st);
+                step_search(env, w.fp, w.gen, key, v0 ? (v1 ? k1 : k0) : (KT)0, need, t, ks, st);
                 if (need) {
                     kc = ks;
                     stored = st;
                 }
             }
         }
-        const bool moves = act && kc != 0xFFFFFFFFu;
+        const bool moves = act && kc != ~(KT)0;
         stg_u64_if(moves && (pick >> l) == 1u, env.T + at, tag);
 
         // Apply the move (walkers that have one).  The flipped entries read as 0 while the
         // sums are taken, which leaves out the pairs whose two ends both flip and lag 0.
-        const int bi = moves ? (int)(kc & 0xFFu) : 0;
+        const int bi = moves ? (int)((uint32_t)kc & 0xFFu) : 0;
         const int pb = bi & 1, vb = bi >> 1, vq = n - 1 - pb - vb;
         const bool centre = bi == c, same = ((pb ^ c) & 1) == 0;  // same: sg = +1 in the flipped class
         const uint32_t wsh = t.shfl(w.word, bi >> 5) << (31 - (bi & 31));
@@ -776,19 +936,22 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
         if (moves) {
             if (lane == (bi >> 5)) w.word ^= 1u << (bi & 31);
             w.fp ^= zk;
-            w.isl += (int)(kc >> 8) - kKeyBias;
+            w.isl += (int)((uint32_t)kc >> 8) - kKeyBias;
+            if constexpr (PSL) w.psl = (int)__half2float(__ushort_as_half((unsigned short)((uint64_t)kc >> 32)));
             w.stag += 1;
-            if (w.isl < w.since) {
+            if (step_better<PSL>(w.psl, w.isl, w.since_psl, w.since)) {
                 w.since = w.isl;
+                w.since_psl = w.psl;
                 w.stag = 0;
             }
             again = w.stag >= env.patience || !stored;
         }
-        if (moves && (w.isl < w.best || w.isl <= w.tisl)) {
+        if (moves && (step_better<PSL>(w.psl, w.isl, w.best_psl, w.best) || w.isl <= w.tisl)) {
             WalkerState* st = env.state();
             const int64_t steps = st->steps_done + it + 1;
-            if (w.isl < w.best) {
+            if (step_better<PSL>(w.psl, w.isl, w.best_psl, w.best)) {
                 w.best = w.isl;
+                w.best_psl = w.psl;
                 if (lane == 0) st->best_step = steps;
                 if (lane < kBitWords) st->best[lane] = w.word;
             }
@@ -820,19 +983,19 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
 // CTAs of 8 warps per SM the walk kernels are compiled for: three (80 registers a thread),
 // but two where three would not fit in shared memory (four walkers per warp, lane blocks
 // from 7)
-__host__ __device__ constexpr int step_ctas(int tile, int R)
+__host__ __device__ constexpr int step_ctas(int tile, int R, bool psl = false)
 {
-    return 3 * 8 * (32 / tile) * step_smem(tile, R).words * 4 <= kSmemBudget ? 3 : 2;
+    return 3 * 8 * (32 / tile) * step_smem(tile, R, psl).words * 4 <= kSmemBudget ? 3 : 2;
 }
 
 // Runs the walkers of the queue: the warp takes W consecutive walkers; when their lengths
 // differ (a group boundary) or fewer are left, it runs them one after the other with the
 // other lane groups idle.
-template <class LG, class RT, int RMAX>
+template <class LG, class RT, int RMAX, bool PSL = false>
 __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
 {
     constexpr int NL = LG::kSize, W = 32 / NL;
-    using LAY = StepLayout<NL, RMAX>;
+    using LAY = StepLayout<NL, RMAX, PSL>;
     constexpr StepSmem SL = LAY::SL;
     const int l = lane_id();
     const LG t(l);
@@ -879,8 +1042,13 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
             const int64_t steps0 = st->steps_done;
             const int len = (int)min((int64_t)p.chunk_steps, max(target - steps0, (int64_t)0));
             bool real = mine && len > 0;
-            const int isl = step_build<LAY>(wb, w.word, G.L, G.n, t);
-            if (real && isl != w.isl) {
+            w.psl = w.best_psl = w.since_psl = 0;
+            const int isl = step_build<LAY>(wb, w.word, G.L, G.n, t, &w.psl);
+            if (PSL) {
+                w.best_psl = st->best_psl;
+                w.since_psl = st->since_psl;
+            }
+            if (real && (isl != w.isl || (PSL && w.psl != st->psl))) {
                 if (t.lane == 0) raise_error(p.status, LABS_ESTATE, (int)mine_w);
                 real = false;
             }
@@ -926,6 +1094,11 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
                     st->stagnation = w.stag;
                     st->gen = w.gen;
                     st->steps_done = steps0 + done;
+                    if (PSL) {
+                        st->psl = w.psl;
+                        st->best_psl = w.best_psl;
+                        st->since_psl = w.since_psl;
+                    }
                 }
             }
             __syncwarp();

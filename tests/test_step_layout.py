@@ -26,7 +26,7 @@ def dump(tmp_path_factory):
         f = line.split()
         v = list(map(int, f[1:]))
         if f[0] == "step":
-            lay[(v[0], v[1])] = dict(zip(FIELDS, v[2:]))
+            lay[(v[0], v[1], v[2])] = dict(zip(FIELDS, v[3:]))
         else:
             shape[(v[0], v[1])] = (v[2], v[3], v[4])
     return lay, shape
@@ -38,9 +38,9 @@ def conflict_free(R, tile):
     return R
 
 
-def check(S, shape, tile, nmax, n, lay):
+def check(S, shape, psl, tile, nmax, n, lay):
     RMAX = S["R"]
-    R = lay[(tile, n)]["R"]
+    R = lay[(psl, tile, n)]["R"]
     if tile == 32:
         R = RMAX if R >= RMAX else (RMAX - 2 if RMAX > 2 else 1)
     else:
@@ -55,8 +55,9 @@ def check(S, shape, tile, nmax, n, lay):
     assert T <= 4 * M and outs >= hw and lags >= n
     if n == nmax:
         assert lags >= S["gneg"] >= 16 * T
-    hlo, hhi = -2 * S["h0"], 2 * (S["ks"] - 4)               # copy 0 of a class, halves (below copy 1's pad)
-    klo, khi = -8, 2 * (S["hc"] - S["h0"] - S["ks"])         # copy 1, halves from its first word
+    pad1 = 2 * S["h0"] if psl else 8                          # copy 1's zero halves below its first word
+    hlo, hhi = -2 * S["h0"], 2 * S["ks"] - pad1               # copy 0 of a class, halves
+    klo, khi = -pad1, 2 * (S["hc"] - S["h0"] - S["ks"])      # copy 1, halves from its first word
 
     def row(u):
         assert hlo <= u < hhi, ("row", u)
@@ -81,6 +82,12 @@ def check(S, shape, tile, nmax, n, lay):
                 m = zi - 2 * r
                 assert -S["zneg"] <= m < lags
                 assert (m < 0) == (not 2 * (v0 + r) + p <= c)
+    if psl:  # pairs at v0 +- m, m = 1 .. n, in the copy of their parity; the list of lags
+        for u in (-n, outs - R + n + R + 1):
+            row(u - 1)
+            row(u)
+            assert klo <= u - 2 and u + 1 < khi
+        assert S["x"] + n + 1 <= S["words"]
     # row blocks of the product: first diagonal -(T-1), last S-1 (with one operand, the load
     # of a last diagonal without a partner reads the next one's too)
     dlast = Sb - 1
@@ -107,12 +114,12 @@ def check(S, shape, tile, nmax, n, lay):
     assert (n - 1) // 32 + 1 < S["bvec"] and S["b"] + 2 * S["bvec"] <= S["words"]
 
 
-@pytest.mark.parametrize("tile", [8, 16, 32])
-def test_step_accesses_stay_in_their_regions(dump, tile):
+@pytest.mark.parametrize("psl,tile", [(0, 8), (0, 16), (0, 32), (1, 16), (1, 32)])
+def test_step_accesses_stay_in_their_regions(dump, psl, tile):
     lay, shape = dump
-    for (t, nmax), S in lay.items():
-        if t != tile:
+    for (q, t, nmax), S in lay.items():
+        if (q, t) != (psl, tile):
             continue
         for n in sorted(set(range(2, nmax + 1, 5)) | {2, 3, 4, 5, nmax - 1, nmax} | set(range(max(2, nmax - 40), nmax + 1))):
             if 2 <= n <= nmax:
-                check(S, shape, tile, nmax, n, lay)
+                check(S, shape, psl, tile, nmax, n, lay)
