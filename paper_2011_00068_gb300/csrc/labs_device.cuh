@@ -1448,208 +1448,6 @@ __device__ __forceinline__ uint64_t warp_max64(uint64_t v)
 // Python statement), each flip costing about a sixth of a rebuild.
 constexpr int kBestFirstMaxFlips = 5;
 
-template <int R>
-__device__ void walk_bestfirst(const WalkEnv& env, Walker& w, int64_t until, int* base, const WarpSmem& SL,
-                               const View& V, int trace_slot, int64_t trace_start, const Tile<32>& t, uint64_t* qkey,
-                               uint32_t* qbits)
-{
-    static_assert(LABS_QUEUE_SIZE == 32, "one queue entry per lane");
-    const KParams& p = *env.p;
-    const int lane = t.lane, n = env.n;
-    const Outs<Tile<32>, R> o(t);
-    const int cap = p.probe_cap;
-    const int tisl = target_isl(p, env.L);
-    uint64_t qk = qkey[lane];
-    // xLastovka's second table (null when off): slot f mod size holds
-    // (generation << 40) | (~f mod 2^40) of an evaluated neighbour f
-    uint64_t* T2 = p.tabu2 != nullptr ? p.tabu2 + (env.T - p.tabu) : nullptr;
-    constexpr uint64_t kLow40 = 0xFFFFFFFFFFull;
-    int64_t hits = 0;
-    float P[R];
-    p_direct(V, n, o, P);
-    StopCheck stop;
-    stop.start(p, lane == 0);
-    while (w.steps < until) {
-        if ((w.steps & (kCheckEvery - 1)) == 0) {
-            const int why = t.shfl(stop.poll(p, lane == 0), 0);
-            if (why) {
-                if (lane == 0) raise_error(p.status, why, (int)env.g);
-                break;
-            }
-        }
-        const int64_t e = w.steps;
-        unsigned key[R];
-        {
-            float X[R];
-            toeplitz_one(V, SL, n, o, t, X);
-            lane_keys(V, n, o, X, P, key);
-        }
-        if (T2 != nullptr) {
-            // neighbours the table holds are skipped (their keys dropped); every other
-            // one is inserted once all lanes have looked (larger word kept: the table
-            // does not depend on the order of the insertions)
-            uint64_t ins[R];
-            int h = 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                ins[r] = 0ull;
-                if (key[r] == 0xFFFFFFFFu) continue;
-                const uint64_t f = w.fp ^ __ldg(env.zk + (key[r] & 0xFFu));
-                const uint64_t tag = ((uint64_t)w.gen << 40) | (~f & kLow40);
-                if (T2[f & env.tmask] == tag) {
-                    key[r] = 0xFFFFFFFFu;
-                    ++h;
-                } else {
-                    ins[r] = f;
-                }
-            }
-            hits += t.radd(h);
-            t.sync();
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if (key[r] != 0xFFFFFFFFu)
-                    atomicMax(reinterpret_cast<unsigned long long*>(T2 + (ins[r] & env.tmask)),
-                              (unsigned long long)(((uint64_t)w.gen << 40) | (~ins[r] & kLow40)));
-            t.sync();
-        }
-        // Neighbours in queue order (ISL, then i: the packed keys' order) while they
-        // come before the queue's last entry or the queue has a free place.  The queue's
-        // last entry only moves forward during the step, so the neighbours after its
-        // value at the start cannot enter; the others are looked up in HT one by one as
-        // the insertion reaches them (HT does not change during the insertion, so this
-        // equals looking them all up first, at a few probes per step instead of one per
-        // neighbour).
-        const bool full0 = t.ballot(qk == ~0ull) == 0u;
-        const uint64_t last0 = full0 ? warp_max64(qk) : ~0ull;
-        bool fresh[R];  // candidate r: before last0
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const unsigned k = key[r];
-            const uint64_t ck = ((uint64_t)(w.isl + (int)(k >> 8) - kKeyBias) << 36) | ((uint64_t)e << 8) |
-                                (uint64_t)(k & 0xFFu);
-            fresh[r] = k != 0xFFFFFFFFu && ck < last0;
-        }
-        unsigned floor = 0u;
-        for (;;) {
-            unsigned b = 0xFFFFFFFFu;
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if (fresh[r] && key[r] > floor) b = min(b, key[r]);
-            const unsigned k = t.rminu(b);
-            if (k == 0xFFFFFFFFu) break;
-            floor = k;
-            const int i = (int)(k & 0xFFu);
-            const int isl_f = w.isl + (int)(k >> 8) - kKeyBias;
-            const uint64_t ck = ((uint64_t)isl_f << 36) | ((uint64_t)e << 8) | (uint64_t)i;
-            const unsigned empty = t.ballot(qk == ~0ull);
-            int dst;
-            if (empty) {
-                dst = __ffs(empty) - 1;
-            } else {
-                const uint64_t last = warp_max64(qk);
-                if (ck > last) break;  // every later neighbour comes after it too
-                dst = __ffs(t.ballot(qk == last)) - 1;
-            }
-            {
-                // HT lookup of this neighbour: up to probe_cap slots, four per round
-                const uint64_t f = w.fp ^ __ldg(env.zk + i);
-                const uint64_t tag = (f & ~kGenMask) | w.gen;
-                bool visited = false;
-                for (int s0 = 0; s0 < cap; s0 += 4) {
-                    const bool mine = lane < 4 && s0 + lane < cap;
-                    const uint64_t x = mine ? env.T[(f + (uint64_t)(s0 + lane)) & env.tmask] : 0ull;
-                    const unsigned bal = t.ballot(mine && (((x & kGenMask) != w.gen) || x == tag));
-                    if (bal) {
-                        visited = t.shfl(x == tag ? 1 : 0, __ffs(bal) - 1) != 0;
-                        break;
-                    }
-                }
-                if (visited) continue;
-            }
-            if (lane == dst) qk = ck;
-            const uint32_t word = w.word ^ (lane == (i >> 5) ? 1u << (i & 31) : 0u);
-            if (lane < kBitWords) qbits[dst * kBitWords + lane] = word;
-            if (isl_f < w.best_isl) {
-                w.best_isl = isl_f;
-                w.best_step = e + 1;
-                if (lane < kBitWords) env.st->best[lane] = word;
-            }
-            if (w.target_step < 0 && isl_f <= tisl) w.target_step = e + 1;
-        }
-        t.sync();
-        // S <- the queue's first entry not in HT (entries that are get dropped)
-        int code = LABS_TRACE_BLOCKED;
-        bool again = true;
-        for (;;) {
-            if (!t.ballot(qk != ~0ull)) {
-                w.blocked += 1;  // empty queue: restart
-                break;
-            }
-            const uint64_t first = warp_min64(qk);
-            const int src = __ffs(t.ballot(qk == first)) - 1;
-            const uint32_t word = lane < kBitWords ? qbits[src * kBitWords + lane] : 0u;
-            if (lane == src) qk = ~0ull;
-            const int i = (int)(first & 0xFFu);
-            const bool nb = ((first >> 8) & 0xFFFFFFFull) == (uint64_t)e;  // a neighbour of S
-            const uint64_t f = nb ? (w.fp ^ __ldg(env.zk + i)) : fingerprint_all(word, env.zk, n, t);
-            const Probe pr = probe_full(env, f, w.gen, cap, t);
-            if (pr.visited) continue;
-            // free variables in which the new S differs from S (1 for a neighbour)
-            uint32_t diff = lane < kBitWords ? (word ^ w.word) : 0u;
-            const int k = nb ? 1 : t.radd(__popc(diff));
-            if (k <= kBestFirstMaxFlips) {
-                // flip them one by one (lowest first) with the walk's incremental update
-                for (int j = 0; j < k; ++j) {
-                    const unsigned bl = t.ballot(diff != 0u);
-                    const int src_lane = __ffs(bl) - 1;
-                    const int fi = nb ? i : 32 * src_lane + t.shfl(__ffs(diff) - 1, src_lane);
-                    apply_flip<Tile<32>, R>(V, n, o, lane, true, fi, P);
-                    t.sync();
-                    if (lane == src_lane) diff &= diff - 1u;
-                }
-            } else {
-                // rebuild from the bits; the walker's padding is still zero, so no clear
-                rows_from_bits(V, word, env.L, n, t);
-                build_table(V, n, t);
-                p_direct(V, n, o, P);
-            }
-            w.word = word;
-            w.isl = (int)(first >> 36);
-            w.fp = f;
-            code = (int)(f & 0xFFFFu);
-            if (pr.slot >= 0) {
-                if (lane == 0) env.T[pr.slot] = (f & ~kGenMask) | w.gen;
-                again = false;
-            } else {
-                w.overflows += 1;  // no free HT slot for the new S: restart
-                code |= LABS_TRACE_RESTART;
-            }
-            break;
-        }
-        w.steps += 1;
-        if (again) {
-            qk = ~0ull;
-            const uint32_t gen0 = w.gen;
-            restart_walker(env, w, base, SL, V, t);
-            if (T2 != nullptr && w.gen < gen0) {  // generations wrapped: HT was zeroed, so is T2
-                for (int64_t i = lane; i <= (int64_t)env.tmask; i += 32) T2[i] = 0ull;
-                t.sync();
-            }
-            p_direct(V, n, o, P);
-        }
-        t.sync();
-        if (trace_slot >= 0 && lane == 0) {
-            const int64_t s = w.steps - 1 - trace_start;
-            if (s >= 0 && s < p.status->trace_capacity) {
-                p.status->trace_code[trace_slot * p.status->trace_capacity + s] = code;
-                p.status->trace_isl[trace_slot * p.status->trace_capacity + s] = w.isl;
-            }
-        }
-    }
-    qkey[lane] = qk;
-    if (lane == 0) env.st->cache_hits += hits;
-}
-
 // One launch advances every walker by up to chunk_steps steps toward the target.  The
 // kernel is compiled for a tile of TILE lanes per walker and a largest lane block RMAX
 // = block_R(n_max, TILE) (register allocation follows it; odd for TILE = 32); walkers
@@ -1818,8 +1616,8 @@ __device__ __forceinline__ uint64_t group_min64(uint64_t v, const LG& t)
     return ((uint64_t)hi << 32) | lo;
 }
 
-template <int TILE, int RMAX, int MODE>
-__global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(KParams p, int chunk_index)
+template <int TILE, int RMAX>
+__global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_learned_kernel(KParams p, int chunk_index)
 {
     extern __shared__ __align__(16) int smem[];
     const WarpSmem SL = warp_smem(p.n_max, TILE);
@@ -1871,7 +1669,7 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
         env.rdump_count = nullptr;
         env.dump_cap = 0;
         DevStatus* S = p.status;
-        if (MODE == 1 && S->learned) {
+        if (S->learned) {
             env.slot = S->l_slot + wi * kBitWords;
             env.slot_valid = S->l_slot_valid + wi;
             if (S->l_score_step[wi] == steps_done) {
@@ -1896,22 +1694,12 @@ __global__ void __launch_bounds__(256, LABS_WALK_MIN_BLOCKS) walk_chunk_kernel(K
                 if (idx < S->log_capacity) ex.rec = S->log + idx;
             }
         }
-        // the learned mode's step (walk_steps) or the best-first search
         constexpr int R2 = RMAX > 2 ? RMAX - 2 : 1;
         const bool full = RMAX <= 2 || block_R(G.n, TILE) >= RMAX;
-        if constexpr (MODE == 2) {
-            uint64_t* qk = p.pq_key + wi * LABS_QUEUE_SIZE;
-            uint32_t* qb = p.pq_bits + wi * LABS_QUEUE_SIZE * kBitWords;
-            if (full)
-                walk_bestfirst<RMAX>(env, w, until, base, SL, V, trace_slot, trace_start, t, qk, qb);
-            else
-                walk_bestfirst<R2>(env, w, until, base, SL, V, trace_slot, trace_start, t, qk, qb);
-        } else {
-            if (full)
-                walk_steps<Tile<TILE>, RMAX>(env, w, until, base, SL, V, trace_slot, trace_start, ex, t);
-            else
-                walk_steps<Tile<TILE>, R2>(env, w, until, base, SL, V, trace_slot, trace_start, ex, t);
-        }
+        if (full)
+            walk_steps<Tile<TILE>, RMAX>(env, w, until, base, SL, V, trace_slot, trace_start, ex, t);
+        else
+            walk_steps<Tile<TILE>, R2>(env, w, until, base, SL, V, trace_slot, trace_start, ex, t);
         save_walker(st, w, t.lane);
         t.sync();
     }

@@ -909,17 +909,15 @@ static WalkFn walk_fn(int tile, int rmax, int mode)
     }
 }
 
-// Lane block and shared memory per warp of a walk kernel (modes 0 and 3: the walk under the
-// ISL and the PSL objective).
+// Lane block and shared memory per warp of a walk kernel (mode 1: the learned mode).
 static int walk_R(int n_max, int tile, int mode)
 {
-    return mode == 0 || mode == 3 ? step_R(n_max, tile) : block_R(n_max, tile);
+    return mode != 1 ? step_R(n_max, tile) : block_R(n_max, tile);
 }
 
 static size_t walk_warp_bytes(int n_max, int tile, int mode)
 {
-    const int words = mode == 0 || mode == 3 ? step_smem(tile, step_R(n_max, tile), mode == 3).words
-                                             : warp_smem(n_max, tile).words;
+    const int words = mode != 1 ? step_smem(tile, step_R(n_max, tile), mode == 3).words : warp_smem(n_max, tile).words;
     return (size_t)words * sizeof(int) * (kWarp / tile);
 }
 

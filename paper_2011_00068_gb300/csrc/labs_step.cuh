@@ -711,6 +711,144 @@ __device__ __forceinline__ void psl_terms(uint32_t list, int top, uint32_t rows,
     }
 }
 
+// ------------------------------------------------------------------ parts of a step
+
+// A lane's base addresses and constants.
+template <class LAY, class LG, int R>
+struct StepLane {
+    using SH = StepShape<LG, R>;
+    StepProduct<LAY, LG, R> prod;
+    uint32_t xr;      // results; coefficients at a fixed distance
+    uint32_t zr, sr;  // Z and s_{3i-L+1} of the outputs
+    uint32_t rows, gw, zw;
+    float sig4, bias;
+    uint32_t ib;  // free variables i of outputs 0-3, one byte each
+    int hw4;      // row words from here on are zero in both copies
+    int wb, n;
+    __device__ __forceinline__ StepLane(int wb0, int n_, const LG& t, const Outs<LG, R>& o)
+        : prod(wb0, t.lane + t.base), wb(wb0 + group_of(t) * LAY::SL.words), n(n_)
+    {
+        constexpr StepSmem SL = LAY::SL;
+        const int c = n - 1;
+        xr = sbyte(wb + SL.x + o.p * SL.xp + o.v0);
+        // a lane without outputs reads Z below 0 (no output) and any finite row entry
+        zr = sbyte(wb + SL.z) + 2 * max(c - o.p - 2 * o.v0, -1);
+        sr = sbyte(wb + SL.h0 + o.p * SL.hc) + 2 * (2 * o.v0 + o.p <= c ? 3 * o.v0 + o.p - n + 1 : 0);
+        rows = sbyte(wb + SL.h0);
+        gw = sbyte(wb + SL.g + 4 * t.lane);
+        zw = sbyte(wb + SL.z + 2 * t.lane);
+        sig4 = ((c - o.p) & 1) ? -4.f : 4.f;
+        bias = (float)(16 * (n - o.p - 3)) + kIntBias;  // 16 (N_p - 2), N_p = n - 1 - p
+        ib = (uint32_t)(2 * o.v0 + o.p) * 0x01010101u + 0x06040200u;
+        hw4 = 4 * ((n + 1) >> 1);
+    }
+};
+
+// Keys (dISL + 2^22) << 8 | i of the lane's outputs after step_toeplitz, ascending in (dISL,
+// i): the FP32 value dISL + 1.5 2^23 holds the integer in its low bits, and one byte
+// permute puts i below its low three bytes.  Outputs that do not exist or are marked have
+// an infinite Z, whose bytes give a key of at least 2^31.  ms (MS): -8 s_i / 2 as FP16 pairs.
+template <bool MS, class LAY, class LG, int R>
+__device__ __forceinline__ void step_keys(const StepLane<LAY, LG, R>& a, unsigned (&key)[R], uint32_t (&ms)[(R + 1) / 2])
+{
+    constexpr StepSmem SL = LAY::SL;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float x = lds_f32(a.xr + 4 * r), r8 = lds_f32(a.xr - 4u * (uint32_t)(SL.x - SL.r8) + 4 * r);
+        const float z = lds_f16(a.zr - 4 * r), s3 = lds_f16(a.sr + 6 * r);
+        const float v = fmaf(r8, fmaf(a.sig4, s3, x), fmaf(8.f, z, a.bias));
+        key[r] = __byte_perm(__float_as_uint(v), r < 4 ? a.ib : r < 8 ? a.ib + 0x08080808u : a.ib + 0x10101010u,
+                             0x2104 + (r & 3));
+        if (MS) {
+            const uint32_t h = __half_as_ushort(__float2half_rn(0.5f * r8));
+            ms[r >> 1] = (r & 1) ? ms[r >> 1] | (h << 16) : h;
+        }
+    }
+}
+
+// Flips free variable bi (and its mirror) of the walkers with `moves` in rows, coefficients,
+// table and Z; neg: 0x80000000 where s_i = -1 before the flip.  mark: the flipped output is
+// no candidate of the next step (the lags' next store of Z takes the mark away).   The flipped entries read as 0 while the sums are
+// taken, which leaves out the pairs whose two ends both flip and lag 0.
+template <class LAY, class LG, int R>
+__device__ __forceinline__ void step_flip(const StepLane<LAY, LG, R>& a, StepLags<StepShape<LG, R>::NB>& lg, bool moves,
+                                          int bi, uint32_t neg, bool mark, const LG& t)
+{
+    constexpr StepSmem SL = LAY::SL;
+    constexpr int NL = LG::kSize, NB = StepShape<LG, R>::NB;
+    const int lane = t.lane, n = a.n, c = n - 1;
+    const int pb = bi & 1, vb = bi >> 1, vq = n - 1 - pb - vb;
+    const bool centre = bi == c, same = ((pb ^ c) & 1) == 0;  // same: sg = +1 in the flipped class
+    const uint32_t rb = a.rows + (pb ? 4 * SL.hc : 0);
+    const bool writer = moves && lane < 2;  // lane 0 writes s_i, lane 1 its mirror
+    const uint32_t ea = rb + 2 * (lane ? vq : vb);
+    sts_u16_if(writer, ea, 0u);
+    sts_u16_if(writer, ea + 4 * SL.ks - 2, 0u);
+    __syncwarp();
+    {
+        // at lag m the flipped class's autocorrelation changes by -2 s_i (a_{vb+m} +
+        // a_{vb-m}) for each flipped end, in all coef (a_{vb+m} + sg a_{vq+m}), coef = -4
+        // s_i (centre: -2 s_c): a_{vb-m} = sg a_{vq+m}
+        const __half2 coef = as_half2(moves ? (centre ? 0xC000C000u : 0xC400C400u) ^ (neg | neg >> 16) : 0u);
+        const __half2 sig = as_half2(same ? 0x3C003C00u : 0xBC00BC00u);
+        // Z: 3 x the lag's own class, 1 x the other, sign (-1)^m
+        const __half2 cz = __hmul2(coef, as_half2(same ? 0xBC004200u : 0xC2003C00u));
+        const uint32_t ub = rb + ((vb & 1) ? 4 * SL.ks : 0), qb = rb + ((vq & 1) ? 4 * SL.ks : 0);
+        const int uo = 2 * (vb & ~1) + 8 * lane, qo = 2 * (vq & ~1) + 8 * lane;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const uint32_t u = ub + min(uo + 8 * NL * b, a.hw4), q = qb + min(qo + 8 * NL * b, a.hw4);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const __half2 s2 = __hfma2(sig, as_half2(lds_u32(q + 4 * j)), as_half2(lds_u32(u + 4 * j)));
+                lg.e[b][j] = as_u32(__hfma2(coef, s2, as_half2(lg.e[b][j])));
+                lg.z[b][j] = as_u32(__hfma2(cz, s2, as_half2(lg.z[b][j])));
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            // the lag after the lane's block: the next lane's first (the next block's first
+            // lane for the last one)
+            const uint32_t give = lane == 0 ? (b + 1 < NB ? lg.e[b + 1 < NB ? b + 1 : b][0] : 0u) : lg.e[b][0];
+            const uint32_t nx = __shfl_sync(kFull, give, t.base + ((lane + 1) & (NL - 1)));
+            const uint32_t e0 = lg.e[b][0], e1 = lg.e[b][1];
+            const uint32_t o0 = __byte_perm(e0, e1, 0x5432), o1 = __byte_perm(e1, nx, 0x5432);
+            if (4 * NL * (b + 1) <= SL.gpos)
+                sts_v4(a.gw + 16 * NL * b, e0, o0, e1, o1);
+            else
+                sts_v4_if(lane < SL.gpos / 4 - NL * b, a.gw + 16 * NL * b, e0, o0, e1, o1);
+            if (4 * NL * b < SL.gneg) {
+                // the mirror: G[-m-1] is G[m] with its halves exchanged
+                const uint32_t m = a.gw - 32 * lane - 16 - 16 * NL * b;
+                const uint32_t r0 = __byte_perm(o1, o1, 0x1032), r1 = __byte_perm(e1, e1, 0x1032),
+                               r2 = __byte_perm(o0, o0, 0x1032), r3 = __byte_perm(e0, e0, 0x1032);
+                if (4 * NL * (b + 1) <= SL.gneg)
+                    sts_v4(m, r0, r1, r2, r3);
+                else
+                    sts_v4_if(lane < SL.gneg / 4 - NL * b, m, r0, r1, r2, r3);
+            }
+            sts_v2(a.zw + 8 * NL * b, lg.z[b][0], lg.z[b][1]);
+        }
+    }
+    __syncwarp();
+    // s_i and, with the class's sign, its mirror, both negated: an entry is +1 exactly when
+    // s_i (lane 1: sg s_i) was -1
+    const uint32_t s = (neg != 0u) == (lane == 0 || same) ? 0x3C00u : 0xBC00u;
+    sts_u16_if(writer, ea, s);
+    sts_u16_if(writer, ea + 4 * SL.ks - 2, s);
+    const bool first = moves && lane == 0;
+    sts_f32_if(first, sbyte(a.wb + SL.r8) + (pb ? 4 * SL.xp : 0) + 4 * vb,
+               __uint_as_float((centre ? 0x40800000u : 0x41000000u) | neg));
+    if (mark) sts_u16_if(first, sbyte(a.wb + SL.z) + 2 * (c - bi), kHalfInf);
+}
+
+// 0x80000000 where free variable i of the walker's bits is -1.
+template <class LG>
+__device__ __forceinline__ uint32_t step_sign(uint32_t word, int i, const LG& t)
+{
+    return (t.shfl(word, i >> 5) << (31 - (i & 31))) & 0x80000000u;
+}
+
 // ------------------------------------------------------------------ the walk's steps
 
 // Advances the warp's walkers by up to len steps each (one per lane group; `real`: the
@@ -721,30 +859,16 @@ template <class LAY, class LG, class RT, int R>
 __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, int len, bool real, int wb0,
                                              unsigned extras, const LG& t, const RT& tt)
 {
-    using SH = StepShape<LG, R>;
     constexpr StepSmem SL = LAY::SL;
-    constexpr int NL = SH::NL, NB = SH::NB;
+    constexpr int NL = LG::kSize, NB = StepShape<LG, R>::NB;
     constexpr int S = NL / 2;  // HT slots probed per candidate in a round
     constexpr bool PSL = LAY::kPsl;
     using KT = typename StepKey<PSL>::type;
     const KParams& p = *env.p;
     const int lane = t.lane, l = lane + t.base, n = env.n, c = n - 1;
-    const int wb = wb0 + group_of(t) * SL.words;
     const Outs<LG, R> o(t);
-
-    // base addresses of the lane
-    const StepProduct<LAY, LG, R> prod(wb0, l);
-    const uint32_t xr = sbyte(wb + SL.x + o.p * SL.xp + o.v0);  // results; coefficients at a fixed distance
-    // a lane without outputs reads Z below 0 (no output) and any finite row entry
-    const uint32_t zr = sbyte(wb + SL.z) + 2 * max(c - o.p - 2 * o.v0, -1);
-    const uint32_t sr = sbyte(wb + SL.h0 + o.p * SL.hc) + 2 * (2 * o.v0 + o.p <= c ? 3 * o.v0 + o.p - n + 1 : 0);
-    const uint32_t rows = sbyte(wb + SL.h0);
-    const uint32_t gw = sbyte(wb + SL.g + 4 * lane), zw = sbyte(wb + SL.z + 2 * lane);
-    const float sig4 = ((c - o.p) & 1) ? -4.f : 4.f;
-    const float bias = (float)(16 * (n - o.p - 3)) + kIntBias;  // 16 (N_p - 2), N_p = n - 1 - p
-    const uint32_t ib = (uint32_t)(2 * o.v0 + o.p) * 0x01010101u + 0x06040200u;  // free variables i of outputs 0-3
-    const int hw4 = 4 * ((n + 1) >> 1);  // row words from here on are zero in both copies
-
+    const StepLane<LAY, LG, R> a(wb0, n, t, o);
+    const int wb = a.wb;
     StepLags<NB> lg;
     step_load_lags<LAY, LG, R>(wb, lane, lg);
     StopCheck stop;
@@ -760,30 +884,16 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
                 break;
             }
         }
-        step_toeplitz<LAY, LG, R>(prod, l);
+        step_toeplitz<LAY, LG, R>(a.prod, l);
 
-        // keys (dISL + 2^22) << 8 | i, ascending in (dISL, i): the FP32 value dISL + 1.5 2^23
-        // holds the integer in its low bits, and one byte permute puts i below its low
-        // three bytes.  Outputs that do not exist and the move back to the state just left
-        // (marked below; that state is always in HT) have an infinite Z, whose bytes give a
-        // key of at least 2^31.  Under the PSL objective the PSL (as FP16 bits, which order
-        // as the integers do) goes above it.
+        // The move back to the state just left is marked (that state is always in HT).  Under
+        // the PSL objective the PSL (as FP16 bits, which order as the integers do) goes above
+        // the key.
         KT key[R];
         {
             unsigned kl[R];
             uint32_t ms[(R + 1) / 2];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float x = lds_f32(xr + 4 * r), r8 = lds_f32(xr - 4u * (uint32_t)(SL.x - SL.r8) + 4 * r);
-                const float z = lds_f16(zr - 4 * r), s3 = lds_f16(sr + 6 * r);
-                const float v = fmaf(r8, fmaf(sig4, s3, x), fmaf(8.f, z, bias));
-                kl[r] = __byte_perm(__float_as_uint(v), r < 4 ? ib : r < 8 ? ib + 0x08080808u : ib + 0x10101010u,
-                                    0x2104 + (r & 3));
-                if (PSL) {  // -8 s_i / 2
-                    const uint32_t h = __half_as_ushort(__float2half_rn(0.5f * r8));
-                    ms[r >> 1] = (r & 1) ? ms[r >> 1] | (h << 16) : h;
-                }
-            }
+            step_keys<PSL>(a, kl, ms);
             if constexpr (PSL) {
                 uint32_t mx[(R + 1) / 2];
 #pragma unroll
@@ -859,79 +969,11 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
         const bool moves = act && kc != ~(KT)0;
         stg_u64_if(moves && (pick >> l) == 1u, env.T + at, tag);
 
-        // Apply the move (walkers that have one).  The flipped entries read as 0 while the
-        // sums are taken, which leaves out the pairs whose two ends both flip and lag 0.
+        // Apply the move (walkers that have one).
         const int bi = moves ? (int)((uint32_t)kc & 0xFFu) : 0;
-        const int pb = bi & 1, vb = bi >> 1, vq = n - 1 - pb - vb;
-        const bool centre = bi == c, same = ((pb ^ c) & 1) == 0;  // same: sg = +1 in the flipped class
-        const uint32_t wsh = t.shfl(w.word, bi >> 5) << (31 - (bi & 31));
-        const uint32_t neg = wsh & 0x80000000u;  // s_i = -1
-        const uint32_t rb = rows + (pb ? 4 * SL.hc : 0);
-        const bool writer = moves && lane < 2;   // lane 0 writes s_i, lane 1 its mirror
-        const uint32_t ea = rb + 2 * (lane ? vq : vb);
-        sts_u16_if(writer, ea, 0u);
-        sts_u16_if(writer, ea + 4 * SL.ks - 2, 0u);
+        const uint32_t neg = step_sign(w.word, bi, t);
         const uint64_t zk = __ldg(env.zk + bi);
-        __syncwarp();
-        {
-            // at lag m the flipped class's autocorrelation changes by -2 s_i (a_{vb+m} +
-            // a_{vb-m}) for each flipped end, in all coef (a_{vb+m} + sg a_{vq+m}), coef = -4
-            // s_i (centre: -2 s_c): a_{vb-m} = sg a_{vq+m}
-            const __half2 coef = as_half2(moves ? (centre ? 0xC000C000u : 0xC400C400u) ^ (neg | neg >> 16) : 0u);
-            const __half2 sig = as_half2(same ? 0x3C003C00u : 0xBC00BC00u);
-            // Z: 3 x the lag's own class, 1 x the other, sign (-1)^m
-            const __half2 cz = __hmul2(coef, as_half2(same ? 0xBC004200u : 0xC2003C00u));
-            const uint32_t ub = rb + ((vb & 1) ? 4 * SL.ks : 0), qb = rb + ((vq & 1) ? 4 * SL.ks : 0);
-            const int uo = 2 * (vb & ~1) + 8 * lane, qo = 2 * (vq & ~1) + 8 * lane;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const uint32_t u = ub + min(uo + 8 * NL * b, hw4), q = qb + min(qo + 8 * NL * b, hw4);
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const __half2 s2 = __hfma2(sig, as_half2(lds_u32(q + 4 * j)), as_half2(lds_u32(u + 4 * j)));
-                    lg.e[b][j] = as_u32(__hfma2(coef, s2, as_half2(lg.e[b][j])));
-                    lg.z[b][j] = as_u32(__hfma2(cz, s2, as_half2(lg.z[b][j])));
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                // the lag after the lane's block: the next lane's first (the next block's
-                // first lane for the last one)
-                const uint32_t give = lane == 0 ? (b + 1 < NB ? lg.e[b + 1 < NB ? b + 1 : b][0] : 0u) : lg.e[b][0];
-                const uint32_t nx = __shfl_sync(kFull, give, t.base + ((lane + 1) & (NL - 1)));
-                const uint32_t e0 = lg.e[b][0], e1 = lg.e[b][1];
-                const uint32_t o0 = __byte_perm(e0, e1, 0x5432), o1 = __byte_perm(e1, nx, 0x5432);
-                if (4 * NL * (b + 1) <= SL.gpos)
-                    sts_v4(gw + 16 * NL * b, e0, o0, e1, o1);
-                else
-                    sts_v4_if(lane < SL.gpos / 4 - NL * b, gw + 16 * NL * b, e0, o0, e1, o1);
-                if (4 * NL * b < SL.gneg) {
-                    // the mirror: G[-m-1] is G[m] with its halves exchanged
-                    const uint32_t m = gw - 32 * lane - 16 - 16 * NL * b;
-                    const uint32_t r0 = __byte_perm(o1, o1, 0x1032), r1 = __byte_perm(e1, e1, 0x1032),
-                                   r2 = __byte_perm(o0, o0, 0x1032), r3 = __byte_perm(e0, e0, 0x1032);
-                    if (4 * NL * (b + 1) <= SL.gneg)
-                        sts_v4(m, r0, r1, r2, r3);
-                    else
-                        sts_v4_if(lane < SL.gneg / 4 - NL * b, m, r0, r1, r2, r3);
-                }
-                sts_v2(zw + 8 * NL * b, lg.z[b][0], lg.z[b][1]);
-            }
-        }
-        __syncwarp();
-        {
-            // s_i and, with the class's sign, its mirror, both negated: an entry is +1
-            // exactly when s_i (lane 1: sg s_i) was -1
-            const uint32_t s = (neg != 0u) == (lane == 0 || same) ? 0x3C00u : 0xBC00u;
-            sts_u16_if(writer, ea, s);
-            sts_u16_if(writer, ea + 4 * SL.ks - 2, s);
-            const bool first = moves && lane == 0;
-            sts_f32_if(first, sbyte(wb + SL.r8) + (pb ? 4 * SL.xp : 0) + 4 * vb,
-                       __uint_as_float((centre ? 0x40800000u : 0x41000000u) | neg));
-            // the move back is no candidate of the next step (the lags' next store of Z takes
-            // the mark away)
-            sts_u16_if(first, sbyte(wb + SL.z) + 2 * (c - bi), kHalfInf);
-        }
+        step_flip(a, lg, moves, bi, neg, true, t);
         bool again = act;
         if (moves) {
             if (lane == (bi >> 5)) w.word ^= 1u << (bi & 31);
@@ -980,6 +1022,239 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
     return min(it, len);
 }
 
+// ------------------------------------------------------------------ best-first search
+//
+// Algorithm 1 as printed (impxLast, Section 3): the neighbourhood of S fills a queue of
+// LABS_QUEUE_SIZE evaluated neighbours ordered by merit factor and the next S is the queue's
+// first entry (the readings are stated with labs_walk in labs.h).  One walker per warp; lane
+// l holds queue entry l as a 64-bit key
+//   ISL << 36 | (steps done before the step that produced it) << 8 | i
+// (ascending = the queue order; ~0 = empty) and the entry's free variables live in global
+// memory.  A new S that differs from S in at most kBestFirstMaxFlips free variables is
+// reached by that many flips, any other by a rebuild from its bits.
+//
+// What bounds it: the queue's insertions and the move, not the neighbourhood (about 3
+// insertions a step, each a minimum over the warp and an HT lookup).
+template <class LAY, int R>
+__device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w, int len, bool real, int wb,
+                                              unsigned extras, const Tile<32>& t)
+{
+    static_assert(LABS_QUEUE_SIZE == 32, "one queue entry per lane");
+    using LG = Tile<32>;
+    const KParams& p = *env.p;
+    const int lane = t.lane, n = env.n;
+    const Outs<LG, R> o(t);
+    const StepLane<LAY, LG, R> a(wb, n, t, o);
+    const int cap = p.probe_cap;
+    const uint32_t tmask = (1u << p.tabu_log2) - 1u;
+    uint64_t* const qkey = p.pq_key + (int64_t)env.g * LABS_QUEUE_SIZE;
+    uint32_t* const qbits = p.pq_bits + (int64_t)env.g * LABS_QUEUE_SIZE * kBitWords;
+    uint64_t qk = qkey[lane];
+    // xLastovka's second table (null when off): slot f mod size holds
+    // (generation << 40) | (~f mod 2^40) of an evaluated neighbour f
+    uint64_t* const T2 = p.tabu2 != nullptr ? p.tabu2 + (env.T - p.tabu) : nullptr;
+    constexpr uint64_t kLow40 = 0xFFFFFFFFFFull;
+    int64_t hits = 0;
+    const int64_t steps0 = env.state()->steps_done;
+    StepLags<StepShape<LG, R>::NB> lg;
+    step_load_lags<LAY, LG, R>(wb, lane, lg);
+    StopCheck stop;
+    stop.start(p, lane == 0);
+    if (!real) len = 0;
+    int it = 0;
+    for (; it < len; ++it) {
+        if ((it & (kCheckEvery - 1)) == 0) {
+            const int why = t.shfl(stop.poll(p, lane == 0), 0);
+            if (why) {
+                if (lane == 0) raise_error(p.status, why, (int)env.g);
+                break;
+            }
+        }
+        const uint64_t e = (uint64_t)(steps0 + it);
+        step_toeplitz<LAY, LG, R>(a.prod, lane);
+        unsigned key[R];
+        {
+            uint32_t ms[(R + 1) / 2];
+            step_keys<false>(a, key, ms);
+        }
+        if (T2 != nullptr) {
+            // neighbours the table holds are skipped (their keys dropped); every other one is
+            // inserted once all lanes have looked (larger word kept: the table does not
+            // depend on the order of the insertions)
+            uint64_t ins[R];
+            int h = 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                ins[r] = 0ull;
+                if ((int)key[r] < 0) continue;
+                const uint64_t f = w.fp ^ __ldg(env.zk + (key[r] & 0xFFu));
+                const uint64_t tag = ((uint64_t)w.gen << 40) | (~f & kLow40);
+                if (T2[(uint32_t)f & tmask] == tag) {
+                    key[r] = 0xFFFFFFFFu;
+                    ++h;
+                } else {
+                    ins[r] = f;
+                }
+            }
+            hits += t.radd(h);
+            t.sync();
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((int)key[r] >= 0)
+                    atomicMax(reinterpret_cast<unsigned long long*>(T2 + ((uint32_t)ins[r] & tmask)),
+                              (unsigned long long)(((uint64_t)w.gen << 40) | (~ins[r] & kLow40)));
+            t.sync();
+        }
+        // Neighbours in queue order (ISL, then i: the packed keys' order) while they come
+        // before the queue's last entry or the queue has a free place.  The last entry only
+        // moves forward during the step, so neighbours after its value at the start cannot
+        // enter; the others are looked up in HT as the insertion reaches them (HT does not
+        // change during the insertion).  A new key orders behind the queue's of equal ISL (its
+        // step is later, or its i is higher), so a candidate comes before the last entry
+        // exactly when its ISL is lower.
+        unsigned qempty = t.ballot(qk == ~0ull);
+        uint64_t last = qempty ? ~0ull : warp_max64(qk);
+        unsigned limit = 0x80000000u;  // keys below it may enter
+        if (!qempty) {
+            const int64_t d = (int64_t)(last >> 36) - w.isl + kKeyBias;
+            limit = d <= 0 ? 0u : (unsigned)min(d << 8, (int64_t)0x80000000ll);
+        }
+        unsigned floor = 0u;
+        for (;;) {
+            unsigned b = 0x80000000u;
+#pragma unroll
+            for (int r = 0; r < R; ++r) b = min(b, key[r] > floor ? key[r] : 0x80000000u);
+            const unsigned k = t.rminu(b);
+            if (k >= limit) break;
+            floor = k;
+            const int i = (int)(k & 0xFFu);
+            {
+                // HT lookup of this neighbour: up to probe_cap slots, four per round
+                const uint64_t f = w.fp ^ __ldg(env.zk + i);
+                const uint64_t tag = (f & ~kGenMask) | w.gen;
+                bool visited = false;
+                for (int s0 = 0; s0 < cap; s0 += 4) {
+                    const bool mine = lane < 4 && s0 + lane < cap;
+                    const uint64_t x = mine ? env.T[((uint32_t)f + (uint32_t)(s0 + lane)) & tmask] : 0ull;
+                    const unsigned bal = t.ballot(mine && ((((uint32_t)x & (uint32_t)kGenMask) != w.gen) || x == tag));
+                    const unsigned mat = t.ballot(mine && x == tag);
+                    if (bal) {
+                        visited = (mat & bal & (0u - bal)) != 0u;
+                        break;
+                    }
+                }
+                if (visited) continue;
+            }
+            const int isl_f = w.isl + (int)(k >> 8) - kKeyBias;
+            const uint64_t ck = ((uint64_t)isl_f << 36) | (e << 8) | (uint64_t)i;
+            const int dst = __ffs(qempty ? qempty : t.ballot(qk == last)) - 1;
+            if (lane == dst) qk = ck;
+            const uint32_t word = w.word ^ (lane == (i >> 5) ? 1u << (i & 31) : 0u);
+            if (lane < kBitWords) qbits[dst * kBitWords + lane] = word;
+            if (isl_f < w.best) {
+                w.best = isl_f;
+                if (lane == 0) env.state()->best_step = (int64_t)e + 1;
+                if (lane < kBitWords) env.state()->best[lane] = word;
+            }
+            if (isl_f <= w.tisl) {
+                w.tisl = -1;
+                if (lane == 0) env.state()->target_step = (int64_t)e + 1;
+            }
+            qempty &= qempty - 1u;
+            if (!qempty) {
+                // the queue is full: the rest enter only below its last entry
+                last = warp_max64(qk);
+                const int64_t d = (int64_t)(last >> 36) - w.isl + kKeyBias;
+                limit = d <= 0 ? 0u : (unsigned)min(d << 8, (int64_t)0x80000000ll);
+            }
+        }
+        t.sync();
+        // S <- the queue's first entry not in HT (entries that are get dropped)
+        int code = LABS_TRACE_BLOCKED;
+        bool again = true, moved = false;
+        for (;;) {
+            if (!t.ballot(qk != ~0ull)) break;  // empty queue: restart
+            const uint64_t first = warp_min64(qk);
+            const int src = __ffs(t.ballot(qk == first)) - 1;
+            const uint32_t word = lane < kBitWords ? qbits[src * kBitWords + lane] : 0u;
+            if (lane == src) qk = ~0ull;
+            const int i = (int)(first & 0xFFu);
+            const bool nb = ((first >> 8) & 0xFFFFFFFull) == e;  // a neighbour of S
+            const uint64_t f = nb ? (w.fp ^ __ldg(env.zk + i)) : fingerprint_all(word, env.zk, n, t);
+            const uint64_t tag = (f & ~kGenMask) | w.gen;
+            bool visited = false;
+            int64_t slot = -1;
+            for (int s0 = 0; s0 < cap; s0 += 32) {
+                const int s = s0 + lane;
+                const uint64_t x = s < cap ? env.T[((uint32_t)f + (uint32_t)s) & tmask] : 0ull;
+                const unsigned bal = t.ballot(s < cap && ((((uint32_t)x & (uint32_t)kGenMask) != w.gen) || x == tag));
+                const unsigned mat = t.ballot(s < cap && x == tag);
+                if (bal) {
+                    visited = (mat & bal & (0u - bal)) != 0u;
+                    slot = ((uint32_t)f + (uint32_t)(s0 + __ffs(bal) - 1)) & tmask;
+                    break;
+                }
+            }
+            if (visited) continue;
+            // free variables in which the new S differs from S (1 for a neighbour)
+            uint32_t diff = lane < kBitWords ? (word ^ w.word) : 0u;
+            const int k = nb ? 1 : t.radd(__popc(diff));
+            if (k <= kBestFirstMaxFlips) {
+                // flip them one by one, lowest first
+                for (int j = 0; j < k; ++j) {
+                    const unsigned bl = t.ballot(diff != 0u);
+                    const int sl = __ffs(bl) - 1;
+                    const int fi = 32 * sl + t.shfl(__ffs(diff) - 1, sl);
+                    const uint32_t neg = step_sign(w.word, fi, t);
+                    step_flip(a, lg, true, fi, neg, false, t);
+                    t.sync();
+                    if (lane == sl) diff &= diff - 1u;
+                }
+            } else {
+                int none;
+                step_build<LAY>(wb, word, 2 * n - 1, n, t, &none);
+                step_load_lags<LAY, LG, R>(wb, lane, lg);
+            }
+            moved = true;
+            w.word = word;
+            w.isl = (int)(first >> 36);
+            w.fp = f;
+            code = (int)(f & 0xFFFFu);
+            if (slot >= 0) {
+                if (lane == 0) env.T[slot] = tag;
+                again = false;
+            } else {
+                code |= LABS_TRACE_RESTART;  // no free HT slot for the new S: restart
+            }
+            break;
+        }
+        if (again) {
+            WalkerState* st = env.state();
+            if (lane == 0) {
+                if (moved)
+                    st->overflows += 1;
+                else
+                    st->blocked += 1;
+            }
+            qk = ~0ull;
+            const uint32_t gen0 = w.gen;
+            step_restart<LAY>(env, w, wb, (int64_t)e + 1, t);
+            if (T2 != nullptr && w.gen < gen0) {  // generations wrapped: HT was zeroed, so is T2
+                for (int64_t i = lane; i <= (int64_t)tmask; i += 32) T2[i] = 0ull;
+                t.sync();
+            }
+            step_load_lags<LAY, LG, R>(wb, lane, lg);
+        }
+        t.sync();
+        if (extras && lane == 0) step_note(env, it, code, w.isl, extras & 1u);
+    }
+    if (real) {
+        qkey[lane] = qk;
+        if (lane == 0) env.state()->cache_hits += hits;
+    }
+    return it;
+}
+
 // CTAs of 8 warps per SM the walk kernels are compiled for: three (80 registers a thread),
 // but two where three would not fit in shared memory (four walkers per warp, lane blocks
 // from 7)
@@ -991,7 +1266,7 @@ __host__ __device__ constexpr int step_ctas(int tile, int R, bool psl = false)
 // Runs the walkers of the queue: the warp takes W consecutive walkers; when their lengths
 // differ (a group boundary) or fewer are left, it runs them one after the other with the
 // other lane groups idle.
-template <class LG, class RT, int RMAX, bool PSL = false>
+template <class LG, class RT, int RMAX, bool PSL = false, bool BEST = false>
 __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
 {
     constexpr int NL = LG::kSize, W = 32 / NL;
@@ -1071,7 +1346,12 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
             int R = step_R(G.n, NL);
             if (R < RMAX - 3) R = conflict_free_R(RMAX - 3, NL);
             int done;
-            if constexpr (NL == 32) {  // lane blocks are odd
+            if constexpr (BEST) {
+                if (R >= RMAX)
+                    done = walk_bestfirst<LAY, RMAX>(env, w, len, real, wb0, extras, t);
+                else
+                    done = walk_bestfirst<LAY, (RMAX > 2 ? RMAX - 2 : 1)>(env, w, len, real, wb0, extras, t);
+            } else if constexpr (NL == 32) {  // lane blocks are odd
                 if (R >= RMAX)
                     done = walk_lockstep<LAY, LG, RT, RMAX>(env, w, len, real, wb0, extras, t, tt);
                 else
