@@ -1050,6 +1050,12 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
     uint64_t* const qkey = p.pq_key + (int64_t)env.g * LABS_QUEUE_SIZE;
     uint32_t* const qbits = p.pq_bits + (int64_t)env.g * LABS_QUEUE_SIZE * kBitWords;
     uint64_t qk = qkey[lane];
+    // the entry's fingerprint (kept beside its key while the chunk runs)
+    uint64_t qf = 0ull;
+    if (qk != ~0ull)
+        for (int j = 0; 32 * j < n; ++j)
+            for (uint32_t x = qbits[lane * kBitWords + j]; x; x &= x - 1u) qf ^= __ldg(env.zk + 32 * j + __ffs(x) - 1);
+    __syncwarp();
     // xLastovka's second table (null when off): slot f mod size holds
     // (generation << 40) | (~f mod 2^40) of an evaluated neighbour f
     uint64_t* const T2 = p.tabu2 != nullptr ? p.tabu2 + (env.T - p.tabu) : nullptr;
@@ -1119,6 +1125,15 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
             const int64_t d = (int64_t)(last >> 36) - w.isl + kKeyBias;
             limit = d <= 0 ? 0u : (unsigned)min(d << 8, (int64_t)0x80000000ll);
         }
+        // the HT lines of the lanes' lowest candidates are on their way before the insertion
+        // asks for them one after the other
+        {
+            unsigned b = key[0];
+#pragma unroll
+            for (int r = 1; r < R; ++r) b = min(b, key[r]);
+            if (b < limit)
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(env.T + ((uint32_t)(w.fp ^ __ldg(env.zk + (b & 0xFFu))) & tmask)));
+        }
         unsigned floor = 0u;
         for (;;) {
             unsigned b = 0x80000000u;
@@ -1128,9 +1143,9 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
             if (k >= limit) break;
             floor = k;
             const int i = (int)(k & 0xFFu);
+            const uint64_t f = w.fp ^ __ldg(env.zk + i);
             {
                 // HT lookup of this neighbour: up to probe_cap slots, four per round
-                const uint64_t f = w.fp ^ __ldg(env.zk + i);
                 const uint64_t tag = (f & ~kGenMask) | w.gen;
                 bool visited = false;
                 for (int s0 = 0; s0 < cap; s0 += 4) {
@@ -1148,7 +1163,10 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
             const int isl_f = w.isl + (int)(k >> 8) - kKeyBias;
             const uint64_t ck = ((uint64_t)isl_f << 36) | (e << 8) | (uint64_t)i;
             const int dst = __ffs(qempty ? qempty : t.ballot(qk == last)) - 1;
-            if (lane == dst) qk = ck;
+            if (lane == dst) {
+                qk = ck;
+                qf = f;
+            }
             const uint32_t word = w.word ^ (lane == (i >> 5) ? 1u << (i & 31) : 0u);
             if (lane < kBitWords) qbits[dst * kBitWords + lane] = word;
             if (isl_f < w.best) {
@@ -1178,9 +1196,8 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
             const int src = __ffs(t.ballot(qk == first)) - 1;
             const uint32_t word = lane < kBitWords ? qbits[src * kBitWords + lane] : 0u;
             if (lane == src) qk = ~0ull;
-            const int i = (int)(first & 0xFFu);
             const bool nb = ((first >> 8) & 0xFFFFFFFull) == e;  // a neighbour of S
-            const uint64_t f = nb ? (w.fp ^ __ldg(env.zk + i)) : fingerprint_all(word, env.zk, n, t);
+            const uint64_t f = ((uint64_t)t.shfl((uint32_t)(qf >> 32), src) << 32) | t.shfl((uint32_t)qf, src);
             const uint64_t tag = (f & ~kGenMask) | w.gen;
             bool visited = false;
             int64_t slot = -1;
