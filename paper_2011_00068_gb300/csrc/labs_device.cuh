@@ -223,6 +223,7 @@ struct View {
     uint32_t* B;  // bit-packed classes and reversals, 4 x bvec words
     __half* H0;   // FP16 copies of A0 and A1 for the tensor-core Toeplitz product (null:
     __half* H1;   // none); every write of a row entry writes its copy too
+    int* wide;    // long tensor-core layout: nonzero when some |E| is above 2^11 (null: none)
     int gpad;
     int bvec;
 };
@@ -236,6 +237,7 @@ __device__ __forceinline__ View make_view(int* base, const WarpSmem& L)
     v.B = reinterpret_cast<uint32_t*>(base + L.boff);
     v.H0 = L.hlen ? reinterpret_cast<__half*>(base + L.hoff) + L.hpad : nullptr;
     v.H1 = L.hlen ? reinterpret_cast<__half*>(base + L.hoff + L.hlen) + L.hpad : nullptr;
+    v.wide = L.foff ? base + L.foff : nullptr;
     v.gpad = L.gpad;
     v.bvec = L.bvec;
     return v;
@@ -246,6 +248,13 @@ __device__ __forceinline__ void set_row(const View& V, int p, int u, float s)
 {
     (p ? V.A1 : V.A0)[u] = s;
     if (V.H0 != nullptr) (p ? V.H1 : V.H0)[u] = __float2half_rn(s);
+}
+
+// Integers above 2^11 in magnitude are not all FP16 numbers: a table that holds one is
+// marked, and its Toeplitz product takes the FP32 pipes until the rows are rebuilt.
+__device__ __forceinline__ void note_wide(const View& V, float e)
+{
+    if (V.wide != nullptr && fabsf(e) > 2048.f) *V.wide = 1;
 }
 
 // E[m] = e (m >= 1) in every pair of G that holds it, mirrored to E[-m].
@@ -511,85 +520,73 @@ __device__ __forceinline__ void toeplitz_tc(const View& V, const WarpSmem& SL, i
     for (int r = 0; r < R; ++r) X[r] = xr[r];
 }
 
-// The same product for one walker whose lane group spans W whole warps (one walker per
-// warp, W = 1, or per CTA): the output blocks form ceil(T/4) column groups of 4 blocks
-// per class, warp w takes groups w, w + W, ..., and for group m the block diagonals run
-// from -(4m+3) (or -(T-1)) up to S-1-4m.  Two accumulator chains per warp (two groups,
-// or the even and odd diagonals of a lone group; integer partial sums, so the split does
-// not change the result).  The results go through the walker's scratch X[2][xp] to the
-// lanes' R outputs; the group's barrier orders them.
+// The same product for one walker on one warp: the output blocks form M = ceil(T/4)
+// column groups of 4 blocks per class (M <= 2 for n <= 256), and for group m the block
+// diagonals run from -(4m+3) (or -(T-1)) up to S-1-4m.  Two accumulator chains (two
+// groups, or the even and odd diagonals of a lone group; integer partial sums, so the
+// split does not change the result).  The results go through the walker's scratch X[2][xp]
+// to the lanes' R outputs.
 template <class LG, int R>
 __device__ __forceinline__ void toeplitz_tc1(const View& V, const WarpSmem& SL, int n, const Outs<LG, R>& o,
                                              const LG& t, float (&X)[R])
 {
-    constexpr int W = LG::kSize / 32;
-    const int warp = W == 1 ? 0 : (int)(threadIdx.x >> 5), l = threadIdx.x & 31, g = l >> 2, tq = l & 3;
+    const int l = threadIdx.x & 31, g = l >> 2, tq = l & 3;
     const int S = (n + 15) >> 4, T = (((n + 1) >> 1) + 15) >> 4, M = (T + 3) >> 2;
     const int pb = g >> 2, tb = g & 3, px = tq >> 1, tx = 2 * (tq & 1);
     int* const base = reinterpret_cast<int*>(V.A0) - SL.apad;
     const float2* G = reinterpret_cast<const float2*>(base + SL.goff) + SL.gpad + (2 * tq - g);
     const uint32_t* H = reinterpret_cast<const uint32_t*>(base + SL.hoff + pb * SL.hlen) + (SL.hpad >> 1) + 8 * tb + tq;
     float* xs = reinterpret_cast<float*>(base + SL.roff) + px * SL.xp + g;
-    // warp w takes groups m and m + W together: a diagonal's table fragment is loaded
-    // once for both (their diagonal ranges are shifted by 4W); a group without a partner
-    // runs alone with two chains (even and odd diagonals)
-    for (int m = warp; m < M; m += 2 * W) {
-        const int mb = m + W;
-        const int dloA = -min(4 * m + 3, T - 1), dhi = S - 1 - 4 * m;  // group m: d = dloA .. dhi
-        if (mb < M) {
-            const int dlo = -min(4 * mb + 3, T - 1), dhiB = dhi - 4 * W;  // group mb: d = dlo .. dhiB
-            const float2* gy = G + 16 * dlo;
-            const uint32_t* ab = H + 8 * (4 * m + dlo);  // group m's operand; mb's is 32 W words further
-            float dA[4] = {0.f, 0.f, 0.f, 0.f}, dB[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t am = half2_bits(gy[-8]);
-            for (int d = dlo; d <= dhi; ++d) {
-                const uint32_t a0 = half2_bits(gy[0]), a2 = half2_bits(gy[8]);
-                if (d >= dloA) mma_16816(dA, a0, am, a2, a0, ab[0], ab[4]);
-                if (d <= dhiB) mma_16816(dB, a0, am, a2, a0, ab[32 * W], ab[32 * W + 4]);
-                am = a2;
-                gy += 16;
-                ab += 8;
-            }
-            const int tA = tx + 4 * m, tB = tx + 4 * mb;
-            if (tA < T) {
-                xs[16 * tA] = dA[0];
-                xs[16 * tA + 8] = dA[2];
-            }
-            if (tA + 1 < T) {
-                xs[16 * tA + 16] = dA[1];
-                xs[16 * tA + 24] = dA[3];
-            }
-            if (tB < T) {
-                xs[16 * tB] = dB[0];
-                xs[16 * tB + 8] = dB[2];
-            }
-            if (tB + 1 < T) {
-                xs[16 * tB + 16] = dB[1];
-                xs[16 * tB + 24] = dB[3];
-            }
-        } else {
-            const int nd = dhi - dloA + 1;
-            const float2* gy = G + 16 * dloA;
-            const uint32_t* ab = H + 8 * (4 * m + dloA);
-            float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t am = half2_bits(gy[-8]);
-            int k = 0;
-            for (; k + 1 < nd; k += 2) {
-                tc_diag(d0, gy, ab, am);
-                tc_diag(d1, gy + 16, ab + 8, am);
-                gy += 32;
-                ab += 16;
-            }
-            if (k < nd) tc_diag(d0, gy, ab, am);
-            const int t0 = tx + 4 * m;
-            if (t0 < T) {
-                xs[16 * t0] = d0[0] + d1[0];
-                xs[16 * t0 + 8] = d0[2] + d1[2];
-            }
-            if (t0 + 1 < T) {
-                xs[16 * t0 + 16] = d0[1] + d1[1];
-                xs[16 * t0 + 24] = d0[3] + d1[3];
-            }
+    const int dloA = -min(3, T - 1), dhi = S - 1;  // group 0: d = dloA .. dhi
+    if (M > 1) {
+        // both groups together: a diagonal's table fragment is loaded once for both
+        const int dlo = -(T - 1), dhiB = dhi - 4;  // group 1: d = dlo .. dhiB
+        const float2* gy = G + 16 * dlo;
+        const uint32_t* ab = H + 8 * dlo;  // group 0's operand; group 1's is 32 words further
+        float dA[4] = {0.f, 0.f, 0.f, 0.f}, dB[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t am = half2_bits(gy[-8]);
+        for (int d = dlo; d <= dhi; ++d) {
+            const uint32_t a0 = half2_bits(gy[0]), a2 = half2_bits(gy[8]);
+            if (d >= dloA) mma_16816(dA, a0, am, a2, a0, ab[0], ab[4]);
+            if (d <= dhiB) mma_16816(dB, a0, am, a2, a0, ab[32], ab[36]);
+            am = a2;
+            gy += 16;
+            ab += 8;
+        }
+        const int tB = tx + 4;
+        xs[16 * tx] = dA[0];
+        xs[16 * tx + 8] = dA[2];
+        xs[16 * tx + 16] = dA[1];
+        xs[16 * tx + 24] = dA[3];
+        if (tB < T) {
+            xs[16 * tB] = dB[0];
+            xs[16 * tB + 8] = dB[2];
+        }
+        if (tB + 1 < T) {
+            xs[16 * tB + 16] = dB[1];
+            xs[16 * tB + 24] = dB[3];
+        }
+    } else {
+        const int nd = dhi - dloA + 1;
+        const float2* gy = G + 16 * dloA;
+        const uint32_t* ab = H + 8 * dloA;
+        float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t am = half2_bits(gy[-8]);
+        int k = 0;
+        for (; k + 1 < nd; k += 2) {
+            tc_diag(d0, gy, ab, am);
+            tc_diag(d1, gy + 16, ab + 8, am);
+            gy += 32;
+            ab += 16;
+        }
+        if (k < nd) tc_diag(d0, gy, ab, am);
+        if (tx < T) {
+            xs[16 * tx] = d0[0] + d1[0];
+            xs[16 * tx + 8] = d0[2] + d1[2];
+        }
+        if (tx + 1 < T) {
+            xs[16 * tx + 16] = d0[1] + d1[1];
+            xs[16 * tx + 24] = d0[3] + d1[3];
         }
     }
     t.sync();
@@ -598,13 +595,138 @@ __device__ __forceinline__ void toeplitz_tc1(const View& V, const WarpSmem& SL, 
     for (int r = 0; r < R; ++r) X[r] = xr[r];
 }
 
+// The product of a walker that a CTA of W warps owns (n > 256, M = ceil(T/4) >= 3 column
+// groups).  A warp's operands are what bounds it, so it takes GC = 2 to 4 column groups at
+// once, and the diagonals in chunks of four: group m + 1 needs at diagonal d the row
+// blocks that group m needs at d + 4, so a chunk's row fragments, loaded once by ldmatrix
+// (two MMAs' operands each), pass through a ring to the next group a chunk later, and the
+// table fragments of a diagonal serve all GC groups: 10 loads for 16 MMAs (two row words
+// and, for every second MMA, two table pairs to convert before, with tests of the diagonal
+// around each).  608 walkers x 512 steps at L = 4095: 11.2 ms from 17.2; the tensor pipe is
+// now busy 45% of the time, the rest is the step around it.  Chunk k of a set of groups that
+// starts at m0 has d = 4k .. 4k+3 and the row blocks 4 (k + m0 + j) + 0..6 for group j;
+// k runs from -(m0 + GC), where the last group meets its first row block, to C - m0, C
+// the chunk of the last row block; what lies outside the class meets the rows' zeros.
+template <int GC>
+__device__ __forceinline__ void tc_chunks(float (&acc)[GC][4], const float2* gy, uint32_t ha, int nk)
+{
+    uint32_t F[GC][8];
+    const auto load = [&](uint32_t (&f)[8], uint32_t a) {
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3])
+                     : "r"(a));
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(f[4]), "=r"(f[5]), "=r"(f[6]), "=r"(f[7])
+                     : "r"(a + 64u));
+    };
+#pragma unroll
+    for (int j = 0; j < GC - 1; ++j) {
+        load(F[j], ha);
+        ha += 128u;
+    }
+    uint32_t am = half2_bits(gy[-8]);
+    for (;;) {
+#pragma unroll
+        for (int s = 0; s < GC; ++s) {
+            load(F[(s + GC - 1) % GC], ha);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t a0 = half2_bits(gy[16 * i]), a2 = half2_bits(gy[16 * i + 8]);
+#pragma unroll
+                for (int j = 0; j < GC; ++j)
+                    mma_16816(acc[j], a0, am, a2, a0, F[(s + j) % GC][2 * i], F[(s + j) % GC][2 * i + 1]);
+                am = a2;
+            }
+            gy += 64;
+            ha += 128u;
+            if (--nk == 0) return;
+        }
+    }
+}
+
+// One set's chunks k0 .. k0 + nk - 1, added to the integer sums xs (whole numbers, so the
+// order of the warps' additions does not change them).
+template <int GC>
+__device__ __forceinline__ void tc_set(const float2* G, uint32_t H, int* xs, int m0, int k0, int nk, int T, int tx)
+{
+    float acc[GC][4];
+#pragma unroll
+    for (int j = 0; j < GC; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+    tc_chunks<GC>(acc, G + 64 * k0, H + 128u * (uint32_t)(k0 + m0), nk);
+#pragma unroll
+    for (int j = 0; j < GC; ++j) {
+        const int t0 = tx + 4 * (m0 + j);
+        if (t0 < T) {
+            atomicAdd(xs + 16 * t0, __float2int_rn(acc[j][0]));
+            atomicAdd(xs + 16 * t0 + 8, __float2int_rn(acc[j][2]));
+        }
+        if (t0 + 1 < T) {
+            atomicAdd(xs + 16 * t0 + 16, __float2int_rn(acc[j][1]));
+            atomicAdd(xs + 16 * t0 + 24, __float2int_rn(acc[j][3]));
+        }
+    }
+}
+
+// The sets (Q = ceil(M/4), of ceil or floor M/Q groups) and their chunks are one line of
+// work, cut into W equal pieces.  The sums start at zero (long_clear) and are zeroed again
+// as they are read.
+template <class LB, int R>
+__device__ __forceinline__ void toeplitz_long(const View& V, const WarpSmem& SL, int n, const Outs<LB, R>& o,
+                                              const LB& t, float (&X)[R])
+{
+    constexpr int W = LB::kSize / 32;
+    const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    const int l = threadIdx.x & 31, g = l >> 2, tq = l & 3, px = tq >> 1, tx = 2 * (tq & 1);
+    const int S = (n + 15) >> 4, T = (((n + 1) >> 1) + 15) >> 4, M = (T + 3) >> 2;
+    const int C = (S - 1) >> 2, Q = (M + 3) >> 2, few = M / Q, more = M - few * Q;
+    int* const base = reinterpret_cast<int*>(V.A0) - SL.apad;
+    const float2* G = V.G + (2 * tq - g);
+    // ldmatrix row of this lane: operand column l & 7 (class, block), half block (l >> 3) & 1,
+    // the chunk's even or odd diagonal l >> 4
+    const uint32_t H =
+        (uint32_t)__cvta_generic_to_shared(reinterpret_cast<__half*>(base + SL.hoff + ((l >> 2) & 1) * SL.hlen) +
+                                           SL.hpad + 16 * ((l & 3) + (l >> 4)) + 8 * ((l >> 3) & 1));
+    int* const xi = base + SL.roff;
+    int* const xs = xi + px * SL.xp + g;
+    const int total = Q * (C + 1) + M;  // chunks of all sets: C + 1 + their groups
+    int at = warp * total / W, left = (warp + 1) * total / W - at;
+    for (int q = 0, m0 = 0; q < Q && left > 0; ++q) {
+        const int gc = few + (q < more ? 1 : 0), nk = C + 1 + gc;
+        if (at < nk) {
+            const int k0 = at - (m0 + gc), take = min(nk - at, left);
+            if (gc == 4) tc_set<4>(G, H, xs, m0, k0, take, T, tx);
+            else if (gc == 3) tc_set<3>(G, H, xs, m0, k0, take, T, tx);
+            else tc_set<2>(G, H, xs, m0, k0, take, T, tx);
+            left -= take;
+            at = nk;
+        }
+        at -= nk;
+        m0 += gc;
+    }
+    t.sync();
+    int* xr = xi + o.p * SL.xp + o.v0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        X[r] = (float)xr[r];
+        xr[r] = 0;
+    }
+}
+
 // The Toeplitz product of a lane group that owns one walker: on the tensor cores when
-// the layout holds the FP16 rows and the results' scratch, else on the FP32 pipes.
+// the layout holds the FP16 rows and the results' scratch (and the table's entries are
+// FP16 numbers), else on the FP32 pipes.
 template <class LG, int R>
 __device__ __forceinline__ void toeplitz_one(const View& V, const WarpSmem& SL, int n, const Outs<LG, R>& o,
                                              const LG& t, float (&X)[R])
 {
-    if constexpr (LG::kSize >= 32) {
+    if constexpr (LG::kSize > 32) {
+        if (SL.xp != 0 && *V.wide == 0) {
+            toeplitz_long(V, SL, n, o, t, X);
+            return;
+        }
+    } else if constexpr (LG::kSize == 32) {
         if (SL.xp != 0) {
             toeplitz_tc1(V, SL, n, o, t, X);
             return;
@@ -978,7 +1100,11 @@ __device__ __forceinline__ void flip_rows_table(const View& V, int n, const Outs
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         const int m = lane + 1 + TL::kSize * k;
-        if (m < n) set_E(V, m, V.G[m].x + dd[k]);
+        if (m < n) {
+            const float e = V.G[m].x + dd[k];
+            set_E(V, m, e);
+            if constexpr (TL::kSize > 32) note_wide(V, e);
+        }
     }
     if (lane == 0) {
         set_row(V, pb, vb, -as);

@@ -160,6 +160,7 @@ struct KParams {
 //       4 vectors x bvec words (kBitVec in the warp layouts), zero beyond the class
 //       length
 constexpr int kTcPad = 48;  // FP16 row entries the tensor-core product reads below u = 0
+constexpr int kTcPadLong = 256;  // ... the long product (16 row blocks) reads below u = 0; above, up to 18 blocks past S
 constexpr int kBitVec = 9;  // 256 bits per class plus one zero word read by the shifts
 struct WarpSmem {
     int apad;   // zero words below index 0 of each row (multiple of 4)
@@ -179,7 +180,8 @@ struct WarpSmem {
                 // u at half index hpad + u, zero around the class
     int hlen;   // words per FP16 row (4 mod 8: the two classes' operand loads use
                 // different banks; 0: no FP16 rows)
-    int hpad;   // FP16 entries below u = 0 (even)
+    int hpad;   // FP16 entries below u = 0 (even; a multiple of 8 in the long layout)
+    int foff = 0;  // long tensor-core layout: word of the flag that an |E| is above 2^11
     int words;  // total words per walker (multiple of 4: walkers stay 16-byte aligned)
 };
 // Outputs per lane (the lane block R) for n free variables and `tile` lanes per walker
@@ -517,11 +519,14 @@ __host__ __device__ inline WarpSmem long_layout(int n_max, int tile, bool tc)
     if (n_max + 2 * R > lo) lo = n_max + 2 * R;
     if (n_max + 2 * R > gtop) gtop = n_max + 2 * R;
     const int S = (n_max + 15) >> 4, T = (((n_max + 1) >> 1) + 15) >> 4;
-    if (tc && gtop < 16 * S) gtop = 16 * S;  // the tensor-core product's table reads
+    // the tensor-core product's table reads: block diagonals from -4 M (M column groups of
+    // four output blocks) up to the last of the chunk of four that holds S - 1
+    const int M = (T + 3) >> 2;
+    if (tc && gtop < 16 * S + 48) gtop = 16 * S + 48;
     w.apad = (lo + 3) & ~3;
     w.alen = w.apad + ((hi + 7) & ~7);
     w.gpad = (tile / 2) * R > span ? (tile / 2) * R : span;
-    if (tc && w.gpad < 16 * T - 1) w.gpad = 16 * T - 1;
+    if (tc && w.gpad < 64 * M + 16) w.gpad = 64 * M + 16;
     w.glen = w.gpad + gtop;
     w.goff = 2 * w.alen;
     w.boff = w.goff + 2 * w.glen;
@@ -534,10 +539,11 @@ __host__ __device__ inline WarpSmem long_layout(int n_max, int tile, bool tc)
     w.hpad = 0;
     w.xoff = (w.boff + 4 * w.bvec + 3) & ~3;
     if (tc) {
-        // FP16 rows (cleared with the rows, below xoff): u from -kTcPad up to 16 S + kTcPad
+        // FP16 rows (cleared with the rows, below xoff): u from -kTcPadLong up to
+        // 16 (S + 18), 16-byte aligned for the operand loads
         w.hoff = w.xoff;
-        w.hpad = kTcPad;
-        w.hlen = ((8 * S + kTcPad + 3) & ~7) + 4;
+        w.hpad = kTcPadLong;
+        w.hlen = ((8 * (S + 18) + kTcPadLong / 2 + 3) & ~7) + 4;
         w.xoff = w.hoff + 2 * w.hlen;
     }
     // scratch, bits, then the best-first search's queue keys (LABS_QUEUE_SIZE 64-bit
@@ -550,7 +556,8 @@ __host__ __device__ inline WarpSmem long_layout(int n_max, int tile, bool tc)
         const int need = 16 * T > (tile / 2) * R ? 16 * T : (tile / 2) * R;
         w.xp = ((need + 15) & ~31) + 16;
         w.roff = (w.words + 3) & ~3;
-        w.words = w.roff + 2 * w.xp;
+        w.foff = w.roff + 2 * w.xp;
+        w.words = w.foff + 4;
     }
     return w;
 }
