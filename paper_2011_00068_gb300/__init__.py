@@ -273,14 +273,14 @@ def close_rows():
 atexit.register(close_rows)
 
 
-def _rows_ctx(L: int, device: torch.device, stream):
-    key = (L, device.index, stream.cuda_stream)
+def _rows_ctx(L: int, device_index: int, stream: int):
+    key = (L, device_index, stream)
     c = _row_ctx.get(key)
     if c is None:
         lib = library()
         ctx = ctypes.c_void_p()
-        with torch.cuda.device(device):
-            rc = lib.labs_init(ctypes.byref(ctx), int(L), 0, 0, None, _stream_handle(stream))
+        with torch.cuda.device(device_index):
+            rc = lib.labs_init(ctypes.byref(ctx), int(L), 0, 0, None, ctypes.c_void_p(stream))
         if rc != 0:
             msg = _err(lib, ctx)
             lib.labs_destroy(ctx)
@@ -295,31 +295,39 @@ def _rows(seqs: torch.Tensor):
     return seqs.contiguous()
 
 
+def _rows_call(name: str, seqs: torch.Tensor, stream, wide: bool) -> torch.Tensor:
+    """One row kernel on `seqs`: an int32 per row, or (wide) per free variable of a row.
+
+    A call on a few rows is all host work, so it takes the short way where there is one:
+    the current stream's handle without a Stream object, plain integers for the pointers
+    (the prototypes convert them), and a device guard only when another device is current."""
+    seqs = _rows(seqs)
+    dev = seqs.get_device()
+    handle = stream.cuda_stream if stream else torch._C._cuda_getCurrentRawStream(dev)
+    batch, L = seqs.shape
+    out = torch.empty((batch, (L + 1) // 2) if wide else batch, dtype=torch.int32, device=seqs.device)
+    lib = library()
+    ctx = _rows_ctx(L, dev, handle)
+    call = getattr(lib, name)
+    if torch.cuda.current_device() == dev:
+        rc = call(ctx, seqs.data_ptr(), batch, out.data_ptr())
+    else:
+        with torch.cuda.device(dev):
+            rc = call(ctx, seqs.data_ptr(), batch, out.data_ptr())
+    if rc != _native.LABS_OK:
+        _check(rc, lib, ctx)
+    return out
+
+
 def isl(seqs: torch.Tensor, stream=None) -> torch.Tensor:
     """Eq. 2 for every row of an int8 [batch, L] +-1 tensor; -1 for rows that are not +-1."""
-    seqs = _rows(seqs)
-    stream = stream or torch.cuda.current_stream(seqs.device)
-    L = seqs.shape[1]
-    out = torch.empty(seqs.shape[0], dtype=torch.int32, device=seqs.device)
-    lib = library()
-    ctx = _rows_ctx(L, seqs.device, stream)
-    with torch.cuda.device(seqs.device):
-        _check(lib.labs_isl(ctx, _ptr(seqs), seqs.shape[0], _ptr(out)), lib, ctx)
-    return out
+    return _rows_call("labs_isl", seqs, stream, False)
 
 
 def neighbor_delta(seqs: torch.Tensor, stream=None) -> torch.Tensor:
     """dISL of flipping each free variable (and its mirror) of every skew-symmetric row:
     int32 [batch, n]; rows that are not +-1 / skew-symmetric are filled with INT32_MIN."""
-    seqs = _rows(seqs)
-    stream = stream or torch.cuda.current_stream(seqs.device)
-    L = seqs.shape[1]
-    out = torch.empty((seqs.shape[0], (L + 1) // 2), dtype=torch.int32, device=seqs.device)
-    lib = library()
-    ctx = _rows_ctx(L, seqs.device, stream)
-    with torch.cuda.device(seqs.device):
-        _check(lib.labs_neighbor_delta(ctx, _ptr(seqs), seqs.shape[0], _ptr(out)), lib, ctx)
-    return out
+    return _rows_call("labs_neighbor_delta", seqs, stream, True)
 
 
 def enumerate_skew(L: int, device=None, stream=None) -> tuple[int, int, int]:
