@@ -232,17 +232,177 @@ __device__ Probe long_probe(const LongWalk& lw, uint64_t f, uint32_t gen, const 
     return pr;
 }
 
+// The walk's neighbourhood in the form of labs_step.cuh: with m = c - i and sg = (-1)^m,
+//   dISL_i = -8 s_i (X_i + 4 sg s_{3i-L+1}) + 8 Z_m + 16 (N_p - 2),
+//   Z_m    = sg (3 C^(p)_m + C^(1-p)_m) = 4 P_i + 2 + sg E_m
+// (the centre: -4 s_c, Z_0 = 6 - c + (c mod 2)).  Each thread keeps the Z of its R outputs in
+// registers.  A move changes C^(pb) of the flipped class pb alone, by the dC_m that the table
+// changes by, so Z by sg dC_m (own class 3 times): two row entries per output, in every warp.
+// P, which it replaces, changes only in the flipped class, i.e. in half of the warps while
+// the others wait, and needs the mirror and C_{q-i} in the assembly.  With the two-candidate
+// rounds of long_lowest: 608 walkers x 512 steps at L = 4095 10.4 ms from 11.2.
+template <class LB, int R>
+__device__ __forceinline__ void long_z(const View& V, int n, const Outs<LB, R>& o, float (&Z)[R])
+{
+    const int c = n - 1;
+    const float sg = ((c - o.p) & 1) ? -1.f : 1.f;
+    p_direct(V, n, o, Z);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int m = c - 2 * (o.v0 + r) - o.p;
+        // outputs that do not exist (m < 0) hold anything finite
+        Z[r] = m == 0 ? (float)(6 - c + (c & 1)) : fmaf(sg, V.G[max(m, 0)].x, fmaf(4.f, Z[r], 2.f));
+    }
+}
+
+// Keys (dISL + 2^24) << 4 | r of the lane's outputs (|dISL| < 2^24 within the exact range, r <
+// R <= 11), kNoKey where an output does not exist.
+constexpr uint32_t kNoKey = ~0u, kNoD = kNoKey >> 4;
+
+template <class LB, int R>
+__device__ __forceinline__ void long_keys(const View& V, int n, const Outs<LB, R>& o, const float (&X)[R],
+                                          const float (&Z)[R], uint32_t (&key)[R])
+{
+    const int c = n - 1, rc = o.p == (c & 1) ? (c >> 1) - o.v0 : -1;
+    const int nv = ((o.p ? n >> 1 : (n + 1) >> 1)) - o.v0;  // outputs r < nv exist
+    const float sig4 = ((c - o.p) & 1) ? -4.f : 4.f, base = (float)(16 * (n - o.p - 3));
+    const float* A = (o.p ? V.A1 : V.A0) + o.v0;
+    const float* A3 = (o.p ? V.A1 : V.A0) + (nv > 0 ? 3 * o.v0 + o.p - n + 1 : 0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float y = A[r] * fmaf(sig4, A3[r < nv ? 3 * r : 0], X[r]);
+        const int d = __float2int_rn(fmaf(r == rc ? -4.f : -8.f, y, fmaf(8.f, Z[r], base)));
+        key[r] = r < nv ? ((uint32_t)(d + (1 << 24)) << 4) | (uint32_t)r : kNoKey;
+    }
+}
+
+// How far down the products read the table's mirror half.
+template <class LB, int R>
+__device__ __forceinline__ int long_table_low(int n)
+{
+    const int M = ((((n + 1) >> 1) + 15) / 16 + 3) >> 2;  // column groups of the product
+    return max(64 * M + 16, (LB::kSize / 2) * R + 1);     // (the FP32 product: its window)
+}
+
+// S <- S_f for free variable bi: the table, Z and the two row entries, all from the values
+// before the flip (flip_rows_table with Z in place of P).  The table's mirror half is kept as
+// far down as the products read.  Ends without a barrier.
+template <class LB, int R>
+__device__ __forceinline__ void long_flip(const View& V, int n, const Outs<LB, R>& o, float (&Z)[R], int bi,
+                                          const LB& t)
+{
+    const int lane = t.lane, c = n - 1;
+    const int pb = bi & 1, vb = bi >> 1;
+    float* Ab = pb ? V.A1 : V.A0;
+    const float as = Ab[vb];
+    const bool centre = bi == c;
+    const int vq = n - 1 - vb - pb, mq = centre ? INT_MAX : vq - vb;  // lag of the mirror: no term above
+    const float coef = (centre ? -2.f : -4.f) * as;
+    float dd[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {  // lags m = lane + 1 + LB::kSize k < n
+        const int m = min(lane + 1 + LB::kSize * k, n);  // (zeros at lag n)
+        const float up = Ab[vb + m];
+        dd[k] = coef * ((m == mq ? 0.f : up) + Ab[vb - m]);
+    }
+    {
+        const float k = (((c - o.p) & 1) ? -coef : coef) * (o.p == pb ? 3.f : 1.f);
+        const int m0 = c - 2 * o.v0 - o.p;
+        const float *U = Ab + vb + m0, *D = Ab + vb - m0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int m = m0 - 2 * r;
+            const float s = (m == mq ? 0.f : U[-2 * r]) + D[2 * r];
+            Z[r] = fmaf(m == 0 ? 0.f : k, s, Z[r]);
+        }
+    }
+    t.sync();
+    const int low = long_table_low<LB, R>(n);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const int m = lane + 1 + LB::kSize * k;
+        if (m < n) {
+            const float e = V.G[m].x + dd[k];
+            V.G[m].x = e;
+            V.G[m - 1].y = e;
+            if (m <= low) {
+                V.G[-m].x = e;
+                V.G[-m - 1].y = e;
+            }
+            note_wide(V, e);
+        }
+    }
+    if (lane == 0) {
+        set_row(V, pb, vb, -as);
+        if (!centre) set_row(V, pb, vq, -Ab[vq]);
+    }
+}
+
+// The two lowest (dISL, i) of the CTA's outputs, known to every thread.
+struct Lowest {
+    uint32_t d1, i1, d2, i2;  // d: dISL + 2^24, or kNoD
+};
+
+// Lowest (d, i) of the warp's lanes; true on the lane that holds it.
+__device__ __forceinline__ bool warp_lowest(uint32_t d, uint32_t i, uint32_t& dm, uint32_t& im)
+{
+    dm = __reduce_min_sync(kFull, d);
+    const uint32_t c = d == dm ? i : ~0u;
+    im = __reduce_min_sync(kFull, c);
+    return c == im;
+}
+
+// Each warp's two lowest go to `buf` (2 (d, i) pairs a warp), then every warp merges them:
+// one barrier.  A CTA alternates between two buffers, so that a warp may write the next
+// round's while another still reads this round's.
+template <class LB, int R>
+__device__ __forceinline__ Lowest long_lowest(const LongWalk& lw, uint64_t fp, const uint32_t (&key)[R],
+                                              const Outs<LB, R>& o, uint2* buf, const LB& t)
+{
+    constexpr int W = LB::kWarps;
+    const int l = t.lane & 31;
+    uint32_t k1 = kNoKey, k2 = kNoKey;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        k2 = min(k2, max(k1, key[r]));
+        k1 = min(k1, key[r]);
+    }
+    const uint32_t i0 = (uint32_t)(2 * o.v0 + o.p);
+    Lowest a;
+    const bool own = warp_lowest(k1 >> 4, i0 + 2u * (k1 & 15u), a.d1, a.i1);
+    const uint32_t k = own ? k2 : k1;
+    warp_lowest(k >> 4, i0 + 2u * (k & 15u), a.d2, a.i2);
+    if (l == 0) {
+        buf[2 * (t.lane >> 5)] = make_uint2(a.d1, a.i1);
+        buf[2 * (t.lane >> 5) + 1] = make_uint2(a.d2, a.i2);
+    }
+    // the lookups' misses start before the merge
+    if (l < 2 && (l ? a.d2 : a.d1) != kNoD)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(lw.e.T + ((fp ^ __ldg(lw.e.zk + (l ? a.i2 : a.i1))) & lw.e.tmask)));
+    t.sync();
+    uint2 e = l < 2 * W ? buf[l] : make_uint2(kNoD, ~0u);
+    if (warp_lowest(e.x, e.y, a.d1, a.i1)) e = make_uint2(kNoD, ~0u);
+    warp_lowest(e.x, e.y, a.d2, a.i2);
+    return a;
+}
+
 // Steps of one long walker until `until` (or a stop request, or the exact-range check).
+// The lowest neighbour not in HT is sought two candidates at a time, by every warp for
+// itself (the same two 128-byte lines of HT, so the first warp's misses serve all): a
+// round costs one barrier, and the choice needs none to be known.  The move's insertion
+// comes after the barrier inside the flip, when no warp looks HT up any more.
 template <class LB, int R>
 __device__ void long_walk(const LongWalk& lw, Walker& w, int64_t until, const WarpSmem& SL, int* base,
                           const View& V, int trace_slot, int64_t trace_start, const LB& t)
 {
     const WalkEnv& env = lw.e;
     const KParams& p = *env.p;
-    const int lane = t.lane, n = env.n;
+    const int lane = t.lane, n = env.n, l = lane & 31, cap = p.probe_cap;
     const Outs<LB, R> o(t);
-    float P[R];
-    p_direct(V, n, o, P);
+    uint2* const bufs = reinterpret_cast<uint2*>(t.x);
+    int turn = 0;
+    float Z[R];
+    long_z(V, n, o, Z);
     StopCheck stop;
     stop.start(p, lane == 0);
     while (w.steps < until) {
@@ -257,41 +417,74 @@ __device__ void long_walk(const LongWalk& lw, Walker& w, int64_t until, const Wa
                 break;
             }
         }
-        int dl[R];
+        uint32_t key[R];
         {
             float X[R];
             toeplitz_one(V, SL, n, o, t, X);
-            assemble(V, n, o, X, P, dl);
+            long_keys(V, n, o, X, Z, key);
         }
         // lowest (dISL, i) whose result is not in HT
-        uint32_t excl = 0;
         int best_i = -1, best_d = 0;
         int64_t slot = -1;
         uint64_t fnew = 0;
         for (;;) {
-            int bd, bi;
-            tile_argmin(dl, excl, o, t, bd, bi);
-            if (bi < 0) break;
-            const uint64_t f = w.fp ^ __ldg(env.zk + bi);
-            const Probe pr = long_probe(lw, f, w.gen, t);
+            const Lowest c = long_lowest(lw, w.fp, key, o, bufs + 2 * LB::kWarps * turn, t);
+            turn ^= 1;
+            if (c.d1 == kNoD) break;
+            const bool two = c.d2 != kNoD;
+            const uint64_t f1 = w.fp ^ __ldg(env.zk + c.i1), f2 = w.fp ^ __ldg(env.zk + (two ? c.i2 : c.i1));
+            // the first 16 slots of both
+            const uint64_t f = l < 16 ? f1 : f2, tag = (f & ~kGenMask) | w.gen;
+            uint64_t e = 0;
+            if ((l & 15) < cap) e = env.T[(f + (uint64_t)(l & 15)) & env.tmask];
+            const bool match = (l & 15) < cap && e == tag;
+            const unsigned hit = __ballot_sync(kFull, match);
+            const unsigned end = __ballot_sync(kFull, match || ((l & 15) < cap && (e & kGenMask) != w.gen));
+            const auto verdict = [&](unsigned e16, unsigned h16, uint64_t fc) {
+                Probe pr{false, -1};
+                if (e16) {
+                    const int fl = __ffs(e16) - 1;
+                    pr.visited = (h16 >> fl) & 1u;
+                    pr.slot = (int64_t)((fc + (uint64_t)fl) & env.tmask);
+                } else if (cap > 16) {
+                    pr = probe_full(env, fc, w.gen, cap, Tile<32>(l));
+                }
+                return pr;
+            };
+            Probe pr = verdict(end & 0xFFFFu, hit & 0xFFFFu, f1);
             if (!pr.visited) {
-                best_i = bi;
-                best_d = bd;
+                best_i = (int)c.i1;
+                best_d = (int)c.d1 - (1 << 24);
                 slot = pr.slot;
-                fnew = f;
+                fnew = f1;
                 break;
             }
-            exclude<LB, R>(excl, bi, t);
+            if (!two) break;
+            pr = verdict(end >> 16, hit >> 16, f2);
+            if (!pr.visited) {
+                best_i = (int)c.i2;
+                best_d = (int)c.d2 - (1 << 24);
+                slot = pr.slot;
+                fnew = f2;
+                break;
+            }
+            // both visited: leave them out and take the next two
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const uint32_t i = (uint32_t)(2 * (o.v0 + r) + o.p);
+                if (i == c.i1 || i == c.i2) key[r] = kNoKey;
+            }
         }
         w.steps += 1;
         int code;
         if (best_i < 0) {
             w.blocked += 1;
+            t.sync();  // no warp looks HT up any more (a restart may zero it)
             long_restart(lw, w, SL, base, V, t);
-            p_direct(V, n, o, P);
+            long_z(V, n, o, Z);
             code = LABS_TRACE_BLOCKED;
         } else {
-            flip_rows_table(V, n, o, P, best_i, t);
+            long_flip(V, n, o, Z, best_i, t);
             const bool stored = slot >= 0;
             if (lane == 0 && stored) env.T[slot] = (fnew & ~kGenMask) | w.gen;
             if (lane == (best_i >> 5)) w.word ^= 1u << (best_i & 31);
@@ -309,7 +502,7 @@ __device__ void long_walk(const LongWalk& lw, Walker& w, int64_t until, const Wa
             code = best_i;
             if (w.stag >= env.patience || !stored) {
                 long_restart(lw, w, SL, base, V, t);
-                p_direct(V, n, o, P);
+                long_z(V, n, o, Z);
                 code |= LABS_TRACE_RESTART;
             }
         }
