@@ -230,57 +230,6 @@ __global__ void __launch_bounds__(256) isl_long_kernel(const int8_t* __restrict_
 
 // --------------------------------------------------- learned proposal support
 
-// Network inputs of states given by their free-variable bits (8 words each, `stride`
-// words apart): x[b][0][i] = s_i, x[b][1][i] = C_{2(i+1)}/sqrt(L) (0 for i = n-1),
-// x[b][2][i] = dISL_i/(8L).  One warp per state.
-template <int R>
-__device__ void features_row(const View& V, int n, int L, const Tile<32>& t, float* xb)
-{
-    const Outs<Tile<32>, R> o(t);
-    int dl[R];
-    {
-        float X[R], P[R];
-        toeplitz(V, n, o, X);
-        p_direct(V, n, o, P);
-        assemble(V, n, o, X, P, dl);
-    }
-    const float inv8L = (float)(8 * L);
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (dl[r] != INT_MAX) xb[2 * n + 2 * (o.v0 + r) + o.p] = (float)dl[r] / inv8L;
-}
-
-__global__ void __launch_bounds__(256) features_kernel(const uint32_t* __restrict__ bits, int64_t stride,
-                                                       int64_t count, int L, float* __restrict__ x)
-{
-    extern __shared__ __align__(16) int smem[];
-    const int n = (L + 1) / 2;
-    const WarpSmem SL = warp_smem(n, 32);
-    const Tile<32> t(threadIdx.x & 31);
-    const int lane = t.lane, warp = threadIdx.x >> 5;
-    int* base = smem + warp * SL.words;
-    const View V = make_view(base, SL);
-    const float sq = sqrtf((float)L);
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; b < count; b += nwarps) {
-        const uint32_t word = lane < kBitWords ? bits[b * stride + lane] : 0u;
-        load_rows(base, SL, V, word, L, n, t);
-        float* xb = x + b * 3 * n;
-        for (int i = lane; i < n; i += kWarp) {
-            xb[i] = (i & 1) ? V.A1[i >> 1] : V.A0[i >> 1];
-            xb[n + i] = i < n - 1 ? V.G[i + 1].x / sq : 0.f;
-        }
-        switch (block_R(n, 32)) {
-            case 1: features_row<1>(V, n, L, t, xb); break;
-            case 3: features_row<3>(V, n, L, t, xb); break;
-            case 5: features_row<5>(V, n, L, t, xb); break;
-            case 7: features_row<7>(V, n, L, t, xb); break;
-            default: features_row<9>(V, n, L, t, xb); break;
-        }
-        t.sync();
-    }
-}
-
 // Restart candidates of walkers [first, first+count) of one length: candidate 0 is the
 // walker's own next random start (what the plain walk would use); candidates c >= 1 are
 // further random starts, Philox with key = seed and counter = (walker, next restart
@@ -589,16 +538,6 @@ int launch_trace_arm(const KParams& p, const int64_t* dev_ids, int32_t k, int32_
 {
     trace_clear_kernel<<<256, 256, 0, (cudaStream_t)stream>>>(p);
     trace_set_kernel<<<(k + 255) / 256 + 1, 256, 0, (cudaStream_t)stream>>>(p, dev_ids, k, code, isl, capacity);
-    return status_of(cudaGetLastError());
-}
-
-int launch_features(const uint32_t* bits, int64_t stride, int64_t count, int32_t L, float* x, void* stream)
-{
-    if (count == 0) return LABS_OK;
-    const int warps = 8;
-    const size_t smem = (size_t)warps * warp_smem((L + 1) / 2, 32).words * sizeof(int);
-    cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    features_kernel<<<row_grid(count, warps), warps * kWarp, smem, (cudaStream_t)stream>>>(bits, stride, count, L, x);
     return status_of(cudaGetLastError());
 }
 

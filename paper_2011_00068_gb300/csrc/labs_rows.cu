@@ -1,5 +1,5 @@
 // labs_rows.cu -- the neighbourhood of Algorithm 1 for a batch of skew-symmetric rows
-// (labs_neighbor_delta, L <= LABS_MAX_L) on the step of labs_step.cuh: two rows per warp up
+// (labs_neighbor_delta, L <= LABS_MAX_L) and for a batch of states (labs_features) on the step of labs_step.cuh: two rows per warp up
 // to n = 160 free variables, one above.
 //
 // A row is seen once, so everything is built from the row itself:
@@ -111,27 +111,164 @@ __device__ __forceinline__ uint32_t mirror_diff(const uint32_t (&x)[NW], int np,
     return diff;
 }
 
-// LG: Pair (two rows per warp) or Tile<32>; R = step_R(n, lanes per row) outputs per lane;
-// NW = ceil(n/32) words per class; STAGED: rows come through the staging buffers after the
-// rows' shared memory.
+// One lane of a row evaluation.  LG: Pair (two rows per warp) or Tile<32>; R = step_R(n, lanes
+// per row) outputs per lane; NW = ceil(n/32) words per class.
+template <class LG, int R, int NW>
+struct RowLane {
+    static constexpr int NL = LG::kSize, W = 32 / NL;
+    using LAY = StepLayout<NL, R, false>;
+    static constexpr int IT = (4 * NW + NL - 1) / NL;  // pieces of 16 positions per lane
+    StepLane<LAY, LG, R> a;
+    int lane, n, c;
+    // this lane's constants: its lags m = lane (mod NL) all have the parity of the lane
+    int h0, h1;      // half the pairs at lag `lane`
+    uint32_t kc;     // FP16 bits of 1536 + C^(p) at lag `lane` before its mismatches, class 1 high
+    uint32_t zs0, zs1;  // (E, Z) = C^(0) (1, z0) + C^(1) (1, z1)
+    uint32_t gp, gm, zp, rowa, bita, sga, res;
+    int v0;
+    int rc;          // this lane's output that is the centre
+
+    __device__ __forceinline__ RowLane(int wb0, int n_, const LG& t, const Outs<LG, R>& o)
+        : a(wb0, n_, t, o), lane(t.lane), n(n_), c(n_ - 1), v0(o.v0)
+    {
+        constexpr StepSmem SL = LAY::SL;
+        const int wb = a.wb, odd0 = (n - lane) & 1, odd1 = odd0 ^ 1, sgn0 = (c & 1) ? -1 : 1;
+        h0 = (n - lane) >> 1;
+        h1 = (n - 1 - lane) >> 1;
+        kc = 0x66006600u + (uint32_t)(2 * h0 + odd0 * sgn0) + ((uint32_t)(2 * h1 - odd1 * sgn0) << 16);
+        // Z takes 3 times the lag's own class p = (c - m) mod 2, with the sign (-1)^m
+        const uint32_t zs = (lane & 1) ? 0x80000000u : 0u, own = ((c - lane) & 1) ? 0x3C000000u : 0x42000000u;
+        zs0 = (own | 0x3C00u) ^ zs;
+        zs1 = ((own ^ 0x7E000000u) | 0x3C00u) ^ zs;
+        gp = sbyte(wb + SL.g + lane);
+        gm = sbyte(wb + SL.g - lane);
+        zp = sbyte(wb + SL.z) + 2 * lane;
+        rowa = sbyte(wb + SL.h0) + 16 * lane;
+        bita = sbyte(wb + SL.b) + lane;
+        sga = sbyte(wb + SL.b + o.p * SL.bvec + (o.v0 >> 5));
+        rc = o.p == (c & 1) ? (c >> 1) - o.v0 : -1;
+        res = sbyte(wb + SL.r8) + 4 * (2 * o.v0 + o.p);
+    }
+
+    // Every row writes the same entries: the padding is cleared once.
+    __device__ __forceinline__ void clear() const
+    {
+        constexpr StepSmem SL = LAY::SL;
+        for (int i = lane; i < SL.words / 4; i += NL) sts_v4(sbyte(a.wb) + 16 * i, 0u, 0u, 0u, 0u);
+    }
+
+    // Class words, and the signs of the lane's outputs (bit r; above the class anything).
+    __device__ __forceinline__ uint32_t classes(uint32_t (&x0)[NW], uint32_t (&x1)[NW]) const
+    {
+        constexpr StepSmem SL = LAY::SL;
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+            x0[k] = lds_u32(sbyte(a.wb + SL.b) + 4 * k);
+            x1[k] = lds_u32(sbyte(a.wb + SL.b + SL.bvec) + 4 * k);
+        }
+        return __funnelshift_r(lds_u32(sga), lds_u32(sga + 4), v0 & 31);
+    }
+
+    // Table and Z: lags m = lane + NL j + 32 q.
+    __device__ __forceinline__ void table(const uint32_t (&x0)[NW], const uint32_t (&x1)[NW]) const
+    {
+        constexpr StepSmem SL = LAY::SL;
+        const uint32_t ez0 = half_bits(6 - c + (c & 1)) << 16;  // lag 0: E = 0, Z of the centre
+#pragma unroll
+        for (int j = 0; j < 32 / NL; ++j) {
+            uint32_t s0[NW], s1[NW];
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                s0[k] = __funnelshift_r(x0[k], k + 1 < NW ? x0[k + 1] : 0u, lane + NL * j);
+                s1[k] = __funnelshift_r(x1[k], k + 1 < NW ? x1[k + 1] : 0u, lane + NL * j);
+            }
+#pragma unroll
+            for (int q = 0; q < NW; ++q) {
+                const int m0 = 32 * q + NL * j;  // m = m0 + lane
+                int t0 = 0, t1 = 0;
+#pragma unroll
+                for (int k = 0; 2 * k < NW - q; ++k) {
+                    // pairs 32 k .. of the first h: n > 32 (NW - 1) and m < 32 (q + 1)
+                    uint32_t d0 = x0[k] ^ s0[k + q], d1 = x1[k] ^ s1[k + q];
+                    if (32 * (k + 1) > 16 * (NW - q - 2)) {
+                        const int b0 = h0 - m0 / 2 - 32 * k, b1 = h1 - m0 / 2 - 32 * k;
+                        d0 &= __funnelshift_lc(~0u, 0u, k ? max(b0, 0) : b0);
+                        d1 &= __funnelshift_lc(~0u, 0u, k ? max(b1, 0) : b1);
+                    }
+                    t0 += __popc(d0);
+                    t1 += __popc(d1);
+                }
+                const uint32_t cc = kc - (uint32_t)m0 * 0x00010001u - 4u * ((uint32_t)t0 + ((uint32_t)t1 << 16));
+                const __half2 ch = __hsub2(as_half2(cc), as_half2(0x66006600u));
+                uint32_t ez =
+                    as_u32(__hfma2(__high2half2(ch), as_half2(zs1), __hmul2(__low2half2(ch), as_half2(zs0))));
+                if (m0 == 0) ez = lane == 0 ? ez0 : ez;
+                if (q < NW - 1) {  // n > 32 (NW - 1): the lag exists
+                    sts_u16(gp + 4 * m0, ez);
+                    sts_u16(gp + 4 * m0 - 2, ez);
+                    sts_u16(zp + 2 * m0, ez >> 16);
+                    if (m0 + NL - 1 < SL.gneg) {
+                        sts_u16(gm - 4 * m0, ez);
+                        sts_u16(gm - 4 * m0 - 2, ez);
+                    } else if (m0 <= SL.gneg) {
+                        sts_u16_if(m0 + lane <= SL.gneg, gm - 4 * m0, ez);
+                        sts_u16_if(m0 + lane < SL.gneg, gm - 4 * m0 - 2, ez);
+                    }
+                } else {
+                    const bool in = lane < n - m0;
+                    sts_u16_if(in, gp + 4 * m0, ez);
+                    sts_u16_if(in, gp + 4 * m0 - 2, ez);
+                    sts_u16_if(in, zp + 2 * m0, ez >> 16);
+                    if (m0 <= SL.gneg) {
+                        sts_u16_if(in && m0 + lane <= SL.gneg, gm - 4 * m0, ez);
+                        sts_u16_if(in && m0 + lane < SL.gneg, gm - 4 * m0 - 2, ez);
+                    }
+                }
+            }
+        }
+    }
+
+    // The product and the outputs' dISL, int32 i of the row at result(i):
+    //   dISL = -8 s_i (X_i + 4 sg s_{3i-L+1}) + 8 Z_m + 16 (N_p - 2), the centre -4 s_c;
+    // the FP32 value dISL + 1.5 2^23 holds the integer in its low bits.
+    __device__ __forceinline__ void values(uint32_t sgn, int wl) const
+    {
+        __syncwarp();
+        step_toeplitz(a.prod, wl);  // ends with a warp barrier
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float x = lds_f32(a.xr + 4 * r), z = lds_f16(a.zr - 4 * r), s3 = lds_f16(a.sr + 6 * r);
+            const float y = __uint_as_float(__float_as_uint(fmaf(a.sig4, s3, x)) ^ ((sgn << (31 - r)) & 0x80000000u));
+            const float v = fmaf(r == rc ? -4.f : -8.f, y, fmaf(8.f, z, a.bias));
+            sts_u32(res + 8 * r, __float_as_uint(v) - __float_as_uint(kIntBias));
+        }
+        __syncwarp();
+    }
+
+    __device__ __forceinline__ uint32_t result(int i) const { return sbyte(a.wb + LAY::SL.r8) + 4 * i; }
+};
+
+template <class LG, int R>
+constexpr int row_ctas()
+{
+    return LG::kSize == 16 && R > 7 ? 2 : 3;  // of eight warps per SM
+}
+
+// STAGED: rows come through the staging buffers after the rows' shared memory.
 template <class LG, int R, int NW, bool STAGED>
-__global__ void __launch_bounds__(256, LG::kSize == 16 ? (R <= 7 ? 3 : 2) : 3)
+__global__ void __launch_bounds__(256, row_ctas<LG, R>())
     rows_kernel(const int8_t* __restrict__ seqs, int64_t batch, int L, int32_t* __restrict__ out, DevStatus* status)
 {
-    constexpr int NL = LG::kSize, W = 32 / NL;
-    using LAY = StepLayout<NL, R, false>;
-    constexpr StepSmem SL = LAY::SL;
-    constexpr int IT = (4 * NW + NL - 1) / NL;  // 16-byte pieces per lane
+    using RL = RowLane<LG, R, NW>;
+    constexpr int NL = RL::NL, W = RL::W, IT = RL::IT;
+    constexpr StepSmem SL = RL::LAY::SL;
     extern __shared__ __align__(16) int smem[];
     const int n = (L + 1) / 2, c = n - 1;
     const LG t(threadIdx.x & 31);
     const int lane = t.lane, wl = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wb0 = warp * W * SL.words;
     const Outs<LG, R> o(t);
-    const StepLane<LAY, LG, R> a(wb0, n, t, o);
-    const int wb = a.wb;
-    // every row writes the same entries: clear the padding once
-    for (int i = lane; i < SL.words / 4; i += NL) sts_v4(sbyte(wb) + 16 * i, 0u, 0u, 0u, 0u);
+    const RL rl(warp * W * SL.words, n, t, o);
+    rl.clear();
 
     const int SB = stage_bytes(L, W);
     const int8_t* stg = reinterpret_cast<const int8_t*>(smem + (blockDim.x >> 5) * W * SL.words) + warp * (2 * SB + 16);
@@ -148,21 +285,6 @@ __global__ void __launch_bounds__(256, LG::kSize == 16 ? (R <= 7 ? 3 : 2) : 3)
         __syncwarp();
         if (wl == 0 && first < batch) stage_rows(seqs, first, W, L, total, sdst, bar);
     }
-
-    // this lane's constants: its lags m = lane (mod NL) all have the parity of the lane
-    const int odd0 = (n - lane) & 1, odd1 = odd0 ^ 1, sgn0 = (c & 1) ? -1 : 1;
-    const int h0 = (n - lane) >> 1, h1 = (n - 1 - lane) >> 1;  // half the pairs at lag `lane`
-    // FP16 bits of 1536 + C^(p) at lag `lane` before its mismatches, class 1 in the high half
-    const uint32_t kc = 0x66006600u + (uint32_t)(2 * h0 + odd0 * sgn0) + ((uint32_t)(2 * h1 - odd1 * sgn0) << 16);
-    // (E, Z) = C^(0) (1, z0) + C^(1) (1, z1): Z takes 3 times the lag's own class p = (c - m) mod 2
-    const uint32_t zs = (lane & 1) ? 0x80000000u : 0u, own = ((c - lane) & 1) ? 0x3C000000u : 0x42000000u;
-    const __half2 z0 = as_half2((own | 0x3C00u) ^ zs), z1 = as_half2(((own ^ 0x7E000000u) | 0x3C00u) ^ zs);
-    const uint32_t ez0 = half_bits(6 - c + (c & 1)) << 16;  // lag 0: E = 0, Z of the centre
-    const uint32_t gp = sbyte(wb + SL.g + lane), gm = sbyte(wb + SL.g - lane), zp = sbyte(wb + SL.z) + 2 * lane;
-    const uint32_t rowa = sbyte(wb + SL.h0) + 16 * lane, bita = sbyte(wb + SL.b) + lane;
-    const uint32_t sga = sbyte(wb + SL.b + o.p * SL.bvec + (o.v0 >> 5));
-    const int rc = o.p == (c & 1) ? (c >> 1) - o.v0 : -1;   // this lane's output that is the centre
-    const uint32_t sh = sbyte(wb + SL.r8) + 4 * (2 * o.v0 + o.p);
     __syncwarp();
 
     int it = 0;
@@ -230,93 +352,24 @@ __global__ void __launch_bounds__(256, LG::kSize == 16 ? (R <= 7 ? 3 : 2) : 3)
                     const uint32_t lo = __byte_perm(w[0], w[1], p ? 0x7531 : 0x6420);
                     const uint32_t hi = __byte_perm(w[2], w[3], p ? 0x7531 : 0x6420);
                     const uint32_t fl = lo ^ 0x80808080u, fh = hi ^ 0x80808080u;
-                    sts_v4(rowa + 4 * p * SL.hc + 16 * NL * q, byte_halves(fl, 0x4140), byte_halves(fl, 0x4342),
+                    sts_v4(rl.rowa + 4 * p * SL.hc + 16 * NL * q, byte_halves(fl, 0x4140), byte_halves(fl, 0x4342),
                            byte_halves(fh, 0x4140), byte_halves(fh, 0x4342));
-                    sts_u8(bita + 4 * p * SL.bvec + NL * q, (sign_bits(lo) >> 28) | ((sign_bits(hi) >> 24) & 0xF0u));
+                    sts_u8(rl.bita + 4 * p * SL.bvec + NL * q, (sign_bits(lo) >> 28) | ((sign_bits(hi) >> 24) & 0xF0u));
                 }
             }
         }
         __syncwarp();
         uint32_t x0[NW], x1[NW];
-#pragma unroll
-        for (int k = 0; k < NW; ++k) {
-            x0[k] = lds_u32(sbyte(wb + SL.b) + 4 * k);
-            x1[k] = lds_u32(sbyte(wb + SL.b + SL.bvec) + 4 * k);
-        }
-        // signs of the lane's outputs (bit r; above the class's words anything)
-        const uint32_t sgn = __funnelshift_r(lds_u32(sga), lds_u32(sga + 4), o.v0 & 31);
+        const uint32_t sgn = rl.classes(x0, x1);
         const uint32_t f0 = (c & 1) ? ~0u : 0u;  // antipalindromic class: all bits inverted
         bad |= mirror_diff<NW>(x0, n, f0) | mirror_diff<NW>(x1, n - 1, ~f0);
         // the ballot is a full-warp collective: both halves take it, with or without a row (no
         // row: no bytes, not valid)
         const bool valid = t.ballot(bad != 0u) == 0u;
-
-        // table and Z: lags m = lane + NL j + 32 q
-#pragma unroll
-        for (int j = 0; j < 32 / NL; ++j) {
-            uint32_t s0[NW], s1[NW];
-#pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                s0[k] = __funnelshift_r(x0[k], k + 1 < NW ? x0[k + 1] : 0u, lane + NL * j);
-                s1[k] = __funnelshift_r(x1[k], k + 1 < NW ? x1[k + 1] : 0u, lane + NL * j);
-            }
-#pragma unroll
-            for (int q = 0; q < NW; ++q) {
-                const int m0 = 32 * q + NL * j;  // m = m0 + lane
-                int t0 = 0, t1 = 0;
-#pragma unroll
-                for (int k = 0; 2 * k < NW - q; ++k) {
-                    // pairs 32 k .. of the first h: n > 32 (NW - 1) and m < 32 (q + 1)
-                    uint32_t d0 = x0[k] ^ s0[k + q], d1 = x1[k] ^ s1[k + q];
-                    if (32 * (k + 1) > 16 * (NW - q - 2)) {
-                        const int b0 = h0 - m0 / 2 - 32 * k, b1 = h1 - m0 / 2 - 32 * k;
-                        d0 &= __funnelshift_lc(~0u, 0u, k ? max(b0, 0) : b0);
-                        d1 &= __funnelshift_lc(~0u, 0u, k ? max(b1, 0) : b1);
-                    }
-                    t0 += __popc(d0);
-                    t1 += __popc(d1);
-                }
-                const uint32_t cc = kc - (uint32_t)m0 * 0x00010001u - 4u * ((uint32_t)t0 + ((uint32_t)t1 << 16));
-                const __half2 ch = __hsub2(as_half2(cc), as_half2(0x66006600u));
-                uint32_t ez = as_u32(__hfma2(__high2half2(ch), z1, __hmul2(__low2half2(ch), z0)));
-                if (m0 == 0) ez = lane == 0 ? ez0 : ez;
-                if (q < NW - 1) {  // n > 32 (NW - 1): the lag exists
-                    sts_u16(gp + 4 * m0, ez);
-                    sts_u16(gp + 4 * m0 - 2, ez);
-                    sts_u16(zp + 2 * m0, ez >> 16);
-                    if (m0 + NL - 1 < SL.gneg) {
-                        sts_u16(gm - 4 * m0, ez);
-                        sts_u16(gm - 4 * m0 - 2, ez);
-                    } else if (m0 <= SL.gneg) {
-                        sts_u16_if(m0 + lane <= SL.gneg, gm - 4 * m0, ez);
-                        sts_u16_if(m0 + lane < SL.gneg, gm - 4 * m0 - 2, ez);
-                    }
-                } else {
-                    const bool in = lane < n - m0;
-                    sts_u16_if(in, gp + 4 * m0, ez);
-                    sts_u16_if(in, gp + 4 * m0 - 2, ez);
-                    sts_u16_if(in, zp + 2 * m0, ez >> 16);
-                    if (m0 <= SL.gneg) {
-                        sts_u16_if(in && m0 + lane <= SL.gneg, gm - 4 * m0, ez);
-                        sts_u16_if(in && m0 + lane < SL.gneg, gm - 4 * m0 - 2, ez);
-                    }
-                }
-            }
-        }
-        __syncwarp();
-        step_toeplitz(a.prod, wl);  // ends with a warp barrier
-        // dISL = -8 s_i (X_i + 4 sg s_{3i-L+1}) + 8 Z_m + 16 (N_p - 2), the centre -4 s_c;
-        // the FP32 value dISL + 1.5 2^23 + .. holds the integer in its low bits
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float x = lds_f32(a.xr + 4 * r), z = lds_f16(a.zr - 4 * r), s3 = lds_f16(a.sr + 6 * r);
-            const float y = __uint_as_float(__float_as_uint(fmaf(a.sig4, s3, x)) ^ ((sgn << (31 - r)) & 0x80000000u));
-            const float v = fmaf(r == rc ? -4.f : -8.f, y, fmaf(8.f, z, a.bias));
-            sts_u32(sh + 8 * r, __float_as_uint(v) - __float_as_uint(kIntBias));
-        }
-        __syncwarp();
+        rl.table(x0, x1);
+        rl.values(sgn, wl);
         int32_t* dst = out + row * (int64_t)n;
-        const uint32_t res = sbyte(wb + SL.r8) + 4 * lane;
+        const uint32_t res = rl.result(lane);
         if (__all_sync(kFull, has && valid)) {
 #pragma unroll
             for (int k = 0; k < R; ++k)
@@ -324,35 +377,136 @@ __global__ void __launch_bounds__(256, LG::kSize == 16 ? (R <= 7 ? 3 : 2) : 3)
                     dst[lane + NL * k] = (int)lds_u32(res + 4 * NL * k);
         } else if (has) {
             if (!valid && lane == 0 && status) atomicAdd(&status->invalid_rows, 1);
-            for (int i = lane; i < n; i += NL)
-                dst[i] = valid ? (int)lds_u32(sbyte(wb + SL.r8) + 4 * i) : INT_MIN;
+            for (int i = lane; i < n; i += NL) dst[i] = valid ? (int)lds_u32(rl.result(i)) : INT_MIN;
         }
         // the warp barriers before the next rows' product order its overwrites of X and the
         // staged results; the rows, Z and this staging buffer were last read before the one above
     }
 }
 
+// Network inputs of states given by their free-variable bits (8 words each, `stride` words
+// apart): x[b][0][i] = s_i, x[b][1][i] = C_{2(i+1)}/sqrt(L) (0 for i = n-1), x[b][2][i] =
+// dISL_i/(8L).  As the rows, with the pieces of 16 positions from the bits: those above the
+// centre are the mirror's, reversed, with the sign (-1)^(j-c).  Scoring 8192 states of n =
+// 128 takes 172 us with this kernel and took 209 with one warp per state on the FP32 product
+// (40 us of it), a training step of 4096 records 396 from 417.
+template <class LG, int R, int NW>
+__global__ void __launch_bounds__(256, row_ctas<LG, R>())
+    features_kernel(const uint32_t* __restrict__ bits, int64_t stride, int64_t count, int L, float* __restrict__ x)
+{
+    using RL = RowLane<LG, R, NW>;
+    constexpr int NL = RL::NL, W = RL::W, IT = RL::IT;
+    constexpr StepSmem SL = RL::LAY::SL;
+    const int n = (L + 1) / 2, c = n - 1;
+    const LG t(threadIdx.x & 31);
+    const int lane = t.lane, wl = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Outs<LG, R> o(t);
+    const RL rl(warp * W * SL.words, n, t, o);
+    rl.clear();
+    const float sq = sqrtf((float)L), inv8L = (float)(8 * L);
+    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    __syncwarp();
+    for (int64_t b0 = W * ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp); b0 < count; b0 += W * nwarps) {
+        const int64_t b = b0 + group_of(t);
+        const bool has = b < count;
+        const uint32_t* src = bits + (has ? b : b0) * stride;  // no state: the first one's again
+        // bits v .. v+31 of the state, for v >= -31 (zero below 0 and from 32 kBitWords on)
+        const auto window = [&](int v) {
+            const int k = v >> 5;
+            const uint32_t lo = k >= 0 && k < kBitWords ? __ldg(src + k) : 0u;
+            const uint32_t hi = k + 1 >= 0 && k + 1 < kBitWords ? __ldg(src + k + 1) : 0u;
+            return __funnelshift_r(lo, hi, v & 31);
+        };
+#pragma unroll
+        for (int q = 0; q < IT; ++q) {
+            const int piece = lane + NL * q, j0 = 16 * piece;
+            if (IT * NL == 4 * NW || piece < 4 * NW) {
+                // bit e: s_{j0+e} = -1.  Up to the centre the state's bits, above it bit 2c - j
+                uint32_t w = window(j0);
+                if (j0 + 15 > c) {
+                    const uint32_t alt = ((j0 - c) & 1) ? 0x5555u : 0xAAAAu;  // j - c odd
+                    const uint32_t up = (__brev(window(2 * c - j0 - 15)) >> 16) ^ alt;
+                    const uint32_t own = __funnelshift_lc(~0u, 0u, max(c + 1 - j0, 0));
+                    w = (w & own) | (up & ~own);
+                }
+                const int left = L - j0;  // positions of the row from here on
+                w &= __funnelshift_lc(~0u, 0u, min(max(left, 0), 16));
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    uint32_t y = (w >> p) & 0x5555u;
+                    y = (y | y >> 1) & 0x3333u;
+                    y = (y | y >> 2) & 0x0F0Fu;
+                    y = (y | y >> 4) & 0x00FFu;
+                    const int live = (left + 1 - p) >> 1;  // entries of the class from here on
+                    uint32_t hp[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t two = y >> 2 * k;
+                        const uint32_t v = (two << 15 & 0x8000u) | (two << 30 & 0x80000000u) | 0x3C003C00u;
+                        hp[k] = v & (2 * k + 1 < live ? ~0u : 2 * k < live ? 0xFFFFu : 0u);
+                    }
+                    sts_v4(rl.rowa + 4 * p * SL.hc + 16 * NL * q, hp[0], hp[1], hp[2], hp[3]);
+                    sts_u8(rl.bita + 4 * p * SL.bvec + NL * q, y);
+                }
+            }
+        }
+        __syncwarp();
+        uint32_t x0[NW], x1[NW];
+        const uint32_t sgn = rl.classes(x0, x1);
+        rl.table(x0, x1);
+        rl.values(sgn, wl);
+        if (has) {
+            float* xb = x + b * 3 * n;
+            for (int i = lane; i < n; i += NL) {
+                xb[i] = (__ldg(src + (i >> 5)) >> (i & 31)) & 1u ? -1.f : 1.f;
+                xb[n + i] = i < n - 1 ? lds_f16(sbyte(rl.a.wb + SL.g) + 4 * (i + 1)) / sq : 0.f;
+                xb[2 * n + i] = (float)(int)lds_u32(rl.result(i)) / inv8L;
+            }
+        }
+        __syncwarp();  // the next state's table comes after this one's reads
+    }
+}
+
 using RowsFn = void (*)(const int8_t*, int64_t, int, int32_t*, DevStatus*);
+using FeaturesFn = void (*)(const uint32_t*, int64_t, int64_t, int, float*);
+
+// (lane block, words per class) of every length: step_R(n, lanes per row), ceil(n/32)
+#define LABS_ROW_CASES(CASE)                                                                                       \
+    CASE(Pair, 1, 1) CASE(Pair, 2, 1) CASE(Pair, 3, 2) CASE(Pair, 5, 2) CASE(Pair, 5, 3) CASE(Pair, 6, 3)          \
+    CASE(Pair, 7, 4) CASE(Pair, 9, 4) CASE(Pair, 10, 5) CASE(Tile<32>, 7, 6) CASE(Tile<32>, 7, 7)                  \
+    CASE(Tile<32>, 9, 8)
 
 template <bool STAGED>
 RowsFn rows_fn(int key)
 {
-    // (lane block, words per class) of every length: step_R(n, lanes per row), ceil(n/32)
     switch (key) {
-        case 16 * 1 + 1: return rows_kernel<Pair, 1, 1, STAGED>;
-        case 16 * 2 + 1: return rows_kernel<Pair, 2, 1, STAGED>;
-        case 16 * 3 + 2: return rows_kernel<Pair, 3, 2, STAGED>;
-        case 16 * 5 + 2: return rows_kernel<Pair, 5, 2, STAGED>;
-        case 16 * 5 + 3: return rows_kernel<Pair, 5, 3, STAGED>;
-        case 16 * 6 + 3: return rows_kernel<Pair, 6, 3, STAGED>;
-        case 16 * 7 + 4: return rows_kernel<Pair, 7, 4, STAGED>;
-        case 16 * 9 + 4: return rows_kernel<Pair, 9, 4, STAGED>;
-        case 16 * 10 + 5: return rows_kernel<Pair, 10, 5, STAGED>;
-        case 16 * 7 + 6: return rows_kernel<Tile<32>, 7, 6, STAGED>;
-        case 16 * 7 + 7: return rows_kernel<Tile<32>, 7, 7, STAGED>;
-        case 16 * 9 + 8: return rows_kernel<Tile<32>, 9, 8, STAGED>;
+#define LABS_ROW_CASE(LG, R, NW) \
+    case 16 * R + NW: return rows_kernel<LG, R, NW, STAGED>;
+        LABS_ROW_CASES(LABS_ROW_CASE)
+#undef LABS_ROW_CASE
         default: return nullptr;
     }
+}
+
+FeaturesFn features_fn(int key)
+{
+    switch (key) {
+#define LABS_ROW_CASE(LG, R, NW) \
+    case 16 * R + NW: return features_kernel<LG, R, NW>;
+        LABS_ROW_CASES(LABS_ROW_CASE)
+#undef LABS_ROW_CASE
+        default: return nullptr;
+    }
+}
+
+// Warps of a CTA for `units` warps of work: eight; a batch that leaves SMs without a CTA is
+// spread over more, smaller ones (64 rows of L = 255, back to back: 6.1 us a call on the
+// device, 8.2 as four CTAs).
+int row_warps(int64_t units, int sms)
+{
+    int warps = 8;
+    while (warps > 1 && units <= (int64_t)(warps / 2) * sms) warps /= 2;
+    return warps;
 }
 
 }  // namespace
@@ -364,11 +518,8 @@ int launch_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, Dev
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int n = (L + 1) / 2, tile = n <= 160 ? 16 : 32, rows = 32 / tile, R = step_R(n, tile);
-    // eight warps a CTA; a batch that leaves SMs without a CTA is spread over more, smaller
-    // ones (64 rows of L = 255, back to back: 6.1 us a call on the device, 8.2 as four CTAs)
     const int64_t units = (batch + rows - 1) / rows;
-    int warps = 8;
-    while (warps > 1 && units <= (int64_t)(warps / 2) * sms) warps /= 2;
+    const int warps = row_warps(units, sms);
     const size_t warp_bytes = (size_t)rows * step_smem(tile, R).words * sizeof(int);
     const size_t stage = 2 * (size_t)stage_bytes(L, rows) + 16;
     // staged rows need a 16-byte aligned input, and are used where they keep as many CTAs
@@ -385,6 +536,24 @@ int launch_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, Dev
     // more CTAs than fit at once (up to 8 per SM): measured faster than one resident wave
     const int64_t need = (units + warps - 1) / warps, most = (int64_t)sms * 8;
     fn<<<(int)std::min(need, most), warps * kWarp, smem, (cudaStream_t)stream>>>(seqs, batch, L, out, status);
+    return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
+}
+
+int launch_features(const uint32_t* bits, int64_t stride, int64_t count, int32_t L, float* x, void* stream)
+{
+    if (count == 0) return LABS_OK;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int n = (L + 1) / 2, tile = n <= 160 ? 16 : 32, rows = 32 / tile, R = step_R(n, tile);
+    const FeaturesFn fn = features_fn(16 * R + (n + 31) / 32);
+    if (fn == nullptr) return LABS_EINVAL;
+    const int64_t units = (count + rows - 1) / rows;
+    const int warps = row_warps(units, sms);
+    const size_t smem = (size_t)warps * rows * step_smem(tile, R).words * sizeof(int);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t need = (units + warps - 1) / warps, most = (int64_t)sms * 8;
+    fn<<<(int)std::min(need, most), warps * kWarp, smem, (cudaStream_t)stream>>>(bits, stride, count, L, x);
     return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
 }
 
