@@ -25,7 +25,7 @@ struct labs_ctx {
     cudaStream_t capture = nullptr;  // private stream used only to record CUDA graphs
     uint64_t seed = 0;
     int device = 0;
-    int sms = 0;
+    int sms = 0, ahead = 0;
     int nG = 0;
     DevGroup groups[LABS_MAX_GROUPS];
     int64_t W = 0;
@@ -125,6 +125,7 @@ KParams params(labs_ctx* c)
     p.chunk_steps = c->chunk;
     p.rmax = c->long_mode ? long_R(c->n_max, c->tile) : 0;
     p.tile = c->tile;
+    p.ahead = c->ahead;
     p.long_mode = c->long_mode ? 1 : 0;
     p.cur_bits = c->long_mode ? at<uint32_t>(c, c->off_cur_bits) : nullptr;
     p.best_bits = c->long_mode ? at<uint32_t>(c, c->off_best_bits) : nullptr;
@@ -367,6 +368,10 @@ int setup(labs_ctx* c, const int32_t* Ls, const int64_t* counts, int32_t nL, uin
         c->warps_per_cta = warps;
         c->grid = c->sms * c->ctas_per_sm;
         spread(c, k.warps_per_cta == 0);
+        if (c->W * c->n_max <= kAheadSlots && !psl && !(k.flags & LABS_FLAG_BEST_FIRST)) {
+            int occ = 0, regs = 0;
+            c->ahead = walk_kernel_config(c->n_max, c->tile, 4, c->warps_per_cta, &occ, &regs) == LABS_OK && occ > 0;
+        }
         c->chunk = k.chunk_steps ? k.chunk_steps : 1024;
     }
     e = cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking);

@@ -113,6 +113,14 @@ struct Control {
     volatile uint64_t deadline_ns;   // GPU %globaltimer deadline, UINT64_MAX = none
 };
 
+// HT slots that the walkers' neighbours have (walkers x n_max) up to which the plain walk
+// looks all of them up at a step's start (walk_lockstep).  Microseconds a step with and
+// without: 64 walkers of L = 41 0.97 / 1.22, of L = 201 1.01 / 1.21, of L = 501 (16064 slots)
+// 1.24 / 1.36; 300 of L = 151 (22800) 1.72 / 1.67, 300 of L = 201 (30300) 1.39 / 1.48, 300 of
+// L = 501 (75300) 2.14 / 1.60, 2432 of L = 201 4.8 / 1.68: past the line the loads fill the
+// path to L2 and HBM.
+constexpr int64_t kAheadSlots = 1 << 14;
+
 struct KParams {
     DevStatus* status;
     const DevGroup* groups;
@@ -135,6 +143,7 @@ struct KParams {
     int32_t best_first;       // 1: best-first search (one walker per warp, queue below)
     int32_t mode;             // walk kernel variant: 0 plain walk, 1 learned mode, 2 best-first,
                               // 3 walk under the PSL objective
+    int32_t ahead;            // 1: the plain walk's kernels for few walkers
     int32_t long_mode;        // 1: lengths above LABS_MAX_L, one walker per CTA
     uint32_t* cur_bits;       // long mode: [W][kBitWordsLong] free variables of the current
     uint32_t* best_bits;      // and of the best sequence (WalkerState.cur / best unused)
@@ -589,6 +598,9 @@ __host__ __device__ inline int long_isl_limit(int L, int n)
 // lane blocks 1-6 and 7-10; labs_walk16a.cu, labs_walk16b.cu: two walkers per warp,
 // lane blocks 1-5 and 6-10; labs_walk32.cu: one walker per warp).
 using WalkFn = void (*)(KParams, int);
+WalkFn walk_fn8f(int rmax);   // for few walkers (8f, 16f, 32f)
+WalkFn walk_fn16f(int rmax);
+WalkFn walk_fn32f(int rmax);
 WalkFn walk_fn8a(int rmax);
 WalkFn walk_fn8b(int rmax);
 WalkFn walk_fn16a(int rmax);

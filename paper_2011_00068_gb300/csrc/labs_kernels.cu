@@ -434,6 +434,7 @@ int launch_prep_walk(const KParams& p, int64_t steps, int nchunks, void* stream)
 
 static WalkFn walk_fn(int tile, int rmax, int mode)
 {
+    if (mode == 4) return tile == 8 ? walk_fn8f(rmax) : tile == 16 ? walk_fn16f(rmax) : walk_fn32f(rmax);
     if (tile == 8) return rmax <= 6 ? walk_fn8a(rmax) : walk_fn8b(rmax);
     if (tile == 16 && mode == 3) return rmax <= 5 ? walk_fn16p(rmax) : walk_fn16q(rmax);
     if (tile == 16) return rmax <= 5 ? walk_fn16a(rmax) : walk_fn16b(rmax);
@@ -445,7 +446,8 @@ static WalkFn walk_fn(int tile, int rmax, int mode)
     }
 }
 
-// Lane block and shared memory per warp of a walk kernel (mode 1: the learned mode).
+// Lane block and shared memory per warp of a walk kernel (mode 1: the learned mode, 4: the
+// plain walk's kernels for few walkers).
 static int walk_R(int n_max, int tile, int mode)
 {
     return mode != 1 ? step_R(n_max, tile) : block_R(n_max, tile);
@@ -481,7 +483,7 @@ int walk_kernel_config(int n_max, int tile, int mode, int warps_per_cta, int* ct
 
 int launch_walk_chunk(const KParams& p, int chunk_index, int grid, int warps_per_cta, void* stream)
 {
-    const WalkFn fn = walk_fn(p.tile, walk_R(p.n_max, p.tile, p.mode), p.mode);
+    const WalkFn fn = walk_fn(p.tile, walk_R(p.n_max, p.tile, p.mode), p.mode == 0 && p.ahead ? 4 : p.mode);
     const size_t smem_bytes = walk_warp_bytes(p.n_max, p.tile, p.mode) * (size_t)warps_per_cta;
     fn<<<grid, warps_per_cta * kWarp, smem_bytes, (cudaStream_t)stream>>>(p, chunk_index);
     return status_of(cudaGetLastError());

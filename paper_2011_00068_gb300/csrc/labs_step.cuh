@@ -859,7 +859,14 @@ __device__ __forceinline__ uint32_t step_sign(uint32_t word, int i, const LG& t)
 // group has one), from shared state built by step_build.  RT is the tile type a group
 // restarts with (divergently).  extras: bit 0 the walker is traced, bit 1 its chunk is
 // logged.  Returns the steps taken.
-template <class LAY, class LG, class RT, int R>
+//
+// AHEAD (few walkers): with a warp or two on a scheduler nothing covers the latency of the HT
+// lookup, which was half of a step.  The states of all neighbours are known when a step
+// starts, so every lane loads the first HT slot of each of its R outputs then, under the
+// product; what is found visited leaves the keys, and the lowest key left is the move (an
+// occupied first slot of another state sends the walker to step_search).  n loads a step
+// instead of one or two: only while the walkers' HT traffic is small (kAheadSlots).
+template <class LAY, class LG, class RT, int R, bool AHEAD = false>
 __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, int len, bool real, int wb0,
                                              unsigned extras, const LG& t, const RT& tt)
 {
@@ -877,6 +884,15 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
     step_load_lags<LAY, LG, R>(wb, lane, lg);
     StopCheck stop;
     stop.start(p, l == 0);
+    const uint32_t tmask = (1u << p.tabu_log2) - 1u;
+    uint64_t zkr[AHEAD ? R : 1], ent[AHEAD ? R : 1];
+    if constexpr (AHEAD) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = 2 * (o.v0 + r) + o.p;
+            zkr[r] = i <= c ? __ldg(env.zk + i) : 0ull;
+        }
+    }
     const int top = __reduce_max_sync(kFull, real ? len : 0);
     int it = 0;
     for (; it < top; ++it) {
@@ -887,6 +903,10 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
                 if (act && lane == 0) raise_error(p.status, why, (int)env.g);
                 break;
             }
+        }
+        if constexpr (AHEAD) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) ent[r] = env.T[(uint32_t)(w.fp ^ zkr[r]) & tmask];
         }
         step_toeplitz<LAY, LG, R>(a.prod, l);
 
@@ -932,46 +952,79 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
                 for (int r = 0; r < R; ++r) key[r] = kl[r];
             }
         }
-        KT b1, b2;
-        key_top2(key, b1, b2);
-
         // Best admissible flip: the lowest key whose state is not in HT.  The two lowest
         // are probed at once, the first S HT slots of each by one half of the walker's
         // lanes; that settles nearly every step, step_search does the others.
-        KT k0, k1;
-        step_min2(b1, b2, t, k0, k1);
-        const int hs = lane & (S - 1);
-        const KT km = lane >= S ? k1 : k0;
-        const bool live = act && !key_none(km) && hs < p.probe_cap;
-        // a key without an output reads past the length's fingerprint keys, within the workspace
-        const uint64_t f = w.fp ^ __ldg(env.zk + ((uint32_t)km & 0xFFu));
-        const uint32_t at = ((uint32_t)f + (uint32_t)hs) & ((1u << p.tabu_log2) - 1u);
-        const uint64_t e = env.T[at], tag = (f & ~kGenMask) | w.gen;
-        const bool match = live && e == tag;
-        const unsigned hb = __ballot_sync(kFull, match || (live && ((uint32_t)e & (uint32_t)kGenMask) != w.gen));
-        const unsigned mb = __ballot_sync(kFull, match);
-        unsigned pick;  // the lane that saw the free slot of the chosen state (0: not settled)
         KT kc;
-        bool stored = true;
-        {
-            const unsigned g0 = hb & (((1u << S) - 1u) << t.base), g1 = hb & (((1u << S) - 1u) << (t.base + S));
-            const unsigned p0 = g0 & (0u - g0), p1 = g1 & (0u - g1);  // each candidate's first hit
-            const bool v0 = (p0 & mb) != 0u, v1 = (p1 & mb) != 0u;
-            kc = v0 ? k1 : k0;
-            pick = v0 ? (v1 ? 0u : p1) : p0;
-            if (__any_sync(kFull, act && pick == 0u)) {
-                const bool need = act && pick == 0u;
+        uint32_t at;
+        uint64_t tag;
+        bool stored = true, insert;  // insert: this lane writes the chosen state to HT
+        if constexpr (AHEAD) {
+            uint32_t occ = 0;  // outputs whose first slot holds a state of this start
+            KT b = ~(KT)0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const uint64_t tr = ((w.fp ^ zkr[r]) & ~kGenMask) | w.gen;
+                if (ent[r] == tr) key[r] = ~(KT)0;
+                occ |= ((uint32_t)ent[r] & (uint32_t)kGenMask) == w.gen ? 1u << r : 0u;
+                b = min(b, key[r]);
+            }
+            kc = group_min(b, t);
+            if (key_none(kc)) kc = ~(KT)0;
+            const int i0 = (int)((uint32_t)kc & 0xFFu), r0 = (i0 >> 1) - o.v0;
+            const bool other = act && kc != ~(KT)0 && (i0 & 1) == o.p && (unsigned)r0 < (unsigned)R && ((occ >> r0) & 1u);
+            const uint64_t f = w.fp ^ __ldg(env.zk + i0);
+            at = (uint32_t)f & tmask;
+            tag = (f & ~kGenMask) | w.gen;
+            insert = lane == 0;
+            if (__any_sync(kFull, other)) {
+                const bool need = t.ballot(other) != 0u;
                 KT ks = ~(KT)0;
                 bool st = false;
-                step_search(env, w.fp, w.gen, key, v0 ? (v1 ? k1 : k0) : (KT)0, need, t, ks, st);
+                step_search(env, w.fp, w.gen, key, (KT)0, need, t, ks, st);
                 if (need) {
                     kc = ks;
                     stored = st;
+                    insert = false;
+                }
+            }
+        } else {
+            KT b1, b2, k0, k1;
+            key_top2(key, b1, b2);
+            step_min2(b1, b2, t, k0, k1);
+            const int hs = lane & (S - 1);
+            const KT km = lane >= S ? k1 : k0;
+            const bool live = act && !key_none(km) && hs < p.probe_cap;
+            // a key without an output reads past the length's fingerprint keys, within the workspace
+            const uint64_t f = w.fp ^ __ldg(env.zk + ((uint32_t)km & 0xFFu));
+            at = ((uint32_t)f + (uint32_t)hs) & tmask;
+            tag = (f & ~kGenMask) | w.gen;
+            const uint64_t e = env.T[at];
+            const bool match = live && e == tag;
+            const unsigned hb = __ballot_sync(kFull, match || (live && ((uint32_t)e & (uint32_t)kGenMask) != w.gen));
+            const unsigned mb = __ballot_sync(kFull, match);
+            {
+                // pick: the lane that saw the free slot of the chosen state (0: not settled)
+                const unsigned g0 = hb & (((1u << S) - 1u) << t.base), g1 = hb & (((1u << S) - 1u) << (t.base + S));
+                const unsigned p0 = g0 & (0u - g0), p1 = g1 & (0u - g1);  // each candidate's first hit
+                const bool v0 = (p0 & mb) != 0u, v1 = (p1 & mb) != 0u;
+                kc = v0 ? k1 : k0;
+                const unsigned pick = v0 ? (v1 ? 0u : p1) : p0;
+                insert = (pick >> l) == 1u;
+                if (__any_sync(kFull, act && pick == 0u)) {
+                    const bool need = act && pick == 0u;
+                    KT ks = ~(KT)0;
+                    bool st = false;
+                    step_search(env, w.fp, w.gen, key, v0 ? (v1 ? k1 : k0) : (KT)0, need, t, ks, st);
+                    if (need) {
+                        kc = ks;
+                        stored = st;
+                    }
                 }
             }
         }
         const bool moves = act && kc != ~(KT)0;
-        stg_u64_if(moves && (pick >> l) == 1u, env.T + at, tag);
+        stg_u64_if(moves && insert, env.T + at, tag);
 
         // Apply the move (walkers that have one).
         const int bi = moves ? (int)((uint32_t)kc & 0xFFu) : 0;
@@ -1287,7 +1340,7 @@ __host__ __device__ constexpr int step_ctas(int tile, int R, bool psl = false)
 // Runs the walkers of the queue: the warp takes W consecutive walkers; when their lengths
 // differ (a group boundary) or fewer are left, it runs them one after the other with the
 // other lane groups idle.
-template <class LG, class RT, int RMAX, bool PSL = false, bool BEST = false>
+template <class LG, class RT, int RMAX, bool PSL = false, bool BEST = false, bool AHEAD = false>
 __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
 {
     constexpr int NL = LG::kSize, W = 32 / NL;
@@ -1374,17 +1427,17 @@ __device__ __forceinline__ void walk_group(const KParams& p, int chunk_index)
                     done = walk_bestfirst<LAY, (RMAX > 2 ? RMAX - 2 : 1)>(env, w, len, real, wb0, extras, t);
             } else if constexpr (NL == 32) {  // lane blocks are odd
                 if (R >= RMAX)
-                    done = walk_lockstep<LAY, LG, RT, RMAX>(env, w, len, real, wb0, extras, t, tt);
+                    done = walk_lockstep<LAY, LG, RT, RMAX, AHEAD>(env, w, len, real, wb0, extras, t, tt);
                 else
-                    done = walk_lockstep<LAY, LG, RT, (RMAX > 2 ? RMAX - 2 : 1)>(env, w, len, real, wb0, extras, t, tt);
+                    done = walk_lockstep<LAY, LG, RT, (RMAX > 2 ? RMAX - 2 : 1), AHEAD>(env, w, len, real, wb0, extras, t, tt);
             } else if (R >= RMAX)
-                done = walk_lockstep<LAY, LG, RT, RMAX>(env, w, len, real, wb0, extras, t, tt);
+                done = walk_lockstep<LAY, LG, RT, RMAX, AHEAD>(env, w, len, real, wb0, extras, t, tt);
             else if (R == RMAX - 1)
-                done = walk_lockstep<LAY, LG, RT, (RMAX > 1 ? RMAX - 1 : 1)>(env, w, len, real, wb0, extras, t, tt);
+                done = walk_lockstep<LAY, LG, RT, (RMAX > 1 ? RMAX - 1 : 1), AHEAD>(env, w, len, real, wb0, extras, t, tt);
             else if (R == RMAX - 2)
-                done = walk_lockstep<LAY, LG, RT, (RMAX > 2 ? RMAX - 2 : 1)>(env, w, len, real, wb0, extras, t, tt);
+                done = walk_lockstep<LAY, LG, RT, (RMAX > 2 ? RMAX - 2 : 1), AHEAD>(env, w, len, real, wb0, extras, t, tt);
             else
-                done = walk_lockstep<LAY, LG, RT, (RMAX > 3 ? RMAX - 3 : 1)>(env, w, len, real, wb0, extras, t, tt);
+                done = walk_lockstep<LAY, LG, RT, (RMAX > 3 ? RMAX - 3 : 1), AHEAD>(env, w, len, real, wb0, extras, t, tt);
             if (real) {
                 if (t.lane < kBitWords) st->cur[t.lane] = w.word;
                 if (t.lane == 0) {

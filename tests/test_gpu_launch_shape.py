@@ -37,3 +37,26 @@ def test_long_walkers_on_as_many_ctas(L, walkers):
     o = oracle.walk(L, 5, min(walkers, 6), 12)
     assert np.array_equal(r["isl"][:6], o["final_isl"])
     assert np.array_equal(r["seq"][:6], o["final_seq"])
+
+
+@pytest.mark.parametrize("L,many", [(41, 1300), (101, 700), (151, 700), (201, 400), (401, 150)])
+@pytest.mark.parametrize("kw", [{}, {"tabu_log2": 4, "probe_cap": 3}, {"tabu_log2": 5, "probe_cap": 1},
+                                {"tabu_log2": 6, "probe_cap": 32, "patience": 30}, {"tabu_log2": 3, "probe_cap": 20}])
+def test_few_and_many_walkers_take_the_same_steps(L, many, kw):
+    """Few walkers look every neighbour up at a step's start, many the lowest two: the first
+    walkers of both searches, and the oracle's, agree step for step, also where HT is nearly
+    full, single slots are probed or every state is taken."""
+    few, steps, got = 9, 90, []
+    for W in (few, many):
+        s = labs.Search(L, W, 11, **kw)
+        code, isl = s.trace(list(range(few)), steps)
+        s.walk(steps)
+        s.sync()
+        r = s.results(seqs=True)
+        got.append((code.cpu().numpy(), isl.cpu().numpy(), r["isl"][:few], r["best_isl"][:few], r["seq"][:few]))
+        s.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+    o = oracle.walk(L, 11, few, steps, trace=True, **kw)
+    assert np.array_equal(got[0][0], o["trace_code"]) and np.array_equal(got[0][1], o["trace_isl"])
+    assert np.array_equal(got[0][4], o["final_seq"])
