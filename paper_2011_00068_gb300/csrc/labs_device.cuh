@@ -1,10 +1,10 @@
-// labs_device.cuh -- device code of the walk shared by the kernel translation units
-// (included by labs_kernels.cu, labs_long.cu and the walk-instantiation units
-// labs_walk8a/8b.cu, labs_walk16a/16b.cu and labs_walk32*.cu).  Not part of the
-// public ABI.
+// labs_device.cuh -- device code shared by the kernel translation units: random starts,
+// lane groups, the rows, table and neighbourhood of a walker on FP32 (the learned walk, the
+// first starts, the long sequences; the other walks and the row kernels evaluate the
+// neighbourhood in the form of labs_step.cuh).  Not part of the public ABI.
 //
-// A tile of lanes owns one walker (or one input row): the whole warp, or half of it when
-// two walkers share a warp.  A walker's sequence is kept in shared
+// A lane group owns one walker (or one input row): the whole warp, a part of it when
+// several walkers share a warp, or a CTA.  A walker's sequence is kept in shared
 // memory split by parity, because for even lags every term of the neighbourhood
 // evaluation pairs positions of equal parity:
 //   A0[u] = s_{2u}   (u = 0..n-1),   A1[u] = s_{2u+1}   (u = 0..n-2),
@@ -429,8 +429,7 @@ __device__ __forceinline__ void toeplitz_part(const float* A, const float2* G, i
     for (int r = 0; r < RC; ++r) X[C0 + r] = acc[r].x + acc[r].y;
 }
 
-// All R outputs in one pass over u (a two-pass split of a 13-output block, fewer
-// registers, ran the four-walker step 13-29% slower than one pass).
+// All R outputs in one pass over u.
 template <class TL, int R>
 __device__ __forceinline__ void toeplitz(const View& V, int n, const Outs<TL, R>& o, float (&X)[R])
 {
@@ -438,8 +437,8 @@ __device__ __forceinline__ void toeplitz(const View& V, int n, const Outs<TL, R>
     toeplitz_part<R, 0, R>(A, V.G - o.v0, (n + 7) & ~7, X);
 }
 
-// The Toeplitz products of both walkers of a warp (two walkers per warp) on the tensor
-// cores, for n <= 128.  In blocks of 16, u = 16 s + j and v = 16 t + i, the product is
+// The Toeplitz product on the tensor cores.  In blocks of 16, u = 16 s + j and v = 16 t + i,
+// it is
 //   X_t = sum_d T_d A_{t+d},   T_d[i][j] = E[16 d + j - i],   A_s[j] = A_p[16 s + j],
 // a sum over the block diagonals d of a 16 x 16 Toeplitz block of the table times the
 // row blocks d further.  One mma.sync.m16n8k16 per diagonal takes T_d (rows i, columns
@@ -449,8 +448,7 @@ __device__ __forceinline__ void toeplitz(const View& V, int n, const Outs<TL, R>
 // is exact), the rows come from their FP16 copies (A = 0, +-1), and the products
 // accumulate in FP32: every partial sum is an integer below 2^24, so the result equals
 // the FP32 product's.  Reads outside the class meet the rows' zero padding, and E is
-// finite (zero) beyond the table.  The warp writes each walker's results to its
-// scratch X[2][xp], and every lane then reads its R outputs.
+// finite (zero) beyond the table.
 __device__ __forceinline__ uint32_t half2_bits(float2 v)
 {
     const __half2 h = __float22half2_rn(v);  // .x in the low half
@@ -476,51 +474,7 @@ __device__ __forceinline__ void tc_diag(float (&d)[4], const float2* gy, const u
     am8 = a2;
 }
 
-template <int R>
-__device__ __forceinline__ void toeplitz_tc(const View& V, const WarpSmem& SL, int n, const Outs<Pair, R>& o, int h,
-                                            float (&X)[R])
-{
-    const int l = threadIdx.x & 31, g = l >> 2, tq = l & 3;
-    const int S = (n + 15) >> 4;               // row blocks
-    const int T = (((n + 1) >> 1) + 15) >> 4;  // output blocks per class (<= 4)
-    const int pb = g >> 2, tb = g & 3;         // this lane's operand column: class, block
-    const int px = tq >> 1, tx = 2 * (tq & 1); // its accumulator columns: class, first block
-    int* const own = reinterpret_cast<int*>(V.A0) - SL.apad;
-    int* const base0 = own - h * SL.words;     // walker 0 of the warp; walker 1 follows
-    const float2* gy = reinterpret_cast<const float2*>(base0 + SL.goff) + SL.gpad + (2 * tq - g - 16 * (T - 1));
-    const uint32_t* ab = reinterpret_cast<const uint32_t*>(base0 + SL.hoff + pb * SL.hlen) + (SL.hpad >> 1) +
-                         8 * (tb - (T - 1)) + tq;
-    const int nd = S + T - 1, w1 = SL.words, g1 = SL.words >> 1;
-    // two independent accumulator chains, one per walker
-    float d0[4] = {0.f, 0.f, 0.f, 0.f}, e0[4] = {0.f, 0.f, 0.f, 0.f};
-    uint32_t am0 = half2_bits(gy[-8]), am1 = half2_bits(gy[g1 - 8]);
-    for (int k = 0; k < nd; ++k) {
-        tc_diag(d0, gy, ab, am0);
-        tc_diag(e0, gy + g1, ab + w1, am1);
-        gy += 16;
-        ab += 8;
-    }
-    float* xp = reinterpret_cast<float*>(base0 + SL.roff) + px * SL.xp + 16 * tx + g;
-    float* xq = xp + w1;
-    if (tx < T) {
-        xp[0] = d0[0];
-        xp[8] = d0[2];
-        xq[0] = e0[0];
-        xq[8] = e0[2];
-    }
-    if (tx + 1 < T) {
-        xp[16] = d0[1];
-        xp[24] = d0[3];
-        xq[16] = e0[1];
-        xq[24] = e0[3];
-    }
-    __syncwarp();
-    const float* xr = reinterpret_cast<const float*>(own + SL.roff) + o.p * SL.xp + o.v0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) X[r] = xr[r];
-}
-
-// The same product for one walker on one warp: the output blocks form M = ceil(T/4)
+// One walker on one warp: the output blocks form M = ceil(T/4)
 // column groups of 4 blocks per class (M <= 2 for n <= 256), and for group m the block
 // diagonals run from -(4m+3) (or -(T-1)) up to S-1-4m.  Two accumulator chains (two
 // groups, or the even and odd diagonals of a lone group; integer partial sums, so the
@@ -1372,169 +1326,10 @@ __device__ void save_scalars(WalkerState* st, const Walker& w)
     }
 }
 
-// ------------------------------------------------------------------ lockstep step
-//
-// The step of walk_steps without the learned extras, written for a warp that runs
-// either one walker (lane group Tile<32>) or two walkers of the same length in
-// lockstep (Pair: lanes 16h..16h+15 run walker h).  With two walkers both halves stay
-// converged through the hot part of every step, so each full-warp collective serves
-// both walkers and what differs between them is carried by predicates; restarts,
-// which are rare, run divergently per half with tile-masked primitives (Tile<16>).
-// The trajectory of each walker is exactly that of walk_steps.
-
-// dISL of the lane's R outputs (returns how many exist): the assembly of `assemble`
-// without bounds tests or branches, for the lockstep layouts (warp_smem pads the rows
-// and the table for every lane output, existing or not), s_{3i-L+1} reading as 0 below
-// index 0, and the centre's formula selected per output.  The results are exact
-// integers below 2^22 in magnitude (|dISL| < 8 L^2 + 48 n for L <= 511), returned as
-// dISL + 1.5 * 2^23 in fp32, whose bit pattern is 0x4B400000 + dISL: the integer sits in
-// the low bits without a float-to-int conversion.  lane_keys packs them as
-// (dISL + 2^22) << 8 | i, ascending in (dISL, i), or 0xFFFFFFFF where the output does
-// not exist (keys are unique, below 2^31 and above 0).
+// dISL + 1.5 * 2^23 in fp32 has the bit pattern 0x4B400000 + dISL (|dISL| < 2^22 for L <=
+// 511): the integer sits in the low bits without a conversion.
 constexpr float kIntBias = 12582912.f;  // 1.5 * 2^23
-constexpr int kIntBiasBits = 0x4B400000;
-constexpr int kKeyBias = 1 << 22;       // dISL = (key >> 8) - kKeyBias
-
-__device__ __forceinline__ float row_value(float a)
-{
-    return a;
-}
-__device__ __forceinline__ float row_value(__half a)
-{
-    return __half2float(a);
-}
-
-// A: the lane's class row (FP32, or FP16 in the row kernels' tensor-core layout).
-template <class LG, int R, class E>
-__device__ __forceinline__ int lane_dlb_rows(const E* A, const View& V, int n, const Outs<LG, R>& o,
-                                             const float (&X)[R], const float (&P)[R], uint32_t (&db)[R])
-{
-    const int p = o.p, c = n - 1;
-    const int rv = (p ? (n >> 1) : ((n + 1) >> 1)) - o.v0;
-    const int rc = (c & 1) == p ? ((c - p) >> 1) - o.v0 : -1;  // the centre's r, if this lane has it
-    const float base = (float)(16 * ((p ? n - 2 : n - 1) - 1)) + kIntBias, cbase = (float)(16 * (c >> 1)) + kIntBias;
-    const E* Av = A + o.v0;                        // s_i          = Av[r]
-    const E* Aq = A + (n - 1 - p - o.v0);          // s_q          = Aq[-r]
-    const E* At = A + (3 * o.v0 + p - n + 1);      // s_{3i-L+1}   = At[3r]
-    const float2* Gc = V.G + (c - p - 2 * o.v0);   // C_{q-i}      = Gc[-2r].x
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const float av = row_value(Av[r]), sq = row_value(Aq[-r]);
-        const float ck0 = Gc[-2 * r].x, st = row_value(At[3 * r]);
-        const bool ctr = r == rc;
-        // every partial sum is an integer of magnitude below 2^24: exact
-        const float add = ctr ? cbase : fmaf(32.f, fmaf(-sq, st, P[r]), base);
-        const float mul = (ctr ? -4.f : -8.f) * av;
-        db[r] = __float_as_uint(fmaf(mul, fmaf(-sq, ck0, X[r]), add));
-    }
-    return rv;  // outputs r below this exist
-}
-
-template <class LG, int R>
-__device__ __forceinline__ int lane_dlb(const View& V, int n, const Outs<LG, R>& o, const float (&X)[R],
-                                        const float (&P)[R], uint32_t (&db)[R])
-{
-    return lane_dlb_rows(o.p ? V.A1 : V.A0, V, n, o, X, P, db);
-}
-
-template <class LG, int R, class E>
-__device__ __forceinline__ int lane_dl_rows(const E* A, const View& V, int n, const Outs<LG, R>& o,
-                                            const float (&X)[R], const float (&P)[R], int (&dl)[R])
-{
-    uint32_t db[R];
-    const int rv = lane_dlb_rows(A, V, n, o, X, P, db);
-#pragma unroll
-    for (int r = 0; r < R; ++r) dl[r] = (int)db[r] - kIntBiasBits;
-    return rv;
-}
-
-template <class LG, int R>
-__device__ __forceinline__ int lane_dl(const View& V, int n, const Outs<LG, R>& o, const float (&X)[R],
-                                       const float (&P)[R], int (&dl)[R])
-{
-    return lane_dl_rows(o.p ? V.A1 : V.A0, V, n, o, X, P, dl);
-}
-
-template <class LG, int R>
-__device__ __forceinline__ void lane_keys(const View& V, int n, const Outs<LG, R>& o, const float (&X)[R],
-                                          const float (&P)[R], unsigned (&key)[R])
-{
-    uint32_t db[R];
-    const int rv = lane_dlb(V, n, o, X, P, db);
-    const unsigned i0 = (unsigned)(2 * o.v0 + o.p);
-    // (0x4B400000 + dISL) << 8 drops the exponent: (2^22 + dISL) << 8
-#pragma unroll
-    for (int r = 0; r < R; ++r) key[r] = r < rv ? (db[r] << 8) + i0 + 2u * r : 0xFFFFFFFFu;
-}
-
-// Flips free variable best_i (and its mirror) in the walker's rows, even-lag table and
-// P, all from the values before the flip, when `moves` (the lanes of a walker without a
-// move rewrite unchanged values).  The rows are padded so that no read or write needs a
-// bounds test (four walkers per warp: reads of s_{i+2m} stay inside the class and the
-// mirror half of the table is kept only as deep as the Toeplitz window reads).
-template <class LG, int R>
-__device__ __forceinline__ void apply_flip(const View& V, int n, const Outs<LG, R>& o, int lane, bool moves,
-                                           int best_i, float (&P)[R])
-{
-    const int c = n - 1;
-    const int m0 = 1 + lane * R;  // this lane's lags 2m of the update, m = m0 .. m0+R-1
-    const int pb = best_i & 1, vb = best_i >> 1;
-    float* Ab = pb ? V.A1 : V.A0;
-    const bool centre = best_i == c;
-    const int vq = centre ? vb : n - 1 - vb - pb;
-    const float as = Ab[vb], aq = centre ? 0.f : Ab[vq];
-    __syncwarp();
-    // The flipped entries read as 0 while the changes are taken: that drops the pairs
-    // whose two ends both flip (unchanged) and the lag-0 terms from every sum below.
-    if (moves && lane == 0) {
-        Ab[vb] = 0.f;
-        Ab[vq] = 0.f;
-    }
-    __syncwarp();
-    // dC_{2m} = -4 s_i (s_{i+2m} + s_{i-2m}) (centre: -2 s_c (..)) for this lane's m
-    const float coef = moves ? (centre ? -2.f : -4.f) * as : 0.f;
-    float dd[R];
-    {
-        const float* up = Ab + vb + m0;
-        const float* dn = Ab + vb - m0;
-#pragma unroll
-        for (int k = 0; k < R; ++k) dd[k] = coef * (up[k] + dn[-k]);
-    }
-    // P_v of the moved class: each pair (v+m, v-m) with exactly one flipped end
-    // changes by -2 x its old product; the partner of w is 2v - w
-    {
-        const float g = (moves && o.p == pb) ? -2.f : 0.f;
-        const float* B1 = Ab + 2 * o.v0 - vb;
-        const float* B2 = Ab + 2 * o.v0 - vq;
-#pragma unroll
-        for (int r = 0; r < R; ++r) P[r] = fmaf(g, fmaf(aq, B2[2 * r], as * B1[2 * r]), P[r]);
-    }
-    {
-        // E[m] += dd for this lane's m, in the pairs G[y] = (E[y], E[y+1]) and their
-        // mirrors at -y (pairs shared with a neighbour lane are written field by field)
-        float e[R + 1];
-        e[R] = 0.f;
-#pragma unroll
-        for (int k = 0; k < R; k += 2) {
-            const float2 g = V.G[m0 + k];
-            e[k] = g.x + dd[k];
-            if (k + 1 < R) e[k + 1] = g.y + dd[k + 1];
-        }
-        V.G[m0 - 1].y = e[0];
-#pragma unroll
-        for (int k = 0; k + 1 < R; ++k) V.G[m0 + k] = make_float2(e[k], e[k + 1]);
-        V.G[m0 + R - 1].x = e[R - 1];
-        V.G[-m0].x = e[0];
-#pragma unroll
-        for (int k = 0; k + 1 < R; ++k) V.G[-m0 - k - 1] = make_float2(e[k + 1], e[k]);
-        V.G[-m0 - R].y = e[R - 1];
-    }
-    __syncwarp();
-    if (moves && lane == 0) {
-        set_row(V, pb, vb, -as);
-        if (!centre) set_row(V, pb, vq, -aq);
-    }
-}
+constexpr int kKeyBias = 1 << 22;       // walk keys: dISL = (key >> 8) - kKeyBias
 
 // ISL at or below which the target merit factor is met (-1: no target).
 __device__ __forceinline__ int target_isl(const KParams& p, int L)
@@ -1543,17 +1338,7 @@ __device__ __forceinline__ int target_isl(const KParams& p, int L)
     return (int)min((int64_t)INT_MAX, (int64_t)p.target_den * L * L / (2 * (int64_t)p.target_num));
 }
 
-// ------------------------------------------------------------- best-first search
-//
-// Algorithm 1 as printed (impxLast, Section 3): the neighbourhood of S fills a queue
-// of LABS_QUEUE_SIZE evaluated neighbours ordered by merit factor and the next S is the
-// queue's first entry (the readings are stated with labs_walk in labs.h).  One walker
-// per warp; lane l holds queue entry l as a 64-bit key
-//   ISL << 36 | (steps done before the step that produced it) << 8 | i
-// (ascending = the queue order; ~0 = empty) and the entry's free variables live in
-// global memory.  An entry produced by the current step is a neighbour of S and is
-// applied incrementally; an older one rebuilds the rows and the table from its bits.
-
+// Lowest and highest 64-bit value of the warp's lanes (the best-first search's queue keys).
 __device__ __forceinline__ uint64_t warp_min64(uint64_t v)
 {
     const unsigned hi = __reduce_min_sync(kFull, (unsigned)(v >> 32));
@@ -1570,16 +1355,10 @@ __device__ __forceinline__ uint64_t warp_max64(uint64_t v)
 
 // A new S that differs from S in at most this many free variables is reached by that
 // many incremental flips (a neighbour of S, about half the steps, by one) rather than
-// a rebuild from its bits; about four of five steps at L = 101..151 (measured with the
-// Python statement), each flip costing about a sixth of a rebuild.
+// a rebuild from its bits; about four of five steps at L = 101..151, each flip costing about
+// a sixth of a rebuild.
 constexpr int kBestFirstMaxFlips = 5;
 
-// One launch advances every walker by up to chunk_steps steps toward the target.  The
-// kernel is compiled for a tile of TILE lanes per walker and a largest lane block RMAX
-// = block_R(n_max, TILE) (register allocation follows it; odd for TILE = 32); walkers
-// whose n needs a smaller block run with RMAX-2, which covers them (any R >=
-// block_R(n) computes the same values).  MODE picks the step: 0 the plain walk, 1 the
-// learned mode, 2 the best-first search (one variant per kernel keeps the code small).
 // ------------------------------------------------------------ PSL objective walk
 
 // Order key of a flip under the PSL objective: PSL' << 43 | ISL' << 13 | i (PSL' < 2^21,

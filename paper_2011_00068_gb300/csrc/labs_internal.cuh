@@ -214,6 +214,8 @@ __host__ __device__ constexpr int block_R(int n, int tile)
 // Shared memory of one SM that the walk layouts may fill (of 228 KB, 1 KB per CTA kept).
 constexpr int kSmemBudget = 226 * 1024;
 
+// The walk kernels that keep this layout are the first starts and the learned walk, 32 lanes
+// per walker; the others have StepSmem.
 // n_max: largest number of free variables served; tile: lanes per walker (32, 16 or 8);
 // tc: with the regions of the tensor-core Toeplitz product (FP16 rows, results); psl:
 // two walkers per warp under the PSL objective (the rows and the table padded for the
@@ -412,7 +414,8 @@ __host__ __device__ constexpr StepSmem step_smem(int tile, int R, bool psl = fal
     return w;
 }
 
-// Layout of one row of the stateless row kernels (labs_neighbor_delta), `tile` lanes per
+// Layout of one row of an FP32 or converted-table row evaluation (no kernel has it any more:
+// labs_rows.cu takes step_smem; its bounds test remains), `tile` lanes per
 // row with lane block R = block_R(n_max, tile) (v0 <= (tile/2 - 1) R):
 //   A rows: the Toeplitz loop reads A_p[0 .. round8(n)) (zero beyond the class), the
 //     assembly A_p[v], A_p[n-1-p-v] and A_p[3v+p-n+1] for every lane output v (down to

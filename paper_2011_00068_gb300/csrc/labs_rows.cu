@@ -1,6 +1,6 @@
 // labs_rows.cu -- the neighbourhood of Algorithm 1 for a batch of skew-symmetric rows
-// (labs_neighbor_delta, L <= LABS_MAX_L) and for a batch of states (labs_features) on the step of labs_step.cuh: two rows per warp up
-// to n = 160 free variables, one above.
+// (labs_neighbor_delta, L <= LABS_MAX_L) and for a batch of states (labs_features), on the
+// step of labs_step.cuh: two rows per warp up to n = 160 free variables, one above.
 //
 // A row is seen once, so everything is built from the row itself:
 //   - a lane takes 16 consecutive bytes, i.e. eight entries of each parity class: as FP16

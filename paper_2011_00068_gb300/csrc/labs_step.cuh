@@ -1,8 +1,8 @@
 // labs_step.cuh -- the walk's step (Algorithm 1, self-avoiding form) for lengths up to
 // LABS_MAX_L under the ISL or the PSL objective: four, two or one walkers per warp (LG =
 // Quad, Pair or Tile<32>), the Toeplitz product on the tensor cores in all three.  The step
-// rule is the one stated at labs_walk in labs.h.  Included by the labs_walk8*.cu,
-// labs_walk16*.cu, labs_walk32.cu and labs_walk32p.cu units.
+// rule is the one stated at labs_walk in labs.h.  Included by the labs_walk*.cu units (but
+// 32l) and, for the layout, the product and the outputs, by labs_rows.cu.
 //
 // The neighbourhood in the form this step evaluates.  With p = i mod 2, v = i / 2, n_p
 // entries in class p, c = n-1, m = c - i and sg = (-1)^m:
