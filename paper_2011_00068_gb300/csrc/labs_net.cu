@@ -636,6 +636,14 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
 // copy one row up and right behind the first, so that columns 8-15 of the operand are the
 // next tap's.  conv1's takes one column (8 channels, 3 in use) per tap from 8 copies of the
 // inputs, each one row further up.
+// CTAs per SM's turn: a weight gradient's accumulator takes the products of a CTA's tiles one
+// after the other, and the tensor core's FP32 additions round toward zero, an error that
+// grows with their number.  304 CTAs add about 110 products each at 4096 samples of n = 128;
+// with 152 the gradients of W2 and W3 were 2e-6 to 3e-6 away (2-norm) from those with 304,
+// with 608 1e-6 the other way.  The second turn costs a training step of 4096 20 us (417
+// from 396): weights loaded and partial sums written twice as often.
+constexpr int kBwdCtas = 2;
+
 template <int MT, bool FIRST>
 struct BwdShape {
     using T = Tile<MT>;
@@ -1047,9 +1055,9 @@ NetWs carve(void* base, int64_t B, int n)
     w.restart = (float*)take((size_t)B * 4);
     w.loss = (float*)take(4);
     w.err = (int*)take(4);
-    w.part1 = (float*)take(sms * 64 * kC * 4);
-    w.part2 = (float*)take(sms * kTaps * kC * kC * 4);
-    w.part3 = (float*)take(sms * kTaps * kC * kC * 4);
+    w.part1 = (float*)take(kBwdCtas * sms * 64 * kC * 4);
+    w.part2 = (float*)take(kBwdCtas * sms * kTaps * kC * kC * 4);
+    w.part3 = (float*)take(kBwdCtas * sms * kTaps * kC * kC * 4);
     w.part4 = (float*)take(sms * 2 * kC * kC * 4);
     w.bytes = off;
     return w;
@@ -1080,7 +1088,7 @@ static int launch_conv_backward(const BwdArgs& a, int sms, cudaStream_t s)
     if (cudaFuncSetAttribute(conv_backward_kernel<MT, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM) !=
         cudaSuccess)
         return LABS_ECUDA;
-    const int grid = (int)std::min<int64_t>(a.tiles, sms);
+    const int grid = (int)std::min<int64_t>(a.tiles, kBwdCtas * sms);
     conv_backward_kernel<MT, FIRST><<<grid, S::THREADS, S::SMEM, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
 }
@@ -1128,8 +1136,8 @@ static int gradients_tiles(FwdArgs a, const NetWs& w, float* grad, int sms, cuda
     b.G = w.dA2, b.IN = w.A1, b.X0 = w.X0, b.wb = w.wpk + pWb2, b.dIN = nullptr, b.part = w.part2, b.part1 = w.part1;
     b.db = grad + oB1;
     if (!rc) rc = launch_conv_backward<MT, true>(b, sms, s);
-    const int ctas = (int)std::min<int64_t>(tiles, sms);
-    const ReduceArgs r{w.part1, w.part2, w.part3, w.part4, ctas, ctas * FwdShape<MT, true>::NG, grad};
+    const int ctas = (int)std::min<int64_t>(tiles, sms), back = (int)std::min<int64_t>(tiles, kBwdCtas * sms);
+    const ReduceArgs r{w.part1, w.part2, w.part3, w.part4, back, ctas * FwdShape<MT, true>::NG, grad};
     wgrad_reduce_kernel<<<2 * kTaps * kC + 128, 256, 0, s>>>(r);
     if (!rc && cudaGetLastError() != cudaSuccess) rc = LABS_ECUDA;
     return rc;

@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(256, row_ctas<LG, R>())
 // dISL_i/(8L).  As the rows, with the pieces of 16 positions from the bits: those above the
 // centre are the mirror's, reversed, with the sign (-1)^(j-c).  Scoring 8192 states of n =
 // 128 takes 172 us with this kernel and took 209 with one warp per state on the FP32 product
-// (40 us of it), a training step of 4096 records 396 from 417.
+// (40 us of it); a training step of 4096 records is 21 us shorter.
 template <class LG, int R, int NW>
 __global__ void __launch_bounds__(256, row_ctas<LG, R>())
     features_kernel(const uint32_t* __restrict__ bits, int64_t stride, int64_t count, int L, float* __restrict__ x)
