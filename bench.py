@@ -43,15 +43,17 @@ def int32_equivalent(lag_terms_per_s, sms, sm_mhz):
             "note": "lag terms per second over the int32 multiply-add rate (%d SMs x %d lanes x %.0f MHz)"
                     % (sms, INT32_MAD_LANES_PER_SM, sm_mhz)}
 # The PSL objective adds, per lag term of every flip, C' = C + cs (a + b) and max |C'|:
-# an add, an FMA and a max beside the Toeplitz FMA, i.e. four FP32 lane operations,
-# against the pipe's 128 lane operations per clock per SM.
+# an add, an FMA and a max beside the Toeplitz FMA, i.e. four lane operations, against the
+# FP32 pipe's 128 lane operations per clock per SM.  (Up to L = 511 the kernel takes only the
+# lags that can decide a neighbour's PSL, as FP16 pairs, so this counts the terms answered,
+# not the operations executed.)
 PSL_LANE_OPS_PER_LAG_TERM = 4
 WALK_KERNELS = {4: "walk_quad_kernel", 2: "walk_pair_kernel", 1: "walk_chunk_kernel"}  # by walkers per warp
 # DRAM bytes per walker step of the L=201 walk kernel (ncu: dram__bytes_read.sum +
 # dram__bytes_write.sum of a 4864-walker x 256-step launch of the current kernel,
-# 373.1 + 33.6 MB over 1,245,184 walker steps, profiles/walk_pair_kernel_L201_16384w.md);
+# 372.1 + 35.5 MB over 1,245,184 walker steps, profiles/step_kernels_small_cases.md);
 # None when not captured for the current kernel
-DRAM_BYTES_PER_WALKER_STEP = 326.7
+DRAM_BYTES_PER_WALKER_STEP = 327.3
 
 
 def parse():
@@ -295,7 +297,7 @@ def delta_kernel_line(args, dev, stream, labs):
     peak = FP32_LANES_PER_SM * 2 * sms * sm_mhz * 1e6
     achieved = ALGO_FLOP_PER_LAG_TERM * (n - 1) * flips
     del out
-    return {"kernel": "delta_kernel", "rows": B, "L": L, "ms_per_launch": ms, "value": flips, "unit": UNIT,
+    return {"kernel": "rows_kernel", "rows": B, "L": L, "ms_per_launch": ms, "value": flips, "unit": UNIT,
             "input_bytes": B * L, "output_bytes": B * n * 4,
             "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": None},
@@ -432,6 +434,8 @@ def run_ours(args):
         peak /= 2
         unit = "Tops/s (FP32 lane operations)"
     kernel = ("walk_psl_pair_kernel" if args.search == "psl" and st["walkers_per_warp"] == 2
+              else "walk_psl_chunk_kernel" if args.search == "psl"
+              else "walk_bestfirst_kernel" if args.search == "bestfirst"
               else WALK_KERNELS[st["walkers_per_warp"]])
     steps_per_launch = args.walkers * args.walk_steps / nchunks
     roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": unit,
@@ -446,8 +450,8 @@ def run_ours(args):
                 "peak_source": "derived: %d SMs x %d FP32 lanes x %s x %.0f MHz (FMA pipe)" % (
                     sms, FP32_LANES_PER_SM, "1 op" if args.search == "psl" else "2 FLOP", sm_mhz),
                 "toeplitz": ("tensor cores: mma.sync.m16n8k16, FP16 operands (exact small integers), FP32 "
-                             "accumulation; the step around it is issue- and latency-bound on the FP32, integer "
-                             "and load/store pipes, so lag terms are counted against the FP32 FMA peak"
+                             "accumulation; the step is bound by the shared-memory pipe and by issue, so lag "
+                             "terms are counted against the FP32 FMA peak"
                              if st.get("tensor_cores") else "FP32 FMA pipe"),
                 "tensor_frac": (ops_per_launch / avg_launch_s / tensor_peak() if args.search != "psl" else None)}
 
