@@ -28,7 +28,7 @@
 // warps per SM.  The step it replaces (FP32 rows and pair table, P per output, table
 // operands converted on load, 128 registers and 16 warps per SM) issued 1017.  16384
 // walkers x 10^4 steps at L = 201: 63.9 ms from 120.7; 16384 x 2000 at L = 501: 35.2 from
-// 58.0; 52 lengths 201..303 x 512 walkers x 2000: 30.2 from 63.5.
+// 58.0; 52 lengths 201..303 x 512 walkers x 2000: 29.9 from 63.4.
 #pragma once
 
 #include "labs_device.cuh"
@@ -1091,7 +1091,9 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
 // reached by that many flips, any other by a rebuild from its bits.
 //
 // What bounds it: the queue's insertions and the move, not the neighbourhood (about 3
-// insertions a step, each a minimum over the warp and an HT lookup).
+// insertions a step, each a minimum over the warp and an HT lookup).  16384 walkers x 1000
+// steps at L = 201: 35.9 ms, 51.6 on FP32 rows and table at 16 warps per SM (38.7 before the
+// entries' fingerprints were kept and the candidates' HT lines prefetched).
 template <class LAY, int R>
 __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w, int len, bool real, int wb,
                                               unsigned extras, const Tile<32>& t)
