@@ -324,7 +324,8 @@ int labs_enumerate_noalloc(int32_t L, int64_t *min_isl, uint64_t *count,
  * W3[64][64][7] b3 W4[64][64] b4 w5[64] b5 w6[64] b6 (labs_net_sizes gives the count);
  * products use bfloat16 copies with float32 accumulation on the tensor cores.
  * Loss per sample: wf * CE(softmax(score), target) + 0.5 (restart - y)^2, batch mean.
- * All pointers are device memory; calls are asynchronous on cuda_stream. */
+ * All pointers are device memory; the workspace starts on a 16-byte boundary (LABS_EINVAL
+ * otherwise); calls are asynchronous on cuda_stream. */
 int labs_net_sizes(int32_t n, int64_t batch, size_t *param_count, size_t *workspace_bytes);
 int labs_net_init(float *dev_params, uint64_t seed, void *cuda_stream);
 int labs_net_forward(const float *dev_params, const float *dev_x, int64_t batch, int32_t n,
@@ -374,7 +375,8 @@ int labs_features(int32_t L, const uint32_t *dev_bits, int64_t stride_words, int
  *     block, c) for candidate c); the one with the highest restart score (ties: lowest
  *     index) is used at the walker's next restart.
  * The exact ISL decides every move; the network only orders candidates.
- * dev_ws: labs_learned_workspace_bytes bytes.  Chunks run without a CUDA graph. */
+ * dev_ws: labs_learned_workspace_bytes bytes, on a 16-byte boundary (LABS_EINVAL
+ * otherwise).  Chunks run without a CUDA graph. */
 int labs_learned_workspace_bytes(const labs_ctx *ctx, int32_t candidates, size_t *bytes);
 int labs_learned(labs_ctx *ctx, const float *dev_params, int32_t tau, int32_t candidates,
                  void *dev_ws, size_t ws_bytes);

@@ -984,6 +984,8 @@ int labs_learned(labs_ctx* c, const float* dev_params, int32_t tau, int32_t cand
         if (tau < 0 || candidates < 1 || candidates > 64) return fail(c, LABS_EINVAL, "bad tau / candidates");
         if (!dev_ws || ws_bytes < learned_ws_bytes(c, candidates))
             return fail(c, LABS_ENOMEM, "learned workspace needs %zu bytes", learned_ws_bytes(c, candidates));
+        // the network's part begins a multiple of 256 bytes into it (bulk copies: 16-byte boundaries)
+        if (((uintptr_t)dev_ws & 15) != 0) return fail(c, LABS_EINVAL, "learned workspace must be 16-byte aligned");
     }
     cudaSetDevice(c->device);
     c->l_params = dev_params;

@@ -1026,6 +1026,12 @@ static size_t align256(size_t x)
     return (x + 255) & ~(size_t)255;
 }
 
+// The kernels' bulk copies and 16-byte stores start on 16-byte boundaries of the workspace.
+static bool aligned_ws(const void* ws)
+{
+    return ((uintptr_t)ws & 15) == 0;
+}
+
 static int sm_count()
 {
     int dev = 0, sms = 0;
@@ -1226,6 +1232,7 @@ int labs_net_forward(const float* dev_params, const float* dev_x, int64_t batch,
     if (batch == 0) return LABS_OK;
     const net::NetWs w = net::carve(dev_ws, batch, n);
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
+    if (!net::aligned_ws(dev_ws)) return LABS_EINVAL;
     return net::forward(dev_params, dev_x, w, batch, n, dev_scores ? dev_scores : w.score,
                         dev_restart ? dev_restart : w.restart, (cudaStream_t)cuda_stream);
 }
@@ -1240,6 +1247,7 @@ int labs_net_gradients(const float* dev_params, const float* dev_x, const int32_
         return LABS_EINVAL;
     const net::NetWs w = net::carve(dev_ws, batch, n);
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
+    if (!net::aligned_ws(dev_ws)) return LABS_EINVAL;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     int rc = net::gradients(dev_params, dev_x, w, dev_target, dev_y, dev_wf, dev_grads, batch, n, s);
     if (!rc && dev_loss) rc = cudaMemcpyAsync(dev_loss, w.loss, 4, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
