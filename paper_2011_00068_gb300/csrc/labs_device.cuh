@@ -377,6 +377,7 @@ __device__ __forceinline__ int build_table(const View& V, int n, const TL& t)
                 const int len0 = n - m, len1 = len0 - 1;
                 const int d = len0 - 2 * c0[g] + (len1 > 0 ? len1 - 2 * c1[g] : 0);
                 set_E(V, m, (float)d);
+                if constexpr (TL::kSize > 32) note_wide(V, (float)d);
                 part += d * d;
             }
         }
@@ -1371,13 +1372,25 @@ __device__ __forceinline__ int psl_key_i(uint64_t k) { return (int)(k & 0x1FFFu)
 __device__ __forceinline__ int psl_key_isl(uint64_t k) { return (int)((k >> 13) & 0x3FFFFFFFull); }
 __device__ __forceinline__ int psl_key_psl(uint64_t k) { return (int)(k >> 43); }
 
+// A pointer into shared memory that the compiler keeps in a register: without this the loops
+// below computed theirs anew from the layout (a select of the class, the base of shared memory)
+// in every iteration, 36 times a step at L = 513.
+template <class T>
+__device__ __forceinline__ const T* held_shared(const T* p)
+{
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("" : "+r"(a));
+    return static_cast<const T*>(__cvta_shared_to_generic(a));
+}
+
 // The same PSL values for the lane block R = 7 in one pass: s_{i-2m} and s_{i+2m} of the
 // R outputs in two windows of R values that slide one class entry per lag (three shared
 // loads per lag), and the mirror's term dropped by a compare and select per lag term.
 template <class TL, int R>
 __device__ __forceinline__ void psl_eval_select(const View& V, int n, const Outs<TL, R>& o, int (&pl)[R])
 {
-    const float* A = (o.p ? V.A1 : V.A0) + o.v0;
+    const float* A = held_shared((o.p ? V.A1 : V.A0) + o.v0);
+    const float2* G = held_shared(V.G);
     const int c = n - 1;
     float cs[R], mx[R], lo[R], hi[R];
     int q0[R];
@@ -1401,7 +1414,7 @@ __device__ __forceinline__ void psl_eval_select(const View& V, int n, const Outs
             lo[j] = A[-m];
             hi[(j + R - 1) % R] = A[m + R - 1];
             if (m == 0) continue;
-            const float C = V.G[m].x;
+            const float C = G[m].x;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const float a = lo[(j - r + R) % R];
@@ -1429,12 +1442,17 @@ __device__ __forceinline__ void psl_eval_select(const View& V, int n, const Outs
 // loop unrolled by P so that the ring indices are constants).  Lags outside 1..n-1 (the
 // first 2 RC - 2 and the last iterations) are masked in the blocks that hold them.
 // Exact in fp32: every value is an integer of magnitude below 2^10.
+// Compiled by itself (not inlined): its registers are then the same whatever surrounds it.
+// Inlined beside the tensor-core product its ring lost register banks (dispatch stalls 0.44 an
+// issue from 0.32).  608 walkers x 128 steps of the long PSL walk, inlined / like this: L = 513
+// 4.10 / 3.61 ms, 1025 7.17 / 6.22, 2047 20.8 / 16.3, 4095 60.7 / 55.2, 11263 437 / 410.
 template <class TL, int R, int C0, int RC>
-__device__ __forceinline__ void psl_ring(const View& V, int n, const Outs<TL, R>& o, int (&pl)[R])
+__device__ __noinline__ void psl_ring(const View& V, int n, const Outs<TL, R>& o, int (&pl)[R])
 {
     constexpr int P = 3 * RC - 2;
     const int w0 = o.v0 + C0;
-    const float* A = (o.p ? V.A1 : V.A0) + w0;
+    const float* A = held_shared((o.p ? V.A1 : V.A0) + w0);
+    const float2* G = held_shared(V.G);
     const int c = n - 1;
     const int tstar = c - o.p - 2 * w0;
     const int tend = n - 1 + 2 * (RC - 1);
@@ -1449,7 +1467,7 @@ __device__ __forceinline__ void psl_ring(const View& V, int n, const Outs<TL, R>
 #pragma unroll
     for (int k = 1; k < P; ++k) {
         ra[k] = A[P - k];
-        rc[k] = V.G[k - P].x;
+        rc[k] = G[k - P].x;
         rb[k] = A[k - P];
     }
     for (int t0 = 0; t0 <= tend; t0 += P) {
@@ -1458,7 +1476,7 @@ __device__ __forceinline__ void psl_ring(const View& V, int n, const Outs<TL, R>
             for (int j = 0; j < P; ++j) {
                 const int t = t0 + j;
                 ra[j] = A[-t];
-                rc[j] = V.G[t].x;
+                rc[j] = G[t].x;
                 rb[j] = A[t];
                 const float z = t == tstar ? 0.f : 1.f;
 #pragma unroll
@@ -1474,7 +1492,7 @@ __device__ __forceinline__ void psl_ring(const View& V, int n, const Outs<TL, R>
                 const int t = t0 + j;
                 if (t > tend) break;
                 ra[j] = A[-t];
-                rc[j] = V.G[t].x;
+                rc[j] = G[t].x;
                 rb[j] = A[t];
                 const float z = t == tstar ? 0.f : 1.f;
 #pragma unroll

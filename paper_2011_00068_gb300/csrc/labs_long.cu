@@ -119,16 +119,6 @@ __device__ __forceinline__ void long_clear(int* base, const WarpSmem& SL, const 
     t.sync();
 }
 
-// The table after the rows: returns the ISL, marks a table that FP16 does not hold.
-template <class LB>
-__device__ __forceinline__ int long_build_table(const View& V, int n, const LB& t)
-{
-    const int isl = build_table(V, n, t);  // ends with barriers
-    for (int m = 1 + t.lane; m < n; m += LB::kSize) note_wide(V, V.G[m].x);
-    t.sync();
-    return isl;
-}
-
 // Rows from the shared bits (Eq. 4: s_j = x_j for j <= c, s_{c+t} = (-1)^t x_{c-t}),
 // then the table; returns the ISL.
 template <class LB>
@@ -145,7 +135,7 @@ __device__ int long_load_rows(const LongWalk& lw, const WarpSmem& SL, int* base,
         set_row(V, j & 1, j >> 1, (float)s);
     }
     t.sync();
-    return long_build_table(V, n, t);
+    return build_table(V, n, t);
 }
 
 // HT fingerprint of the shared bits (long_load_rows ran first).
@@ -1047,7 +1037,7 @@ __global__ void __launch_bounds__(NT, kLongThreads / NT) long_delta_kernel(const
             t.sync();
             continue;
         }
-        const int isl = long_build_table(V, n, t);
+        const int isl = build_table(V, n, t);
         if (isl > long_isl_limit(L, n)) {
             for (int i = t.lane; i < n; i += LB::kSize) dst[i] = INT32_MIN;
             if (t.lane == 0 && status) raise_error(status, LABS_ERANGE, (int)row);
