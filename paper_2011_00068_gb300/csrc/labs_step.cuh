@@ -419,6 +419,19 @@ struct StepEnv {
     __device__ __forceinline__ WalkerState* state() const { return p->states + g; }
 };
 
+// The step loops count from the warp's phase, its first walker's step count modulo kCheckEvery,
+// so that stop requests are asked for at the same steps whatever the chunks.  (The question
+// waits for host memory: asked at every chunk's start, it took a third of a one-step chunk's
+// time, 16384 walkers of L = 201 173 us a chunk from 118.  The phase is read again where it is
+// needed, which is rare: held, it cost a register and 1.4% of the walk at L = 201.)
+template <class LG>
+__device__ __forceinline__ int step_phase(const StepEnv& env, const LG& t)
+{
+    uint32_t h = 0;  // (a group past the last walker stands on one that exists: any valid state)
+    if constexpr (LG::kSize < 32) h = min((uint32_t)t.h, env.g);
+    return (int)env.p->states[env.g - h].steps_done & (kCheckEvery - 1);
+}
+
 // The lags of a lane: E and Z at lags 4 (lane + NL b) .. +3 as FP16 pairs.
 template <int NB>
 struct StepLags {
@@ -893,8 +906,9 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
             zkr[r] = i <= c ? __ldg(env.zk + i) : 0ull;
         }
     }
+    int it = __shfl_sync(kFull, step_phase(env, t), 0);
+    len += it;
     const int top = __reduce_max_sync(kFull, real ? len : 0);
-    int it = 0;
     for (; it < top; ++it) {
         const bool act = real && it < len;
         if ((it & (kCheckEvery - 1)) == 0) {
@@ -1047,7 +1061,7 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
         }
         if (moves && (step_better<PSL>(w.psl, w.isl, w.best_psl, w.best) || w.isl <= w.tisl)) {
             WalkerState* st = env.state();
-            const int64_t steps = st->steps_done + it + 1;
+            const int64_t steps = st->steps_done + (it - step_phase(env, t)) + 1;
             if (step_better<PSL>(w.psl, w.isl, w.best_psl, w.best)) {
                 w.best = w.isl;
                 w.best_psl = w.psl;
@@ -1067,16 +1081,16 @@ __device__ __forceinline__ int walk_lockstep(const StepEnv& env, StepWalker& w, 
                 else if (!stored)
                     st->overflows += 1;
             }
-            step_restart<LAY>(env, w, wb, st->steps_done + it + 1, tt);
+            step_restart<LAY>(env, w, wb, st->steps_done + (it - step_phase(env, t)) + 1, tt);
             step_load_lags<LAY, LG, R>(wb, lane, lg);
         }
         __syncwarp();
         if (extras && act && lane == 0) {
             const int code = !moves ? LABS_TRACE_BLOCKED : again ? bi | LABS_TRACE_RESTART : bi;
-            if (!step_note(env, it, code, w.isl, extras)) extras &= ~2u;
+            if (!step_note(env, it - step_phase(env, t), code, w.isl, extras)) extras &= ~2u;
         }
     }
-    return min(it, len);
+    return min(it, len) - __shfl_sync(kFull, step_phase(env, t), 0);
 }
 
 // ------------------------------------------------------------------ best-first search
@@ -1120,13 +1134,13 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
     uint64_t* const T2 = p.tabu2 != nullptr ? p.tabu2 + (env.T - p.tabu) : nullptr;
     constexpr uint64_t kLow40 = 0xFFFFFFFFFFull;
     int64_t hits = 0;
-    const int64_t steps0 = env.state()->steps_done;
+    int it = step_phase(env, t);
+    const int64_t steps0 = env.state()->steps_done - it;  // before step it = 0
     StepLags<StepShape<LG, R>::NB> lg;
     step_load_lags<LAY, LG, R>(wb, lane, lg);
     StopCheck stop;
     stop.start(p, lane == 0);
-    if (!real) len = 0;
-    int it = 0;
+    len = real ? len + it : 0;
     for (; it < len; ++it) {
         if ((it & (kCheckEvery - 1)) == 0) {
             const int why = t.shfl(stop.poll(p, lane == 0), 0);
@@ -1322,13 +1336,13 @@ __device__ __forceinline__ int walk_bestfirst(const StepEnv& env, StepWalker& w,
             step_load_lags<LAY, LG, R>(wb, lane, lg);
         }
         t.sync();
-        if (extras && lane == 0) step_note(env, it, code, w.isl, extras & 1u);
+        if (extras && lane == 0) step_note(env, it - step_phase(env, t), code, w.isl, extras & 1u);
     }
     if (real) {
         qkey[lane] = qk;
         if (lane == 0) env.state()->cache_hits += hits;
     }
-    return it;
+    return it - step_phase(env, t);
 }
 
 // CTAs of 8 warps per SM the walk kernels are compiled for: three (80 registers a thread),
