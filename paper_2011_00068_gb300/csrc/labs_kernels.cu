@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "labs_device.cuh"
+#include "labs_launch.h"
 
 namespace labsgpu {
 
@@ -420,7 +421,7 @@ int launch_zobrist(const KParams&, uint64_t* zkeys, const DevGroup* host_groups,
 int launch_reset(const KParams& p, int grid, int block, void* stream)
 {
     const size_t smem = (size_t)(block / kWarp) * warp_smem(p.n_max, 32).words * sizeof(int);
-    cudaFuncSetAttribute(reset_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (allow_shared((const void*)reset_kernel) != cudaSuccess) return LABS_ECUDA;
     reset_kernel<<<grid, block, smem, (cudaStream_t)stream>>>(p);
     return status_of(cudaGetLastError());
 }
@@ -463,7 +464,6 @@ int walk_kernel_config(int n_max, int tile, int mode, int warps_per_cta, int* ct
 {
     const WalkFn fn = walk_fn(tile, walk_R(n_max, tile, mode), mode);
     const size_t smem_bytes = walk_warp_bytes(n_max, tile, mode) * (size_t)warps_per_cta;
-    // the limit is the device's, not this context's need: contexts share the kernels
     int dev = 0, most = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -471,10 +471,7 @@ int walk_kernel_config(int n_max, int tile, int mode, int warps_per_cta, int* ct
     *ctas_per_sm = 0;
     if (smem_bytes > (size_t)most) return LABS_EINVAL;
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, fn);
-    if (e != cudaSuccess) return LABS_ECUDA;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
-    if (e != cudaSuccess) return LABS_ECUDA;
+    if (allow_shared((const void*)fn, &fa) != cudaSuccess) return LABS_ECUDA;
     if (regs) *regs = fa.numRegs;
     if (warps_per_cta * kWarp > fa.maxThreadsPerBlock) return LABS_EINVAL;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, warps_per_cta * kWarp, smem_bytes);

@@ -1,0 +1,25 @@
+// labs_launch.h -- host side of launches whose shared memory is above the default 48 KB.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace labsgpu {
+
+// A kernel's limit of dynamic shared memory belongs to the process (per device): several
+// contexts, lengths and host threads share a kernel and ask for different sizes.  So the limit
+// is always set to what the device allows, never to one launch's need, which another thread's
+// smaller one could replace between that call and the launch.
+inline cudaError_t allow_shared(const void* fn, cudaFuncAttributes* attributes = nullptr)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    if (attributes != nullptr) *attributes = fa;
+    return e;
+}
+
+}  // namespace labsgpu

@@ -6,6 +6,7 @@
 // The per-lane arithmetic is the warp kernels' (labs_device.cuh), run by a lane group
 // that spans the CTA; the collectives go through shared memory.
 #include "labs_device.cuh"
+#include "labs_launch.h"
 
 namespace labsgpu {
 
@@ -1141,16 +1142,11 @@ ResetFn long_reset_fn(int n_max, bool psl)
 int long_kernel_config(int n_max, int mode, size_t smem_bytes, int* ctas_per_sm, int* regs)
 {
     const LongFn fn = long_fn(n_max, mode);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) return LABS_ECUDA;
-    e = cudaFuncSetAttribute(long_reset_fn(n_max, mode == 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes);
-    if (e != cudaSuccess) return LABS_ECUDA;
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, fn);
-    if (e != cudaSuccess) return LABS_ECUDA;
+    if (allow_shared((const void*)fn, &fa) != cudaSuccess) return LABS_ECUDA;
+    if (allow_shared((const void*)long_reset_fn(n_max, mode == 1)) != cudaSuccess) return LABS_ECUDA;
     if (regs) *regs = fa.numRegs;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, long_threads(n_max, mode == 1), smem_bytes);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, long_threads(n_max, mode == 1), smem_bytes);
     return e == cudaSuccess ? LABS_OK : LABS_ECUDA;
 }
 
@@ -1179,8 +1175,7 @@ int launch_long_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out
     const int n = (L + 1) / 2;
     const size_t smem = (size_t)long_smem(n, long_threads(n)).words * sizeof(int);
     const LongDeltaFn fn = long_delta_fn(n);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return LABS_ECUDA;
+    if (allow_shared((const void*)fn) != cudaSuccess) return LABS_ECUDA;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

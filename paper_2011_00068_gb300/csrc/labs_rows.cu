@@ -27,6 +27,7 @@
 // lanes held them) 1277.  2^20 rows of L = 201: 524 us from 810; 2^18 rows: L = 255 148 us,
 // L = 303 231, L = 511 352.
 #include "labs_async.cuh"
+#include "labs_launch.h"
 #include "labs_step.cuh"
 
 #include <algorithm>
@@ -532,7 +533,7 @@ int launch_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, Dev
     const RowsFn fn = staged ? rows_fn<true>(key) : rows_fn<false>(key);
     if (fn == nullptr) return LABS_EINVAL;
     const size_t smem = warps * (warp_bytes + (staged ? stage : 0));
-    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024 && allow_shared((const void*)fn) != cudaSuccess) return LABS_ECUDA;
     // more CTAs than fit at once (up to 8 per SM): measured faster than one resident wave
     const int64_t need = (units + warps - 1) / warps, most = (int64_t)sms * 8;
     fn<<<(int)std::min(need, most), warps * kWarp, smem, (cudaStream_t)stream>>>(seqs, batch, L, out, status);
@@ -551,7 +552,7 @@ int launch_features(const uint32_t* bits, int64_t stride, int64_t count, int32_t
     const int64_t units = (count + rows - 1) / rows;
     const int warps = row_warps(units, sms);
     const size_t smem = (size_t)warps * rows * step_smem(tile, R).words * sizeof(int);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024 && allow_shared((const void*)fn) != cudaSuccess) return LABS_ECUDA;
     const int64_t need = (units + warps - 1) / warps, most = (int64_t)sms * 8;
     fn<<<(int)std::min(need, most), warps * kWarp, smem, (cudaStream_t)stream>>>(bits, stride, count, L, x);
     return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
