@@ -218,7 +218,11 @@ struct FwdShape {
     static constexpr int SCB = (2 * T::M + T::M / 4 + 32) * 4;
     static constexpr int SUMS = SC + (TRAIN ? NG * SCB : 0);
     static constexpr int SMEM = SUMS + (TRAIN ? 4 * kC * 4 : 0) + 128;  // + alignment slack
-    static constexpr int TMEM_USED = NG * MT * 64 + (TRAIN ? NG * 64 : 0);
+    // Accumulators of dW4 per group, taken in turn by its tiles: two per SM either way.  A chain
+    // of products loses what the tensor core's additions round toward zero, so it is kept as
+    // short as two CTAs per SM had it (one accumulator above n = 128 made it twice as long).
+    static constexpr int ACC4 = 2 / NG > 1 ? 2 / NG : 1;
+    static constexpr int TMEM_USED = NG * MT * 64 + (TRAIN ? NG * ACC4 * 64 : 0);
     static constexpr int TMEM = TMEM_USED <= 128 ? 128 : 256;
 };
 
@@ -236,7 +240,7 @@ struct FwdArgs {
     const float* y;
     const float* wf;
     bf16 *X0, *A1, *A2, *dA3;  // tiles in global memory
-    float* part4;              // [CTA x group][64 channels][64 outputs] partial dW4
+    float* part4;              // [accumulator x CTA x group][64 channels][64 outputs] partial dW4
     float* grad;
     float* loss;
 };
@@ -311,7 +315,7 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + S::BAR + 48);
-    const uint32_t acc0 = tmem + grp * MT * 64, acc4 = tmem + S::NG * MT * 64 + grp * 64;
+    const uint32_t acc0 = tmem + grp * MT * 64, acc4 = tmem + S::NG * MT * 64 + grp * S::ACC4 * 64;
     // the group's first warp issues its products, from uniform values
     const bool issuer = uniform(wq) == 0;
     const uint32_t u_sb = uniform(sb), u_gx = uniform(gx), u_ga = uniform(ga), u_bar = uniform(bar), u_acc0 = uniform(acc0),
@@ -548,7 +552,7 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
                 for (int mt = 0; mt < MT; ++mt)
                     issue_product<kC, 1, T::COL>(el, u_acc0 + 64 * mt, u_gd + 48 + 2048 * mt, u_sb + S::WB4);
                 // dW4: its rows 64-127 (the columns after a3's, i.e. dh's) are dropped
-                issue_wgrad<T::M, T::COL>(el, u_acc4, u_ga + 48, u_gd + 48, done == 0);
+                issue_wgrad<T::M, T::COL>(el, u_acc4 + 64 * (done % S::ACC4), u_ga + 48, u_gd + 48, done < S::ACC4);
                 tc_commit(el, u_bar);
             }
             wait_products();
@@ -597,14 +601,19 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
             atomicAdd(a.loss, lsum);
         }
         // this group's partial dW4 (channel x output)
-        float4* dst = reinterpret_cast<float4*>(a.part4 + ((int64_t)blockIdx.x * S::NG + grp) * kC * kC) + t * (kC / 4);
-        float acc[64];
-        if (done > 0) load_acc(acc4, wq, acc);  // a warp-wide load: done is the same for the group
+        for (int q = 0; q < S::ACC4; ++q) {
+            if (q > 0 && tiles <= gridDim.x * S::NG) break;  // no tile took it
+            const int64_t slot4 = ((int64_t)q * gridDim.x + blockIdx.x) * S::NG + grp;
+            float4* dst = reinterpret_cast<float4*>(a.part4 + slot4 * kC * kC) + t * (kC / 4);
+            const bool used = done > q;  // the same for the group: the load is warp-wide
+            float acc[64];
+            if (used) load_acc(acc4 + 64 * q, wq, acc);
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-            if (t < kC)
-                dst[i] = done > 0 ? make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3])
+            for (int i = 0; i < 16; ++i)
+                if (t < kC)
+                    dst[i] = used ? make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3])
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -1142,8 +1151,10 @@ static int gradients_tiles(FwdArgs a, const NetWs& w, float* grad, int sms, cuda
     b.G = w.dA2, b.IN = w.A1, b.X0 = w.X0, b.wb = w.wpk + pWb2, b.dIN = nullptr, b.part = w.part2, b.part1 = w.part1;
     b.db = grad + oB1;
     if (!rc) rc = launch_conv_backward<MT, true>(b, sms, s);
+    constexpr int NG = FwdShape<MT, true>::NG, ACC4 = FwdShape<MT, true>::ACC4;
     const int ctas = (int)std::min<int64_t>(tiles, sms), back = (int)std::min<int64_t>(tiles, kBwdCtas * sms);
-    const ReduceArgs r{w.part1, w.part2, w.part3, w.part4, back, ctas * FwdShape<MT, true>::NG, grad};
+    const ReduceArgs r{w.part1, w.part2, w.part3, w.part4, back, ctas * NG * (tiles > ctas * NG ? ACC4 : 1),
+                       grad};
     wgrad_reduce_kernel<<<2 * kTaps * kC + 128, 256, 0, s>>>(r);
     if (!rc && cudaGetLastError() != cudaSuccess) rc = LABS_ECUDA;
     return rc;
