@@ -325,7 +325,9 @@ int labs_enumerate_noalloc(int32_t L, int64_t *min_isl, uint64_t *count,
  * products use bfloat16 copies with float32 accumulation on the tensor cores.
  * Loss per sample: wf * CE(softmax(score), target) + 0.5 (restart - y)^2, batch mean.
  * All pointers are device memory; the workspace starts on a 16-byte boundary (LABS_EINVAL
- * otherwise); calls are asynchronous on cuda_stream. */
+ * otherwise); calls are asynchronous on cuda_stream.  Every wait inside the kernels is
+ * bounded; a pass in which one gives up (a copy or product that never completed) returns
+ * NaN: the scores it could not compute, or the loss and every gradient. */
 int labs_net_sizes(int32_t n, int64_t batch, size_t *param_count, size_t *workspace_bytes);
 int labs_net_init(float *dev_params, uint64_t seed, void *cuda_stream);
 int labs_net_forward(const float *dev_params, const float *dev_x, int64_t batch, int32_t n,

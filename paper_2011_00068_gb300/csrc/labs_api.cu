@@ -470,6 +470,7 @@ int proposal_pass(labs_ctx* c)
     void* nws = c->l_ws + (learned_ws_bytes(c, P) - net_workspace_bytes(kProposalBatch, c->n_max));
     const int64_t S = std::max<int64_t>(1, kProposalBatch / P);
     const WalkerState* states = at<WalkerState>(c, c->off_states);
+    DevStatus* const status = at<DevStatus>(c, c->off_status);
     for (int g = 0; g < c->nG; ++g) {
         const DevGroup& G = c->groups[g];
         for (int64_t s0 = G.first; s0 < G.first + G.count; s0 += S) {
@@ -479,12 +480,12 @@ int proposal_pass(labs_ctx* c)
             if (!(c->cfg.flags & LABS_FLAG_LEARNED_RESTARTS)) {  // flip scores: the full learned mode
                 rc = launch_features(reinterpret_cast<const uint32_t*>(states + s0), sizeof(WalkerState) / 4, cnt,
                                      G.L, x, c->stream);
-                if (!rc) rc = net_forward_ws(c->l_params, x, cnt, G.n, nws, &sc, &rs, c->stream);
+                if (!rc) rc = net_forward_ws(c->l_params, x, cnt, G.n, nws, &sc, &rs, status, c->stream);
                 if (!rc) rc = launch_scores(p, s0, cnt, G.n, sc, c->stream);
             }
             if (!rc) rc = launch_candidates(p, s0, cnt, G.n, P, cand, c->stream);
             if (!rc) rc = launch_features(cand, kBitWords, cnt * P, G.L, x, c->stream);
-            if (!rc) rc = net_forward_ws(c->l_params, x, cnt * P, G.n, nws, &sc, &rs, c->stream);
+            if (!rc) rc = net_forward_ws(c->l_params, x, cnt * P, G.n, nws, &sc, &rs, status, c->stream);
             if (!rc) rc = launch_select(p, s0, cnt, P, rs, cand, c->stream);
             if (rc) return fail(c, rc, "proposal pass: %s", cudaGetErrorString(cudaGetLastError()));
         }

@@ -68,10 +68,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 }
 
 // Waits until the phase with the given parity of bar has completed; false when it did
-// not within kWaitTries attempts.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+// not within `tries` attempts.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int tries = kWaitTries)
 {
-    for (int i = 0; i < kWaitTries; ++i)
+    for (int i = 0; i < tries; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }

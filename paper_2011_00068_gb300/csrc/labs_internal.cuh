@@ -646,10 +646,10 @@ int launch_labels(const labs_log_record* rec, int64_t count, int32_t* target, fl
 
 // Learned network (labs_net.cu): forward of a batch of float inputs [B][3][n] into the
 // caller's workspace; scores [B][n] and restart [B] are returned as device pointers
-// inside that workspace.
+// inside that workspace.  A device wait that gives up raises LABS_ECUDA in *status (nullable).
 size_t net_workspace_bytes(int64_t B, int n);
 int net_forward_ws(const float* params, const float* x, int64_t B, int n, void* ws, const float** scores,
-                   const float** restart, void* stream);
+                   const float** restart, DevStatus* status, void* stream);
 
 // Partial / final result of the exhaustive skew search (labs_enum.cu).
 struct EnumPart {

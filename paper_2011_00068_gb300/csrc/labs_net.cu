@@ -52,6 +52,25 @@ namespace {
 
 constexpr int kTcThreads = 128;  // threads of a tile group: one TMEM lane (output row) each
 
+// Attempts of the kernels' waits, by what is waited for (a test builds this file with none).
+// A wait that gives up is repeated once, with kWaitTries attempts, so that nothing is left under
+// way where that can be helped; then it marks a word of its tile group's that the group's
+// threads read only between two of their barriers which no such mark can come between, so that
+// they leave together; and it sets the pass's error word.  (A reduction in the group's barriers
+// instead of the mark took 1 to 2% of a pass, a test around the epilogue after a wait up to 25%
+// in spilled registers: until the group leaves, its epilogues run on whatever there is.)
+#ifndef LABS_NET_TRIES_WEIGHTS
+#define LABS_NET_TRIES_WEIGHTS kWaitTries
+#endif
+#ifndef LABS_NET_TRIES_TILES
+#define LABS_NET_TRIES_TILES kWaitTries
+#endif
+#ifndef LABS_NET_TRIES_PRODUCTS
+#define LABS_NET_TRIES_PRODUCTS kWaitTries
+#endif
+constexpr int kTriesWeights = LABS_NET_TRIES_WEIGHTS, kTriesTiles = LABS_NET_TRIES_TILES,
+              kTriesProducts = LABS_NET_TRIES_PRODUCTS;
+
 // A tile of MT x 128 output rows.
 template <int MT>
 struct Tile {
@@ -226,6 +245,14 @@ struct FwdShape {
     static constexpr int TMEM = TMEM_USED <= 128 ? 128 : 256;
 };
 
+// A wait gave up: the pass's error word (its gradients become NaN) and, in a walk, the
+// context's status.
+__device__ __forceinline__ void net_failed(int* err, DevStatus* status)
+{
+    atomicExch(err, 1);
+    if (status != nullptr) atomicCAS(&status->error, 0, LABS_ECUDA);
+}
+
 struct FwdArgs {
     const float* x;
     const bf16* wpk;
@@ -233,6 +260,7 @@ struct FwdArgs {
     float* score;
     float* restart;
     int* err;
+    DevStatus* status;  // of the walk's context, or null
     int64_t B;
     int n;
     // training
@@ -282,7 +310,7 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
     float* bias = reinterpret_cast<float*>(sm + S::BIAS);
     const uint32_t s_bias = sb + S::BIAS;
     const uint32_t bar_w = sb + S::BAR, bar = bar_w + 8 + 8 * grp, slot = sb + S::BAR + 48;
-    volatile int* failed = reinterpret_cast<volatile int*>(sm + S::BAR + 56);
+    volatile int* failed = reinterpret_cast<volatile int*>(sm + S::BAR + 32) + grp;  // the group's mark
     const uint32_t gx = sb + S::GROUPS + grp * S::GROUP + S::X0, ga = sb + S::GROUPS + grp * S::GROUP + S::ACT,
                    gd = sb + S::GROUPS + grp * S::GROUP + S::DH;
     float* s_score = reinterpret_cast<float*>(sm + S::SC + grp * S::SCB);
@@ -305,8 +333,8 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
     for (int i = threadIdx.x; i < S::NG * S::GROUP / 16; i += S::THREADS)
         sts128(sb + S::GROUPS + 16 * i, make_uint4(0u, 0u, 0u, 0u));
     if (threadIdx.x < 32) tmem_alloc(slot, S::TMEM);
+    if (t == 0) *failed = 0;
     if (threadIdx.x == 0) {
-        *failed = 0;
         mbar_init(bar_w, 1);
         for (int g = 0; g < S::NG; ++g) mbar_init(bar_w + 8 + 8 * g, 1);
         mbar_init_fence();
@@ -328,7 +356,7 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
         bulk_copy_g2s(sb + S::W4, a.wpk + pWf4, kC * 128, bar_w);
         if (TRAIN) bulk_copy_g2s(sb + S::WB4, a.wpk + pWb4, kC * 128, bar_w);
     }
-    bool ok = mbar_wait(bar_w, 0);
+    bool ok = !__syncthreads_or(!mbar_wait(bar_w, 0, kTriesWeights));
     uint32_t phase = 0;
     int done = 0;           // tiles of this group
     float2 gw6 = {0.f, 0.f};  // this warp's samples: the gradients of w6's channels 2 lane and 2 lane + 1
@@ -354,9 +382,12 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
             for (int f = 0; f < 3; ++f) xin[mt][f] = in ? a.x[(b * 3 + f) * n + rpos[mt]] : 0.f;
         }
     };
-    // waits for the group's products; a wait that gives up ends the CTA's work
+    // waits for the group's products; a wait that gives up ends the group's work with this tile
     auto wait_products = [&]() {
-        if (!mbar_wait(bar, phase)) *failed = 1;
+        if (!mbar_wait(bar, phase, kTriesProducts)) {
+            mbar_wait(bar, phase);
+            *failed = 1;
+        }
         phase ^= 1;
         tc_fence_after();
     };
@@ -588,9 +619,25 @@ __global__ void __launch_bounds__(FwdShape<MT, TRAIN>::THREADS, 1) net_forward_k
         tc_fence_before();
         group_sync(1 + grp);
         tc_fence_after();
+        // the same for the whole group: the mark is made before this barrier, or after the next
+        // tile's first one
         ok = *failed == 0;
     }
-    if (!ok || *failed) atomicExch(a.err, 1);
+    if (!ok) {
+        mbar_wait(bar_w, 0);  // the weights' copies end before the CTA does
+        if (t == 0) net_failed(a.err, a.status);
+        if (!TRAIN) {
+            // the scores that this group owes, from the tile it gave up at
+            for (tile = (int64_t)grp * gridDim.x + blockIdx.x + max(done - 1, 0) * stride; tile < tiles; tile += stride) {
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    if (rk[mt] >= 0 && tile * K + rk[mt] < a.B) {
+                        a.score[(tile * K + rk[mt]) * n + rpos[mt]] = NAN;
+                        a.restart[tile * K + rk[mt]] = NAN;
+                    }
+            }
+        }
+    }
     if constexpr (TRAIN) {
         add_channels(sums + 3 * kC, lane, gw6);
 #pragma unroll
@@ -663,7 +710,9 @@ struct BwdShape {
     // 8-15 fall on G and their rows of the result are dropped), G, IN, IN one row up (its
     // first row lies 16 bytes before it)
     static constexpr int XC = 0, G = FIRST ? 8 * T::COL : 0, IN = G + T::ACT, GROUP = IN + 2 * T::ACT;
-    static constexpr int BAR = GROUPS + NG * GROUP, SUMS = BAR + 160;
+    // barriers, the TMEM slot, the CTA's mark (a part of it gave up), two marks per group
+    static constexpr int BAR = GROUPS + NG * GROUP, MARKS = BAR + 152, SUMS = BAR + 192;
+    static_assert(4 + 8 * NG <= SUMS - MARKS, "marks");
     static constexpr int SMEM = SUMS + kC * 4 + 128;
     static constexpr int ACC_W = 0, ACC_W1 = 256, ACC_D = FIRST ? 320 : 256;  // TMEM columns
     static constexpr int TMEM = 512;
@@ -701,7 +750,7 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
     auto wbar = [&](int g) { return bars + 40 * g + 16; };
     auto rbar = [&](int g) { return bars + 40 * g + 24; };
     auto fbar = [&](int g) { return bars + 40 * g + 32; };
-    volatile int* failed = reinterpret_cast<volatile int*>(sm + S::BAR + 152);
+    volatile int* failed = reinterpret_cast<volatile int*>(sm + S::MARKS);
     float* sums = reinterpret_cast<float*>(sm + S::SUMS);
     auto buf = [&](int g) { return sb + S::GROUPS + g * S::GROUP; };
     if (threadIdx.x < kC) sums[threadIdx.x] = 0.f;
@@ -709,8 +758,8 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
     for (int i = threadIdx.x; i < S::NG * S::GROUP / 16; i += S::THREADS)
         sts128(sb + S::GROUPS + 16 * i, make_uint4(0u, 0u, 0u, 0u));
     if (issuer) tmem_alloc(slot, S::TMEM);
+    if (threadIdx.x <= 2 * S::NG) failed[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
-        *failed = 0;
         mbar_init(bar_w, 1);
         for (int i = 0; i < 5 * S::NG; ++i) mbar_init(bars + 8 * i, 1);
         mbar_init_fence();
@@ -735,8 +784,14 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                 bulk_copy_g2s(b + S::XC + k * (T::COL - 16),
                               reinterpret_cast<const unsigned char*>(a.X0) + tile * T::COL, T::COL, f);
     };
+    int loads = 0;  // a group's first thread: its tiles' copies
     if (issuer) {
-        // the whole warp, with uniform values; one lane issues
+        // the whole warp, with uniform values; one lane issues.  Its waits are over, too, once a
+        // group has given up
+        auto wait = [&](uint32_t bar, uint32_t parity, int tries) {
+            return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, tries)) != 0;
+        };
+        uint32_t last = 0, last_parity = 0;  // the barrier of the last products, its phase
         const uint32_t el = elect_one(), u_sb = uniform(sb), u_tmem = uniform(tmem), u_bars = uniform(bars);
         bool fresh = true, fresh1 = true;
         if (el) {
@@ -746,11 +801,11 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                 if (tile_of(g, 0) < a.tiles) load(g, tile_of(g, 0));
         }
         __syncwarp();
-        bool ok = mbar_wait(bar_w, 0);
+        bool ok = wait(bar_w, 0, kTriesWeights);
         for (int it = 0; ok && tile_of(0, it) < a.tiles; ++it) {
             for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
                 const uint32_t b = u_sb + S::GROUPS + g * S::GROUP, br = u_bars + 40 * g;
-                ok = __all_sync(0xFFFFFFFFu, mbar_wait(br, it & 1));
+                ok = wait(br, it & 1, kTriesTiles);
                 if (!ok) break;
                 tc_fence_after();
 #pragma unroll
@@ -763,20 +818,39 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                     issue_wgrad<T::M, T::COL>(el, u_tmem + S::ACC_W + 64 * q, b + S::IN + 32 * q, b + S::G + 48, fresh);
                 fresh = false;
                 tc_commit(el, br + 16);
+                last = br + 16, last_parity = it & 1;
             }
             if (FIRST)
                 for (int g = 0; ok && g < S::NG && tile_of(g, it) < a.tiles; ++g) {
                     const uint32_t b = u_sb + S::GROUPS + g * S::GROUP, br = u_bars + 40 * g;
-                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(br + 24, it & 1));
+                    ok = wait(br + 24, it & 1, kTriesTiles);
                     if (!ok) break;
                     tc_fence_after();
                     issue_wgrad<T::M, T::COL>(el, u_tmem + S::ACC_W1, b + S::XC, b + S::G + 48, fresh1);
                     fresh1 = false;
                     tc_commit(el, br + 32);
+                    last = br + 32, last_parity = it & 1;
                 }
         }
-        if (!ok) *failed = 1;
+        if (!ok) {
+            *failed = 1;  // the groups' waits are over
+            // the copies and products under way end before the CTA does (a commit covers all before it)
+            mbar_wait(bar_w, 0);
+            if (last != 0u) mbar_wait(last, last_parity);
+        }
     } else {
+        // Marks: a thread makes the one of its iteration's parity before the group's barrier,
+        // all read it after the barrier, and the next iteration but one cannot make it before
+        // they have: the same for the whole group.  What the first thread waits for after the
+        // barrier (`late`) it tells in the next iteration.
+        bool late = false;
+        volatile int* const marks = failed + 1 + 2 * grp;
+        auto await = [&](uint32_t bar, uint32_t parity) {  // over, too, once the issuer or a group has given up
+            if (mbar_wait(bar, parity, kTriesProducts)) return true;
+            if (*failed == 0) mbar_wait(bar, parity);
+            return false;
+        };
+        if (t == 0 && tile_of(grp, 0) < a.tiles) loads = 1;  // (the issuer's)
         const int K = tile_samples(a.n);
         float2 gb = {0.f, 0.f};
         int rk[MT];
@@ -787,13 +861,13 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
         }
         for (int it = 0; tile_of(grp, it) < a.tiles; ++it) {
             const int64_t tile = tile_of(grp, it);
-            if (!mbar_wait(dbar(grp), it & 1)) *failed = 1;
+            if (late || !await(dbar(grp), it & 1)) marks[it & 1] = 1;
             tc_fence_after();
             unsigned char* const gout = FIRST ? nullptr : reinterpret_cast<unsigned char*>(a.dIN) + tile * T::ACT;
             if (!FIRST) zero_pad_rows<MT, 8>(gout, t);
             if (FIRST) {
                 // da1 takes G's place: the weight gradient has read it
-                if (!mbar_wait(wbar(grp), it & 1)) *failed = 1;
+                if (!late && !await(wbar(grp), it & 1)) marks[it & 1] = 1;
                 tc_fence_after();
             }
 #pragma unroll
@@ -826,27 +900,31 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
                 fence_async_shared();
                 tc_fence_before();
                 group_sync(1 + grp);
+                if (marks[it & 1]) break;
                 if (t == 0) {
                     mbar_arrive(rbar(grp));
-                    if (!mbar_wait(fbar(grp), it & 1)) *failed = 1;
-                    if (tile_of(grp, it + 1) < a.tiles && *failed == 0) {
+                    late = !await(fbar(grp), it & 1);
+                    if (tile_of(grp, it + 1) < a.tiles && !late) {
                         fence_async_shared();
                         load(grp, tile_of(grp, it + 1));
+                        ++loads;
                     }
                 }
             } else {
                 tc_fence_before();
                 group_sync(1 + grp);  // every row's mask has been read
+                if (marks[it & 1]) break;
                 if (t == 0) {
-                    if (!mbar_wait(wbar(grp), it & 1)) *failed = 1;
-                    if (tile_of(grp, it + 1) < a.tiles && *failed == 0) {
+                    late = !await(wbar(grp), it & 1);
+                    if (tile_of(grp, it + 1) < a.tiles && !late) {
                         fence_async_shared();
                         load(grp, tile_of(grp, it + 1));
+                        ++loads;
                     }
                 }
             }
-            if (*failed) break;
         }
+        if (late || marks[0] || marks[1]) *failed = 1;
         add_channels(sums, lane, gb);
     }
     __syncwarp();
@@ -854,7 +932,8 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
     __syncthreads();
     tc_fence_after();
     if (*failed) {
-        if (threadIdx.x == 0) atomicExch(a.err, 1);
+        if (loads > 0) mbar_wait(full(grp), (loads - 1) & 1);  // the tiles' copies end before the CTA does
+        if (threadIdx.x == 0) net_failed(a.err, nullptr);
     } else if (grp == 0) {
         // every product has completed: each group's last waits covered its own
         for (int q = 0; q < 4; ++q) {
@@ -890,13 +969,22 @@ __global__ void __launch_bounds__(BwdShape<MT, FIRST>::THREADS, 1) conv_backward
 // slices of the CTAs each.
 struct ReduceArgs {
     const float *p1, *p2, *p3, *p4;
-    int c23, c4;  // CTAs of the convolutions' partials, CTA groups of W4's
+    int c23, c4;  // CTAs of the convolutions' partials, accumulators of W4's
     float* grad;
+    float* loss;
+    const int* err;  // nonzero: a wait of the pass gave up, everything it returns is NaN
 };
 
 __global__ void __launch_bounds__(256) wgrad_reduce_kernel(ReduceArgs a)
 {
     __shared__ float4 sh[16][17];
+    const bool failed = *a.err != 0;
+    if (failed && blockIdx.x == 0) {
+        // the gradients that are added up elsewhere
+        for (int i = threadIdx.x; i < kParams; i += blockDim.x)
+            if (!(i < oB1 || (i >= oW2 && i < oB2) || (i >= oW3 && i < oB3) || (i >= oW4 && i < oB4))) a.grad[i] = NAN;
+        if (threadIdx.x == 0) *a.loss = NAN;
+    }
     const int col = threadIdx.x & 15, sl = threadIdx.x >> 4;
     // rows of 64 outputs: W2 448, W3 448, W1 64 (tap * 8 + channel), W4 64
     int row = blockIdx.x, ctas = a.c23, rows = kTaps * kC;
@@ -920,13 +1008,14 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(ReduceArgs a)
         const int o = threadIdx.x;
         float t = 0.f;
         for (int k = 0; k < 16; ++k) t += reinterpret_cast<const float*>(&sh[k][o >> 2])[o & 3];
+        if (failed) t = NAN;
         if (which == 4) {
             a.grad[oW4 + o * kC + row] = t;  // dW4[j][c]
         } else if (which == 1) {
             const int k = row >> 3, c = row & 7;
             if (k < kTaps) {
                 a.grad[oW1 + (o * kCin + c) * kTaps + k] = t;
-                a.grad[oW1 + (o * kCin + c + 8) * kTaps + k] = 0.f;  // channels 8-15 carry no input
+                a.grad[oW1 + (o * kCin + c + 8) * kTaps + k] = failed ? NAN : 0.f;  // channels 8-15 carry no input
             }
         } else {
             const int k = row / kC, c = row % kC;
@@ -935,10 +1024,11 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(ReduceArgs a)
     }
 }
 
-// Packed bf16 copies of the float32 master weights: element e of a layer's K x 64 operand is
+// Packed bf16 copies of the float32 master weights (and the pass's error word cleared): element e of a layer's K x 64 operand is
 // K index 8 (e / 512) + e % 8 of output (e / 8) % 64.
-__global__ void pack_kernel(const float* __restrict__ prm, bf16* __restrict__ wpk)
+__global__ void pack_kernel(const float* __restrict__ prm, bf16* __restrict__ wpk, int* __restrict__ err)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *err = 0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < kPacked; t += gridDim.x * blockDim.x) {
         float v;
         if (t < pWf2) {  // Wf1: K index k*16+c, W1[o][c][k]
@@ -1025,7 +1115,7 @@ __global__ void init_kernel(float* __restrict__ prm, uint64_t seed)
 struct NetWs {
     bf16 *X0, *A1, *A2, *dA3, *dA2, *wpk;
     float *score, *restart, *loss;
-    int* err;  // set by a tensor-core kernel whose copy or product wait gave up
+    int* err;  // cleared by pack_kernel, set by a tensor-core kernel whose wait gave up
     float *part1, *part2, *part3, *part4;  // per-CTA partial weight gradients
     size_t bytes;
 };
@@ -1124,15 +1214,17 @@ static FwdArgs forward_args(const float* prm, const float* x, const NetWs& w, in
 
 int pack(const float* prm, const NetWs& w, cudaStream_t s)
 {
-    pack_kernel<<<4 * sm_count(), 256, 0, s>>>(prm, w.wpk);
+    pack_kernel<<<4 * sm_count(), 256, 0, s>>>(prm, w.wpk, w.err);
     return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
 }
 
-int forward(const float* prm, const float* x, const NetWs& w, int64_t B, int n, float* score, float* restart, cudaStream_t s)
+int forward(const float* prm, const float* x, const NetWs& w, int64_t B, int n, float* score, float* restart, DevStatus* status,
+            cudaStream_t s)
 {
     int rc = pack(prm, w, s);
     if (rc) return rc;
-    const FwdArgs a = forward_args(prm, x, w, B, n, score, restart);
+    FwdArgs a = forward_args(prm, x, w, B, n, score, restart);
+    a.status = status;
     return n <= 128 ? launch_forward<1, false>(a, sm_count(), s) : launch_forward<2, false>(a, sm_count(), s);
 }
 
@@ -1154,7 +1246,7 @@ static int gradients_tiles(FwdArgs a, const NetWs& w, float* grad, int sms, cuda
     constexpr int NG = FwdShape<MT, true>::NG, ACC4 = FwdShape<MT, true>::ACC4;
     const int ctas = (int)std::min<int64_t>(tiles, sms), back = (int)std::min<int64_t>(tiles, kBwdCtas * sms);
     const ReduceArgs r{w.part1, w.part2, w.part3, w.part4, back, ctas * NG * (tiles > ctas * NG ? ACC4 : 1),
-                       grad};
+                       grad, a.loss, w.err};
     wgrad_reduce_kernel<<<2 * kTaps * kC + 128, 256, 0, s>>>(r);
     if (!rc && cudaGetLastError() != cudaSuccess) rc = LABS_ECUDA;
     return rc;
@@ -1205,10 +1297,10 @@ size_t net_workspace_bytes(int64_t B, int n)
 }
 
 int net_forward_ws(const float* params, const float* x, int64_t B, int n, void* ws, const float** scores,
-                   const float** restart, void* stream)
+                   const float** restart, DevStatus* status, void* stream)
 {
     const net::NetWs w = net::carve(ws, B, n);
-    const int rc = net::forward(params, x, w, B, n, w.score, w.restart, (cudaStream_t)stream);
+    const int rc = net::forward(params, x, w, B, n, w.score, w.restart, status, (cudaStream_t)stream);
     if (scores) *scores = w.score;
     if (restart) *restart = w.restart;
     return rc;
@@ -1245,7 +1337,7 @@ int labs_net_forward(const float* dev_params, const float* dev_x, int64_t batch,
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
     if (!net::aligned_ws(dev_ws)) return LABS_EINVAL;
     return net::forward(dev_params, dev_x, w, batch, n, dev_scores ? dev_scores : w.score,
-                        dev_restart ? dev_restart : w.restart, (cudaStream_t)cuda_stream);
+                        dev_restart ? dev_restart : w.restart, nullptr, (cudaStream_t)cuda_stream);
 }
 
 int labs_net_gradients(const float* dev_params, const float* dev_x, const int32_t* dev_target, const float* dev_y,
