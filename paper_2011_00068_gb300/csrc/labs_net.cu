@@ -1117,6 +1117,7 @@ struct NetWs {
     float *score, *restart, *loss;
     int* err;  // cleared by pack_kernel, set by a tensor-core kernel whose wait gave up
     float *part1, *part2, *part3, *part4;  // per-CTA partial weight gradients
+    float* grad;  // gradients of a pass whose result overlaps its inputs
     size_t bytes;
 };
 
@@ -1129,6 +1130,22 @@ static size_t align256(size_t x)
 static bool aligned_ws(const void* ws)
 {
     return ((uintptr_t)ws & 15) == 0;
+}
+
+// Memory that a pass reads while it writes its results: a result that overlaps some of it (in
+// place of an input, say) goes to the workspace first and is copied at the end.
+struct Span {
+    const void* p;
+    size_t bytes;
+};
+
+template <int N>
+static bool apart(const void* out, size_t bytes, const Span (&in)[N])
+{
+    const uintptr_t a = (uintptr_t)out;
+    bool ok = out != nullptr;
+    for (const Span& s : in) ok = ok && (a + bytes <= (uintptr_t)s.p || (uintptr_t)s.p + s.bytes <= a);
+    return ok;
 }
 
 static int sm_count()
@@ -1164,6 +1181,7 @@ NetWs carve(void* base, int64_t B, int n)
     w.part2 = (float*)take(kBwdCtas * sms * kTaps * kC * kC * 4);
     w.part3 = (float*)take(kBwdCtas * sms * kTaps * kC * kC * 4);
     w.part4 = (float*)take(sms * 2 * kC * kC * 4);
+    w.grad = (float*)take(kParams * 4);
     w.bytes = off;
     return w;
 }
@@ -1336,8 +1354,17 @@ int labs_net_forward(const float* dev_params, const float* dev_x, int64_t batch,
     const net::NetWs w = net::carve(dev_ws, batch, n);
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
     if (!net::aligned_ws(dev_ws)) return LABS_EINVAL;
-    return net::forward(dev_params, dev_x, w, batch, n, dev_scores ? dev_scores : w.score,
-                        dev_restart ? dev_restart : w.restart, nullptr, (cudaStream_t)cuda_stream);
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    const size_t sb = (size_t)batch * n * 4, rb = (size_t)batch * 4;
+    const net::Span in[] = {{dev_params, net::kParams * 4}, {dev_x, 3 * sb}, {dev_ws, ws_bytes}};
+    float* const score = net::apart(dev_scores, sb, in) ? dev_scores : w.score;
+    float* const restart = net::apart(dev_restart, rb, in) ? dev_restart : w.restart;
+    int rc = net::forward(dev_params, dev_x, w, batch, n, score, restart, nullptr, s);
+    if (!rc && dev_scores && score != dev_scores)
+        rc = cudaMemcpyAsync(dev_scores, score, sb, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
+    if (!rc && dev_restart && restart != dev_restart)
+        rc = cudaMemcpyAsync(dev_restart, restart, rb, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
+    return rc;
 }
 
 int labs_net_gradients(const float* dev_params, const float* dev_x, const int32_t* dev_target, const float* dev_y,
@@ -1352,7 +1379,12 @@ int labs_net_gradients(const float* dev_params, const float* dev_x, const int32_
     if (!dev_ws || ws_bytes < w.bytes) return LABS_ENOMEM;
     if (!net::aligned_ws(dev_ws)) return LABS_EINVAL;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    int rc = net::gradients(dev_params, dev_x, w, dev_target, dev_y, dev_wf, dev_grads, batch, n, s);
+    const size_t gb = net::kParams * 4, rb = (size_t)batch * 4;
+    const net::Span in[] = {{dev_params, gb}, {dev_x, 3 * n * rb}, {dev_target, rb}, {dev_y, rb}, {dev_wf, rb}};
+    float* const grad = net::apart(dev_grads, gb, in) ? dev_grads : w.grad;
+    int rc = net::gradients(dev_params, dev_x, w, dev_target, dev_y, dev_wf, grad, batch, n, s);
+    if (!rc && grad != dev_grads)
+        rc = cudaMemcpyAsync(dev_grads, grad, gb, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
     if (!rc && dev_loss) rc = cudaMemcpyAsync(dev_loss, w.loss, 4, cudaMemcpyDeviceToDevice, s) ? LABS_ECUDA : 0;
     return rc;
 }
