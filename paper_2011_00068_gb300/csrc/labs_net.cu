@@ -1160,6 +1160,9 @@ NetWs carve(void* base, int64_t B, int n)
 {
     NetWs w;
     const size_t tiles = (size_t)tile_count(B, n), col = (size_t)(tile_rows(n) + 9) * 16, sms = (size_t)sm_count();
+    // the CTAs that write partial sums: a small batch has fewer than the GPU could run (80 MB of
+    // partials for all of them, 1 MB for one state)
+    const size_t fwd = std::min(tiles, sms), bwd = std::min(tiles, kBwdCtas * sms);
     char* p = static_cast<char*>(base);
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -1177,10 +1180,10 @@ NetWs carve(void* base, int64_t B, int n)
     w.restart = (float*)take((size_t)B * 4);
     w.loss = (float*)take(4);
     w.err = (int*)take(4);
-    w.part1 = (float*)take(kBwdCtas * sms * 64 * kC * 4);
-    w.part2 = (float*)take(kBwdCtas * sms * kTaps * kC * kC * 4);
-    w.part3 = (float*)take(kBwdCtas * sms * kTaps * kC * kC * 4);
-    w.part4 = (float*)take(sms * 2 * kC * kC * 4);
+    w.part1 = (float*)take(bwd * 64 * kC * 4);
+    w.part2 = (float*)take(bwd * kTaps * kC * kC * 4);
+    w.part3 = (float*)take(bwd * kTaps * kC * kC * 4);
+    w.part4 = (float*)take(fwd * 2 * kC * kC * 4);
     w.grad = (float*)take(kParams * 4);
     w.bytes = off;
     return w;

@@ -53,6 +53,21 @@ def test_unaligned_learned_workspace_is_refused(flags):
     s.close()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [2, 41, 101, 128, 152, 256])
+def test_small_batches_need_small_workspaces(n):
+    """A batch's workspace holds what its own tiles use (a few MB for one state, where the
+    partial sums of every CTA that the GPU could run take 80 MB), and never shrinks with the
+    batch, so that one sized for the largest batch serves all."""
+    sizes = []
+    for B in (1, 2, 8, 64, 151, 152, 153, 303, 304, 305, 1000, 4096, 8192):
+        nbytes = ctypes.c_size_t()
+        assert labs.library().labs_net_sizes(n, B, None, ctypes.byref(nbytes)) == 0
+        sizes.append(nbytes.value)
+    assert sizes[0] < 2 << 20 and sizes[2] < 12 << 20
+    assert sizes == sorted(sizes)
+
+
 def _param_count():
     k = ctypes.c_size_t()
     assert labs.library().labs_net_sizes(21, 1, ctypes.byref(k), None) == 0
