@@ -9,15 +9,22 @@ namespace labsgpu {
 // contexts, lengths and host threads share a kernel and ask for different sizes.  So the limit
 // is always set to what the device allows, never to one launch's need, which another thread's
 // smaller one could replace between that call and the launch.
-inline cudaError_t allow_shared(const void* fn, cudaFuncAttributes* attributes = nullptr)
+// static_bytes: the kernel's own shared arrays.
+inline cudaError_t allow_shared(const void* fn, int static_bytes)
 {
     int dev = 0, most = 0;
-    cudaFuncAttributes fa;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - static_bytes);
+    return e;
+}
+
+// The same with the kernel's attributes asked for (about 1 us more).
+inline cudaError_t allow_shared(const void* fn, cudaFuncAttributes* attributes = nullptr)
+{
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess) e = allow_shared(fn, (int)fa.sharedSizeBytes);
     if (attributes != nullptr) *attributes = fa;
     return e;
 }

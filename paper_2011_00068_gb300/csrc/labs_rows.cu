@@ -471,6 +471,20 @@ __global__ void __launch_bounds__(256, row_ctas<LG, R>())
 using RowsFn = void (*)(const int8_t*, int64_t, int, int32_t*, DevStatus*);
 using FeaturesFn = void (*)(const uint32_t*, int64_t, int64_t, int, float*);
 
+// A kernel and the shared memory of one of its warps' rows.  (The layout is a loop over all
+// lengths: worked out in every call instead of by the compiler it took 1.5 us of a 4 us call.)
+template <class Fn>
+struct RowKernel {
+    Fn fn = nullptr;
+    size_t warp_bytes = 0;
+};
+template <class LG, int R>
+constexpr size_t row_warp_bytes()
+{
+    constexpr StepSmem SL = step_smem(LG::kSize, R);
+    return (size_t)(32 / LG::kSize) * SL.words * sizeof(int);
+}
+
 // (lane block, words per class) of every length: step_R(n, lanes per row), ceil(n/32)
 #define LABS_ROW_CASES(CASE)                                                                                       \
     CASE(Pair, 1, 1) CASE(Pair, 2, 1) CASE(Pair, 3, 2) CASE(Pair, 5, 2) CASE(Pair, 5, 3) CASE(Pair, 6, 3)          \
@@ -478,25 +492,25 @@ using FeaturesFn = void (*)(const uint32_t*, int64_t, int64_t, int, float*);
     CASE(Tile<32>, 9, 8)
 
 template <bool STAGED>
-RowsFn rows_fn(int key)
+RowKernel<RowsFn> rows_fn(int key)
 {
     switch (key) {
 #define LABS_ROW_CASE(LG, R, NW) \
-    case 16 * R + NW: return rows_kernel<LG, R, NW, STAGED>;
+    case 16 * R + NW: return {rows_kernel<LG, R, NW, STAGED>, row_warp_bytes<LG, R>()};
         LABS_ROW_CASES(LABS_ROW_CASE)
 #undef LABS_ROW_CASE
-        default: return nullptr;
+        default: return {};
     }
 }
 
-FeaturesFn features_fn(int key)
+RowKernel<FeaturesFn> features_fn(int key)
 {
     switch (key) {
 #define LABS_ROW_CASE(LG, R, NW) \
-    case 16 * R + NW: return features_kernel<LG, R, NW>;
+    case 16 * R + NW: return {features_kernel<LG, R, NW>, row_warp_bytes<LG, R>()};
         LABS_ROW_CASES(LABS_ROW_CASE)
 #undef LABS_ROW_CASE
-        default: return nullptr;
+        default: return {};
     }
 }
 
@@ -521,7 +535,10 @@ int launch_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, Dev
     const int n = (L + 1) / 2, tile = n <= 160 ? 16 : 32, rows = 32 / tile, R = step_R(n, tile);
     const int64_t units = (batch + rows - 1) / rows;
     const int warps = row_warps(units, sms);
-    const size_t warp_bytes = (size_t)rows * step_smem(tile, R).words * sizeof(int);
+    const int key = 16 * R + (n + 31) / 32;
+    const RowKernel<RowsFn> plain = rows_fn<false>(key);
+    if (plain.fn == nullptr) return LABS_EINVAL;
+    const size_t warp_bytes = plain.warp_bytes;
     const size_t stage = 2 * (size_t)stage_bytes(L, rows) + 16;
     // staged rows need a 16-byte aligned input, and are used where they keep as many CTAs
     // of eight warps on an SM as the rows alone (three, two with lane blocks 9 and 10)
@@ -529,11 +546,9 @@ int launch_delta(const int8_t* seqs, int64_t batch, int32_t L, int32_t* out, Dev
     const size_t cap = tile == 32 || R <= 7 ? 3 : 2;  // the kernels' launch bounds
     const bool staged = ((uintptr_t)seqs & 15) == 0 &&
                         std::min(cap, sm_bytes / (warp_bytes + stage)) >= std::min(cap, sm_bytes / warp_bytes);
-    const int key = 16 * R + (n + 31) / 32;
-    const RowsFn fn = staged ? rows_fn<true>(key) : rows_fn<false>(key);
-    if (fn == nullptr) return LABS_EINVAL;
+    const RowsFn fn = staged ? rows_fn<true>(key).fn : plain.fn;
     const size_t smem = warps * (warp_bytes + (staged ? stage : 0));
-    if (smem > 48 * 1024 && allow_shared((const void*)fn) != cudaSuccess) return LABS_ECUDA;
+    if (smem > 48 * 1024 && allow_shared((const void*)fn, 0) != cudaSuccess) return LABS_ECUDA;
     // more CTAs than fit at once (up to 8 per SM): measured faster than one resident wave
     const int64_t need = (units + warps - 1) / warps, most = (int64_t)sms * 8;
     fn<<<(int)std::min(need, most), warps * kWarp, smem, (cudaStream_t)stream>>>(seqs, batch, L, out, status);
@@ -547,12 +562,12 @@ int launch_features(const uint32_t* bits, int64_t stride, int64_t count, int32_t
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int n = (L + 1) / 2, tile = n <= 160 ? 16 : 32, rows = 32 / tile, R = step_R(n, tile);
-    const FeaturesFn fn = features_fn(16 * R + (n + 31) / 32);
+    const auto [fn, warp_bytes] = features_fn(16 * R + (n + 31) / 32);
     if (fn == nullptr) return LABS_EINVAL;
     const int64_t units = (count + rows - 1) / rows;
     const int warps = row_warps(units, sms);
-    const size_t smem = (size_t)warps * rows * step_smem(tile, R).words * sizeof(int);
-    if (smem > 48 * 1024 && allow_shared((const void*)fn) != cudaSuccess) return LABS_ECUDA;
+    const size_t smem = warps * warp_bytes;
+    if (smem > 48 * 1024 && allow_shared((const void*)fn, 0) != cudaSuccess) return LABS_ECUDA;
     const int64_t need = (units + warps - 1) / warps, most = (int64_t)sms * 8;
     fn<<<(int)std::min(need, most), warps * kWarp, smem, (cudaStream_t)stream>>>(bits, stride, count, L, x);
     return cudaGetLastError() == cudaSuccess ? LABS_OK : LABS_ECUDA;
