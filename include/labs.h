@@ -206,7 +206,8 @@ int labs_neighbor_delta(labs_ctx *ctx, const int8_t *dev_seqs, int64_t batch,
                         int32_t *dev_delta_out);
 
 /* Advances every walker by `steps` steps of the walk (Algorithm 1, self-avoiding
- * form; the step rule is stated here and implemented in csrc/labs_device.cuh):
+ * form; the step rule is stated here and implemented in csrc/labs_step.cuh, for long
+ * lengths in csrc/labs_long.cu):
  *   evaluate all n flips; take the flip with the lowest dISL whose result is not in
  *   the walker's HT (ties to the lowest i); move there and insert it into HT; keep
  *   the best sequence (strictly lower ISL); restart from a new random sequence with

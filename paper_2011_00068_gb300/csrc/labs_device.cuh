@@ -1511,7 +1511,7 @@ __device__ __noinline__ void psl_ring(const View& V, int n, const Outs<TL, R>& o
 
 // All R outputs of the lane: one ring pass up to R = 6; wider lane blocks, whose three
 // rings of 3R - 2 entries would not fit the registers, take the compare-and-select form
-// at R = 7 (measured 2% faster there, two walkers per warp at L = 201) and two ring
+// at R = 7 (2% faster there when a walk of two per warp had that lane block) and two ring
 // passes of (R+1)/2 and R - (R+1)/2 outputs from R = 9 (each pass reloads its rings:
 // about twice the shared loads of one pass, but three instructions per lag term instead
 // of a compare and select per term; 21-40% faster for the long lane blocks 9 and 11).

@@ -117,8 +117,9 @@ struct Control {
 // looks all of them up at a step's start (walk_lockstep).  Microseconds a step with and
 // without: 64 walkers of L = 41 0.97 / 1.22, of L = 201 1.01 / 1.21, of L = 501 (16064 slots)
 // 1.24 / 1.36; 300 of L = 151 (22800) 1.72 / 1.67, 300 of L = 201 (30300) 1.39 / 1.48, 300 of
-// L = 501 (75300) 2.14 / 1.60, 2432 of L = 201 4.8 / 1.68: past the line the loads fill the
-// path to L2 and HBM.
+// L = 501 (75300) 2.14 / 1.60, 2432 of L = 201 4.8 / 1.68: with many walkers the loads fill the
+// path to L2 and HBM.  The slots do not order the cases between 2^14 and 2^15 (four walkers per
+// warp lose where two still gain): the line lies below the first loss that was measured.
 constexpr int64_t kAheadSlots = 1 << 14;
 
 struct KParams {
@@ -415,7 +416,7 @@ __host__ __device__ constexpr StepSmem step_smem(int tile, int R, bool psl = fal
 }
 
 // Layout of one row of an FP32 or converted-table row evaluation (no kernel has it any more:
-// labs_rows.cu takes step_smem; its bounds test remains), `tile` lanes per
+// labs_rows.cu takes step_smem; kept for the bounds test that includes it), `tile` lanes per
 // row with lane block R = block_R(n_max, tile) (v0 <= (tile/2 - 1) R):
 //   A rows: the Toeplitz loop reads A_p[0 .. round8(n)) (zero beyond the class), the
 //     assembly A_p[v], A_p[n-1-p-v] and A_p[3v+p-n+1] for every lane output v (down to

@@ -1,7 +1,8 @@
 // labs_kernels.cu -- sm_103a kernels of the skew-symmetric LABS search
-// (Brest & Boskovic, arXiv 2011.00068): walker starts, the stateless row kernels
-// (ISL, neighbourhood), learned-proposal support, reductions and the launchers.
-// The walk itself is in labs_device.cuh, instantiated by the labs_walk*.cu units.
+// (Brest & Boskovic, arXiv 2011.00068): walker starts, the ISL of rows, learned-proposal
+// support, reductions and the launchers.  The walks themselves are in labs_step.cuh (the
+// learned mode's in labs_device.cuh), instantiated by the labs_walk*.cu units, and in
+// labs_long.cu; the row neighbourhoods and the network's inputs in labs_rows.cu.
 #include <algorithm>
 
 #include "labs_device.cuh"

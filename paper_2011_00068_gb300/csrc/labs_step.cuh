@@ -304,7 +304,7 @@ struct StepProduct {
 };
 
 // X_v for all outputs of the warp's W walkers into their scratch: the block-diagonal sum
-// of toeplitz_tc (labs_device.cuh), with the table kept as FP16 pairs G[y] = (E[y],
+// of toeplitz_tc1 (labs_device.cuh), with the table kept as FP16 pairs G[y] = (E[y],
 // E[y+1]) (one 4-byte load per operand register, no conversion) and the row blocks of
 // two (walker, column group) operands loaded by one ldmatrix per diagonal.
 template <class LAY, class LG, int R>

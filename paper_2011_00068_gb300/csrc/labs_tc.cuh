@@ -1,7 +1,7 @@
 // labs_tc.cuh -- 5th-generation tensor cores on sm_103a as inline PTX: tensor memory
 // (TMEM) allocation, tcgen05.mma with BF16 operands in shared memory and an FP32
-// accumulator in TMEM, tcgen05.ld of the accumulator, and two-dimensional tiled TMA loads
-// (cp.async.bulk.tensor) that stage the operands.  Used by the network's GEMMs.
+// accumulator in TMEM and tcgen05.ld of the accumulator.  Used by the network's products, whose
+// operands come by bulk copies (labs_async.cuh).
 //
 // Operand layouts in shared memory, without swizzling; a core matrix is 8 rows of 16
 // bytes stored contiguously (128 bytes).
@@ -16,8 +16,6 @@
 //    along K (the next 8 rows) and the stride byte offset `sbo` along M (N); the same
 //    staged columns serve, with lbo = 128 and sbo = one column.
 #pragma once
-
-#include <cuda.h>
 
 #include <cstdint>
 
@@ -129,17 +127,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 __device__ __forceinline__ void tc_wait_ld()
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Tile (x, y) of a two-dimensional tensor map into shared memory at dst, counted on
-// barrier bar; coordinates outside the tensor read zeros.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-            "r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
 }
 
 }  // namespace labsgpu
