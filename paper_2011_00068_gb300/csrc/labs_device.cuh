@@ -669,6 +669,55 @@ __device__ __forceinline__ void toeplitz_long(const View& V, const WarpSmem& SL,
     }
 }
 
+// The product of a walker that a CTA of four warps owns with no more column groups than warps:
+// a warp takes one group, its even and odd diagonals as the two chains (toeplitz_tc1's form),
+// and no sums meet; the pieces of toeplitz_long are too short there for its ring.  608 walkers x
+// 256 steps of L = 513 / 769 / 897 0.881 / 1.065 / 1.122 ms like this and 0.911 / 1.079 / 1.106
+// with toeplitz_long, best-first x 128 2.21 / 2.75 / 2.84 and 2.25 / 2.80 / 2.85: the line lies
+// between the last two.  (The PSL walk, on eight warps there, keeps toeplitz_long: 3.61 ms at
+// L = 513, 3.65 like this.)
+constexpr int kGroupsMaxN = 400;
+template <class LB, int R>
+__device__ __forceinline__ void toeplitz_groups(const View& V, const WarpSmem& SL, int n, const Outs<LB, R>& o,
+                                                const LB& t, float (&X)[R])
+{
+    const int m = threadIdx.x >> 5, l = threadIdx.x & 31, g = l >> 2, tq = l & 3;
+    const int S = (n + 15) >> 4, T = (((n + 1) >> 1) + 15) >> 4, M = (T + 3) >> 2;
+    const int pb = g >> 2, tb = g & 3, px = tq >> 1, tx = 2 * (tq & 1);
+    int* const base = reinterpret_cast<int*>(V.A0) - SL.apad;
+    float* const xf = reinterpret_cast<float*>(base + SL.roff);
+    if (m < M) {
+        const int dlo = -min(4 * m + 3, T - 1), nd = S - 4 * m - dlo;  // d = dlo .. S-1-4m
+        const float2* gy = V.G + (2 * tq - g) + 16 * dlo;
+        const uint32_t* ab = reinterpret_cast<const uint32_t*>(base + SL.hoff + pb * SL.hlen) + (SL.hpad >> 1) +
+                             8 * (tb + 4 * m + dlo) + tq;
+        float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t am = half2_bits(gy[-8]);
+        int k = 0;
+        for (; k + 1 < nd; k += 2) {
+            tc_diag(d0, gy, ab, am);
+            tc_diag(d1, gy + 16, ab + 8, am);
+            gy += 32;
+            ab += 16;
+        }
+        if (k < nd) tc_diag(d0, gy, ab, am);
+        float* const xs = xf + px * SL.xp + g;
+        const int t0 = tx + 4 * m;
+        if (t0 < T) {
+            xs[16 * t0] = d0[0] + d1[0];
+            xs[16 * t0 + 8] = d0[2] + d1[2];
+        }
+        if (t0 + 1 < T) {
+            xs[16 * t0 + 16] = d0[1] + d1[1];
+            xs[16 * t0 + 24] = d0[3] + d1[3];
+        }
+    }
+    t.sync();
+    const float* const xr = xf + o.p * SL.xp + o.v0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) X[r] = xr[r];
+}
+
 // The Toeplitz product of a lane group that owns one walker: on the tensor cores when
 // the layout holds the FP16 rows and the results' scratch (and the table's entries are
 // FP16 numbers), else on the FP32 pipes.
@@ -678,6 +727,13 @@ __device__ __forceinline__ void toeplitz_one(const View& V, const WarpSmem& SL, 
 {
     if constexpr (LG::kSize > 32) {
         if (SL.xp != 0 && *V.wide == 0) {
+            // (lane blocks that such a length can have; a context of longer ones takes the other)
+            if constexpr (LG::kSize == 128 && R <= 5) {
+                if (n <= kGroupsMaxN) {
+                    toeplitz_groups(V, SL, n, o, t, X);
+                    return;
+                }
+            }
             toeplitz_long(V, SL, n, o, t, X);
             return;
         }

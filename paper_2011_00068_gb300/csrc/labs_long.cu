@@ -108,15 +108,16 @@ struct LongWalk {
     int isl_limit;    // exact-range bound of the ISL (long_isl_limit)
 };
 
-// Zeroes rows, table and bit vectors (everything below the scratch and the bits).
-template <class LB>
+// Zeroes rows, table and bit vectors (everything below the scratch and the bits), the mark of a
+// table that FP16 does not hold and, unless SUMS is false, the product's sums (every product
+// leaves them zero).
+template <bool SUMS = true, class LB>
 __device__ __forceinline__ void long_clear(int* base, const WarpSmem& SL, const LB& t)
 {
     int4* b4 = reinterpret_cast<int4*>(base);
     for (int i = t.lane; i < SL.xoff / 4; i += LB::kSize) b4[i] = make_int4(0, 0, 0, 0);
-    // the product's sums, and the mark of a table that FP16 does not hold
     if (SL.xp != 0)
-        for (int i = SL.roff / 4 + t.lane; i <= SL.foff / 4; i += LB::kSize) b4[i] = make_int4(0, 0, 0, 0);
+        for (int i = (SUMS ? SL.roff : SL.foff) / 4 + t.lane; i <= SL.foff / 4; i += LB::kSize) b4[i] = make_int4(0, 0, 0, 0);
     t.sync();
 }
 
@@ -1014,9 +1015,10 @@ __global__ void __launch_bounds__(NT, kLongThreads / NT) long_delta_kernel(const
     const LB t(threadIdx.x, smem + SL.xoff);
     const View V = make_view(smem, SL);
     const Outs<LB, R> o(t);
+    long_clear(smem, SL, t);
     for (int64_t row = blockIdx.x; row < batch; row += gridDim.x) {
         const int8_t* src = seqs + row * (int64_t)L;
-        long_clear(smem, SL, t);
+        long_clear<false>(smem, SL, t);
         bool ok = true;
         for (int j = t.lane; j < L; j += LB::kSize) {
             const int v = src[j];
